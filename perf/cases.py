@@ -259,3 +259,80 @@ def tolerance(case):
     if kind == "layer" and case["out"] == "fp32":
         return {"rel": 1e-6, "max": 1e-5}   # seen 8.6e-8 / 4.0e-7 at K <= 4736; grows with K
     return {"rel": 1.6e-4, "max": 0.016}    # seen 4.7e-5 / 7.8e-3: one BF16 step where the FP32 sums round apart
+
+
+# ---- the same in 64 bits ---------------------------------------------------------------------------
+# Every FP8 operand, code and scale is decided by single FP32 operations that torch performs alike;
+# the products, sums and output scales below are float64, the outputs unrounded.
+def _e4m3(v):
+    return v.clamp(-448.0, 448.0).to(torch.float8_e4m3fn).to(torch.float32)
+
+
+def _pow2_ceil(s):
+    m, e = torch.frexp(s)
+    return torch.where(m == 0.5, s, torch.ldexp(torch.ones_like(s), e))
+
+
+def _exact_weight(g, N, K, weights, per_channel):
+    """The float64 weights that inference multiplies with: FP8 values times their weight scale."""
+    W = torch.randn((N, K), generator=g, device="cuda") * 0.02
+    amax = W.abs().amax(dim=1, keepdim=True) if per_channel else W.abs().max().reshape(1, 1)
+    s_w = amax / torch.full_like(amax, 448.0)
+    w8 = _e4m3(W / s_w).view(N, K // 128, 128)
+    del W
+    if weights == "signmag":
+        a = w8.abs().amax(dim=2, keepdim=True)
+        s = (a / torch.full_like(a, 7.0)).bfloat16().float()
+        q = (w8 / s).round().clamp(-7.0, 7.0)
+    else:
+        lo, hi = w8.amin(dim=2, keepdim=True).clamp(max=0.0), w8.amax(dim=2, keepdim=True).clamp(min=0.0)
+        s = ((hi - lo) / torch.full_like(hi, 15.0)).bfloat16().float()
+        z = (-lo / s).round().clamp(0.0, 15.0)
+        q = (w8 / s + z).round().clamp(0.0, 15.0) - z
+    return _e4m3(q * s).view(N, K).double() * s_w.double()
+
+
+def _exact_linear(x, w, scale="exact"):
+    x = x.float()
+    amax = x.abs().amax(dim=1, keepdim=True)
+    top = torch.full_like(amax, 448.0)
+    s = amax / top
+    inv = top / amax
+    if scale == "pow2":
+        s = _pow2_ceil(s)
+        inv = torch.ones_like(s) / s
+    return (_e4m3(x * inv).double() @ w.T).mul_(s.double())
+
+
+def exact(case, seed):
+    g = _gen(seed)
+    kind = case["kind"]
+    if kind == "layer":
+        x = _activation(g, case["M"], case["K"])
+        return _exact_linear(x, _exact_weight(g, case["N"], case["K"], case["weights"], case["per_channel"]),
+                             case["scale"])
+    if kind == "block":
+        out = {}
+        for name, N, K in _block_shapes(case):
+            x = _activation(g, case["M"], K)
+            out[name] = _exact_linear(x, _exact_weight(g, N, K, case["weights"], case["per_channel"]))
+        return out
+    if kind == "chain":
+        out = []
+        for i in range(case["count"]):
+            M = (case["M0"], case["M1"], case["M2"])[i % 3]
+            w = _exact_weight(g, case["N"], case["K"], case["weights"], False)
+            out.append(_exact_linear(_activation(g, M, case["K"]), w))
+        return out
+    if kind == "chain_mlp":
+        M, h, f = case["M"], case["hidden"], case["ffn"]
+        w = _exact_weight(g, 2 * f, h, case["weights"], False)
+        gate_up = _exact_linear(_activation(g, M, h), w)
+        w = _exact_weight(g, h, f, case["weights"], False)
+        stored = gate_up.bfloat16().double()          # what the second layer reads is BF16 by definition
+        act = (stored[:, :f] * torch.sigmoid(stored[:, :f]) * stored[:, f:]).bfloat16()
+        return [gate_up, _exact_linear(act, w)]
+    if kind == "hessian":
+        x = _activation(g, case["T"], case["K"]).double()
+        return x.T @ x
+    return None                                       # the quantizer: whole numbers
