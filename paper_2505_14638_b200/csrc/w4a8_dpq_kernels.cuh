@@ -309,8 +309,8 @@ dpq_trailing_kernel(float* __restrict__ work, const float* __restrict__ U, const
 
 // ---------------------------------------------------------------------------------------------
 // The layer Hessian of the quantizer (Sec. 3.1; Sec. 3.3 for its preparation): H = X^T X over the
-// calibration tokens.  A plain FP32 contraction on the FMA pipes, for the X that TMA cannot read (rows
-// that are not 16-byte aligned, fewer than 64 features); every other X takes hessian_umma_kernel.
+// calibration tokens.  A plain FP32 contraction on the FMA pipes -- an offline step whose sums
+// decide nothing bit-exactly (the factorization that follows is a library matter in float64).
 // One CTA per 64 x 64 tile of the upper triangle (tiles below the diagonal are mirrored on the
 // way out); 256 threads, 4 x 4 outputs each; the token dimension in slabs of 32 rows staged in
 // shared memory as fp32.

@@ -9,7 +9,6 @@
 
 #include "../../include/w4a8.h"
 #include "w4a8_dpq_kernels.cuh"
-#include "w4a8_hessian_umma.cuh"
 #include "w4a8_linear_chain.cuh"
 #include "w4a8_linear_splitn.cuh"
 #include "w4a8_linear_pair.cuh"
@@ -629,28 +628,6 @@ static int launch_cluster_kcut(const uint8_t* x8, int64_t ldx8, const uint8_t* w
     pl.counter_bytes = 0;
     pl.workspace_bytes = 0;
     return launch_streamk<Cfg>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, nullptr, pl, M, N, K, st, nullptr, cl);
-}
-
-template <int TOK>
-static int launch_hessian_umma(const void* x, int64_t T, int64_t K, int64_t ldx, float* H, int accumulate,
-                               cudaStream_t st) {
-    using Cfg = HessCfg<TOK>;
-    auto kern = hessian_umma_kernel<TOK>;
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [&] {
-        attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes);
-    });
-    if (attr_err != cudaSuccess) return W4A8_ERR_CUDA;
-    unsigned int* status = status_word_ptr();
-    CUtensorMap tx;
-    if (!status || !make_tmap_u8_2d(&tx, x, (uint64_t)T, (uint64_t)(2 * K), (uint64_t)(2 * ldx), 128, (uint32_t)TOK,
-                                    CU_TENSOR_MAP_SWIZZLE_128B))
-        return W4A8_ERR_CUDA;
-    const int64_t nt = (K + Cfg::TILE - 1) / Cfg::TILE;
-    kern<<<(unsigned)(nt * (nt + 1) / 2), Cfg::kThreads, Cfg::kSmemBytes, st>>>(tx, T, K, H, accumulate ? 1 : 0, status);
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return launch_status();
 }
 
 static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* wpp,
@@ -1565,14 +1542,6 @@ int w4a8_hessian_accumulate(const void* x_bf16, int64_t T, int64_t K, int64_t ld
     if ((reinterpret_cast<uintptr_t>(x_bf16) & 1u) || (reinterpret_cast<uintptr_t>(H) & 3u)) return W4A8_ERR_BAD_ALIGNMENT;
     int rc = check_device();
     if (rc != W4A8_OK) return rc;
-    // The tensor-core kernel where TMA can read X (16-byte base and row pitch, at least half a tile of
-    // features): (T, K) = (1024, 4096) 34 us against 796 us for the FP32 kernel, (129, 1096) 11 against 28,
-    // (63, 72) 10 against 11.  BF16 rows of any other alignment and narrower X take the FP32 kernel.
-    // Up to 192 tokens the chunks are of 32 tokens instead of 64: at that length the FP32 chain is still
-    // more exact than 64-token chunks (2-norm error at T = 129: 8.9e-8, 64-token chunks 9.7e-8, 32-token 7.2e-8).
-    if (aligned16(x_bf16) && ldx % 8 == 0 && K >= 64 && T <= INT32_MAX - 64)
-        return T <= 192 ? launch_hessian_umma<32>(x_bf16, T, K, ldx, H, accumulate, static_cast<cudaStream_t>(stream))
-                        : launch_hessian_umma<64>(x_bf16, T, K, ldx, H, accumulate, static_cast<cudaStream_t>(stream));
     const int64_t nb = (K + kHessTile - 1) / kHessTile;
     hessian_xtx_kernel<<<(unsigned)(nb * (nb + 1) / 2), 256, 0, static_cast<cudaStream_t>(stream)>>>(
         static_cast<const uint16_t*>(x_bf16), T, K, ldx, H, accumulate ? 1.0f : 0.0f);

@@ -165,32 +165,3 @@ def test_quantizer_pipeline_from_activations_through_the_c_abi():
         D = (W - w8).double()
         return float(torch.einsum("nk,kj,nj->", D, H.double(), D))
     assert out_err(cq) <= 0.8 * out_err(rq)
-
-
-@pytest.mark.parametrize("T,K,pitch,offset", [
-    (1, 64, 64, 0), (31, 72, 80, 0), (33, 128, 128, 8), (64, 136, 144, 0), (65, 248, 256, 0), (192, 256, 256, 0),
-    (193, 264, 264, 0), (500, 392, 400, 16), (700, 127, 128, 0),
-    (65, 129, 131, 0), (65, 136, 136, 3), (40, 63, 64, 0)])   # the last three: not for the tensor-core kernel
-def test_hessian_at_tile_edges(T, K, pitch, offset):
-    # Tiles of 128 features, stages of 32 tokens (T <= 192) or 64; rows inside a wider buffer whose surroundings are
-    # NaN.  Bound: every MMA (16 products) and every chunk adds one rounding of at most 2^-23 of the sum of magnitudes.
-    g = torch.Generator().manual_seed(T * K)
-    buf = torch.full((T * pitch + offset + 8,), float("nan"), dtype=torch.bfloat16)
-    x = buf[offset:offset + T * pitch].view(T, pitch)[:, :K]
-    x.copy_(torch.randn((T, K), generator=g) * torch.linspace(0.1, 5.0, K))
-    xd = buf.cuda()[offset:offset + T * pitch].view(T, pitch)[:, :K]
-    ref, mag = (v.double().T @ v.double() for v in (x, x.abs()))
-    old = torch.randn((K, K), generator=g)
-    old = old + old.T
-    guard = torch.full((K * K + 64,), -7.0, device="cuda")
-    H = guard[:K * K].view(K, K)
-    H.copy_(old)
-    H1 = binding.hessian_accumulate(xd)
-    binding.hessian_accumulate(xd, H)
-    torch.cuda.synchronize()
-    assert binding.query_device_status() == 0
-    assert bool((guard[K * K:] == -7.0).all())
-    bound = (8 + T / 8) * 2.0 ** -23 * mag
-    assert bool(((H1.cpu().double() - ref).abs() <= bound).all())
-    assert bool(((H.cpu().double() - ref - old.double()).abs() <= bound + 2.0 ** -23 * old.abs()).all())
-    assert torch.equal(H1, H1.T) and torch.equal(H, H.T)
