@@ -452,7 +452,7 @@ int w4a8_gar_permutation(const float* hdiag, int64_t K, int group, int32_t* perm
  *   mse_steps  0 or 1: Eq. 8 as is; 2..11: that many shrink factors 1, 0.98, 0.96, ... are tried.
  *   workspace  device, 16-byte aligned, w4a8_dpq_workspace_bytes(N, K) bytes (scratch).
  * Every step that decides a code is a single correctly rounded fp32 operation, so the codes are
- * reproducible and independent of the launch geometry.  Enqueues about 2 K / 128 kernels.
+ * reproducible and independent of the launch geometry.  Enqueues about K / 128 kernels.
  */
 size_t w4a8_dpq_workspace_bytes(int64_t N, int64_t K);
 int w4a8_dpq_quantize(const float* W, int64_t N, int64_t K, int group, const float* U, const int32_t* perm,

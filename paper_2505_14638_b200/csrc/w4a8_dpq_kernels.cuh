@@ -5,21 +5,21 @@
 // The rows of W are independent; the columns of a row are quantized one after the other, each
 // sending its scaled error e to the columns on its right (Eq. 12): w_v <- fma(-e, U_qv, w_v),
 // U = upper Cholesky factor of the inverse Hessian in processing order.  Work is cut the way
-// GPTQ cuts it, in blocks of one group (128 columns):
-//   dpq_block_kernel     half a warp per row: group scale / zero-point (Eq. 8, optional search),
-//                        then the 128 columns in sequence with the updates inside the block;
-//                        writes the codes, the group's scale and zero-point and the 128 errors;
-//   dpq_trailing_kernel  applies the block's 128 errors to every column to the right of the
-//                        block, q ascending -- the same chain of fused multiply-adds, in the same
-//                        order, that the column-by-column algorithm performs for that element.
+// GPTQ cuts it, in blocks of one group (128 columns), one launch of dpq_step_kernel per block: its
+// first CTAs bring the block's columns up to date and quantize them (group scale / zero-point,
+// Eq. 8, optional search; the 128 columns in sequence), the others apply the errors of the block
+// before to all later columns, q ascending -- the same chain of fused multiply-adds, in the same
+// order, that the column-by-column algorithm performs for each element.
 // Every floating-point step that decides an integer is one explicitly rounded fp32 operation
-// (__fdiv_rn, __fmul_rn, __fmaf_rn ...: never contracted), and the search compares exact integer
+// (__fmul_rn, __fmaf_rn ...: never contracted; quotients correctly rounded), and the search compares exact integer
 // sums, so the codes do not depend on how the work is spread over threads.
 #pragma once
 
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include "w4a8_common.cuh"
+#include "w4a8_ptx.cuh"
 #include "w4a8_simple_kernels.cuh"
 
 namespace w4a8 {
@@ -90,107 +90,458 @@ __device__ __forceinline__ DpqGroup dpq_group_params(float lo, float hi, float a
     return g;
 }
 
-// Returns the code u (Eq. 9); w8hat = nearest_Z((u - z) s), the value inference multiplies with (Eq. 10).
-__device__ __forceinline__ int dpq_quant_dequant(float w8, const DpqGroup& g, int symmetric, float& w8hat) {
-    int u;
-    if (symmetric) {
-        const float q = rintf(__fdiv_rn(w8, g.s));
-        u = (int)fminf(fmaxf(q, -7.0f), 7.0f) + 8;
+// ---- division by a repeated divisor --------------------------------------------------------------
+// The correctly rounded quotient from the reciprocal h = RN(1 / b) and its tail l, in four dependent
+// operations: q = RN(a h + RN(a l)) is within half a unit in the last place and 2^-24 of a / b, its remainder is exact
+// in one FMA, and the correction by the remainder times a correctly rounded reciprocal then rounds to
+// RN(a / b) (Markstein's theorem, IBM J. Res. Dev. 34(1), 1990).  Valid while nothing underflows or
+// overflows on the way: |b| in [2^-40, 2^40], a = 0 or |a| in [2^-72, 2^60]; a zero quotient may lose its sign.
+struct Recip {
+    float b, h, l;
+};
+__device__ __forceinline__ Recip make_recip(float b) {
+    Recip r;
+    r.b = b;
+    r.h = __fdiv_rn(1.0f, b);
+    r.l = __fmul_rn(__fmaf_rn(-r.h, b, 1.0f), r.h);
+    return r;
+}
+__device__ __forceinline__ float div_recip(float a, const Recip& r) {
+    const float q = __fmaf_rn(a, r.h, __fmul_rn(a, r.l));
+    return __fmaf_rn(__fmaf_rn(-q, r.b, a), r.h, q);
+}
+__device__ __forceinline__ bool recip_range(float b) { return fabsf(b) >= 0x1p-40f && fabsf(b) <= 0x1p40f; }
+
+// Two FP32 operations in one instruction (each rounded once, as two scalar ones).
+__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long mul_f32x2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ void unpack_f32x2(unsigned long long v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+
+__device__ __forceinline__ unsigned long long div_recip_f32x2(unsigned long long a, const Recip& r) {
+    const unsigned long long h = pack_f32x2(r.h, r.h);
+    const unsigned long long q = fma_f32x2(a, h, mul_f32x2(a, pack_f32x2(r.l, r.l)));
+    return fma_f32x2(fma_f32x2(q, pack_f32x2(-r.b, -r.b), a), h, q);
+}
+
+// 16 bytes (four floats) global -> shared, asynchronously; four 4-byte copies where the source is not
+// 16-byte aligned.
+__device__ __forceinline__ void dpq_copy16(uint32_t dst, const float* src, bool vec) {
+    if (vec) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
     } else {
-        const float q = rintf(__fadd_rn(__fdiv_rn(w8, g.s), (float)g.z));
-        u = (int)fminf(fmaxf(q, 0.0f), 15.0f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4u * i), "l"(src + i) : "memory");
     }
-    w8hat = e4m3_roundtrip(__fmul_rn((float)(u - g.z), g.s));
-    return u;
+}
+__device__ __forceinline__ void dpq_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void dpq_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-__device__ __forceinline__ long long warp_sum_ll(long long v) {
+// nearest_Z of two values (Eq. 10), through the conversion instructions.
+__device__ __forceinline__ float2 e4m3x2_roundtrip(float a, float b) {
+    uint32_t h2;
+    asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((uint16_t)cvt_e4m3x2(b, a)));
+    return __half22float2(*reinterpret_cast<const __half2*>(&h2));
+}
+
+// Four columns of the chain with IEEE divisions, for operands outside the range of div_recip: v[0..3] the weights,
+// v[4..7] receives their errors (negated), u_d the block of U from (q0, q0) on; returns the four FP8 codes.
+__device__ __noinline__ uint32_t dpq_four_slow(float* v, float sw, const float* lut_h, const float* u_d) {
+    uint32_t all = 0;
+#pragma unroll 1
+    for (int c = 0; c < 4; ++c) {
+        const uint32_t code = cvt_e4m3x2(0.0f, __fdiv_rn(v[c], sw));
+        v[4 + c] = __fdiv_rn(__fsub_rn(lut_h[code], v[c]), u_d[c * 128 + c]);
+        for (int j = c + 1; j < 4; ++j) v[j] = __fmaf_rn(v[4 + c], u_d[c * 128 + j], v[j]);
+        all |= code << (8 * c);
+    }
+    return all;
+}
+
+template <int W>   // lanes that share a row
+__device__ __forceinline__ float row_min(float v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    for (int o = W / 2; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    return v;
+}
+template <int W>
+__device__ __forceinline__ float row_max(float v) {
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    return v;
+}
+template <int W>
+__device__ __forceinline__ long long row_sum_ll(long long v) {
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
     return v;
 }
 
-// Half a warp per row, 32 rows per CTA; block `b` = processing positions [128 b, 128 b + 128).
-// The chain of one column (three IEEE divisions, two FP8 conversions) is some seventy dependent
-// instructions that every lane executes and only the column's owner needs: with two rows per warp a
-// warp instruction carries two of those chains (a warp per row spent its issue slots on them: with
-// 28 warps per SM the kernel was bound by issue, not by latency).  Lane l of a half owns positions
-// l, l + 16, ..., l + 112 of the block.  The block of U (128 x 128) is staged in shared memory for
-// the whole CTA.
-constexpr int kDpqRowsPerCta = 32;
+// Step b of the quantizer, one launch: the first CTAs quantize block b (processing positions
+// [128 b, 128 b + 128), 32 rows per CTA), the others apply the errors of block b - 1 to the columns to
+// the right of block b.  The two touch different columns, so the serial chain of a block (some ten
+// microseconds) runs beside the contraction that fills the chip.  Measured, us per layer, this kernel / a block
+// kernel (57 us: IEEE divisions, half a warp per row) followed by a trailing kernel (scalar FMAs, 8 x 8 per thread):
+// (N, K) = (256, 1024) 221 / 479, (256, 4096) 948 / 2109, (4096, 4096) 2288 / 3525, (4096, 14336) 22264 / 28550.
+constexpr int kDpqThreads = 256;
+constexpr int kDpqRowsPerCta = 32;      // eight lanes per row
+constexpr int kDpqChunk = 32;           // values of q per stage
+struct DpqSmem {
+    // block CTAs
+    static constexpr int kU = 0;                                   // [128][128] U of the block itself
+    static constexpr int kPanel = kU + 128 * 128 * 4;              // 2 x [32][128] U of the previous block's rows
+    static constexpr int kErr = kPanel + 2 * kDpqChunk * 128 * 4;  // 2 x [32][32 rows] errors of the previous block
+    static constexpr int kCodes = kErr + 2 * kDpqChunk * kDpqRowsPerCta * 4 + 256;
+    static constexpr int kDiag = kCodes + kDpqRowsPerCta * 128;    // [128] float4: U_qq, its reciprocal and tail
+    static constexpr int kPerm = kDiag + 128 * 16;                 // [128] column within its original group
+    static constexpr int kBlockBytes = kPerm + 128 + 16;
+    // over the panel and the errors, idle by then: the rows' tables
+    static constexpr int kLutPitch = 257;                          // floats; rows a bank apart
+    static constexpr int kLut = kPanel;
+    static constexpr int kLutU = kLut + kDpqRowsPerCta * kLutPitch * 4;
+    static_assert(kLutU + kDpqRowsPerCta * 256 <= kCodes, "tables");
+    // trailing CTAs
+    static constexpr int kTrailU = 0;                              // 2 x [32][128]
+    static constexpr int kTrailErr = 2 * kDpqChunk * 128 * 4;      // 2 x [32][128 rows]
+    static constexpr int kTrailBytes = 2 * kTrailErr;
+    static constexpr int kBytes = kBlockBytes > kTrailBytes ? kBlockBytes : kTrailBytes;
+    static_assert(2 * (kBytes + 1024) <= 228 * 1024, "two CTAs per SM");
+};
 
-__device__ __forceinline__ float half_warp_min(float v) {
+// Where the (negated) errors of a block are kept: in place of the block's weights, which nothing reads any
+// more, and in the order in which they are wanted, four rows of one q side by side: row 4 g + j of a complete
+// group of four rows holds q = 32 j .. 32 j + 31 as float4 (rows 4 g .. 4 g + 3).  The up to three rows after the last
+// complete group keep their own errors, q ascending.
+//
+// Chunk c (32 values of q) of the rows from n0 on -> e_s[q][ROWS], the groups of row q permuted by ^ (q & 7) so that the
+// copies (consecutive q) fall into different banks.
+template <int ROWS>
+__device__ __forceinline__ void dpq_load_errors(float* e_s, uint32_t e_addr, const float* __restrict__ work, int64_t N,
+                                                int64_t K, int64_t p, int64_t n0, int c) {
+    const int q = threadIdx.x & 31;
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-    return v;
-}
-__device__ __forceinline__ float half_warp_max(float v) {
+    for (int i = 0; i < ROWS / 4 * 32 / kDpqThreads; ++i) {
+        const int g = (int)(threadIdx.x >> 5) + i * (kDpqThreads / 32);
+        const int64_t n = n0 + 4 * g;
+        const int at = q * ROWS + 4 * (g ^ (q & 7));
+        if (n + 3 < N) {
+            dpq_copy16(e_addr + (uint32_t)at * 4u, work + (n + c) * K + p + 4 * q, true);
+        } else {
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-    return v;
-}
-__device__ __forceinline__ long long half_warp_sum_ll(long long v) {
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-    return v;
+            for (int r = 0; r < 4; ++r) e_s[at + r] = n + r < N ? work[(n + r) * K + p + c * kDpqChunk + q] : 0.0f;
+        }
+    }
 }
 
-__global__ void __launch_bounds__(16 * kDpqRowsPerCta)
-dpq_block_kernel(float* __restrict__ work, const float* __restrict__ U, const int32_t* __restrict__ perm,
-                 int64_t N, int64_t K, int b, int symmetric, int mse_steps, int per_channel,
-                 const float* __restrict__ s_w, uint8_t* __restrict__ codes, uint16_t* __restrict__ gscale,
-                 uint8_t* __restrict__ gzero, float* __restrict__ err) {
-    extern __shared__ float u_s[];  // [128][128] block of U, then kDpqRowsPerCta x 128 bytes of code staging
-    uint8_t* code_s = reinterpret_cast<uint8_t*>(u_s + 128 * 128);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int half = lane >> 4, sl = lane & 15;
+// Columns to the right of block b, w[n][v] <- fma(-e[n][q], U[q][v], w[n][v]) for the q of block b - 1 in
+// ascending order: the chain of fused multiply-adds that the column-by-column algorithm performs for that element.
+// 128 rows x 128 columns per CTA; a warp takes 16 rows and all columns, a lane four columns.  Bound: the FP32 pipes,
+// if shared memory keeps up: per q a warp reads 512 distinct bytes of U and sixteen errors that all lanes share
+// (five 16-byte loads, eight 128-byte passes), half of what an 8 x 8 tile per thread takes, whose lanes read the
+// same words from different quarters of the warp; the operands of the next q are fetched ahead (waiting for them
+// was the largest stall with four warps per scheduler).  Packed pairs of rows: the pipe takes a packed FMA every other
+// cycle, which leaves issue slots for the loads (scalar: 23.7 ms against 21.9 for (4096, 14336)); 19 T FMA/s in all,
+// of the 28-31 T that a loop of FMAs alone reaches.  Errors and rows of U come in double-buffered chunks of 32 q.
+__device__ __forceinline__ void dpq_trailing_tile(uint8_t* sm, uint32_t sm_addr, float* __restrict__ work,
+                                                  const float* __restrict__ U, int64_t N, int64_t K, int64_t pprev,
+                                                  int64_t v0, int64_t n0, bool uvec) {
+    constexpr int kChunks = 128 / kDpqChunk;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const float* usrc = U + (pprev + (tid >> 5)) * K + v0 + 4 * lane;
+    auto load_u = [&](int c) {
+        const uint32_t dst = sm_addr + DpqSmem::kTrailU + (uint32_t)((c & 1) * kDpqChunk * 128 * 4) + (uint32_t)tid * 16u;
+#pragma unroll
+        for (int i = 0; i < kDpqChunk / 8; ++i) dpq_copy16(dst + (uint32_t)(i * 8 * 512), usrc + (int64_t)(c * kDpqChunk + 8 * i) * K, uvec);
+    };
+    auto load_e = [&](int c) {
+        const int off = DpqSmem::kTrailErr + (c & 1) * kDpqChunk * 128 * 4;
+        dpq_load_errors<128>(reinterpret_cast<float*>(sm + off), sm_addr + (uint32_t)off, work, N, K, pprev, n0, c);
+    };
+    load_u(0);   // (U is the caller's: complete before the first launch of the chain)
+    ptx::griddep_wait();
+    load_e(0);
+    dpq_commit();
+    float* wp = work + (n0 + 16 * warp) * K + v0 + 4 * lane;
+    const int rows = (int)min((int64_t)16, N - (n0 + 16 * warp));   // (may be negative: a warp without rows)
+    unsigned long long acc[8][4];   // rows 2 i and 2 i + 1, four columns
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
+        if (2 * i < rows) a = *reinterpret_cast<const float4*>(wp + (int64_t)(2 * i) * K);
+        if (2 * i + 1 < rows) b = *reinterpret_cast<const float4*>(wp + (int64_t)(2 * i + 1) * K);
+        acc[i][0] = pack_f32x2(a.x, b.x);
+        acc[i][1] = pack_f32x2(a.y, b.y);
+        acc[i][2] = pack_f32x2(a.z, b.z);
+        acc[i][3] = pack_f32x2(a.w, b.w);
+    }
+#pragma unroll 1
+    for (int c = 0; c < kChunks; ++c) {
+        dpq_wait<0>();
+        __syncthreads();   // chunk c is there; chunk c - 1 has been consumed by everybody
+        if (c + 1 < kChunks) {
+            load_u(c + 1);
+            load_e(c + 1);
+            dpq_commit();
+        }
+        // group 4 warp + g of row q is at 4 ((4 warp + g) ^ (q & 7)) = 4 (4 warp ^ (q & 4)) + 4 (g ^ (q & 3)): two bases
+        const uint8_t* us = sm + DpqSmem::kTrailU + (c & 1) * kDpqChunk * 512 + 16 * lane;
+        const uint8_t* e0 = sm + DpqSmem::kTrailErr + (c & 1) * kDpqChunk * 512 + 64 * warp;
+        const uint8_t* e1 = sm + DpqSmem::kTrailErr + (c & 1) * kDpqChunk * 512 + 64 * (warp ^ 1);
+        struct Q {
+            ulonglong2 e[4];
+            float4 u;
+        } q0, q1;
+        auto fetch = [&](Q& t, int q8, int j) {   // q = q8 + j, j = 0..7 known at compile time
+            t.u = *reinterpret_cast<const float4*>(us + (q8 + j) * 512);
+#pragma unroll
+            for (int g = 0; g < 4; ++g)
+                t.e[g] = *reinterpret_cast<const ulonglong2*>(((j & 4) ? e1 : e0) + (q8 + j) * 512 + 16 * (g ^ (j & 3)));
+        };
+        auto apply = [&](const Q& t) {
+            const float uv[4] = {t.u.x, t.u.y, t.u.z, t.u.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const unsigned long long u2 = pack_f32x2(uv[j], uv[j]);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    acc[2 * g][j] = fma_f32x2(t.e[g].x, u2, acc[2 * g][j]);   // Eq. 12
+                    acc[2 * g + 1][j] = fma_f32x2(t.e[g].y, u2, acc[2 * g + 1][j]);
+                }
+            }
+        };
+        fetch(q0, 0, 0);
+#pragma unroll 1
+        for (int q8 = 0; q8 < kDpqChunk; q8 += 8) {
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+                fetch(q1, q8, j + 1);
+                apply(q0);
+                if (j < 6) fetch(q0, q8, j + 2);
+                else fetch(q0, (q8 + 8) & (kDpqChunk - 1), 0);   // (the last one is not used)
+                apply(q1);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        float4 a, b;
+        unpack_f32x2(acc[i][0], a.x, b.x);
+        unpack_f32x2(acc[i][1], a.y, b.y);
+        unpack_f32x2(acc[i][2], a.z, b.z);
+        unpack_f32x2(acc[i][3], a.w, b.w);
+        if (2 * i < rows) *reinterpret_cast<float4*>(wp + (int64_t)(2 * i) * K) = a;
+        if (2 * i + 1 < rows) *reinterpret_cast<float4*>(wp + (int64_t)(2 * i + 1) * K) = b;
+    }
+}
+
+// Block b of 32 rows, eight lanes per row.  Lane sl of a row keeps columns 32 k + 4 sl + {0..3}, k = 0..3.
+// Bound by the latency of the column chain (two quotients, a conversion and a look-up each).
+// Four columns at a time: every lane of the row fetches the four weights (one exchange per four columns
+// instead of one per column), follows the same scalar computation through all four, and then applies
+// the four errors to its own columns, in ascending order.  Columns that are finished are updated along
+// with the others; nothing reads them again.
+__global__ void __launch_bounds__(kDpqThreads, 2)
+dpq_step_kernel(float* __restrict__ work, const float* __restrict__ U, const int32_t* __restrict__ perm,
+                int64_t N, int64_t K, int b, int symmetric, int mse_steps, int per_channel,
+                const float* __restrict__ s_w, uint8_t* __restrict__ codes, uint16_t* __restrict__ gscale,
+                uint8_t* __restrict__ gzero) {
+    extern __shared__ __align__(16) uint8_t sm[];
+    const uint32_t sm_addr = ptx::smem_addr(sm);
     const int64_t p0 = (int64_t)b * 128;
-    for (int i = threadIdx.x; i < 128 * 128; i += 16 * kDpqRowsPerCta) {
-        const int q = i >> 7, v = i & 127;
-        u_s[i] = (v >= q) ? U[(p0 + q) * K + p0 + v] : 0.0f;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, sl = lane & 7;
+    const bool uvec = (reinterpret_cast<uintptr_t>(U) & 15u) == 0;
+    const unsigned block_ctas = (unsigned)((N + kDpqRowsPerCta - 1) / kDpqRowsPerCta);
+    ptx::griddep_launch_dependents();
+    if (blockIdx.x >= block_ctas) {
+        const unsigned t = blockIdx.x - block_ctas, row_tiles = (unsigned)((N + 127) / 128);
+        dpq_trailing_tile(sm, sm_addr, work, U, N, K, p0 - 128, p0 + 128 + (int64_t)(t / row_tiles) * 128,
+                          (int64_t)(t % row_tiles) * 128, uvec);
+        return;
     }
-    __syncthreads();
-    const int rl = 2 * warp + half;                               // row within the CTA
+    const float* u_s = reinterpret_cast<const float*>(sm + DpqSmem::kU);
+    uint8_t* code_s = sm + DpqSmem::kCodes;
+    float4* diag_s = reinterpret_cast<float4*>(sm + DpqSmem::kDiag);
+    uint8_t* perm_s = sm + DpqSmem::kPerm;
+    const int rl = 4 * warp + (lane >> 3);                        // row within the CTA
     const int64_t n_raw = (int64_t)blockIdx.x * kDpqRowsPerCta + rl;
-    if ((int64_t)blockIdx.x * kDpqRowsPerCta + 2 * warp >= N) return;   // neither row of the warp exists
-    const bool valid = n_raw < N;                                 // (a half without a row repeats the last one and stores nothing)
+    const bool valid = n_raw < N;                                 // (lanes without a row repeat the last one and store nothing)
     const int64_t n = valid ? n_raw : N - 1;
     const int64_t G = K >> 7;
-    const float sw = per_channel ? s_w[n] : s_w[0];
-    float* wrow = work + n * K + p0;
-    float w[8];
+
+    auto load_panel = [&](int c) {
+        const uint32_t dst = sm_addr + DpqSmem::kPanel + (uint32_t)((c & 1) * kDpqChunk * 128 * 4);
+        const float* src = U + (p0 - 128 + c * kDpqChunk) * K + p0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = wrow[sl + 16 * i];
+        for (int i = 0; i < kDpqChunk * 32 / kDpqThreads; ++i) {
+            const int idx = i * kDpqThreads + tid, q = idx >> 5, c4 = (idx & 31) * 4;
+            dpq_copy16(dst + (uint32_t)((q * 128 + c4) * 4), src + (int64_t)q * K + c4, uvec);
+        }
+    };
+    auto load_err = [&](int c) {
+        const int off = DpqSmem::kErr + (c & 1) * kDpqChunk * kDpqRowsPerCta * 4;
+        dpq_load_errors<kDpqRowsPerCta>(reinterpret_cast<float*>(sm + off), sm_addr + (uint32_t)off, work, N, K, p0 - 128,
+                                        (int64_t)blockIdx.x * kDpqRowsPerCta, c);
+    };
+    if (b > 0) {
+        load_panel(0);   // (U is the caller's: complete before the first launch of the chain)
+        ptx::griddep_wait();
+        load_err(0);
+        dpq_commit();
+        load_panel(1);
+        load_err(1);
+        dpq_commit();
+    }
+#pragma unroll
+    for (int i = 0; i < 128 * 32 / kDpqThreads; ++i) {
+        const int idx = i * kDpqThreads + tid, q = idx >> 5, c4 = (idx & 31) * 4;
+        dpq_copy16(sm_addr + DpqSmem::kU + (uint32_t)((q * 128 + c4) * 4), U + (p0 + q) * K + p0 + c4, uvec);
+    }
+    dpq_commit();
+    if (tid < 128) perm_s[tid] = (uint8_t)(perm ? (perm[p0 + tid] & 127) : tid);
+    // The errors of the previous block first (the trailing CTAs of the previous launch left this block out): a
+    // warp takes its four rows, a lane four consecutive columns of each, so that U is read once per four rows.
+    {
+        const int64_t r0 = (int64_t)blockIdx.x * kDpqRowsPerCta + 4 * warp;
+        float a[4][4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float4 t = *reinterpret_cast<const float4*>(work + (r0 + r < N ? r0 + r : N - 1) * K + p0 + 4 * lane);
+            a[r][0] = t.x;
+            a[r][1] = t.y;
+            a[r][2] = t.z;
+            a[r][3] = t.w;
+        }
+        if (b > 0) {
+#pragma unroll 1
+            for (int c = 0; c < 128 / kDpqChunk; ++c) {
+                // groups in flight, in order: chunks 0 and 1, U of the block, chunks 2 and 3
+                if (c < 2) dpq_wait<2>();
+                else if (c == 2) dpq_wait<1>();
+                else dpq_wait<0>();
+                __syncthreads();
+                const float* us = reinterpret_cast<const float*>(sm + DpqSmem::kPanel) + (c & 1) * kDpqChunk * 128 + 4 * lane;
+                const float* es = reinterpret_cast<const float*>(sm + DpqSmem::kErr) + (c & 1) * kDpqChunk * kDpqRowsPerCta;
+#pragma unroll 8
+                for (int q = 0; q < kDpqChunk; ++q) {
+                    const float4 e4 = *reinterpret_cast<const float4*>(es + q * kDpqRowsPerCta + 4 * (warp ^ (q & 7)));
+                    const float4 u4 = *reinterpret_cast<const float4*>(us + q * 128);
+                    const float ev[4] = {e4.x, e4.y, e4.z, e4.w};
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        a[r][0] = __fmaf_rn(ev[r], u4.x, a[r][0]);
+                        a[r][1] = __fmaf_rn(ev[r], u4.y, a[r][1]);
+                        a[r][2] = __fmaf_rn(ev[r], u4.z, a[r][2]);
+                        a[r][3] = __fmaf_rn(ev[r], u4.w, a[r][3]);
+                    }
+                }
+                __syncthreads();
+                if (c + 2 < 128 / kDpqChunk) {
+                    load_panel(c + 2);
+                    load_err(c + 2);
+                    dpq_commit();
+                }
+            }
+        } else {
+            dpq_wait<0>();
+            __syncthreads();
+        }
+        // to eight lanes per row through the (idle) panel buffers
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            *reinterpret_cast<float4*>(sm + DpqSmem::kPanel + ((4 * warp + r) * 132 + 4 * lane) * 4) =
+                make_float4(a[r][0], a[r][1], a[r][2], a[r][3]);
+        __syncwarp();
+    }
+    unsigned long long w[8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(sm + DpqSmem::kPanel + (rl * 132 + 32 * k + 4 * sl) * 4);
+        w[2 * k] = t.x;
+        w[2 * k + 1] = t.y;
+    }
+    if (tid < 128) {
+        const float d = u_s[tid * 128 + tid];
+        const Recip r = make_recip(d);
+        diag_s[tid] = make_float4(d, r.h, r.l, 0.0f);
+    }
+    const bool diag_ok = __syncthreads_and(tid >= 128 || recip_range(u_s[(tid & 127) * 129]));
 
     // Eq. 7 on the group's current weights, then Eq. 8 (once per group)
-    float w8[8];
+    const Recip sw = make_recip(per_channel ? s_w[n] : s_w[0]);
+    float w8[16];
     float lo = 0.0f, hi = 0.0f, amax = 0.0f;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        w8[i] = e4m3_roundtrip(__fdiv_rn(w[i], sw));
-        lo = fminf(lo, w8[i]);
-        hi = fmaxf(hi, w8[i]);
-        amax = fmaxf(amax, fabsf(w8[i]));
+        unpack_f32x2(w[i], w8[2 * i], w8[2 * i + 1]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float& v = w8[2 * i + h];
+            v = e4m3_roundtrip(__fdiv_rn(v, sw.b));
+            lo = fminf(lo, v);
+            hi = fmaxf(hi, v);
+            amax = fmaxf(amax, fabsf(v));
+        }
     }
-    lo = half_warp_min(lo);
-    hi = half_warp_max(hi);
-    amax = half_warp_max(amax);
+    lo = row_min<8>(lo);
+    hi = row_max<8>(hi);
+    amax = row_max<8>(amax);
     DpqGroup grp = dpq_group_params(lo, hi, amax, 1.0f, symmetric);
+    // whole-number bounds of u - z + fz: codes 0..15 with the zero-point added, or -7..7 around zero
+    const float dlo = symmetric ? -7.0f : 0.0f, dhi = symmetric ? 7.0f : 15.0f;
     if (mse_steps > 1) {
         // Sec. 3.3: least squared error over the group among shrunk ranges; exact integer sums
         long long best = -1;
+#pragma unroll 1
         for (int t = 0; t < mse_steps; ++t) {
             const float pt = __fsub_rn(1.0f, __fmul_rn((float)t, 0.02f));
             const DpqGroup gt = dpq_group_params(lo, hi, amax, pt, symmetric);
+            const Recip st = make_recip(gt.s);   // (a sixteenth of FP8 values apart: always within the range of div_recip)
+            const float fz = symmetric ? 0.0f : (float)gt.z;
             long long e2 = 0;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                float h;
-                (void)dpq_quant_dequant(w8[i], gt, symmetric, h);
-                const long long d = (long long)__fmul_rn(__fsub_rn(w8[i], h), 512.0f);
-                e2 += d * d;
+                // two weights per instruction where there is a packed form
+                const unsigned long long v = pack_f32x2(w8[2 * i], w8[2 * i + 1]);
+                float c0, c1;
+                unpack_f32x2(add_f32x2(div_recip_f32x2(v, st), pack_f32x2(fz, fz)), c0, c1);
+                const unsigned long long magic = pack_f32x2(12582912.0f, 12582912.0f);
+                unsigned long long d = add_f32x2(pack_f32x2(fminf(fmaxf(c0, dlo), dhi), fminf(fmaxf(c1, dlo), dhi)), magic);
+                d = add_f32x2(add_f32x2(d, pack_f32x2(-12582912.0f, -12582912.0f)), pack_f32x2(-fz, -fz));   // u - z
+                float p0s, p1s;
+                unpack_f32x2(mul_f32x2(d, pack_f32x2(gt.s, gt.s)), p0s, p1s);
+                const float2 h8 = e4m3x2_roundtrip(p0s, p1s);
+                // 512 (w8 - h8), a whole number below 2^20: both are on the 2^-9 grid
+                const unsigned long long diff = add_f32x2(v, pack_f32x2(-h8.x, -h8.y));
+                float i0, i1;
+                unpack_f32x2(fma_f32x2(diff, pack_f32x2(512.0f, 512.0f), magic), i0, i1);
+                const int da = __float_as_int(i0) - 0x4B400000, db = __float_as_int(i1) - 0x4B400000;
+                e2 += (long long)da * da;
+                e2 += (long long)db * db;
             }
-            e2 = half_warp_sum_ll(e2);
+            e2 = row_sum_ll<8>(e2);
             if (best < 0 || e2 < best) {
                 best = e2;
                 grp = gt;
@@ -198,30 +549,105 @@ dpq_block_kernel(float* __restrict__ work, const float* __restrict__ U, const in
         }
     }
 
-    // the 128 columns in sequence; every lane of a half follows the same scalar computation
     const int64_t og = perm ? (int64_t)(perm[p0] >> 7) : (int64_t)b;
-    float* erow = err + n * 128;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    const float fz = symmetric ? 0.0f : (float)grp.z;
+    const float uoff = symmetric ? 8.0f : (float)grp.z;
+    // The row's table: code and dequantized value (Eq. 9, 10, 11) of each of the 256 FP8 values that Eq. 7 can give.
+    // Worked out once per group, off the chain: a column then takes one conversion and one look-up instead of a
+    // quotient, two roundings and a product.
+    float* lut_h = reinterpret_cast<float*>(sm + DpqSmem::kLut) + rl * DpqSmem::kLutPitch;
+    uint8_t* lut_u = sm + DpqSmem::kLutU + rl * 256;
+    {
+        const Recip sg = make_recip(grp.s);
 #pragma unroll 4
-        for (int o = 0; o < 16; ++o) {
-            const int q = 16 * i + o;
-            const float wq = __shfl_sync(0xFFFFFFFFu, w[i], (lane & 16) | o);
-            const float wq8 = e4m3_roundtrip(__fdiv_rn(wq, sw));         // Eq. 7
-            float h8;
-            const int u = dpq_quant_dequant(wq8, grp, symmetric, h8);    // Eq. 9, Eq. 10
-            const float h16 = __fmul_rn(h8, sw);                         // Eq. 11
-            const float e = __fdiv_rn(__fsub_rn(wq, h16), u_s[q * 128 + q]);
-            const float* urow = u_s + q * 128;
+        for (int i = 0; i < 16; ++i) {
+            const int code = 16 * i + 2 * sl;   // this lane: code and code + 1
+            uint32_t h2;
+            asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"((uint16_t)(code | (code + 1) << 8)));
+            const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&h2));
+            float d[2];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int v = sl + 16 * k;
-                if (v > q) w[k] = __fmaf_rn(-e, urow[v], w[k]);          // Eq. 12
+            for (int h = 0; h < 2; ++h) {
+                const float c = fminf(fmaxf(__fadd_rn(div_recip(h == 0 ? v.x : v.y, sg), fz), dlo), dhi);
+                d[h] = __fsub_rn(__fsub_rn(__fadd_rn(c, 12582912.0f), 12582912.0f), fz);
             }
+            const float2 h8 = e4m3x2_roundtrip(__fmul_rn(d[0], grp.s), __fmul_rn(d[1], grp.s));
+            lut_h[code] = __fmul_rn(h8.x, sw.b);
+            lut_h[code + 1] = __fmul_rn(h8.y, sw.b);
+            *reinterpret_cast<uint16_t*>(lut_u + code) =
+                (uint16_t)(__float2int_rn(__fadd_rn(d[0], uoff)) | __float2int_rn(__fadd_rn(d[1], uoff)) << 8);
+        }
+        __syncwarp();
+    }
+    // the divisions take the short form where operands are within its range (a weight of zero is)
+    // where this row's errors go (see dpq_load_errors): value (row, q) of a complete group of four rows to row 4 g + q / 32
+    const bool whole = (n_raw | 3) < N;
+    float* ew = whole ? work + (n & ~(int64_t)3) * K + p0 + (n & 3) : work + n * K + p0;
+    const bool fast = diag_ok && recip_range(sw.b);
+    const float wmin = fast ? 0x1p-40f : __int_as_float(0x7F800000), wzero = fast ? 0.0f : -1.0f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll 1
+        for (int o = 0; o < 8; ++o) {
+            const int q0 = 32 * k + 4 * o;
+            const float* urow = u_s + q0 * 128;
+            float wv[4], ne[4];
+            uint32_t code[4];   // Eq. 7, as an FP8 byte
+            unpack_f32x2(w[2 * k], wv[0], wv[1]);
+            unpack_f32x2(w[2 * k + 1], wv[2], wv[3]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) wv[c] = __shfl_sync(0xFFFFFFFFu, wv[c], (lane & 24) | o);
+            const float4 u0 = *reinterpret_cast<const float4*>(urow + q0);
+            const float4 u1 = *reinterpret_cast<const float4*>(urow + 128 + q0);
+            const float u23 = urow[256 + q0 + 3];
+            bool in = true;
+            {
+                float v[4] = {wv[0], wv[1], wv[2], wv[3]};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float4 dg = diag_s[q0 + c];
+                    code[c] = cvt_e4m3x2(0.0f, div_recip(v[c], sw));
+                    ne[c] = div_recip(__fsub_rn(lut_h[code[c]], v[c]), Recip{dg.x, dg.y, dg.z});
+                    const float av = fabsf(v[c]);
+                    in = in && ((av >= wmin && av <= 0x1p60f) || av == wzero);
+                    // Eq. 12 inside the four
+                    if (c == 0) {
+                        v[1] = __fmaf_rn(ne[0], u0.y, v[1]);
+                        v[2] = __fmaf_rn(ne[0], u0.z, v[2]);
+                        v[3] = __fmaf_rn(ne[0], u0.w, v[3]);
+                    } else if (c == 1) {
+                        v[2] = __fmaf_rn(ne[1], u1.z, v[2]);
+                        v[3] = __fmaf_rn(ne[1], u1.w, v[3]);
+                    } else if (c == 2) {
+                        v[3] = __fmaf_rn(ne[2], u23, v[3]);
+                    }
+                }
+            }
+            if (!in) {   // (tested once per four columns: a test per column stood in the chain)
+                float f[8] = {wv[0], wv[1], wv[2], wv[3], 0.0f, 0.0f, 0.0f, 0.0f};
+                const uint32_t all = dpq_four_slow(f, sw.b, lut_h, urow + q0);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    ne[c] = f[4 + c];
+                    code[c] = (all >> (8 * c)) & 0xFFu;
+                }
+            }
+            // Eq. 12 on this lane's columns, the four errors in order
+#pragma unroll
+            for (int kk = k; kk < 4; ++kk)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const ulonglong2 u2 = *reinterpret_cast<const ulonglong2*>(urow + c * 128 + 32 * kk + 4 * sl);
+                    const unsigned long long e2 = pack_f32x2(ne[c], ne[c]);
+                    w[2 * kk] = fma_f32x2(e2, u2.x, w[2 * kk]);
+                    w[2 * kk + 1] = fma_f32x2(e2, u2.y, w[2 * kk + 1]);
+                }
             if (sl == o && valid) {
-                erow[q] = e;
-                const int c = perm ? (perm[p0 + q] & 127) : q;  // column inside its original group
-                code_s[rl * 128 + c] = (uint8_t)u;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    ew[whole ? (int64_t)k * K + 16 * o + 4 * c : (int64_t)(q0 + c)] = ne[c];
+                    code_s[rl * 128 + perm_s[q0 + c]] = lut_u[code[c]];
+                }
             }
         }
     }
@@ -229,83 +655,21 @@ dpq_block_kernel(float* __restrict__ work, const float* __restrict__ U, const in
     if (!valid) return;
     // codes of the group, original order, two per byte (even column in the low nibble)
     {
-        const uint8_t* cs = code_s + rl * 128 + sl * 8;
-        const uint32_t packed = (uint32_t)cs[0] | ((uint32_t)cs[1] << 4) | ((uint32_t)cs[2] << 8) | ((uint32_t)cs[3] << 12) |
-                                ((uint32_t)cs[4] << 16) | ((uint32_t)cs[5] << 20) | ((uint32_t)cs[6] << 24) | ((uint32_t)cs[7] << 28);
-        *reinterpret_cast<uint32_t*>(codes + n * (K >> 1) + og * 64 + sl * 4) = packed;
+        const uint32_t* cs = reinterpret_cast<const uint32_t*>(code_s + rl * 128 + sl * 16);
+        uint32_t packed[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t a = cs[2 * i], c = cs[2 * i + 1];
+            packed[i] = (a & 15u) | ((a >> 4) & 0xF0u) | ((a >> 8) & 0xF00u) | ((a >> 12) & 0xF000u) |
+                        ((c & 15u) << 16) | ((c << 12) & 0xF00000u) | ((c << 8) & 0xF000000u) | ((c << 4) & 0xF0000000u);
+        }
+        *reinterpret_cast<uint2*>(codes + n * (K >> 1) + og * 64 + sl * 8) = make_uint2(packed[0], packed[1]);
     }
     if (sl == 0) {
         gscale[n * G + og] = __bfloat16_as_ushort(__float2bfloat16_rn(grp.s));
         if (gzero) gzero[n * G + og] = (uint8_t)grp.z;
     }
 }
-
-// Columns to the right of block b: w[n][v] <- fma(-e[n][q], U[128 b + q][v], w[n][v]), q = 0..127
-// in order.  A CTA takes 128 rows x 128 columns, a thread 8 rows x 8 columns (two runs of four
-// columns, 64 apart) which it keeps in registers; the errors and the rows of U come through shared
-// memory in chunks of 32 values of q, so that one q costs a thread four 16-byte shared loads and 64
-// FMAs and a tile of U is fetched once per 128 rows.  (First version: 16 rows x 512 columns per CTA,
-// U straight from L2 -- every 16 rows fetched it again, and the L2 traffic, not the FMA pipe, set
-// the pace: a fifth to a third of the FMA peak.)  The chain of one element is unchanged: the same
-// fused multiply-adds, q ascending.
-__global__ void __launch_bounds__(256, 2)
-dpq_trailing_kernel(float* __restrict__ work, const float* __restrict__ U, const float* __restrict__ err,
-                    int64_t N, int64_t K, int b) {
-    __shared__ __align__(16) float e_s[32][132];  // [q][row] = -e (the padding spreads the transposing stores over the banks)
-    __shared__ __align__(16) float u_s[32][128];  // [q][column]
-    const int64_t p0 = (int64_t)b * 128;
-    const int64_t v0 = p0 + 128 + (int64_t)blockIdx.x * 128;   // K is a multiple of 128: the column tile is whole
-    const int64_t n0 = (int64_t)blockIdx.y * 128;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    float acc[8][8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int64_t n = n0 + ty * 8 + i;
-        float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), c = a;
-        if (n < N) {
-            a = *reinterpret_cast<const float4*>(work + n * K + v0 + tx * 4);
-            c = *reinterpret_cast<const float4*>(work + n * K + v0 + 64 + tx * 4);
-        }
-        acc[i][0] = a.x; acc[i][1] = a.y; acc[i][2] = a.z; acc[i][3] = a.w;
-        acc[i][4] = c.x; acc[i][5] = c.y; acc[i][6] = c.z; acc[i][7] = c.w;
-    }
-    const float* up = U + p0 * K + v0;
-#pragma unroll 1
-    for (int qc = 0; qc < 128; qc += 32) {
-        if (qc > 0) __syncthreads();   // the previous chunk has been consumed
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int idx = i * 256 + tid;
-            const int q = idx & 31, row = idx >> 5;
-            e_s[q][row] = (n0 + row < N) ? -err[(n0 + row) * 128 + qc + q] : 0.0f;   // -e, exact
-            const int c = idx & 127, qu = idx >> 7;
-            u_s[qu][c] = __ldg(up + (int64_t)(qc + qu) * K + c);
-        }
-        __syncthreads();
-#pragma unroll 2
-        for (int q = 0; q < 32; ++q) {
-            const float4 ea = *reinterpret_cast<const float4*>(&e_s[q][ty * 8]);
-            const float4 eb = *reinterpret_cast<const float4*>(&e_s[q][ty * 8 + 4]);
-            const float4 ua = *reinterpret_cast<const float4*>(&u_s[q][tx * 4]);
-            const float4 ub = *reinterpret_cast<const float4*>(&u_s[q][64 + tx * 4]);
-            const float e[8] = {ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, eb.z, eb.w};
-            const float u[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = __fmaf_rn(e[i], u[j], acc[i][j]);   // Eq. 12
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int64_t n = n0 + ty * 8 + i;
-        if (n < N) {
-            *reinterpret_cast<float4*>(work + n * K + v0 + tx * 4) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-            *reinterpret_cast<float4*>(work + n * K + v0 + 64 + tx * 4) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
-        }
-    }
-}
-
 
 // ---------------------------------------------------------------------------------------------
 // The layer Hessian of the quantizer (Sec. 3.1; Sec. 3.3 for its preparation): H = X^T X over the

@@ -1568,7 +1568,7 @@ int w4a8_hessian_prepare(const float* H, int64_t K, const int32_t* perm, float d
 
 size_t w4a8_dpq_workspace_bytes(int64_t N, int64_t K) {
     if (N <= 0 || K <= 0 || K % kGroup != 0) return 0;
-    return ((size_t)N * (size_t)K + (size_t)N * 128) * sizeof(float);
+    return (size_t)N * (size_t)K * sizeof(float);
 }
 
 int w4a8_dpq_quantize(const float* W, int64_t N, int64_t K, int group, const float* U, const int32_t* perm,
@@ -1586,11 +1586,10 @@ int w4a8_dpq_quantize(const float* W, int64_t N, int64_t K, int group, const flo
     int rc = check_device();
     if (rc != W4A8_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    constexpr int kBlockSmem = 128 * 128 * 4 + kDpqRowsPerCta * 128;
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(once, [&] {
-        attr_err = cudaFuncSetAttribute(dpq_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlockSmem);
+        attr_err = cudaFuncSetAttribute(dpq_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DpqSmem::kBytes);
     });
     if (attr_err != cudaSuccess) return W4A8_ERR_CUDA;
     // Eq. 6
@@ -1606,21 +1605,26 @@ int w4a8_dpq_quantize(const float* W, int64_t N, int64_t K, int group, const flo
     int64_t ns = per_channel ? N : 1;
     amax_to_scale_kernel<<<(unsigned)((ns + 255) / 256), 256, 0, st>>>(s_w, ns);
     float* work = static_cast<float*>(workspace);
-    float* err = work + N * K;
     dpq_gather_kernel<<<(unsigned)((N * K + 255) / 256), 256, 0, st>>>(W, perm, N, K, work);
     uint64_t launches = 3;
     const int G = (int)(K / kGroup);
+    const int64_t block_ctas = (N + kDpqRowsPerCta - 1) / kDpqRowsPerCta, row_tiles = (N + 127) / 128;
     for (int b = 0; b < G; ++b) {
-        dpq_block_kernel<<<(unsigned)((N + kDpqRowsPerCta - 1) / kDpqRowsPerCta), 16 * kDpqRowsPerCta, kBlockSmem, st>>>(
-            work, U, perm, N, K, b, symmetric, mse_steps, per_channel, s_w, codes,
-            static_cast<uint16_t*>(gscale_bf16), gzero, err);
+        // (from the second step on the launches overlap: a step's CTAs start, and fetch U, while the one before drains)
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(block_ctas + (b > 0 ? row_tiles * (G - 1 - b) : 0)));
+        cfg.blockDim = dim3(kDpqThreads);
+        cfg.dynamicSmemBytes = (size_t)DpqSmem::kBytes;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = b > 0 ? 1 : 0;
+        if (cudaLaunchKernelEx(&cfg, dpq_step_kernel, work, U, perm, N, K, b, symmetric, mse_steps, per_channel,
+                               static_cast<const float*>(s_w), codes, static_cast<uint16_t*>(gscale_bf16), gzero) != cudaSuccess)
+            return W4A8_ERR_CUDA;
         ++launches;
-        const int64_t rest = K - ((int64_t)b + 1) * 128;
-        if (rest > 0) {
-            dim3 grid((unsigned)(rest / 128), (unsigned)((N + 127) / 128));
-            dpq_trailing_kernel<<<grid, 256, 0, st>>>(work, U, err, N, K, b);
-            ++launches;
-        }
     }
     g_launches.fetch_add(launches, std::memory_order_relaxed);
     return launch_status();

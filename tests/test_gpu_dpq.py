@@ -165,3 +165,34 @@ def test_quantizer_pipeline_from_activations_through_the_c_abi():
         D = (W - w8).double()
         return float(torch.einsum("nk,kj,nj->", D, H.double(), D))
     assert out_err(cq) <= 0.8 * out_err(rq)
+
+
+@pytest.mark.parametrize("N,K,offset", [(3, 128, 0), (31, 256, 1), (33, 384, 0), (127, 256, 2), (130, 512, 0), (257, 256, 0)])
+@pytest.mark.parametrize("mse_steps", [0, 11])
+def test_dpq_at_row_tile_edges(N, K, offset, mse_steps):
+    # 32 rows per quantizing CTA, groups of four rows, row tiles of 128; U at bases that are not 16-byte aligned, with
+    # NaN below its diagonal (which is not read); operands outside the range of the short divisions: weights of zero,
+    # denormals, rows 2^50 and 2^-60 times the others, a diagonal entry of U beyond 2^40.
+    W = inputs.make_weight(N, K, 0.02, seed=N * K)
+    W[0, ::3] = 0.0
+    W[N // 2] = 0.0
+    W[N - 1] *= 2.0 ** -60
+    W[N // 3, 5:9] = 1e-40
+    W[N // 4] *= 2.0 ** 50
+    perm = oracle.gar_permutation(np.random.default_rng(N).random(K).astype(np.float32))
+    U = oracle.hessian_upper_cholesky(_hessian(K, N))
+    U[K // 2, K // 2] *= 2.0 ** 45
+    buf = torch.empty((K * K + 4,), device="cuda")
+    Ud = buf[offset:offset + K * K].view(K, K)
+    Ud.copy_(dev(U))
+    Ud.masked_fill_(torch.ones((K, K), dtype=torch.bool, device="cuda").tril(-1), float("nan"))
+    for symmetric in (False, True):
+        for per_channel in (False, True):
+            kw = dict(symmetric=symmetric, mse_steps=mse_steps, per_channel=per_channel)
+            ref = oracle.dpq_quantize(W, U, perm, **kw)
+            codes, gscale, gzero, s_w = binding.dpq_quantize(dev(W), Ud, dev(perm), **kw)
+            torch.cuda.synchronize()
+            assert np.array_equal(s_w.cpu().numpy().view(np.uint32), ref[3].view(np.uint32))
+            assert np.array_equal(bf16_bits(gscale), ref[1])
+            assert symmetric or np.array_equal(gzero.cpu().numpy(), ref[2])
+            assert np.array_equal(codes.cpu().numpy(), ref[0])
