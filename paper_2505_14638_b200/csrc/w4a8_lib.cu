@@ -1542,9 +1542,15 @@ int w4a8_hessian_accumulate(const void* x_bf16, int64_t T, int64_t K, int64_t ld
     if ((reinterpret_cast<uintptr_t>(x_bf16) & 1u) || (reinterpret_cast<uintptr_t>(H) & 3u)) return W4A8_ERR_BAD_ALIGNMENT;
     int rc = check_device();
     if (rc != W4A8_OK) return rc;
-    const int64_t nb = (K + kHessTile - 1) / kHessTile;
-    hessian_xtx_kernel<<<(unsigned)(nb * (nb + 1) / 2), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const uint16_t*>(x_bf16), T, K, ldx, H, accumulate ? 1.0f : 0.0f);
+    const int64_t n128 = (K + 127) / 128, n64 = (K + 63) / 64;
+    const uint16_t* xb = static_cast<const uint16_t*>(x_bf16);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    // Tiles of 128 features once there are half as many as SMs, of 64 below (measured with 128 / 64, us:
+    // (T, K) = (2000, 1024) 191 / 76, (1024, 1536) 105 / 113, (1024, 2560) 193 / 217, (1024, 4096) 367 / 507).
+    if (n128 * (n128 + 1) / 2 >= kNominalSMs / 2)
+        hessian_xtx_kernel<128><<<(unsigned)(n128 * (n128 + 1) / 2), 256, 0, st>>>(xb, T, K, ldx, H, accumulate ? 1 : 0);
+    else
+        hessian_xtx_kernel<64><<<(unsigned)(n64 * (n64 + 1) / 2), 256, 0, st>>>(xb, T, K, ldx, H, accumulate ? 1 : 0);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return launch_status();
 }

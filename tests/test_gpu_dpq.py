@@ -196,3 +196,28 @@ def test_dpq_at_row_tile_edges(N, K, offset, mse_steps):
             assert np.array_equal(bf16_bits(gscale), ref[1])
             assert symmetric or np.array_equal(gzero.cpu().numpy(), ref[2])
             assert np.array_equal(codes.cpu().numpy(), ref[0])
+
+
+@pytest.mark.parametrize("T,K,pitch,offset", [
+    (1, 1, 8, 0), (15, 63, 72, 0), (16, 64, 64, 8), (17, 72, 80, 0), (33, 250, 250, 3), (40, 1501, 1501, 1),
+    (33, 1544, 1544, 0), (16, 1660, 1664, 8), (50, 1672, 1680, 0)])   # tiles of 64, and of 128 features from K = 1409 on
+def test_hessian_at_tile_edges(T, K, pitch, offset):
+    # Small whole numbers: every sum is exact in FP32.  Rows inside a wider buffer whose surroundings are NaN; the
+    # words behind H are not touched.
+    g = torch.Generator().manual_seed(T * K)
+    buf = torch.full((T * pitch + offset + 8,), float("nan"), dtype=torch.bfloat16)
+    x = buf[offset:offset + T * pitch].view(T, pitch)[:, :K]
+    x.copy_(torch.randint(-15, 16, (T, K), generator=g))
+    xd = buf.cuda()[offset:offset + T * pitch].view(T, pitch)[:, :K]
+    ref = (x.double().T @ x.double()).float()
+    old = torch.randint(-1000, 1000, (K, K), generator=g).float()
+    old = old + old.T
+    guard = torch.full((K * K + 64,), -7.5, device="cuda")
+    H = guard[:K * K].view(K, K)
+    H.copy_(old)
+    H1 = binding.hessian_accumulate(xd)
+    binding.hessian_accumulate(xd, H)
+    torch.cuda.synchronize()
+    assert torch.equal(H1.cpu(), ref)
+    assert torch.equal(H.cpu(), ref + old)
+    assert bool((guard[K * K:] == -7.5).all())
