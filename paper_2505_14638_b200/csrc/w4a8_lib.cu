@@ -290,7 +290,8 @@ static void make_sk_plan(int64_t M, int64_t N, int64_t K, int sms, SkPlan* pl) {
 template <class Cfg>
 static int launch_streamk(const CUtensorMap& tx, const uint8_t* wpp, const float* s_x, const float* s_w,
                           int sw_stride, void* y, int64_t ldy, int out_dtype, void* workspace, const SkPlan& pl,
-                          int M, int N, int K, cudaStream_t st, const CUtensorMap* tw8 = nullptr, int cl = 0) {
+                          int M, int N, int K, cudaStream_t st, const CUtensorMap* tw8 = nullptr, int cl = 0,
+                          const uint8_t* gzero = nullptr) {
     auto kern = linear_streamk_kernel<Cfg>;
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
@@ -323,8 +324,8 @@ static int launch_streamk(const CUtensorMap& tx, const uint8_t* wpp, const float
         attr[1].val.clusterDim.z = 1;
         cfg.numAttrs = 2;
     }
-    // (the second tensor map is read only by the FP8-weight variant)
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tx, tw8 ? *tw8 : tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype,
+    // (the second tensor map is read only by the FP8-weight and canonical variants)
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tx, tw8 ? *tw8 : tx, wpp, gzero, s_x, s_w, sw_stride, y, ldy, out_dtype,
                                        counters, slots, M, N, K, pl.TM, pl.TN, aligned, cl, status);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     if (e != cudaSuccess) return W4A8_ERR_CUDA;
@@ -586,7 +587,7 @@ static int cluster_kcut_ctas(int64_t M, int64_t N, int64_t K, int sms) {
 template <class Cfg>
 static int launch_cluster_kcut(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, const float* s_x, const float* s_w,
                                int sw_stride, void* y, int64_t ldy, int out_dtype, int M, int N, int K, int cl,
-                               cudaStream_t st) {
+                               cudaStream_t st, const CUtensorMap* tw = nullptr, const uint8_t* gzero = nullptr) {
     const int TN = (N + 127) / 128;
     static std::atomic<int> fits[9];   // clusters of size cl resident at once (0: not asked yet)
     int have = fits[cl].load(std::memory_order_relaxed);
@@ -627,7 +628,7 @@ static int launch_cluster_kcut(const uint8_t* x8, int64_t ldx8, const uint8_t* w
     pl.P = (int64_t)TN * cl;
     pl.counter_bytes = 0;
     pl.workspace_bytes = 0;
-    return launch_streamk<Cfg>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, nullptr, pl, M, N, K, st, nullptr, cl);
+    return launch_streamk<Cfg>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, nullptr, pl, M, N, K, st, tw, cl, gzero);
 }
 
 static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* wpp,
@@ -743,6 +744,62 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
     return rc;
 }
 
+// Weights in the boundary format, kernel chosen by the library: the kernels of the prepacked formats on canonical
+// arrays, as far as they need no workspace (the caller's is not zero-filled).  Returns -1 (nothing launched) where
+// linear_umma_kernel is the better one: up to sixteen tokens its small CTAs, two per SM and K cut between them,
+// stream a wide layer faster ((2, 24064, 4608) 33 us against 39 on tiles of 64 tokens).
+static int linear_canonical_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* codes,
+                                 const uint16_t* gscale, const uint8_t* gzero, const float* s_w, int sw_stride, int64_t N,
+                                 int64_t K, void* y, int64_t ldy, int out_dtype, cudaStream_t st) {
+    const int sms = sm_count();
+    if (sms <= 0) return W4A8_ERR_CUDA;
+    if (M <= 16) return -1;
+    const uint8_t* gs = reinterpret_cast<const uint8_t*>(gscale);
+    CUtensorMap tw;
+    if (!make_tmap_u8_2d(&tw, codes, (uint64_t)N, (uint64_t)(K / 2), (uint64_t)(K / 2), 64, 128, CU_TENSOR_MAP_SWIZZLE_64B))
+        return W4A8_ERR_CUDA;
+    for (int cl = cluster_kcut_ctas(M, N, K, sms); cl >= 2; --cl) {
+        const int rc = M <= 64 ? launch_cluster_kcut<SkCfg<64, 4, 8, 4, kFmtCanonical, 1, false, true>>(
+                                     x8, ldx8, gs, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st, &tw, gzero)
+                               : launch_cluster_kcut<SkCfg<128, 3, 6, 3, kFmtCanonical, 1, false, true>>(
+                                     x8, ldx8, gs, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st, &tw, gzero);
+        if (rc != -1) return rc;
+    }
+    // Whole tiles of 128 channels x 64 / 128 / 256 tokens (no workspace): rounds of tiles times the measured time of a
+    // k-block step, us.  Measured (us, chosen in brackets; one tile per CTA of linear_umma_kernel before):
+    // (64, 28672, 4096) [32] 44 46, before 57; (256, 6144, 4096) 31 [23] 26, before 51; (512, 4096, 14336) 94 [69] 84,
+    // before 110; (2048, 6144, 4096) 148 99 [63], before 148; (3000, 28672, 4096) 940 630 [408], before 899.  Tiles of
+    // 256 x 256 were slower: (2048, 4096, 4096) 46 against 45, (8192, 28672, 4096) 1288 against 1170.
+    double best = 1e30;
+    SkPlan pl = {};
+    for (int bnx = 256; bnx >= 64; bnx >>= 1) {
+        const int64_t TM = (M + bnx - 1) / bnx, TN = (N + 127) / 128, tiles = TM * TN;
+        const double unit = bnx == 64 ? 0.425 : (bnx == 128 ? 0.55 : 0.70);
+        const double t = (double)((tiles + sms - 1) / sms) * (double)(K / 128) * unit;
+        if (t < best) {
+            best = t;
+            pl.bnx = bnx;
+            pl.TM = (int)TM;
+            pl.TN = (int)TN;
+            pl.aligned = 1;
+            pl.U = tiles * (K / 128);
+            pl.P = tiles < sms ? tiles : sms;
+        }
+    }
+    CUtensorMap tx;
+    if (!make_tmap_u8_2d(&tx, x8, (uint64_t)M, (uint64_t)K, (uint64_t)ldx8, 128, (uint32_t)pl.bnx, CU_TENSOR_MAP_SWIZZLE_128B))
+        return W4A8_ERR_CUDA;
+#define W4A8_SKC(BNX, G, S1, S2)                                                                                       \
+    return launch_streamk<SkCfg<BNX, G, S1, S2, kFmtCanonical>>(tx, gs, s_x, s_w, sw_stride, y, ldy, out_dtype, nullptr, \
+                                                                pl, (int)M, (int)N, (int)K, st, &tw, 0, gzero)
+    switch (pl.bnx) {
+        case 64: W4A8_SKC(64, 4, 8, 4);
+        case 128: W4A8_SKC(128, 4, 4, 4);
+        default: W4A8_SKC(256, 4, 4, 3);
+    }
+#undef W4A8_SKC
+}
+
 static int linear_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* codes,
                        const void* gscale, const uint8_t* gzero, int fmt, const float* s_w, int sw_stride,
                        int64_t N, int64_t K, int group, void* y, int64_t ldy, int out_dtype, void* workspace,
@@ -778,6 +835,10 @@ static int linear_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_
     if (rc != W4A8_OK) return rc;
 
     const uint16_t* gs = static_cast<const uint16_t*>(gscale);
+    if (algo == W4A8_ALGO_AUTO && split_k == 0 && !g_idx) {
+        rc = linear_canonical_impl(x8, ldx8, s_x, M, codes, gs, gzero, s_w, sw_stride, N, K, y, ldy, out_dtype, st);
+        if (rc != -1) return rc;
+    }
     if (plan.algo == W4A8_ALGO_SIMT) {
         dim3 grid((unsigned)((N + 31) / 32), (unsigned)((M + 7) / 8));
         linear_simt_kernel<<<grid, 256, 0, st>>>(x8, ldx8, s_x, M, codes, gs, gzero, s_w, sw_stride, N, K, y, ldy,

@@ -58,6 +58,12 @@ namespace w4a8 {
 // At 128 tokens a CTA exchanges 64 KB, which the SM-to-SM network moves in about 2.5 us (some
 // 25 bytes per clock and SM): little is gained there.  Needs no workspace.
 //
+// FMT = canonical (weights as they are stored at the boundary, not prepacked): a TMA tile load of 64 bytes x 128 (256)
+// rows per k-block takes the place of the two bulk copies, and the expanding threads fetch their row's scale
+// and zero-point of a stage from the canonical arrays while they expand the stage before.  Whole tiles or
+// the cluster exchange only (the canonical entry points have no workspace that is zero-filled once), and nothing is
+// requested before griddepcontrol.wait.
+//
 // W16 = true (the W4A16 comparison scheme of Sec. 4.3 on this kernel's skeleton): activations stay
 // BF16 (two TMA loads of 64 values per k-block and token tile), the INT4 codes are expanded to BF16
 // through a table of the group's eight magnitudes (two 128-byte panels per row and k-block), the
@@ -73,10 +79,11 @@ struct SkCfg {
     static constexpr int S1 = S1_;     // ring of TMA stages (packed chunk + activation tile)
     static constexpr int S2 = S2_;     // ring of dequantized E4M3 weight tiles
     static constexpr int FMT = FMT_;
+    static constexpr bool CANON = FMT_ == kFmtCanonical;   // see the kernel's comment
     static constexpr int kMeta = meta_bytes(FMT);
     static constexpr int RB = RB_;     // 128-row blocks per tile
     static constexpr int kCodeBytes = RB_ * 8192;   // packed codes of the tile's rows for one k-block
-    static constexpr int kWStage = RB_ * 9216;  // rows x (64 code bytes + meta), padded to keep the activation tile 1024-aligned
+    static constexpr int kWStage = RB_ * (CANON ? 8192 : 9216);  // rows x (64 code bytes + meta), padded to keep the activation tile 1024-aligned
     static constexpr int kXBytes = BNX * 128 * (W16_ ? 2 : 1);
     static constexpr int kStage1 = kWStage + kXBytes;
     static constexpr int kW8Bytes = RB_ * 128 * 128 * (W16_ ? 2 : 1);   // expanded weights of one k-block: E4M3 (W16: BF16, two panels)
@@ -121,8 +128,9 @@ struct SkCfg {
 template <class Cfg>
 __global__ void __launch_bounds__(Cfg::kThreads)
 linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K], box 128 x BNX, 128B swizzle
-                      const __grid_constant__ CUtensorMap tmap_w,  // W8 only: FP8 weights u8 [N][K], box 128 x 128, 128B swizzle
-                      const uint8_t* __restrict__ wpp,             // tiled weights (panels, k-block major)
+                      const __grid_constant__ CUtensorMap tmap_w,  // W8: FP8 weights u8 [N][K], box 128 x 128, 128B swizzle; canonical: codes u8 [N][K/2], box 64 x 128 RB, 64B swizzle
+                      const uint8_t* __restrict__ wpp,             // tiled weights (panels, k-block major); canonical: the BF16 group scales [N][K/128]
+                      const uint8_t* __restrict__ gzero,           // canonical only: zero-points u8 [N][K/128] or NULL
                       const float* __restrict__ s_x, const float* __restrict__ s_w, int sw_stride,
                       void* __restrict__ y, int64_t ldy, int out_dtype, unsigned int* counters,
                       float* slots, int M, int N, int K, int TM, int TN, int aligned, int cl,
@@ -326,6 +334,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                 }
             }
             int it0 = 0;
+            if constexpr (Cfg::CANON) ptx::griddep_wait();
             if constexpr (!Cfg::W8) {
                 // The weights-only prologue as straight-line code: every slot is free, nothing to wait
                 // for, and the requests of the ring-full go out back to back (as iterations of the
@@ -339,9 +348,14 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                         const uint8_t* msrc = meta_base + row0 * Cfg::kMeta;
                         const uint32_t cbytes = (uint32_t)(rows * kRowCodeBytes), mbytes = (uint32_t)(rows * Cfg::kMeta);
                         if (ptx::elect_one()) {
-                            ptx::mbar_arrive_expect_tx(bar_full(i), cbytes + mbytes);
-                            ptx::bulk_load(stage_w(i), csrc, cbytes, bar_full(i));
-                            ptx::bulk_load(stage_w(i) + (uint32_t)Cfg::kCodeBytes, msrc, mbytes, bar_full(i));
+                            if constexpr (Cfg::CANON) {
+                                ptx::mbar_arrive_expect_tx(bar_full(i), (uint32_t)Cfg::kCodeBytes);
+                                ptx::tma_load_2d(stage_w(i), &tmap_w, kb * 64, nt * TR, bar_full(i));
+                            } else {
+                                ptx::mbar_arrive_expect_tx(bar_full(i), cbytes + mbytes);
+                                ptx::bulk_load(stage_w(i), csrc, cbytes, bar_full(i));
+                                ptx::bulk_load(stage_w(i) + (uint32_t)Cfg::kCodeBytes, msrc, mbytes, bar_full(i));
+                            }
                         }
                         r1.advance(S1);
                         ++issued;
@@ -378,6 +392,11 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                     if (ptx::elect_one()) {
                         ptx::mbar_arrive_expect_tx(bar_w8_full(s2), (uint32_t)Cfg::kW8Bytes);
                         ptx::tma_load_2d(stage_w8(s2), &tmap_w, kb * 128, nt * TR, bar_w8_full(s2));
+                    }
+                } else if constexpr (Cfg::CANON) {
+                    if (ptx::elect_one()) {
+                        ptx::mbar_arrive_expect_tx(full, (uint32_t)Cfg::kCodeBytes);
+                        ptx::tma_load_2d(wdst, &tmap_w, kb * 64, nt * TR, full);
                     }
                 } else if (ptx::elect_one()) {
                     ptx::mbar_arrive_expect_tx(full, cbytes + mbytes);
@@ -771,6 +790,29 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
         const int dw = warp - 10;
         const int g = dw >> 2;
         const int r = (dw & 3) * 32 + lane;
+        // canonical: scale and zero-point of this thread's rows, fetched one of the group's stages ahead
+        uint32_t meta[RB];
+        int mkb = kb_begin + g, mnt = (int)(tile_begin / TM), mmt = (int)(tile_begin % TM);
+        auto next_meta = [&](int step) {   // of the stage `step` k-blocks further
+            mkb += step;
+            while (mkb >= KB) {
+                mkb -= KB;
+                if (++mmt == TM) {
+                    mmt = 0;
+                    ++mnt;
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < RB; ++b) {
+                const int n = mnt * TR + b * 128 + r;
+                const int64_t i = (int64_t)n * KB + mkb;
+                meta[b] = n < N ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(wpp) + i) | (gzero ? (uint32_t)__ldg(gzero + i) : 8u) << 16 : 0u;
+            }
+        };
+        if constexpr (Cfg::CANON) {
+            ptx::griddep_wait();
+            next_meta(0);
+        }
         for (int it = Cfg::W8 ? n_it : g; it < n_it; it += G) {   // (W8: nothing to expand)
             const int s1 = it % S1, s2 = it % S2;
             if (!ptx::mbar_wait(bar_full(s1), (uint32_t)((it / S1) & 1), abort_flag, status_word)) break;
@@ -780,7 +822,16 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
             if constexpr (Cfg::W16)
                 dequant_row_to_smem_bf16(stage_w(s1) + tiled_row_offset(r), stage_w(s1) + (uint32_t)Cfg::kCodeBytes + (uint32_t)(r * Cfg::kMeta), r,
                                          stage_w8(s2) + (uint32_t)r * 128u);
-            else
+            else if constexpr (Cfg::CANON) {
+                uint32_t m[RB];
+#pragma unroll
+                for (int b = 0; b < RB; ++b) m[b] = meta[b];
+                next_meta(G);   // (past the last stage: a row that does not exist, or one that is not used)
+#pragma unroll
+                for (int b = 0; b < RB; ++b)
+                    dequant_canonical_row_to_smem(stage_w(s1) + (uint32_t)(b * 8192), m[b], r,
+                                                  stage_w8(s2) + (uint32_t)(b * 16384) + (uint32_t)r * 128u);
+            } else
 #pragma unroll
             for (int b = 0; b < RB; ++b)
                 dequant_row_to_smem<Cfg::FMT>(stage_w(s1) + tiled_row_offset(b * 128 + r),

@@ -34,7 +34,9 @@ constexpr uint32_t kChunkStride = 128;  // bytes between two chunks of one row
 __host__ __device__ constexpr uint32_t tiled_row_offset(int row) {
     return (uint32_t)(row >> 3) * 512u + (uint32_t)(row & 7) * 16u;
 }
-__host__ __device__ constexpr int meta_bytes(int fmt) { return fmt == kFmtTiledSignMag ? 2 : (fmt == kFmtTiledFp8 ? 0 : 4); }
+__host__ __device__ constexpr int meta_bytes(int fmt) {
+    return fmt == kFmtTiledSignMag ? 2 : (fmt == kFmtTiled ? 4 : 0);   // (FP8: none; canonical: in arrays of their own)
+}
 // Bytes of one row of one k-block, and the offset of a row's first 16-byte chunk within a piece that
 // starts on a multiple of eight rows (chunk c of the row sits c * 128 bytes further), per format.
 __host__ __device__ constexpr int row_bytes(int fmt) { return fmt == kFmtTiledFp8 ? 128 : kRowCodeBytes; }
@@ -109,6 +111,30 @@ __device__ __forceinline__ void dequant_row_to_smem(uint32_t src, uint32_t meta,
         asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (((uint32_t)c ^ sw128) << 4)), "r"(o0),
                      "r"(o1), "r"(o2), "r"(o3)
                      : "memory");
+    }
+}
+
+// The same for a row of a canonical tile: the TMA tile of 64 bytes per row with the 64-byte swizzle at `tile`; scale
+// (BF16 bits) and zero-point (from bit 16 on) in `meta`.
+__device__ __forceinline__ void dequant_canonical_row_to_smem(uint32_t tile, uint32_t meta, int row, uint32_t dst) {
+    const uint32_t sw64 = (uint32_t)((row >> 1) & 3), sw128 = (uint32_t)(row & 7), src = tile + (uint32_t)row * 64u;
+    DequantLut lut;
+    lut.build(bf16_bits_to_float(meta & 0xFFFFu), (int)(meta >> 16));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        uint32_t p[4];
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(p[0]), "=r"(p[1]), "=r"(p[2]), "=r"(p[3])
+                     : "r"(src + (((uint32_t)j ^ sw64) << 4)));
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            uint32_t o0, o1, o2, o3;
+            lut.dequant8(p[2 * c], o0, o1);
+            lut.dequant8(p[2 * c + 1], o2, o3);
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (((uint32_t)(2 * j + c) ^ sw128) << 4)), "r"(o0),
+                         "r"(o1), "r"(o2), "r"(o3)
+                         : "memory");
+        }
     }
 }
 

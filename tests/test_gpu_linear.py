@@ -285,3 +285,44 @@ def test_host_forward_many_tokens_takes_the_copy_path():
     torch.cuda.synchronize()
     ok, dist = bf16_gate(bf16_bits(y_host), ref["y64"])
     assert ok, dist
+
+
+@pytest.mark.parametrize("M,N,K", [
+    # few tokens, weights to registers: K below and above 512 columns per unit of work, one to four 8-row units per CTA, odd
+    # counts, several row tiles in progress, eight and sixteen tokens
+    (1, 1024, 128), (8, 1040, 512), (9, 1200, 640), (16, 1024, 3584), (3, 2384, 1152), (16, 3600, 1024), (5, 6144, 256),
+    (2, 1024, 7808), (13, 4112, 2048),
+    # canonical weights: K cut inside clusters at up to 64 and 128 tokens, whole tiles of 64, 128 and 256 tokens
+    (17, 144, 1152), (65, 272, 384), (128, 1040, 896), (20, 9616, 128), (100, 9616, 256), (130, 400, 640), (257, 1296, 256),
+    (300, 9488, 128)])
+def test_formats_at_tile_edges(M, N, K):
+    # Small whole numbers (exact in any order), rows of X8 and Y inside wider buffers; the elements of Y beyond N
+    # and beyond M are not touched.
+    rng = np.random.default_rng(M * 7 + N * 3 + K)
+    tab = e4m3_value_table()
+    ints = np.zeros(13, dtype=np.uint8)
+    for c, v in enumerate(tab):
+        if np.isfinite(v) and v == int(v) and abs(v) <= 6:
+            ints[int(v) + 6] = c
+    x8 = ints[rng.integers(0, 13, size=(M, K))]
+    s_x = 2.0 ** rng.integers(-3, 4, size=M).astype(np.float32)
+    codes = pack_codes(rng.integers(1, 16, size=(N, K)).astype(np.uint8))
+    gs = inputs.f32_to_bf16_bits(np.ones((N, K // 128), dtype=np.float32))
+    gz = rng.integers(4, 12, size=(N, K // 128)).astype(np.uint8)
+    s_w = 2.0 ** rng.integers(-3, 4, size=N).astype(np.float32)
+    xd = torch.zeros((M, K + 48), dtype=torch.uint8, device="cuda")
+    xd[:, :K] = dev(x8)
+    for zero in (gz, None):
+        want = oracle.linear(x8, s_x, oracle.dequant_weight(codes, gs, zero), s_w, want=("y32",))["y32"]
+        wd = weights_to_dev(codes, gs, zero, s_w)
+        runs = [lambda y, wd=wd: binding.linear(xd[:, :K], dev(s_x), *wd, out_dtype=binding.OUT_FP32, out=y)]
+        for fmt in ([binding.FMT_TILED] if zero is not None else [binding.FMT_TILED, binding.FMT_TILED_SIGNMAG]):
+            tw = binding.prepack_weight(*wd, weight_format=fmt)
+            runs.append(lambda y, tw=tw: binding.linear_tiled(xd[:, :K], dev(s_x), tw, out_dtype=binding.OUT_FP32, out=y))
+        for run in runs:
+            buf = torch.full((M + 1, N + 12), -7.5, device="cuda")
+            run(buf[:M, :N])
+            torch.cuda.synchronize()
+            assert binding.query_device_status() == 0
+            assert np.array_equal(buf[:M, :N].cpu().numpy(), want)
+            assert bool((buf[M:] == -7.5).all()) and bool((buf[:, N:] == -7.5).all())
