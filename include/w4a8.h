@@ -204,7 +204,8 @@ int w4a8_linear_static_scratch(const uint8_t* x8, int64_t ldx8, const float* s_x
  *   in_i = BF16( silu(G) * U ), G|U = x_i        (W4A8_CHAIN_INPUT_SILU_MUL: x_i has 2 K columns, gate
  *                                                 first, exactly as w4a8_silu_mul_quantize defines it),
  * and the results are those of w4a8_quantize_act (or w4a8_silu_mul_quantize) followed by
- * w4a8_linear on the same tiled weights with K not cut: same scales, same FP8 codes, same
+ * w4a8_linear on the same tiled weights with K not cut (layers with at least 96 output channels per
+ * SM; smaller ones w4a8_linear may cut along K): same scales, same FP8 codes, same
  * accumulation order -- for the output channels whose K range one CTA walks alone; where the chain
  * cuts K (see below) the FP32 partial sums are added in a fixed order, so results still repeat bit
  * for bit from call to call, and agree with w4a8_linear within its output tolerance.  Problems run

@@ -6,10 +6,12 @@
 #include <atomic>
 #include <cstdlib>
 #include <mutex>
+#include <type_traits>
 
 #include "../../include/w4a8.h"
 #include "w4a8_dpq_kernels.cuh"
 #include "w4a8_linear_chain.cuh"
+#include "w4a8_linear_direct.cuh"
 #include "w4a8_linear_splitn.cuh"
 #include "w4a8_linear_pair.cuh"
 #include "w4a8_linear_streamk.cuh"
@@ -631,9 +633,111 @@ static int launch_cluster_kcut(const uint8_t* x8, int64_t ldx8, const uint8_t* w
     return launch_streamk<Cfg>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, nullptr, pl, M, N, K, st, tw, cl, gzero);
 }
 
+// ------------------------------------------------------------------------------ few tokens, weights to registers
+constexpr int kDirMaxSmem = 227 * 1024;
+
+static int64_t direct_xpitch(int64_t K) { return (K / 128 * 144 + 64 + 127) / 128 * 128 + 64; }
+
+static size_t direct_smem(int64_t M, int64_t K, int nt) {
+    return (size_t)M * (size_t)direct_xpitch(K) + (size_t)((M + 3) & ~(int64_t)3) * 4 + (size_t)2 * 16 * 8 * nt * 20 * 4;
+}
+
+template <class Cfg>
+static int launch_direct_cfg(const uint8_t* x8, int64_t ldx8, const uint8_t* w, const uint16_t* gscale,
+                             const uint8_t* gzero, const float* s_x, const float* s_w, int sw_stride, void* y,
+                             int64_t ldy, int out_dtype, int M, int N, int K, const DirPlan& plan, cudaStream_t st) {
+    auto kern = linear_direct_kernel<Cfg>;
+    static std::once_flag once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(once, [&] {
+        attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDirMaxSmem);
+    });
+    if (attr_err != cudaSuccess) return W4A8_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)plan.P);
+    cfg.blockDim = dim3(Cfg::kThreads);
+    cfg.dynamicSmemBytes = direct_smem(M, K, Cfg::NT);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, x8, ldx8, w, gscale, gzero, s_x, s_w, sw_stride, y, ldy, out_dtype,
+                                             M, N, K, plan);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    if (e != cudaSuccess) return W4A8_ERR_CUDA;
+    return launch_status();
+}
+
+// Arrangement of the sixteen warps of a CTA with the fewest rounds (units of work per warp); returns those.
+static int64_t make_direct_plan(int64_t N, int64_t K, int sms, DirPlan* plan) {
+    const int64_t NU = N / 8;
+    plan->P = (int)(sms < NU ? sms : NU);
+    plan->xpitch = (int)direct_xpitch(K);
+    const int64_t T = ((NU + plan->P - 1) / plan->P + 1) / 2, Q = (K / 128 + 3) / 4;
+    int64_t best = INT64_MAX;
+    for (int wq = 1; wq <= 16 && wq <= Q; ++wq) {
+        const int64_t tc = 16 / wq, rounds = ((T + tc - 1) / tc) * ((Q + wq - 1) / wq);
+        if (rounds < best) {
+            best = rounds;
+            plan->Wq = wq;
+            plan->Tc = (int)tc;
+        }
+    }
+    return best;
+}
+
+// Small layers at up to sixteen tokens, where the latencies of a launch outweigh the weights: at most two units of
+// work per warp, and no more weights than this kernel's expansion -- whose FP8 fragments the hardware converts to
+// 16 bits for the MMA, on the pipe that expands -- keeps up with.  Measured (us, linear alone, this kernel / the
+// split-N kernel, canonical: the kernel of one tile per CTA):
+//   sign-magnitude M = 8: (1024, 1024) 3.4 / 6.3, (4096, 1024) 3.6 / 6.6, (4096, 4096) 6.8 / 7.6, (6144, 4096) 8.3 / 9.3,
+//   (28672, 4096) 22 / 17.5; M = 1: (2048, 2048) 3.3 / 5.4, (4096, 4096) 6.5 / 6.5; M = 16: (6144, 4096) 9.8 / 10.7
+//   generic M = 8: (1024, 1024) 3.5 / 6.4, (6144, 4096) 9.4 / 10.2; M = 1: (2048, 2048) 3.6 / 5.4, (1536, 8192) 7.4 / 6.4;
+//   M = 16: (4096, 4096) 8.8 / 9.2, (6144, 4096) 11.3 / 11.4
+//   canonical M = 8: (1024, 1024) 3.5 / 8.4, (6144, 4096) 11.0 / 13.2; M = 16: (2048, 2048) 4.9 / 8.6, (1536, 8192) 10.1 / 10.0,
+//   (6144, 4096) 12.7 / 13.7
+//   24 tokens: level at (1024, 1024), slower everywhere else.
+// Prepacked layers with a 96-row block for every SM keep the kernel that walks all of K in one chain of MMAs: a chain launch
+// gives the same bits there.
+static bool direct_applies(int64_t M, int64_t N, int64_t K, int fmt, int sms, DirPlan* plan) {
+    if (fmt != kFmtCanonical && N >= (int64_t)96 * sms) return false;
+    if (M > 16 || N < 1024 || direct_smem(M, K, M <= 8 ? 1 : 2) > (size_t)kDirMaxSmem) return false;
+    const int64_t most = fmt == kFmtCanonical ? 26 : (M < 4 ? 8 : (fmt == kFmtTiled && M > 8 ? 17 : 26));
+    return N * K <= most * 1000000 && make_direct_plan(N, K, sms, plan) <= 2;
+}
+
+static int launch_direct(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* w,
+                         const uint16_t* gscale, const uint8_t* gzero, int fmt, const float* s_w, int sw_stride, int64_t N,
+                         int64_t K, void* y, int64_t ldy, int out_dtype, const DirPlan& plan, cudaStream_t st) {
+#define W4A8_DIR(FMT, NT)                                                                                              \
+    return launch_direct_cfg<DirCfg<FMT, NT>>(x8, ldx8, w, gscale, gzero, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, \
+                                              (int)N, (int)K, plan, st)
+    if (fmt == kFmtCanonical) {
+        if (M <= 8) W4A8_DIR(kFmtCanonical, 1);
+        W4A8_DIR(kFmtCanonical, 2);
+    }
+    if (fmt == kFmtTiled) {
+        if (M <= 8) W4A8_DIR(kFmtTiled, 1);
+        W4A8_DIR(kFmtTiled, 2);
+    }
+    if (M <= 8) W4A8_DIR(kFmtTiledSignMag, 1);
+    W4A8_DIR(kFmtTiledSignMag, 2);
+#undef W4A8_DIR
+}
+
 static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* wpp,
                              int fmt, const float* s_w, int sw_stride, int64_t N, int64_t K, void* y, int64_t ldy,
                              int out_dtype, void* workspace, size_t workspace_bytes, cudaStream_t st) {
+    if (M <= 16) {
+        const int rc = check_device();
+        if (rc != W4A8_OK) return rc;
+        const int sms_d = sm_count();
+        DirPlan plan;
+        if (sms_d > 0 && direct_applies(M, N, K, fmt, sms_d, &plan))
+            return launch_direct(x8, ldx8, s_x, M, wpp, nullptr, nullptr, fmt, s_w, sw_stride, N, K, y, ldy, out_dtype, plan, st);
+    }
     if (M > 16) {
         // 17..128 tokens on a layer with few 128-row tiles: K cut between the CTAs of a cluster (measured, us,
         // against the split-N kernel or the persistent kernel with its exchange through L2:
@@ -753,6 +857,10 @@ static int linear_canonical_impl(const uint8_t* x8, int64_t ldx8, const float* s
                                  int64_t K, void* y, int64_t ldy, int out_dtype, cudaStream_t st) {
     const int sms = sm_count();
     if (sms <= 0) return W4A8_ERR_CUDA;
+    DirPlan plan;
+    if (direct_applies(M, N, K, kFmtCanonical, sms, &plan))
+        return launch_direct(x8, ldx8, s_x, M, codes, gscale, gzero, kFmtCanonical, s_w, sw_stride, N, K, y, ldy, out_dtype,
+                             plan, st);
     if (M <= 16) return -1;
     const uint8_t* gs = reinterpret_cast<const uint8_t*>(gscale);
     CUtensorMap tw;
