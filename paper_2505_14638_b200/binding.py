@@ -1,4 +1,5 @@
-"""ctypes binding of the C-ABI library declared in include/w4a8.h.
+"""Binding of the C-ABI library declared in include/w4a8.h: ctypes, and for the calls that a serving loop
+makes once per layer an extension module (csrc/w4a8_host.cpp).
 
 Argument marshalling only: every step of the W4A8 path (Eq. 13 activation quantization, Eq. 10
 weight dequantization, FP8 matmul, Eq. 4 / Eq. 11 epilogue) runs in the library's CUDA kernels.
@@ -55,6 +56,8 @@ class ChainProblem(ctypes.Structure):
     ]
 
 _lib = None
+_host = None
+HOST_PATH = os.path.join(_HERE, "_w4a8_host.so")
 
 
 class W4A8Error(RuntimeError):
@@ -144,6 +147,24 @@ def lib():
     return L
 
 
+def _load_host():
+    """The extension module with the per-layer calls; raises when it (or the CUDA library) is missing."""
+    global _host
+    lib()
+    if not os.path.exists(HOST_PATH):
+        raise RuntimeError("extension module %s is missing: build it with "
+                           "`python -m paper_2505_14638_b200.build` (there is no fallback path)" % HOST_PATH)
+    import importlib.machinery
+    import importlib.util
+
+    import torch  # noqa: F401  (its libraries have to be loaded first)
+    loader = importlib.machinery.ExtensionFileLoader("_w4a8_host", HOST_PATH)
+    mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_w4a8_host", loader))
+    loader.exec_module(mod)
+    _host = mod
+    return mod
+
+
 def status_string(status: int) -> str:
     return lib().w4a8_status_string(int(status)).decode()
 
@@ -183,17 +204,16 @@ def _check(fn, rc):
 def quantize_act(x, scale_mode=SCALE_EXACT, static_scale=None, out=None):
     """w4a8_quantize_act: x BF16 [M, K] (row stride in elements = x.stride(0)).
     Returns (x8 uint8 [M, K], s_x float32 [M])."""
-    import torch
-    assert x.is_cuda and x.dtype == torch.bfloat16 and x.dim() == 2 and x.stride(1) == 1
-    M, K = x.shape
     if out is None:
-        x8 = torch.empty((M, K), dtype=torch.uint8, device=x.device)
-        s_x = torch.empty((M,), dtype=torch.float32, device=x.device)
-    else:
-        x8, s_x = out
-    rc = lib().w4a8_quantize_act(_ptr(x), M, K, x.stride(0), _ptr(x8), x8.stride(0), _ptr(s_x),
-                                 int(scale_mode), _ptr(static_scale), _stream())
-    _check("w4a8_quantize_act", rc)
+        import torch
+        assert x.is_cuda and x.dtype == torch.bfloat16 and x.dim() == 2 and x.stride(1) == 1
+        M, K = x.shape
+        out = (torch.empty((M, K), dtype=torch.uint8, device=x.device),
+               torch.empty((M,), dtype=torch.float32, device=x.device))
+    x8, s_x = out
+    rc = (_host or _load_host()).quantize_act(x, x8, s_x, int(scale_mode), static_scale)
+    if rc != OK:
+        _check("w4a8_quantize_act", rc)
     return x8, s_x
 
 
@@ -335,25 +355,26 @@ def new_workspace(M, N, K, weight_format=FMT_CANONICAL, device="cuda"):
 def linear(x8, s_x, codes, gscale, gzero, s_w, out_dtype=OUT_BF16, out=None, workspace=None,
            algo=ALGO_AUTO, split_k=0):
     """w4a8_linear / w4a8_linear_ex on canonical weights: returns Y [M, N] (BF16 or FP32)."""
-    import torch
     M, K = x8.shape
     N = codes.shape[0]
     if out is None:
+        import torch
         dt = torch.bfloat16 if out_dtype == OUT_BF16 else torch.float32
         out = torch.empty((M, N), dtype=dt, device=x8.device)
-    need = linear_workspace_bytes(M, N, K, algo, split_k)
+    auto = algo == ALGO_AUTO and split_k == 0
+    host = _host or _load_host()
+    need = host.linear_workspace_bytes(M, N, K, FMT_CANONICAL) if auto else linear_workspace_bytes(M, N, K, algo, split_k)
     if need and (workspace is None or workspace.numel() * workspace.element_size() < need):
+        import torch
         workspace = torch.empty((need,), dtype=torch.uint8, device=x8.device)
-    wbytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    sw_stride = 0 if s_w.numel() == 1 else 1
-    L = lib()
-    if algo == ALGO_AUTO and split_k == 0:
-        rc = L.w4a8_linear(_ptr(x8), x8.stride(0), _ptr(s_x), M, _ptr(codes), _ptr(gscale),
-                           _ptr(gzero), FMT_CANONICAL, _ptr(s_w), sw_stride, N, K, GROUP, _ptr(out),
-                           out.stride(0), int(out_dtype), _ptr(workspace), wbytes, _stream())
-        _check("w4a8_linear", rc)
+    if auto:
+        rc = host.linear(x8, s_x, codes, gscale, gzero, FMT_CANONICAL, s_w, N, K, GROUP, out, int(out_dtype), workspace)
+        if rc != OK:
+            _check("w4a8_linear", rc)
     else:
-        rc = L.w4a8_linear_ex(_ptr(x8), x8.stride(0), _ptr(s_x), M, _ptr(codes), _ptr(gscale),
+        wbytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
+        sw_stride = 0 if s_w.numel() == 1 else 1
+        rc = lib().w4a8_linear_ex(_ptr(x8), x8.stride(0), _ptr(s_x), M, _ptr(codes), _ptr(gscale),
                               _ptr(gzero), _ptr(s_w), sw_stride, N, K, GROUP, _ptr(out),
                               out.stride(0), int(out_dtype), _ptr(workspace), wbytes, int(algo),
                               int(split_k), _stream())
@@ -385,19 +406,19 @@ def linear_static_scratch(x8, s_x, codes, gscale, gzero, s_w, out_dtype=OUT_BF16
 def linear_tiled(x8, s_x, tw, out_dtype=OUT_BF16, out=None, workspace=None):
     """w4a8_linear on a TiledWeight.  `workspace` must come from new_workspace (zero-filled once);
     one is created when none is given."""
-    import torch
-    M, K = x8.shape
-    assert K == tw.K
-    if out is None:
-        dt = torch.bfloat16 if out_dtype == OUT_BF16 else torch.float32
-        out = torch.empty((M, tw.N), dtype=dt, device=x8.device)
-    if workspace is None:
-        workspace = new_workspace(M, tw.N, K, tw.fmt, x8.device)
-    rc = lib().w4a8_linear(_ptr(x8), x8.stride(0), _ptr(s_x), M, _ptr(tw.buf), None, None, tw.fmt,
-                           _ptr(tw.s_w), 0 if tw.s_w.numel() == 1 else 1, tw.N, K, GROUP, _ptr(out),
-                           out.stride(0), int(out_dtype), _ptr(workspace),
-                           workspace.numel() * workspace.element_size(), _stream())
-    _check("w4a8_linear", rc)
+    if out is None or workspace is None:
+        import torch
+        M, K = x8.shape
+        assert K == tw.K
+        if out is None:
+            dt = torch.bfloat16 if out_dtype == OUT_BF16 else torch.float32
+            out = torch.empty((M, tw.N), dtype=dt, device=x8.device)
+        if workspace is None:
+            workspace = new_workspace(M, tw.N, K, tw.fmt, x8.device)
+    rc = (_host or _load_host()).linear(x8, s_x, tw.buf, None, None, tw.fmt, tw.s_w, tw.N, tw.K, GROUP, out, int(out_dtype),
+                                        workspace)
+    if rc != OK:
+        _check("w4a8_linear", rc)
     return out
 
 

@@ -1,4 +1,5 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a (no JIT cache, no torch extension)."""
+"""Builds the CUDA library in-tree with nvcc for sm_100a, and the binding's per-layer calls (a small
+extension module against torch's headers) with the host compiler.  No JIT cache."""
 from __future__ import annotations
 
 import os
@@ -8,11 +9,13 @@ import sys
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB_PATH = os.path.join(_HERE, "libw4a8_b200.so")
+HOST_PATH = os.path.join(_HERE, "_w4a8_host.so")
 SOURCES = [os.path.join(CSRC, "w4a8_lib.cu")]
+HOST_SOURCE = os.path.join(CSRC, "w4a8_host.cpp")
 
 
 def _deps():
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")]
     deps.append(os.path.join(os.path.dirname(_HERE), "include", "w4a8.h"))
     return deps
 
@@ -30,18 +33,44 @@ def nvcc_command(out_path: str, verbose: bool = False):
     return cmd + SOURCES + ["-lcudart"]
 
 
+def host_command(out_path: str):
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    return [
+        os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", "-fvisibility=hidden",
+        "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+        "-I" + os.path.join(root, "include"), "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"),
+        "-I" + os.path.join(cuda, "include"), "-I" + sysconfig.get_paths()["include"],
+        "-o", out_path, HOST_SOURCE,
+        "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda",
+        "-L" + _HERE, "-l:" + os.path.basename(LIB_PATH), "-Wl,-rpath,$ORIGIN",
+    ]
+
+
+def _run(cmd, out, tmp, what, verbose=False):
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose:
+        sys.stderr.write(res.stderr)
+    if res.returncode != 0:
+        raise RuntimeError(what + " failed:\n" + res.stdout + res.stderr)
+    os.replace(tmp, out)
+
+
+def _stale(out, deps):
+    return not os.path.exists(out) or any(os.path.getmtime(d) > os.path.getmtime(out) for d in deps)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile when the library is missing or older than a source. Returns the .so path."""
-    stale = force or not os.path.exists(LIB_PATH) or any(
-        os.path.getmtime(d) > os.path.getmtime(LIB_PATH) for d in _deps())
-    if stale:
+    """Compile what is missing or older than a source. Returns the CUDA library's path."""
+    if force or _stale(LIB_PATH, _deps()):
         tmp = LIB_PATH + ".tmp%d" % os.getpid()
-        res = subprocess.run(nvcc_command(tmp, verbose), capture_output=True, text=True)
-        if verbose:
-            sys.stderr.write(res.stderr)
-        if res.returncode != 0:
-            raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
-        os.replace(tmp, LIB_PATH)
+        _run(nvcc_command(tmp, verbose), LIB_PATH, tmp, "nvcc", verbose)
+    if force or _stale(HOST_PATH, [HOST_SOURCE, _deps()[-1]]):
+        tmp = HOST_PATH + ".tmp%d" % os.getpid()
+        _run(host_command(tmp), HOST_PATH, tmp, "g++")
     return LIB_PATH
 
 

@@ -132,3 +132,23 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(RuntimeError, match="no fallback"):
         binding.lib()
+
+
+def test_extension_module_marshals_and_refuses(L):
+    # sizes agree with the ctypes route; arguments that are not tensors, or not as many, raise; CPU tensors are refused
+    # before anything is launched; a status of the library comes back as one
+    import torch
+    h = binding._load_host()
+    for M, N, K, fmt in ((16, 14336, 4096, 0), (2048, 4096, 4096, 0), (5, 1024, 1024, 2), (16, 14336, 100, 0)):
+        assert h.linear_workspace_bytes(M, N, K, fmt) == int(L.w4a8_linear_workspace_bytes(M, N, K, fmt))
+    x = torch.zeros((4, 128), dtype=torch.bfloat16)
+    with pytest.raises(AssertionError):
+        h.quantize_act(x, x, x, 0, None)
+    with pytest.raises(TypeError):
+        h.quantize_act(x, 1, x, 0, None)
+    with pytest.raises(TypeError):
+        h.quantize_act(x)
+    x8 = torch.zeros((4, 128), dtype=torch.uint8)
+    s = torch.ones(1)
+    with pytest.raises(AssertionError):   # K differs
+        h.linear(x8, s, x8, None, None, binding.FMT_TILED, s, 16, 256, 128, s, 0, None)
