@@ -752,15 +752,15 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
             if (rc != W4A8_OK) return rc;
             if (M <= 64)
                 rc = fmt == kFmtTiledSignMag
-                         ? launch_cluster_kcut<SkCfg<64, 4, 8, 4, kFmtTiledSignMag, 1, false, true>>(
+                         ? launch_cluster_kcut<SkCfg<64, 4, 12, 12, kFmtTiledSignMag, 1, false, true>>(
                                x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st)
-                         : launch_cluster_kcut<SkCfg<64, 4, 8, 4, kFmtTiled, 1, false, true>>(
+                         : launch_cluster_kcut<SkCfg<64, 4, 12, 12, kFmtTiled, 1, false, true>>(
                                x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st);
             else
                 rc = fmt == kFmtTiledSignMag
-                         ? launch_cluster_kcut<SkCfg<128, 3, 6, 3, kFmtTiledSignMag, 1, false, true>>(
+                         ? launch_cluster_kcut<SkCfg<128, 4, 8, 8, kFmtTiledSignMag, 1, false, true>>(
                                x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st)
-                         : launch_cluster_kcut<SkCfg<128, 3, 6, 3, kFmtTiled, 1, false, true>>(
+                         : launch_cluster_kcut<SkCfg<128, 4, 8, 8, kFmtTiled, 1, false, true>>(
                                x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st);
             if (rc != -1) return rc;
         }
@@ -840,8 +840,8 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
              : launch_streamk<SkCfg<BNX, G, S1, S2, kFmtTiled>>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, \
                                                                 workspace, pl, Mi, Ni, Ki, st)
     switch (pl.bnx) {
-        case 64: W4A8_SK(64, 4, 8, 4); break;
-        case 128: W4A8_SK(128, 4, 4, 4); break;
+        case 64: W4A8_SK(64, 4, 12, 12); break;
+        case 128: W4A8_SK(128, 4, 8, 8); break;
         default: W4A8_SK(256, 4, 4, 3); break;
     }
 #undef W4A8_SK
@@ -867,9 +867,9 @@ static int linear_canonical_impl(const uint8_t* x8, int64_t ldx8, const float* s
     if (!make_tmap_u8_2d(&tw, codes, (uint64_t)N, (uint64_t)(K / 2), (uint64_t)(K / 2), 64, 128, CU_TENSOR_MAP_SWIZZLE_64B))
         return W4A8_ERR_CUDA;
     for (int cl = cluster_kcut_ctas(M, N, K, sms); cl >= 2; --cl) {
-        const int rc = M <= 64 ? launch_cluster_kcut<SkCfg<64, 4, 8, 4, kFmtCanonical, 1, false, true>>(
+        const int rc = M <= 64 ? launch_cluster_kcut<SkCfg<64, 4, 12, 12, kFmtCanonical, 1, false, true>>(
                                      x8, ldx8, gs, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st, &tw, gzero)
-                               : launch_cluster_kcut<SkCfg<128, 3, 6, 3, kFmtCanonical, 1, false, true>>(
+                               : launch_cluster_kcut<SkCfg<128, 4, 8, 8, kFmtCanonical, 1, false, true>>(
                                      x8, ldx8, gs, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st, &tw, gzero);
         if (rc != -1) return rc;
     }
@@ -901,8 +901,8 @@ static int linear_canonical_impl(const uint8_t* x8, int64_t ldx8, const float* s
     return launch_streamk<SkCfg<BNX, G, S1, S2, kFmtCanonical>>(tx, gs, s_x, s_w, sw_stride, y, ldy, out_dtype, nullptr, \
                                                                 pl, (int)M, (int)N, (int)K, st, &tw, 0, gzero)
     switch (pl.bnx) {
-        case 64: W4A8_SKC(64, 4, 8, 4);
-        case 128: W4A8_SKC(128, 4, 4, 4);
+        case 64: W4A8_SKC(64, 4, 12, 12);
+        case 128: W4A8_SKC(128, 4, 8, 8);
         default: W4A8_SKC(256, 4, 4, 3);
     }
 #undef W4A8_SKC

@@ -58,6 +58,17 @@ namespace w4a8 {
 // At 128 tokens a CTA exchanges 64 KB, which the SM-to-SM network moves in about 2.5 us (some
 // 25 bytes per clock and SM): little is gained there.  Needs no workspace.
 //
+// Token tiles of up to 128 (TA): the expanded weights go to tensor memory instead of shared memory, and the MMAs
+// take their A operand from there.  With a small token tile the A operand is as large as the B operand; written to and
+// read back from shared memory beside the copies in and the code reads, it made a 128 x 128 step move 82 KB through
+// shared memory.  What then paced a step was the requests and the issue themselves, so there one ring serves both (a
+// tensor-memory slot is free when its stage's weights have landed), one barrier per stage collects the expanding
+// threads' arrivals and the activation tile, one commit frees the stage, and a warp of its own requests the
+// activation tiles.  Measured, us (operand in shared memory / in tensor memory / with the single ring / and the extra
+// warp): (512, 4096, 4096) 17.4 16.0 15.5 13.0, (256, 6144, 4096) 17.6 15.6 15.0 12.6, K cut in clusters (17, 6144,
+// 4096) 10.3 9.7 8.8 8.5, (77, 4096, 14336) 17.7 16.8 16.5 14.3.  With 256-token tiles the extra warp gained nothing
+// ((2048, 4096, 4096) 32.3 / 32.6): there a step's eight (four) long MMAs cover the requests.
+//
 // FMT = canonical (weights as they are stored at the boundary, not prepacked): a TMA tile load of 64 bytes x 128 (256)
 // rows per k-block takes the place of the two bulk copies, and the expanding threads fetch their row's scale
 // and zero-point of a stage from the canonical arrays while they expand the stage before.  Whole tiles or
@@ -86,11 +97,14 @@ struct SkCfg {
     static constexpr int kWStage = RB_ * (CANON ? 8192 : 9216);  // rows x (64 code bytes + meta), padded to keep the activation tile 1024-aligned
     static constexpr int kXBytes = BNX * 128 * (W16_ ? 2 : 1);
     static constexpr int kStage1 = kWStage + kXBytes;
-    static constexpr int kW8Bytes = RB_ * 128 * 128 * (W16_ ? 2 : 1);   // expanded weights of one k-block: E4M3 (W16: BF16, two panels)
-    static constexpr int kBarBytes = 512;
+    // TA: expanded weights in tensor memory (see the kernel's comment); S2 slots of 32 columns behind the accumulators
+    static constexpr bool TA = !W8_ && !W16_ && RB_ == 1 && BNX_ <= 128;
+    static constexpr int kACol = 2 * BNX_;
+    static constexpr int kW8Bytes = TA ? 0 : RB_ * 128 * 128 * (W16_ ? 2 : 1);   // expanded weights of one k-block in shared memory: E4M3 (W16: BF16, two panels)
+    static constexpr int kBarBytes = 640;
     static constexpr int kSmemBytes = S1 * kStage1 + S2 * kW8Bytes + kBarBytes + 1024;
-    static constexpr int kTmemCols = 2 * BNX < 32 ? 32 : 2 * BNX;   // RB = 1: two accumulators (double buffer); RB = 2: one per row block
-    static constexpr int kThreads = 32 * (10 + 4 * G);
+    static constexpr int kTmemCols = TA ? 512 : (2 * BNX < 32 ? 32 : 2 * BNX);   // RB = 1: two accumulators (double buffer); RB = 2: one per row block
+    static constexpr int kThreads = 32 * (10 + 4 * G + (TA ? 1 : 0));   // (TA: a warp of its own requests the activation tiles)
     static constexpr int kSlotFloats = BNX * 128;
     static_assert(BNX == 16 || BNX == 32 || BNX == 64 || BNX == 128 || BNX == 256, "token tile");
     static_assert(RB_ == 1 || (RB_ == 2 && BNX_ == 256), "two row blocks per tile only with 256-token tiles");
@@ -99,7 +113,8 @@ struct SkCfg {
     static_assert(!CL_ || (RB_ == 1 && !W8_ && BNX_ <= 128), "the cluster exchange serves one row block and at most 128 tokens");
     // the exchange happens in the ring memory, idle by then in every CTA of the cluster: the CTA's own partial
     // tile (BNX columns x 128 channels, fp32) and behind it the slices it receives (C x ceil(BNX / C) columns)
-    static_assert(!CL_ || S1_ * (RB_ * 9216 + BNX_ * 128) + S2_ * RB_ * 16384 >= (2 * BNX_ + 8) * 512, "room for the exchange");
+    static_assert(!CL_ || S1_ * kStage1 + S2_ * kW8Bytes >= (2 * BNX_ + 8) * 512, "room for the exchange");
+    static_assert(!TA || (S1_ == S2_ && kACol + S2_ * 32 <= 512), "one ring; tensor memory columns");
     // A dequantization group handles every G-th stage, so it skips phases of the barriers it
     // waits on, and an mbarrier wait tells phases apart by parity only: the wait for use k of a
     // slot is sound only if use k-1 has completed before it starts.  That holds because a stage's
@@ -194,7 +209,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
         // barrier (W8: the TMA load), the draining threads on an "accumulator drained" barrier, one elsewhere
         for (int i = lane; i < kNumBars; i += 32) {
             uint32_t count = 1u;
-            if (i >= 2 * S1 && i < 2 * S1 + S2) count = Cfg::W8 ? 1u : 128u;
+            if (i >= 2 * S1 && i < 2 * S1 + S2) count = Cfg::W8 ? 1u : (Cfg::TA ? 129u : 128u);   // (TA: and the activation tile's request)
             if (i >= 2 * S1 + 2 * S2 + 2 && i < 2 * S1 + 2 * S2 + 4) count = RB == 2 ? 256u + 128u * G : 256u;   // (RB = 2: the expansion warps drain too)
             ptx::mbar_init(bars_addr + 8u * (uint32_t)i, count);
         }
@@ -415,7 +430,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                 if (it + 1 < ahead) continue;  // still inside the weight-only prologue
                 if (it + 1 == ahead) ptx::griddep_wait();
                 // activation tiles of every stage whose weights have been requested
-                for (; it_x <= it; ++it_x) {
+                for (; !Cfg::TA && it_x <= it; ++it_x) {
                     const uint32_t xfull = bar_xfull(rx.idx), xdst = stage_x(rx.idx);
                     const int x0 = xkb * (Cfg::W16 ? 256 : 128), y0 = xmt * BNX;   // (W16: X as bytes, 256 per k-block)
                     if (ptx::elect_one()) {
@@ -452,7 +467,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                                ptx::globaltimer_ns() - t0 < ptx::kWaitLimitNs) {
                         }
                     }
-                    const bool x_issued = issued - 1 - i < it_x;  // this stage's activation tile was requested too
+                    const bool x_issued = !Cfg::TA && issued - 1 - i < it_x;  // this stage's activation tile was requested too
                     while (x_issued && !ptx::mbar_try_wait(bar_xfull(rb.idx), rb.phase) &&
                            ptx::globaltimer_ns() - t0 < ptx::kWaitLimitNs) {
                     }
@@ -472,18 +487,19 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
             ptx::Ring r1, r2;
             int j = 0;
             int64_t u = u_begin;
-            {
+            if constexpr (!Cfg::TA) {
                 // The activation tiles of the first ring-full (every slot is free): requested here, while
                 // the producer warp requests the weights -- one lane after the other, the first
                 // activation tile went out only after the last of those, a microsecond late.
                 ptx::griddep_wait();
                 int xkb = kb_begin, xmt = (int)(tile_begin % TM);
                 for (int i = 0; i < n_it && i < S1; ++i) {
+                    const uint32_t xfull = bar_xfull(i);
                     if (ptx::elect_one()) {
-                        ptx::mbar_arrive_expect_tx(bar_xfull(i), (uint32_t)Cfg::kXBytes);
-                        ptx::tma_load_2d(stage_x(i), &tmap_x, xkb * (Cfg::W16 ? 256 : 128), xmt * BNX, bar_xfull(i));
+                        ptx::mbar_arrive_expect_tx(xfull, (uint32_t)Cfg::kXBytes);
+                        ptx::tma_load_2d(stage_x(i), &tmap_x, xkb * (Cfg::W16 ? 256 : 128), xmt * BNX, xfull);
                         if constexpr (Cfg::W16)
-                            ptx::tma_load_2d(stage_x(i) + (uint32_t)(BNX * 128), &tmap_x, xkb * 256 + 128, xmt * BNX, bar_xfull(i));
+                            ptx::tma_load_2d(stage_x(i) + (uint32_t)(BNX * 128), &tmap_x, xkb * 256 + 128, xmt * BNX, xfull);
                     }
                     if (++xkb == KB) {
                         xkb = 0;
@@ -505,7 +521,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                 const uint32_t tmem_acc = tmem_base + (uint32_t)(buf * BNX);
                 uint32_t accumulate = 0;
                 for (int i = 0; i < len; ++i) {
-                    ok = ptx::mbar_wait(bar_xfull(r1.idx), r1.phase, abort_flag, status_word);
+                    ok = Cfg::TA || ptx::mbar_wait(bar_xfull(r1.idx), r1.phase, abort_flag, status_word);
                     ok = ok && ptx::mbar_wait(bar_w8_full(r2.idx), r2.phase, abort_flag, status_word);
                     if (!ok) break;
                     ptx::tc_fence_after_sync();
@@ -522,6 +538,12 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                                                   (accumulate | (uint32_t)k) != 0u ? 1u : 0u);
                             ptx::umma_commit(f1);
                             ptx::umma_commit(f2);
+                        }
+                    } else if constexpr (Cfg::TA) {
+                        const uint32_t a_col = tmem_base + (uint32_t)(Cfg::kACol + r2.idx * 32);
+                        if (ptx::elect_one()) {
+                            ptx::umma_f8_kblock_ts(tmem_acc, a_col, b_lo, idesc, accumulate);
+                            ptx::umma_commit(f1);
                         }
                     } else if (ptx::elect_one()) {
                         ptx::umma_f8_kblock(tmem_acc, a_lo, b_lo, idesc, accumulate);
@@ -545,6 +567,43 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                 while (!ptx::mbar_try_wait(bar_drain, 0u) && ptx::globaltimer_ns() - t0 < ptx::kWaitLimitNs) {
                 }
             }
+        }
+        __syncwarp();
+        if constexpr (Cfg::CL) {
+            ptx::cluster_arrive();
+            cl_arrived = true;
+        }
+    } else if (Cfg::TA && warp == 10 + 4 * G) {
+        // ------------------------------------------------------------------ activation tiles (whole warp, one lane issues)
+        // (a stage's requests cost one lane some 600 cycles if it issues all of them)
+        bool ok = true;
+        int issued = 0;
+        ptx::Ring r;
+        int kb = kb_begin, mt = (int)(tile_begin % TM);
+        ptx::griddep_wait();
+        for (int it = 0; it < n_it; ++it) {
+            if (it >= S1) ok = ptx::mbar_wait(bar_free1(r.idx), r.phase ^ 1u, abort_flag, status_word);
+            if (!ok) break;
+            const uint32_t full = bar_w8_full(r.idx), dst = stage_x(r.idx);
+            if (ptx::elect_one()) {
+                ptx::mbar_arrive_expect_tx(full, (uint32_t)Cfg::kXBytes);
+                ptx::tma_load_2d(dst, &tmap_x, kb * 128, mt * BNX, full);
+            }
+            issued = it + 1;
+            r.advance(S1);
+            if (++kb == KB) {
+                kb = 0;
+                if (++mt == TM) mt = 0;
+            }
+        }
+        if (!ok && lane == 0) {
+            // Gave up: let the copies already in flight land.  The barriers count the expanding threads as well,
+            // which may have given up too, so this waits for a part of the limit only.
+            const uint64_t t0 = ptx::globaltimer_ns();
+            for (int it = issued > S1 ? issued - S1 : 0; it < issued; ++it)
+                while (!ptx::mbar_try_wait(bar_w8_full(it % S1), (uint32_t)((it / S1) & 1)) &&
+                       ptx::globaltimer_ns() - t0 < ptx::kWaitLimitNs / 20) {
+                }
         }
         __syncwarp();
         if constexpr (Cfg::CL) {
@@ -789,7 +848,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
         // ------------------------------------------------------------------ dequantization groups
         const int dw = warp - 10;
         const int g = dw >> 2;
-        const int r = (dw & 3) * 32 + lane;
+        const int r = (warp & 3) * 32 + lane;   // (a warp reaches the tensor-memory lanes of its quarter)
         // canonical: scale and zero-point of this thread's rows, fetched one of the group's stages ahead
         uint32_t meta[RB];
         int mkb = kb_begin + g, mnt = (int)(tile_begin / TM), mmt = (int)(tile_begin % TM);
@@ -816,8 +875,26 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
         for (int it = Cfg::W8 ? n_it : g; it < n_it; it += G) {   // (W8: nothing to expand)
             const int s1 = it % S1, s2 = it % S2;
             if (!ptx::mbar_wait(bar_full(s1), (uint32_t)((it / S1) & 1), abort_flag, status_word)) break;
-            if (it >= S2) {
+            // (TA: the packed weights of a stage are requested when the MMAs of the slot's previous stage have completed, so
+            // its tensor-memory slot is free once they have landed)
+            if (!Cfg::TA && it >= S2) {
                 if (!ptx::mbar_wait(bar_free2(s2), (uint32_t)((it / S2 - 1) & 1), abort_flag, status_word)) break;
+            }
+            if constexpr (Cfg::TA) {
+                const uint32_t a_col = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(Cfg::kACol + s2 * 32);
+                ptx::tc_fence_after_sync();
+                if constexpr (Cfg::CANON) {
+                    const uint32_t m = meta[0];
+                    next_meta(G);   // (past the last stage: a row that does not exist, or one that is not used)
+                    dequant_canonical_row_to_tmem(stage_w(s1), m, r, a_col);
+                } else {
+                    dequant_row_to_tmem<Cfg::FMT>(stage_w(s1) + tiled_row_offset(r),
+                                                  stage_w(s1) + (uint32_t)Cfg::kCodeBytes + (uint32_t)(r * Cfg::kMeta), a_col);
+                }
+                ptx::tmem_st_wait();
+                ptx::tc_fence_before_sync();
+                ptx::mbar_arrive(bar_w8_full(s2));
+                continue;
             }
             if constexpr (Cfg::W16)
                 dequant_row_to_smem_bf16(stage_w(s1) + tiled_row_offset(r), stage_w(s1) + (uint32_t)Cfg::kCodeBytes + (uint32_t)(r * Cfg::kMeta), r,

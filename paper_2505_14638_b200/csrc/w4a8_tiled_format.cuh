@@ -266,6 +266,18 @@ __device__ __forceinline__ void expand_row_to_tmem(const uint32_t (&pk)[16], uin
     }
 }
 
+// A row of a canonical tile (see dequant_canonical_row_to_smem) to tensor memory.
+__device__ __forceinline__ void dequant_canonical_row_to_tmem(uint32_t tile, uint32_t meta, int row, uint32_t taddr) {
+    const uint32_t sw64 = (uint32_t)((row >> 1) & 3), src = tile + (uint32_t)row * 64u;
+    uint32_t p[16];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(p[4 * j]), "=r"(p[4 * j + 1]), "=r"(p[4 * j + 2]), "=r"(p[4 * j + 3])
+                     : "r"(src + (((uint32_t)j ^ sw64) << 4)));
+    expand_row_to_tmem<kFmtTiled>(p, meta, taddr);
+}
+
 __device__ __forceinline__ uint32_t load_meta_word(uint32_t meta, int fmt) {
     uint32_t mbits;
     if (fmt == kFmtTiledSignMag)
