@@ -487,6 +487,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
             ptx::Ring r1, r2;
             int j = 0;
             int64_t u = u_begin;
+            if constexpr (Cfg::TA) ptx::griddep_wait();   // (its waits are bounded: the time earlier kernels take must not count)
             if constexpr (!Cfg::TA) {
                 // The activation tiles of the first ring-full (every slot is free): requested here, while
                 // the producer warp requests the weights -- one lane after the other, the first
