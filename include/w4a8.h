@@ -105,7 +105,7 @@ int w4a8_dequant_weight(const uint8_t* codes, const void* gscale_bf16, const uin
  * `workspace` holds fp32 partial tiles when the reduction over K is split between CTAs (they are
  * added in a fixed order: results repeat bit for bit).  Calls with M <= 128 on tiled
  * weights use it only for layers with few output channels and run without it, somewhat slower,
- * when it is NULL or too small; larger M requires it.  (With 17..128 tokens such layers normally
+ * when it is NULL or too small (up to 16 tokens K is then not cut at all); larger M requires it.  (With 17..128 tokens such layers normally
  * need none: the CTAs that share a tile form a thread-block cluster and exchange their partial
  * sums through shared memory, again added in a fixed order.)  It
  * needs w4a8_linear_workspace_bytes(M, N, K, weight_format) bytes and may be NULL when that is
@@ -204,9 +204,8 @@ int w4a8_linear_static_scratch(const uint8_t* x8, int64_t ldx8, const float* s_x
  *   in_i = BF16( silu(G) * U ), G|U = x_i        (W4A8_CHAIN_INPUT_SILU_MUL: x_i has 2 K columns, gate
  *                                                 first, exactly as w4a8_silu_mul_quantize defines it),
  * and the results are those of w4a8_quantize_act (or w4a8_silu_mul_quantize) followed by
- * w4a8_linear on the same tiled weights with K not cut (layers with at least 96 output channels per
- * SM; smaller ones w4a8_linear may cut along K): same scales, same FP8 codes, same
- * accumulation order -- for the output channels whose K range one CTA walks alone; where the chain
+ * w4a8_linear on the same tiled weights with K not cut (called without a workspace): same scales,
+ * same FP8 codes, same accumulation order -- for the output channels whose K range one CTA walks alone; where the chain
  * cuts K (see below) the FP32 partial sums are added in a fixed order, so results still repeat bit
  * for bit from call to call, and agree with w4a8_linear within its output tolerance.  Problems run
  * in array order on one grid of one CTA per SM that stays resident for the whole chain; the packed

@@ -344,6 +344,11 @@ static_assert(kSnCounterBytes == (size_t)kSchedWsOffset, "the kernel finds the p
 static_assert(kLinearCtlSplitN + kSnCounterBytes + kSnSchedBytes == kLinearCtlBytes, "split-N control data at the end of the common control area");
 constexpr size_t kSnWorkspaceBytes = kLinearCtlBytes + (size_t)kMaxSMs * 128 * 128 * sizeof(float);
 
+// K is cut only when the caller gave the (zero-initialised) workspace for the partial sums.
+static bool sn_workspace_usable(const void* workspace, size_t bytes) {
+    return workspace != nullptr && bytes >= kSnWorkspaceBytes && aligned16(workspace);
+}
+
 template <class Cfg>
 static bool make_sn_plan(int64_t N, int64_t K, int sms, bool may_split_k, SnPlan* pl) {
     const int64_t NU = N / 8;
@@ -406,8 +411,7 @@ static int launch_splitn_cfg(const CUtensorMap& tx, const uint8_t* wpp, const fl
     const int sms = sm_count();
     if (sms <= 0) return W4A8_ERR_CUDA;
     SnPlan pl;
-    // K is cut only when the caller gave the (zero-initialised) workspace for the partial sums
-    const bool ws_usable = workspace != nullptr && workspace_bytes >= kSnWorkspaceBytes && aligned16(workspace);
+    const bool ws_usable = sn_workspace_usable(workspace, workspace_bytes);
     if (!make_sn_plan<Cfg>(N, K, sms, ws_usable, &pl)) return W4A8_ERR_BAD_SHAPE;
     if (pl.KSPLIT > 1)
         return launch_splitn_planned<SnCfg<MT, G, FMT, true>>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K,
@@ -730,7 +734,9 @@ static int launch_direct(const uint8_t* x8, int64_t ldx8, const float* s_x, int6
 static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* wpp,
                              int fmt, const float* s_w, int sw_stride, int64_t N, int64_t K, void* y, int64_t ldy,
                              int out_dtype, void* workspace, size_t workspace_bytes, cudaStream_t st) {
-    if (M <= 16) {
+    if (M <= 16 && sn_workspace_usable(workspace, workspace_bytes)) {
+        // (linear_direct_kernel cuts K between the warps of a CTA.  Without a workspace K is never cut, which is how a
+        // caller asks for the bits of a chain launch.)
         const int rc = check_device();
         if (rc != W4A8_OK) return rc;
         const int sms_d = sm_count();

@@ -114,6 +114,21 @@ def test_whole_blocks_match_the_per_launch_path_bit_for_bit():
         assert worst <= 2e-3, (rounds, worst)
 
 
+@pytest.mark.parametrize("M,N,K", [(16, 2064, 512), (5, 1040, 384), (8, 4096, 512), (1, 1024, 128)])
+@pytest.mark.parametrize("asym", [False, True])
+def test_small_layers_whose_k_the_chain_does_not_cut_match_bit_for_bit(M, N, K, asym):
+    # up to four k-blocks: a run of k-blocks is a whole 96-row block, walked by one CTA; without a workspace
+    # w4a8_linear cuts no K either, however small the layer
+    _, tw = _weights(N, K, N + K, asym)
+    x = bf16_dev(inputs.make_activation(M, K, M + K, 0.01, 20.0))
+    y = torch.zeros((M, N), dtype=torch.float32, device="cuda")
+    binding.LinearChain([dict(x=x, weight=tw, y=y)])()
+    want = _per_launch(x, tw, binding.OUT_FP32)
+    torch.cuda.synchronize()
+    assert binding.query_device_status() == 0
+    assert torch.equal(y.view(torch.int32), want.view(torch.int32))
+
+
 def test_dependent_chain_and_gated_block():
     # x -> gate_up (BF16) -> silu(gate) * up quantized in the chain -> down (BF16) -> next layer on
     # the down projection's output: every hand-over goes through the chain's counters.  Each stage is
