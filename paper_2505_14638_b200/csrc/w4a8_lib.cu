@@ -692,24 +692,65 @@ static int64_t make_direct_plan(int64_t N, int64_t K, int sms, DirPlan* plan) {
     return best;
 }
 
-// Small layers at up to sixteen tokens, where the latencies of a launch outweigh the weights: at most two units of
-// work per warp, and no more weights than this kernel's expansion -- whose FP8 fragments the hardware converts to
-// 16 bits for the MMA, on the pipe that expands -- keeps up with.  Measured (us, linear alone, this kernel / the
-// split-N kernel, canonical: the kernel of one tile per CTA):
-//   sign-magnitude M = 8: (1024, 1024) 3.4 / 6.3, (4096, 1024) 3.6 / 6.6, (4096, 4096) 6.8 / 7.6, (6144, 4096) 8.3 / 9.3,
-//   (28672, 4096) 22 / 17.5; M = 1: (2048, 2048) 3.3 / 5.4, (4096, 4096) 6.5 / 6.5; M = 16: (6144, 4096) 9.8 / 10.7
-//   generic M = 8: (1024, 1024) 3.5 / 6.4, (6144, 4096) 9.4 / 10.2; M = 1: (2048, 2048) 3.6 / 5.4, (1536, 8192) 7.4 / 6.4;
-//   M = 16: (4096, 4096) 8.8 / 9.2, (6144, 4096) 11.3 / 11.4
-//   canonical M = 8: (1024, 1024) 3.5 / 8.4, (6144, 4096) 11.0 / 13.2; M = 16: (2048, 2048) 4.9 / 8.6, (1536, 8192) 10.1 / 10.0,
-//   (6144, 4096) 12.7 / 13.7
-//   24 tokens: level at (1024, 1024), slower everywhere else.
+// Layers at up to sixteen tokens for which the kernel above is the faster one: by and large those whose K the split-N
+// kernel would cut (see make_sn_plan), which costs it an exchange, up to a number of weights that this kernel's
+// expansion keeps up with (its FP8 fragments are converted to 16 bits for the MMA on the pipe that expands).  Time of
+// this kernel over that of the split-N kernel, activation quantization and linear layer back to back, weights not in L2,
+// sign-magnitude (generic) format; at M = 8 (1024, 1024) takes 7.5 us there and 4.3 here, (4096, 4096) 9.2 and 8.8:
+//   (N, K)          M = 4          M = 8          M = 9          M = 16
+//   (2048, 128)     0.96 (0.98)    1.05 (1.03)    1.05 (1.19)    1.17 (1.29)    K not cut
+//   (2048, 512)     0.91 (0.97)    1.04 (1.03)    1.13 (1.20)    1.25 (1.30)    K not cut
+//   (2048, 896)     0.81 (0.90)    0.91 (0.90)    1.01 (1.03)    1.10 (1.14)    K not cut
+//   (6144, 896)     0.93 (0.98)    0.97 (1.03)    1.08 (1.17)    1.19 (1.26)    K not cut
+//   (9472, 1536)    0.86 (0.94)    0.82 (0.91)    0.88 (0.98)    0.82 (0.89)
+//   (8192, 2048)    0.87 (0.91)    0.87 (0.91)    0.96 (1.01)    0.97 (1.00)
+//   (9472, 2048)    1.00 (1.06)    0.95 (1.01)    1.05           0.94
+//   (8192, 2560)    0.90 (0.95)    0.91 (0.94)    1.00           1.00
+//   (5120, 2560)    0.86 (0.94)    0.82 (0.88)    0.89 (0.97)    0.90 (0.96)
+//   (4096, 3072)    0.82 (0.91)    0.86 (0.93)    0.96 (1.02)    1.02 (1.08)
+//   (6144, 3072)    1.02 (1.13)    1.00 (1.09)    1.11           1.06
+//   (4096, 4096)    0.96 (0.99)    0.96 (1.02)    1.07 (1.13)    1.04 (1.13)
+//   (5120, 4096)    0.91 (0.88)    0.90 (0.88)    1.03           1.02
+//   (1552, 7168)    0.88 (0.96)    0.85 (0.96)    0.94 (1.04)    0.84 (0.89)
+//   (2048, 7168)    0.96 (1.04)    0.90 (1.00)    1.01 (1.08)    0.96 (1.03)
+//   (3072, 7168)    1.05 (1.09)    1.01 (1.06)    1.12           1.04
+//   (1552, 8192)    0.92 (1.02)    0.91 (0.98)    1.01 (1.11)    0.91 (0.97)
+//   (1296, 11008)   1.04 (1.17)    1.04 (1.11)    1.16 (1.27)
+//   (12288, 1024)   1.21 (1.30)    1.26 (1.28)    1.38 (1.46)    1.42 (1.46)    K not cut
+//   (12288, 1536)   1.33 (1.37)    1.43 (1.41)    1.61           1.64           K not cut
+//   (10240, 2048)   0.82 (0.89)    0.87 (0.95)    1.02           1.00           K not cut, candidates placed at run time
+//   (12288, 2048)   0.87 (1.00)    0.92 (1.05)    1.06           1.12           the same
+// M = 1: (2048, 512) 0.89 (0.93), (1024, 7168) 0.84 (0.90).  Canonical, against the kernel of one tile per CTA: M = 8
+// (1024, 1024) 0.46, (6144, 4096) 0.87, (12288, 2048) 0.81; M = 16 (6144, 4096) 0.98, (2048, 8192) 1.05; (1552, 14336) M = 4
+// 1.01, M = 8 1.05, M = 9 1.15; (4096, 6144) M = 12 1.06.  24 tokens: level at (1024, 1024), slower everywhere else.
 // Prepacked layers with a 96-row block for every SM keep the kernel that walks all of K in one chain of MMAs: a chain launch
 // gives the same bits there.
 static bool direct_applies(int64_t M, int64_t N, int64_t K, int fmt, int sms, DirPlan* plan) {
-    if (fmt != kFmtCanonical && N >= (int64_t)96 * sms) return false;
     if (M > 16 || N < 1024 || direct_smem(M, K, M <= 8 ? 1 : 2) > (size_t)kDirMaxSmem) return false;
-    const int64_t most = fmt == kFmtCanonical ? 26 : (M < 4 ? 8 : (fmt == kFmtTiled && M > 8 ? 17 : 26));
-    return N * K <= most * 1000000 && make_direct_plan(N, K, sms, plan) <= 2;
+    if (make_direct_plan(N, K, sms, plan) > 2) return false;
+    const int64_t weights = N * K;
+    const bool sm = fmt == kFmtTiledSignMag, few = M <= 8;
+    if (fmt == kFmtCanonical) return weights <= (few || K <= 4096 || K > 8192 ? 26 : 16) * (int64_t)1000000 && (K <= 11008 || M <= 4);
+    const int64_t blocks = (N + 127) / 128;
+    int64_t most;   // million weights
+    if (K < 1024) {                       // the split-N kernel does not cut K
+        if (M <= 4 ? !(sm ? N <= 8192 : K >= 512 && N <= 4096) : !(few && K > 512 && N <= (sm ? 6144 : 4096))) return false;
+        most = 8;
+    } else if (2 * blocks > sms) {        // nor here
+        if (K < 2048 || M < 4 || !few || N >= (int64_t)96 * sms) return false;
+        most = sm ? 26 : 24;
+    } else if (M < 4) {
+        most = 8;
+    } else if (K <= 2048) {
+        most = sm ? 20 : (few ? 17 : 15);
+    } else if (sm) {
+        if (K <= 4096) most = few ? 26 : (K <= 2560 ? 21 : 13);
+        else most = K <= 7168 ? 15 : (K <= 8192 ? 13 : 0);
+    } else {
+        if (few && K <= 6144 && blocks * (sms / blocks) < sms * 7 / 8) most = 26;   // the cut leaves an eighth of the SMs idle
+        else most = K <= 7168 ? (few ? 13 : (K <= 3072 ? 12 : 14)) : 0;
+    }
+    return weights <= most * 1000000;
 }
 
 static int launch_direct(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* w,
