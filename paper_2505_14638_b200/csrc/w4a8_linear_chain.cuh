@@ -200,6 +200,10 @@ __device__ __forceinline__ bool chain_mbar_wait(uint32_t bar, uint32_t parity, v
         if (ptx::mbar_try_wait(bar, parity)) return true;
         if ((++spins & 63u) == 0u) {
             if (*abort_flag) return false;
+            if (spins == ptx::kWaitAlone) {   // (see ptx::mbar_wait)
+                ptx::griddep_wait();
+                t0 = 0;
+            }
             const uint64_t now = ptx::globaltimer_ns();
             if (t0 == 0) {
                 t0 = now;
@@ -451,9 +455,6 @@ linear_chain_kernel(const __grid_constant__ ChainParams prm, uint8_t* __restrict
                 const uint8_t* mptr = q.wpp + (int64_t)KB * code_step + (int64_t)sg.kb0 * meta_step + (int64_t)sg.n0 * MB;
                 const uint32_t meta_off = (uint32_t)KS * cbytes;
                 for (int kb = 0; kb < sg.nkb;) {
-                    // (Slots are freed by the expansion, of which the first S2 stages need nothing of an earlier kernel and the
-                    // others wait for MMAs: from there on the time earlier kernels take must not count against the limit.)
-                    if (issued == S1 + S2) ptx::griddep_wait();
                     ok = warp_all(chain_mbar_wait(bar_wfree0 + 8u * (uint32_t)r1.idx, r1.phase ^ 1u, abort_flag, gabort,
                                                   status_word, limit));
                     if (!ok) break;
@@ -504,7 +505,6 @@ linear_chain_kernel(const __grid_constant__ ChainParams prm, uint8_t* __restrict
         const uint32_t b_lo0 = ptx::umma_desc_lo(x_ring);
         constexpr uint32_t b_step = (uint32_t)(2 * kChainXTileBytes) >> 4;
         constexpr uint32_t idesc = ptx::umma_idesc_e4m3_f32(128, kChainMaxM);
-        ptx::griddep_wait();   // (its waits are bounded: the time earlier kernels take must not count)
         for (int i = 0; i < count && ok; ++i) {
             const ChainProblem& q = prm.prob[i];
             const int nseg = nseg_tab[i];
@@ -934,7 +934,6 @@ linear_chain_kernel(const __grid_constant__ ChainParams prm, uint8_t* __restrict
         r1.idx = g;   // (G <= S2 <= S1)
         r2.idx = g;
         int turn = g;  // stages until this group's next turn
-        bool waited = false;
         bool ok = true;
         for (int i = 0; i < count && ok; ++i) {
             const ChainProblem& q = prm.prob[i];
@@ -998,9 +997,6 @@ linear_chain_kernel(const __grid_constant__ ChainParams prm, uint8_t* __restrict
                     if (r2.idx >= S2) {
                         r2.idx -= S2;
                         r2.phase ^= 1u;
-                        // (from the second round of the ring on a stage waits for MMAs: the time earlier kernels take must not count)
-                        if (!waited) ptx::griddep_wait();
-                        waited = true;
                     }
                 }
                 turn = st - nst;

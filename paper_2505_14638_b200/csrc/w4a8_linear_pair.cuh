@@ -176,7 +176,6 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
             constexpr uint32_t idesc = ptx::umma_idesc_e4m3_f32(256, BNX);
             bool ok = true;
             ptx::Ring r1, r2;
-            ptx::griddep_wait();   // (its waits are bounded: the time earlier kernels take must not count)
             for (int j = 0; j < n_tiles && ok; ++j) {
                 const int buf = j & 1;
                 if (j >= 2) {
@@ -271,7 +270,6 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
         const int r = (dw & 3) * 32 + lane;
         for (int it = g; it < n_it; it += G) {
             const int s1 = it % S1, s2 = it % S2;
-            if (it >= S2 && it - G < S2) ptx::griddep_wait();   // (these waits are for MMAs: the time earlier kernels take must not count)
             if (!ptx::mbar_wait(bar_full(s1), (uint32_t)((it / S1) & 1), abort_flag, status_word)) break;
             if (it >= S2) {
                 if (!ptx::mbar_wait(bar_free2(s2), (uint32_t)((it / S2 - 1) & 1), abort_flag, status_word)) break;

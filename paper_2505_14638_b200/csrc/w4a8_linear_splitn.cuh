@@ -463,7 +463,6 @@ linear_splitn_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K
             constexpr uint32_t idesc = ptx::umma_idesc_e4m3_f32(128, MT);
             const uint32_t d0 = tmem_base + (uint32_t)Cfg::kDCol;
             bool first_tile = true;
-            ptx::griddep_wait();   // (its waits are bounded: the time earlier kernels take must not count)
             for (int t = p; t < T && ok; t += P) {
                 if (!first_tile) {
                     ok = ptx::mbar_wait(bar_acc_empty, acc_phase, abort_flag, status_word);
@@ -626,9 +625,6 @@ linear_splitn_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K
                 // round, a group ahead of a late copy could pass one phase early.)
                 const uint32_t full_bar = bar_full0 + 8u * (uint32_t)r1.idx;
                 const uint32_t free_bar = bar_free10 + 8u * (uint32_t)rl.idx;
-                // (Only the first S2 stages of the first tile need nothing of an earlier kernel.  The others wait for
-                // MMAs, or for weights requested after activations: the time earlier kernels take must not count.)
-                if (done >= S2 || t != p) ptx::griddep_wait();
                 if (done >= S2 && !ptx::mbar_test_wait(free_bar, rl.phase))
                     ok = ptx::mbar_wait(free_bar, rl.phase, abort_flag, status_word);
                 if (ok && !ptx::mbar_test_wait(full_bar, r1.phase))

@@ -487,7 +487,6 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
             ptx::Ring r1, r2;
             int j = 0;
             int64_t u = u_begin;
-            if constexpr (Cfg::TA) ptx::griddep_wait();   // (its waits are bounded: the time earlier kernels take must not count)
             if constexpr (!Cfg::TA) {
                 // The activation tiles of the first ring-full (every slot is free): requested here, while
                 // the producer warp requests the weights -- one lane after the other, the first
@@ -873,13 +872,8 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
             ptx::griddep_wait();
             next_meta(0);
         }
-        // From this stage on a group waits for MMAs (a slot to free, or weights requested once one is free), and those
-        // wait for earlier kernels: these are waited for first, or their run time would count against the limit
-        // of the waits.
-        constexpr int kFirstDep = Cfg::TA || S1 < S2 ? S1 : S2;
         for (int it = Cfg::W8 ? n_it : g; it < n_it; it += G) {   // (W8: nothing to expand)
             const int s1 = it % S1, s2 = it % S2;
-            if (it >= kFirstDep && it - G < kFirstDep) ptx::griddep_wait();
             if (!ptx::mbar_wait(bar_full(s1), (uint32_t)((it / S1) & 1), abort_flag, status_word)) break;
             // (TA: the packed weights of a stage are requested when the MMAs of the slot's previous stage have completed, so
             // its tensor-memory slot is free once they have landed)
