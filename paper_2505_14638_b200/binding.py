@@ -201,6 +201,25 @@ def _check(fn, rc):
         raise W4A8Error(fn, rc)
 
 
+# The extension module reads torch tensors.  Buffers of another kind that know their data_ptr(), shape and
+# stride() -- a wrapper, another library's array -- take the ctypes route.
+def _quantize_act_any(x, x8, s_x, scale_mode, static_scale):
+    import torch
+    assert x.is_cuda and x.dtype == torch.bfloat16 and x.dim() == 2 and x.stride(1) == 1
+    M, K = x.shape
+    return lib().w4a8_quantize_act(_ptr(x), M, K, x.stride(0), _ptr(x8), x8.stride(0), _ptr(s_x), int(scale_mode),
+                                   _ptr(static_scale), _stream())
+
+
+def _linear_any(x8, s_x, w, gscale, gzero, fmt, s_w, N, K, out, out_dtype, workspace):
+    M, Kx = x8.shape
+    assert Kx == K
+    return lib().w4a8_linear(_ptr(x8), x8.stride(0), _ptr(s_x), M, _ptr(w), _ptr(gscale), _ptr(gzero), int(fmt), _ptr(s_w),
+                             0 if s_w.numel() == 1 else 1, N, K, GROUP, _ptr(out), out.stride(0), int(out_dtype),
+                             _ptr(workspace), 0 if workspace is None else workspace.numel() * workspace.element_size(),
+                             _stream())
+
+
 def quantize_act(x, scale_mode=SCALE_EXACT, static_scale=None, out=None):
     """w4a8_quantize_act: x BF16 [M, K] (row stride in elements = x.stride(0)).
     Returns (x8 uint8 [M, K], s_x float32 [M])."""
@@ -211,7 +230,11 @@ def quantize_act(x, scale_mode=SCALE_EXACT, static_scale=None, out=None):
         out = (torch.empty((M, K), dtype=torch.uint8, device=x.device),
                torch.empty((M,), dtype=torch.float32, device=x.device))
     x8, s_x = out
-    rc = (_host or _load_host()).quantize_act(x, x8, s_x, int(scale_mode), static_scale)
+    host = _host or _load_host()
+    try:
+        rc = host.quantize_act(x, x8, s_x, int(scale_mode), static_scale)
+    except TypeError:
+        rc = _quantize_act_any(x, x8, s_x, scale_mode, static_scale)
     if rc != OK:
         _check("w4a8_quantize_act", rc)
     return x8, s_x
@@ -368,7 +391,10 @@ def linear(x8, s_x, codes, gscale, gzero, s_w, out_dtype=OUT_BF16, out=None, wor
         import torch
         workspace = torch.empty((need,), dtype=torch.uint8, device=x8.device)
     if auto:
-        rc = host.linear(x8, s_x, codes, gscale, gzero, FMT_CANONICAL, s_w, N, K, GROUP, out, int(out_dtype), workspace)
+        try:
+            rc = host.linear(x8, s_x, codes, gscale, gzero, FMT_CANONICAL, s_w, N, K, GROUP, out, int(out_dtype), workspace)
+        except TypeError:
+            rc = _linear_any(x8, s_x, codes, gscale, gzero, FMT_CANONICAL, s_w, N, K, out, out_dtype, workspace)
         if rc != OK:
             _check("w4a8_linear", rc)
     else:
@@ -415,8 +441,11 @@ def linear_tiled(x8, s_x, tw, out_dtype=OUT_BF16, out=None, workspace=None):
             out = torch.empty((M, tw.N), dtype=dt, device=x8.device)
         if workspace is None:
             workspace = new_workspace(M, tw.N, K, tw.fmt, x8.device)
-    rc = (_host or _load_host()).linear(x8, s_x, tw.buf, None, None, tw.fmt, tw.s_w, tw.N, tw.K, GROUP, out, int(out_dtype),
-                                        workspace)
+    host = _host or _load_host()
+    try:
+        rc = host.linear(x8, s_x, tw.buf, None, None, tw.fmt, tw.s_w, tw.N, tw.K, GROUP, out, int(out_dtype), workspace)
+    except TypeError:
+        rc = _linear_any(x8, s_x, tw.buf, None, None, tw.fmt, tw.s_w, tw.N, tw.K, out, out_dtype, workspace)
     if rc != OK:
         _check("w4a8_linear", rc)
     return out

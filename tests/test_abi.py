@@ -152,3 +152,35 @@ def test_extension_module_marshals_and_refuses(L):
     s = torch.ones(1)
     with pytest.raises(AssertionError):   # K differs
         h.linear(x8, s, x8, None, None, binding.FMT_TILED, s, 16, 256, 128, s, 0, None)
+
+
+class _Wrapped:
+    """A buffer that is not a torch tensor: what it knows it asks the tensor it holds."""
+
+    def __init__(self, t):
+        self._t = t
+
+    def __getattr__(self, name):
+        return getattr(self._t, name)
+
+
+def test_buffers_that_are_not_torch_tensors_reach_the_library(L, monkeypatch):
+    # (addresses that are not 16-byte aligned: the library refuses them before it touches a device)
+    import torch
+    monkeypatch.setattr(binding, "_stream", lambda: None)
+    raw = torch.zeros(4 * 128 + 32, dtype=torch.uint8)
+    at = 1 + (-raw.data_ptr()) % 16
+    x8, s, out = raw[at:at + 4 * 128].view(4, 128), torch.ones(4), torch.zeros((4, 16), dtype=torch.bfloat16)
+    w = torch.zeros(16 * 128, dtype=torch.uint8)
+    tw = binding.TiledWeight(_Wrapped(w), binding.FMT_TILED, 16, 128, _Wrapped(torch.ones(1)))
+    codes, gs = _Wrapped(torch.zeros((16, 64), dtype=torch.uint8)), _Wrapped(torch.ones((16, 1), dtype=torch.bfloat16))
+    for call in (lambda: binding.linear_tiled(_Wrapped(x8), _Wrapped(s), tw, out=_Wrapped(out), workspace=_Wrapped(raw)),
+                 lambda: binding.linear(_Wrapped(x8), _Wrapped(s), codes, gs, None, _Wrapped(s[:1]), out=_Wrapped(out),
+                                        workspace=_Wrapped(torch.zeros(1 << 20, dtype=torch.uint8)))):
+        with pytest.raises(binding.W4A8Error) as e:
+            call()
+        assert binding.status_string(binding.ERR_BAD_ALIGNMENT) in str(e.value)
+    with pytest.raises(AssertionError):      # not on the device
+        binding.quantize_act(_Wrapped(torch.zeros((4, 128), dtype=torch.bfloat16)), out=(_Wrapped(x8), _Wrapped(s)))
+    with pytest.raises(AttributeError):      # not a buffer at all
+        binding.linear_tiled(3, s, tw, out=out, workspace=raw)
