@@ -1,5 +1,6 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a, and the binding's per-layer calls (a small
-extension module against torch's headers) with the host compiler.  No JIT cache."""
+"""Builds the CUDA library in-tree with nvcc for sm_100a, and, where torch is installed, the binding's per-layer
+calls (a small extension module against torch's headers) with the host compiler.  No JIT cache.
+`--library-only` builds the C-ABI library alone, which needs nvcc and nothing else."""
 from __future__ import annotations
 
 import os
@@ -63,11 +64,28 @@ def _stale(out, deps):
     return not os.path.exists(out) or any(os.path.getmtime(d) > os.path.getmtime(out) for d in deps)
 
 
-def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile what is missing or older than a source. Returns the CUDA library's path."""
+def _has_torch():
+    try:
+        import torch  # noqa: F401
+    except ImportError:
+        return False
+    return True
+
+
+def build_library(force: bool = False, verbose: bool = False) -> str:
+    """The C-ABI library alone."""
     if force or _stale(LIB_PATH, _deps()):
         tmp = LIB_PATH + ".tmp%d" % os.getpid()
         _run(nvcc_command(tmp, verbose), LIB_PATH, tmp, "nvcc", verbose)
+    return LIB_PATH
+
+
+def build(force: bool = False, verbose: bool = False) -> str:
+    """Compile what is missing or older than a source. Returns the CUDA library's path."""
+    build_library(force, verbose)
+    if not _has_torch():
+        sys.stderr.write("torch is not installed: the C library is complete, the Python binding's extension module is not built\n")
+        return LIB_PATH
     if force or _stale(HOST_PATH, [HOST_SOURCE, _deps()[-1]]):
         tmp = HOST_PATH + ".tmp%d" % os.getpid()
         _run(host_command(tmp), HOST_PATH, tmp, "g++")
@@ -75,4 +93,5 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 
 if __name__ == "__main__":
-    print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))
+    make = build_library if "--library-only" in sys.argv else build
+    print(make(force="--force" in sys.argv, verbose="-v" in sys.argv))

@@ -3,6 +3,7 @@ rejects bad arguments before touching a device (no GPU needed)."""
 import ctypes
 import os
 import re
+import sys
 
 import pytest
 
@@ -184,3 +185,12 @@ def test_buffers_that_are_not_torch_tensors_reach_the_library(L, monkeypatch):
         binding.quantize_act(_Wrapped(torch.zeros((4, 128), dtype=torch.bfloat16)), out=(_Wrapped(x8), _Wrapped(s)))
     with pytest.raises(AttributeError):      # not a buffer at all
         binding.linear_tiled(3, s, tw, out=out, workspace=raw)
+
+
+def test_the_c_library_builds_without_torch(L, monkeypatch, tmp_path):
+    # (the library itself is there; the extension module would have to be built)
+    monkeypatch.setattr(build, "HOST_PATH", str(tmp_path / "_w4a8_host.so"))
+    monkeypatch.setattr(build, "host_command", lambda out: pytest.fail("needs torch"))
+    monkeypatch.setitem(sys.modules, "torch", None)      # import torch raises ImportError
+    assert build.build() == build.LIB_PATH
+    assert not os.path.exists(build.HOST_PATH)
