@@ -34,6 +34,12 @@ def nvcc_command(out_path: str, verbose: bool = False):
     return cmd + SOURCES + ["-lcudart"]
 
 
+def host_versions() -> str:
+    """What the extension module is compiled against; it carries this text."""
+    import torch
+    return "torch %s, Python %d.%d" % (torch.__version__, sys.version_info[0], sys.version_info[1])
+
+
 def host_command(out_path: str):
     import sysconfig
 
@@ -43,6 +49,7 @@ def host_command(out_path: str):
     return [
         os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", "-fvisibility=hidden",
         "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+        '-DW4A8_HOST_VERSIONS="%s"' % host_versions(),
         "-I" + os.path.join(root, "include"), "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"),
         "-I" + os.path.join(cuda, "include"), "-I" + sysconfig.get_paths()["include"],
         "-o", out_path, HOST_SOURCE,
@@ -62,6 +69,11 @@ def _run(cmd, out, tmp, what, verbose=False):
 
 def _stale(out, deps):
     return not os.path.exists(out) or any(os.path.getmtime(d) > os.path.getmtime(out) for d in deps)
+
+
+def _built_against(path, versions):
+    with open(path, "rb") as f:
+        return (versions + "\0").encode() in f.read()
 
 
 def _has_torch():
@@ -86,7 +98,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not _has_torch():
         sys.stderr.write("torch is not installed: the C library is complete, the Python binding's extension module is not built\n")
         return LIB_PATH
-    if force or _stale(HOST_PATH, [HOST_SOURCE, _deps()[-1]]):
+    if force or _stale(HOST_PATH, [HOST_SOURCE, _deps()[-1]]) or not _built_against(HOST_PATH, host_versions()):
         tmp = HOST_PATH + ".tmp%d" % os.getpid()
         _run(host_command(tmp), HOST_PATH, tmp, "g++")
     return LIB_PATH

@@ -118,7 +118,8 @@ PyMethodDef methods[] = {
     {"linear", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(linear)), METH_FASTCALL, nullptr},
     {"linear_workspace_bytes", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(linear_workspace_bytes)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
-PyModuleDef module = {PyModuleDef_HEAD_INIT, "_w4a8_host", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+// (the versions that it was compiled against: the build looks for them and compiles again for others)
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_w4a8_host", W4A8_HOST_VERSIONS, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
 

@@ -194,3 +194,15 @@ def test_the_c_library_builds_without_torch(L, monkeypatch, tmp_path):
     monkeypatch.setitem(sys.modules, "torch", None)      # import torch raises ImportError
     assert build.build() == build.LIB_PATH
     assert not os.path.exists(build.HOST_PATH)
+
+
+def test_the_extension_module_is_built_again_for_another_torch(L, monkeypatch):
+    import torch
+    assert torch.__version__ in binding._load_host().__doc__
+    built = []
+    monkeypatch.setattr(build, "_run", lambda cmd, out, *a: built.append(out))
+    build.build()
+    assert built == []
+    monkeypatch.setattr(torch, "__version__", "99.0")
+    build.build()
+    assert built == [build.HOST_PATH]
