@@ -753,6 +753,14 @@ static bool direct_applies(int64_t M, int64_t N, int64_t K, int fmt, int sms, Di
     return weights <= most * 1000000;
 }
 
+// Canonical weights, kernel chosen by the library: whether linear_umma_kernel runs, whose K cut needs the caller's
+// workspace.  The kernels that take its place need none.  By the nominal number of SMs, so that the size query,
+// which touches no device, and the launch agree.
+static bool canonical_takes_umma(int64_t M, int64_t N, int64_t K) {
+    DirPlan plan;
+    return M <= 16 && !direct_applies(M, N, K, kFmtCanonical, kNominalSMs, &plan);
+}
+
 static int launch_direct(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* w,
                          const uint16_t* gscale, const uint8_t* gzero, int fmt, const float* s_w, int sw_stride, int64_t N,
                          int64_t K, void* y, int64_t ldy, int out_dtype, const DirPlan& plan, cudaStream_t st) {
@@ -904,11 +912,13 @@ static int linear_canonical_impl(const uint8_t* x8, int64_t ldx8, const float* s
                                  int64_t K, void* y, int64_t ldy, int out_dtype, cudaStream_t st) {
     const int sms = sm_count();
     if (sms <= 0) return W4A8_ERR_CUDA;
-    DirPlan plan;
-    if (direct_applies(M, N, K, kFmtCanonical, sms, &plan))
+    if (canonical_takes_umma(M, N, K)) return -1;
+    if (M <= 16) {
+        DirPlan plan;
+        make_direct_plan(N, K, sms, &plan);
         return launch_direct(x8, ldx8, s_x, M, codes, gscale, gzero, kFmtCanonical, s_w, sw_stride, N, K, y, ldy, out_dtype,
                              plan, st);
-    if (M <= 16) return -1;
+    }
     const uint8_t* gs = reinterpret_cast<const uint8_t*>(gscale);
     CUtensorMap tw;
     if (!make_tmap_u8_2d(&tw, codes, (uint64_t)N, (uint64_t)(K / 2), (uint64_t)(K / 2), 64, 128, CU_TENSOR_MAP_SWIZZLE_64B))
@@ -982,7 +992,8 @@ static int linear_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_
     LinearPlan plan;
     int rc = make_plan(M, N, K, algo, split_k, &plan);
     if (rc != W4A8_OK) return rc;
-    if (plan.workspace_bytes > 0) {
+    const bool chosen = algo == W4A8_ALGO_AUTO && split_k == 0 && !g_idx;   // by the library
+    if (plan.workspace_bytes > 0 && (!chosen || canonical_takes_umma(M, N, K))) {
         if (!workspace || workspace_bytes < plan.workspace_bytes) return W4A8_ERR_WORKSPACE_TOO_SMALL;
         if (reinterpret_cast<uintptr_t>(workspace) & 15u) return W4A8_ERR_BAD_ALIGNMENT;
     }
@@ -990,7 +1001,7 @@ static int linear_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_
     if (rc != W4A8_OK) return rc;
 
     const uint16_t* gs = static_cast<const uint16_t*>(gscale);
-    if (algo == W4A8_ALGO_AUTO && split_k == 0 && !g_idx) {
+    if (chosen) {
         rc = linear_canonical_impl(x8, ldx8, s_x, M, codes, gs, gzero, s_w, sw_stride, N, K, y, ldy, out_dtype, st);
         if (rc != -1) return rc;
     }
@@ -1691,6 +1702,7 @@ size_t w4a8_linear_ex_workspace_bytes(int64_t M, int64_t N, int64_t K, int algo,
     if (M <= 0 || N <= 0 || K <= 0 || K % kGroup != 0) return 0;
     LinearPlan plan;
     if (make_plan(M, N, K, algo, split_k, &plan) != W4A8_OK) return 0;
+    if (algo == W4A8_ALGO_AUTO && split_k == 0 && !canonical_takes_umma(M, N, K)) return 0;
     return plan.workspace_bytes;
 }
 

@@ -206,3 +206,12 @@ def test_the_extension_module_is_built_again_for_another_torch(L, monkeypatch):
     monkeypatch.setattr(torch, "__version__", "99.0")
     build.build()
     assert built == [build.HOST_PATH]
+
+
+@pytest.mark.parametrize("M,N,K", [(33, 6144, 4096), (64, 1024, 4096), (17, 144, 8192), (8, 1024, 1024), (16, 4096, 2048)])
+def test_no_workspace_is_asked_for_where_none_is_used(L, M, N, K):
+    # canonical weights, kernel chosen by the library; the kernel that cuts K through the workspace still asks for it
+    assert L.w4a8_linear_workspace_bytes(M, N, K, binding.FMT_CANONICAL) == 0
+    assert L.w4a8_linear_ex_workspace_bytes(M, N, K, binding.ALGO_AUTO, 0) == 0
+    assert L.w4a8_linear_ex_workspace_bytes(M, N, K, binding.ALGO_UMMA, 0) > 0
+    assert L.w4a8_linear_workspace_bytes(16, 14336, 4096, binding.FMT_CANONICAL) > 0

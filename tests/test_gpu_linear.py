@@ -1,6 +1,8 @@
 """GPU parity: w4a8_linear against the oracle (Sec. 3 flow: Eq. 13 -> Eq. 10 -> FP8 matmul ->
 Eq. 4 / Eq. 11).  FP8 operands must be bit-exact (checked in the other GPU tests); the output
 gate is max relative error 2e-3 before the BF16 cast and 1 BF16 step after it."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -357,3 +359,19 @@ def test_a_workspace_does_not_make_a_layer_slower(M, N, K):
                 torch.cuda.synchronize()
                 b[0] = min(b[0], t0.elapsed_time(t1) * 25)
         assert best[0][0] <= 1.2 * best[1][0], (asym, best[0][0], best[1][0])
+
+
+@pytest.mark.parametrize("M,N,K", [(33, 6144, 512), (64, 1024, 1024), (20, 9616, 256), (8, 1024, 1024), (16, 2048, 512)])
+def test_canonical_calls_without_a_workspace_where_none_is_used(M, N, K):
+    x8, s_x, wq = _gaussian_case(M, N, K, seed=9)
+    xd, sd, (codes, gs, gz, sw) = dev(x8), dev(s_x), weights_to_dev(*wq)
+    y = torch.full((M, N), float("nan"), device="cuda")
+    rc = binding.lib().w4a8_linear(xd.data_ptr(), K, sd.data_ptr(), M, codes.data_ptr(), gs.data_ptr(), None, binding.FMT_CANONICAL,
+                                   sw.data_ptr(), 0, N, K, 128, y.data_ptr(), N, binding.OUT_FP32, None, 0,
+                                   ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == binding.OK
+    torch.cuda.synchronize()
+    assert binding.query_device_status() == 0
+    ref = oracle.linear(x8, s_x, oracle.dequant_weight(*wq[:3]), wq[3])
+    worst, _ = fp32_gate(y.cpu().numpy(), ref["y64"])
+    assert worst <= 2e-3, worst
