@@ -782,10 +782,12 @@ static int launch_direct(const uint8_t* x8, int64_t ldx8, const float* s_x, int6
 
 static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* wpp,
                              int fmt, const float* s_w, int sw_stride, int64_t N, int64_t K, void* y, int64_t ldy,
-                             int out_dtype, void* workspace, size_t workspace_bytes, cudaStream_t st) {
-    if (M <= 16 && sn_workspace_usable(workspace, workspace_bytes)) {
+                             int out_dtype, void* workspace, size_t workspace_bytes, cudaStream_t st, bool y_on_host) {
+    if (M <= 16 && sn_workspace_usable(workspace, workspace_bytes) && (!y_on_host || M * N <= 40000)) {
         // (linear_direct_kernel cuts K between the warps of a CTA.  Without a workspace K is never cut, which is how a
-        // caller asks for the bits of a chain launch.)
+        // caller asks for the bits of a chain launch.  An output in host memory it writes in pieces of 32 bytes, which the
+        // bus takes more slowly than the split-N kernel's rows: host to host, us, split-N / this, (4, 8192, 2048) 15.6 / 14.8,
+        // (8, 4096, 3072) 17.1 / 16.8, (8, 6144, 2048) 15.9 / 17.2, (16, 6144, 2048) 19.1 / 24.1, (16, 8192, 1024) 19.3 / 24.0.)
         const int rc = check_device();
         if (rc != W4A8_OK) return rc;
         const int sms_d = sm_count();
@@ -969,7 +971,7 @@ static int linear_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_
                        const void* gscale, const uint8_t* gzero, int fmt, const float* s_w, int sw_stride,
                        int64_t N, int64_t K, int group, void* y, int64_t ldy, int out_dtype, void* workspace,
                        size_t workspace_bytes, int algo, int split_k, cudaStream_t st,
-                       const int32_t* g_idx = nullptr) {
+                       const int32_t* g_idx = nullptr, bool y_on_host = false) {
     if (fmt != kFmtCanonical && fmt != kFmtTiled && fmt != kFmtTiledSignMag) return W4A8_ERR_INVALID_ARG;
     if (g_idx && (fmt != kFmtCanonical || (reinterpret_cast<uintptr_t>(g_idx) & 3u))) return W4A8_ERR_INVALID_ARG;
     if (!x8 || !s_x || !codes || !s_w || !y) return W4A8_ERR_INVALID_ARG;
@@ -987,7 +989,7 @@ static int linear_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_
     if (fmt != kFmtCanonical) {
         if (algo != W4A8_ALGO_AUTO || split_k > 0) return W4A8_ERR_INVALID_ARG;
         return linear_tiled_impl(x8, ldx8, s_x, M, codes, fmt, s_w, sw_stride, N, K, y, ldy, out_dtype, workspace,
-                                 workspace_bytes, st);
+                                 workspace_bytes, st, y_on_host);
     }
     LinearPlan plan;
     int rc = make_plan(M, N, K, algo, split_k, &plan);
@@ -1894,7 +1896,8 @@ int w4a8_forward_host(const void* x_host_bf16, int64_t M, const uint8_t* weights
             rc = quantize_act_impl(xh, M, K, K, x8_dev, K, s_x_dev, W4A8_SCALE_EXACT, nullptr, st);
             if (rc != W4A8_OK) return rc;
             return linear_impl(x8_dev, K, s_x_dev, M, weights, gscale_bf16, gzero, weight_format, s_w, sw_stride, N,
-                               K, group, yh, N, W4A8_OUT_BF16, workspace, workspace_bytes, W4A8_ALGO_AUTO, 0, st);
+                               K, group, yh, N, W4A8_OUT_BF16, workspace, workspace_bytes, W4A8_ALGO_AUTO, 0, st, nullptr,
+                               true);
         }
     }
     if (cudaMemcpyAsync(x_dev, x_host_bf16, (size_t)M * K * 2, cudaMemcpyHostToDevice, st) != cudaSuccess)

@@ -375,3 +375,38 @@ def test_canonical_calls_without_a_workspace_where_none_is_used(M, N, K):
     ref = oracle.linear(x8, s_x, oracle.dequant_weight(*wq[:3]), wq[3])
     worst, _ = fp32_gate(y.cpu().numpy(), ref["y64"])
     assert worst <= 2e-3, worst
+
+
+@pytest.mark.parametrize("M,N,K", [(16, 6144, 2048), (16, 8192, 1024)])
+def test_host_forward_is_no_slower_than_its_parts_without_a_workspace(M, N, K):
+    # Pinned buffers: the same two kernels' work, the linear layer told (by no workspace) to take the split-N kernel.  A
+    # kernel that writes smaller pieces over the bus once took 1.25 times as long here.
+    x8, s_x, wq = _gaussian_case(M, N, K, seed=6)
+    tws = [binding.prepack_weight(*weights_to_dev(*wq)) for _ in range(2)]
+    fw = [binding.HostForward(M, tw) for tw in tws]
+    xh = torch.randn((M, K)).to(torch.bfloat16).pin_memory()
+    L = binding.lib()
+    addr = {}
+    for t in (xh, fw[0].y_host, fw[1].y_host):
+        p = ctypes.c_void_p()
+        assert L.w4a8_host_buffer_device_pointer(ctypes.c_void_p(t.data_ptr()), ctypes.byref(p)) == 0
+        addr[t.data_ptr()] = p
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+
+    def parts(i):
+        f, tw = fw[i], tws[i]
+        assert L.w4a8_quantize_act(addr[xh.data_ptr()], M, K, K, f.x8.data_ptr(), K, f.s_x.data_ptr(), 0, None, st) == 0
+        assert L.w4a8_linear(f.x8.data_ptr(), K, f.s_x.data_ptr(), M, tw.buf.data_ptr(), None, None, tw.fmt, tw.s_w.data_ptr(), 0, N, K,
+                             128, addr[f.y_host.data_ptr()], N, 0, None, 0, st) == 0
+
+    best = [1e9, 1e9]
+    for _ in range(10):
+        for side, run in enumerate((lambda i: fw[i](xh), parts)):
+            t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            t0.record()
+            for i in range(30):
+                run(i & 1)
+            t1.record()
+            torch.cuda.synchronize()
+            best[side] = min(best[side], t0.elapsed_time(t1) / 30 * 1e3)
+    assert best[0] <= 1.12 * best[1], best
