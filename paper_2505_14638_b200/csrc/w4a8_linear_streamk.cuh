@@ -69,7 +69,7 @@ namespace w4a8 {
 // 4096) 10.3 9.7 8.8 8.5, (77, 4096, 14336) 17.7 16.8 16.5 14.3.  With 256-token tiles the extra warp gained nothing
 // ((2048, 4096, 4096) 32.3 / 32.6): there a step's eight (four) long MMAs cover the requests.
 //
-// FMT = canonical (weights as they are stored at the boundary, not prepacked): a TMA tile load of 64 bytes x 128 (256)
+// FMT = canonical (weights as they are stored at the boundary, not prepacked): a TMA tile load of 64 bytes x 128
 // rows per k-block takes the place of the two bulk copies, and the expanding threads fetch their row's scale
 // and zero-point of a stage from the canonical arrays while they expand the stage before.  Whole tiles or
 // the cluster exchange only (the canonical entry points have no workspace that is zero-filled once), and nothing is
@@ -108,7 +108,7 @@ struct SkCfg {
     static constexpr int kSlotFloats = BNX * 128;
     static_assert(BNX == 16 || BNX == 32 || BNX == 64 || BNX == 128 || BNX == 256, "token tile");
     static_assert(RB_ == 1 || (RB_ == 2 && BNX_ == 256), "two row blocks per tile only with 256-token tiles");
-    static_assert(!W8_ || RB_ == 1, "the FP8-weight variant uses one row block per tile");
+    static_assert((!W8_ && !CANON) || RB_ == 1, "the FP8-weight and canonical variants use one row block per tile");
     static_assert(!W16_ || (RB_ == 1 && !W8_ && !CL_ && FMT_ == kFmtTiledSignMag), "the BF16 variant: one row block, sign-magnitude codes, whole tiles");
     static_assert(!CL_ || (RB_ == 1 && !W8_ && BNX_ <= 128), "the cluster exchange serves one row block and at most 128 tokens");
     // the exchange happens in the ring memory, idle by then in every CTA of the cluster: the CTA's own partial
@@ -143,7 +143,7 @@ struct SkCfg {
 template <class Cfg>
 __global__ void __launch_bounds__(Cfg::kThreads)
 linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K], box 128 x BNX, 128B swizzle
-                      const __grid_constant__ CUtensorMap tmap_w,  // W8: FP8 weights u8 [N][K], box 128 x 128, 128B swizzle; canonical: codes u8 [N][K/2], box 64 x 128 RB, 64B swizzle
+                      const __grid_constant__ CUtensorMap tmap_w,  // W8: FP8 weights u8 [N][K], box 128 x 128, 128B swizzle; canonical: codes u8 [N][K/2], box 64 x 128, 64B swizzle
                       const uint8_t* __restrict__ wpp,             // tiled weights (panels, k-block major); canonical: the BF16 group scales [N][K/128]
                       const uint8_t* __restrict__ gzero,           // canonical only: zero-points u8 [N][K/128] or NULL
                       const float* __restrict__ s_x, const float* __restrict__ s_w, int sw_stride,
@@ -849,8 +849,8 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
         const int dw = warp - 10;
         const int g = dw >> 2;
         const int r = (warp & 3) * 32 + lane;   // (a warp reaches the tensor-memory lanes of its quarter)
-        // canonical: scale and zero-point of this thread's rows, fetched one of the group's stages ahead
-        uint32_t meta[RB];
+        // canonical: scale and zero-point of this thread's row, fetched one of the group's stages ahead
+        uint32_t meta = 0u;
         int mkb = kb_begin + g, mnt = (int)(tile_begin / TM), mmt = (int)(tile_begin % TM);
         auto next_meta = [&](int step) {   // of the stage `step` k-blocks further
             mkb += step;
@@ -861,12 +861,9 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                     ++mnt;
                 }
             }
-#pragma unroll
-            for (int b = 0; b < RB; ++b) {
-                const int n = mnt * TR + b * 128 + r;
-                const int64_t i = (int64_t)n * KB + mkb;
-                meta[b] = n < N ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(wpp) + i) | (gzero ? (uint32_t)__ldg(gzero + i) : 8u) << 16 : 0u;
-            }
+            const int n = mnt * TR + r;
+            const int64_t i = (int64_t)n * KB + mkb;
+            meta = n < N ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(wpp) + i) | (gzero ? (uint32_t)__ldg(gzero + i) : 8u) << 16 : 0u;
         };
         if constexpr (Cfg::CANON) {
             ptx::griddep_wait();
@@ -884,7 +881,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                 const uint32_t a_col = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(Cfg::kACol + s2 * 32);
                 ptx::tc_fence_after_sync();
                 if constexpr (Cfg::CANON) {
-                    const uint32_t m = meta[0];
+                    const uint32_t m = meta;
                     next_meta(G);   // (past the last stage: a row that does not exist, or one that is not used)
                     dequant_canonical_row_to_tmem(stage_w(s1), m, r, a_col);
                 } else {
@@ -900,14 +897,9 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                 dequant_row_to_smem_bf16(stage_w(s1) + tiled_row_offset(r), stage_w(s1) + (uint32_t)Cfg::kCodeBytes + (uint32_t)(r * Cfg::kMeta), r,
                                          stage_w8(s2) + (uint32_t)r * 128u);
             else if constexpr (Cfg::CANON) {
-                uint32_t m[RB];
-#pragma unroll
-                for (int b = 0; b < RB; ++b) m[b] = meta[b];
+                const uint32_t m = meta;
                 next_meta(G);   // (past the last stage: a row that does not exist, or one that is not used)
-#pragma unroll
-                for (int b = 0; b < RB; ++b)
-                    dequant_canonical_row_to_smem(stage_w(s1) + (uint32_t)(b * 8192), m[b], r,
-                                                  stage_w8(s2) + (uint32_t)(b * 16384) + (uint32_t)r * 128u);
+                dequant_canonical_row_to_smem(stage_w(s1), m, r, stage_w8(s2) + (uint32_t)r * 128u);
             } else
 #pragma unroll
             for (int b = 0; b < RB; ++b)
