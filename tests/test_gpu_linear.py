@@ -330,35 +330,20 @@ def test_formats_at_tile_edges(M, N, K):
             assert bool((buf[M:] == -7.5).all()) and bool((buf[:, N:] == -7.5).all())
 
 
-@pytest.mark.parametrize("M,N,K", [(16, 12288, 1536), (9, 14144, 1024), (4, 12288, 1536), (16, 4096, 256), (9, 8192, 128), (16, 14144, 128)])
-def test_a_workspace_does_not_make_a_layer_slower(M, N, K):
-    # Layers whose K the split-N kernel walks whole: with a workspace another kernel may be chosen, without one
-    # it may not.  Both sides in turn, several layers after one another (the kernels that were chosen here once took
-    # 1.3 to 1.6 times as long).
+@pytest.mark.parametrize("M,N,K", [(16, 12288, 1536), (9, 14144, 1024), (4, 12288, 1536), (16, 4096, 512), (9, 8192, 384), (16, 14144, 640)])
+def test_layers_whose_k_the_split_n_kernel_walks_whole_stay_with_it(M, N, K):
+    # With a workspace another kernel may be chosen, without one it may not: here it took 1.3 to 1.6 times as long.  The same
+    # kernel on both sides gives the same bits; the other one cuts K and rounds its sums elsewhere.
     for asym in (False, True):
         x8, s_x, wq = _gaussian_case(M, N, K, seed=4, asym=asym)
-        tws = [binding.prepack_weight(*weights_to_dev(*wq)) for _ in range(4)]
+        tw = binding.prepack_weight(*weights_to_dev(*wq))
         xd, sd = dev(x8), dev(s_x)
-        y = torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
         tiny = torch.zeros((16,), dtype=torch.uint8, device="cuda")
-        best = []
-        for ws in (binding.new_workspace(M, N, K, tws[0].fmt), tiny):
-            binding.linear_tiled(xd, sd, tws[0], out=y, workspace=ws)
-            torch.cuda.synchronize()
-            g = torch.cuda.CUDAGraph()
-            with torch.cuda.graph(g):
-                for i in range(40):
-                    binding.linear_tiled(xd, sd, tws[i % 4], out=y, workspace=ws)
-            best.append([1e9, g])
-        for _ in range(8):
-            for b in best:
-                t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-                t0.record()
-                b[1].replay()
-                t1.record()
-                torch.cuda.synchronize()
-                b[0] = min(b[0], t0.elapsed_time(t1) * 25)
-        assert best[0][0] <= 1.2 * best[1][0], (asym, best[0][0], best[1][0])
+        a, b = (binding.linear_tiled(xd, sd, tw, out_dtype=binding.OUT_FP32, workspace=ws)
+                for ws in (binding.new_workspace(M, N, K, tw.fmt), tiny))
+        torch.cuda.synchronize()
+        assert binding.query_device_status() == 0
+        assert torch.equal(a.view(torch.int32), b.view(torch.int32)), asym
 
 
 @pytest.mark.parametrize("M,N,K", [(33, 6144, 512), (64, 1024, 1024), (20, 9616, 256), (8, 1024, 1024), (16, 2048, 512)])
@@ -377,36 +362,46 @@ def test_canonical_calls_without_a_workspace_where_none_is_used(M, N, K):
     assert worst <= 2e-3, worst
 
 
-@pytest.mark.parametrize("M,N,K", [(16, 6144, 2048), (16, 8192, 1024)])
-def test_host_forward_is_no_slower_than_its_parts_without_a_workspace(M, N, K):
-    # Pinned buffers: the same two kernels' work, the linear layer told (by no workspace) to take the split-N kernel.  A
-    # kernel that writes smaller pieces over the bus once took 1.25 times as long here.
+@pytest.mark.parametrize("M,N,K,register_kernel", [(16, 6144, 2048, False), (16, 8192, 1024, False), (10, 4096, 1024, False),
+                                                   (9, 4096, 1024, True), (8, 2048, 2048, True)])
+def test_host_forward_on_pinned_buffers_leaves_large_outputs_to_the_split_n_kernel(M, N, K, register_kernel):
+    # The kernel for small layers writes smaller pieces over the bus: 24 us host to host at (16, 6144, 2048), 19 us with the
+    # split-N kernel.  The latter cuts K here and leaves its partial sums behind the workspace's 64 KB of control data; the
+    # former does not touch the workspace.
     x8, s_x, wq = _gaussian_case(M, N, K, seed=6)
-    tws = [binding.prepack_weight(*weights_to_dev(*wq)) for _ in range(2)]
-    fw = [binding.HostForward(M, tw) for tw in tws]
-    xh = torch.randn((M, K)).to(torch.bfloat16).pin_memory()
-    L = binding.lib()
-    addr = {}
-    for t in (xh, fw[0].y_host, fw[1].y_host):
-        p = ctypes.c_void_p()
-        assert L.w4a8_host_buffer_device_pointer(ctypes.c_void_p(t.data_ptr()), ctypes.byref(p)) == 0
-        addr[t.data_ptr()] = p
-    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    xb = inputs.make_activation(M, K, 8, 0.01, 20.0)
+    fw = binding.HostForward(M, binding.prepack_weight(*weights_to_dev(*wq)))
+    y = fw(torch.from_numpy(xb.view(np.int16)).view(torch.bfloat16).pin_memory())
+    torch.cuda.synchronize()
+    assert binding.query_device_status() == 0
+    assert bool(fw.ws[65536:].any()) != register_kernel
+    ok, dist = bf16_gate(bf16_bits(y), oracle.forward(xb, *wq)["y64"])
+    assert ok, dist
 
-    def parts(i):
-        f, tw = fw[i], tws[i]
-        assert L.w4a8_quantize_act(addr[xh.data_ptr()], M, K, K, f.x8.data_ptr(), K, f.s_x.data_ptr(), 0, None, st) == 0
-        assert L.w4a8_linear(f.x8.data_ptr(), K, f.s_x.data_ptr(), M, tw.buf.data_ptr(), None, None, tw.fmt, tw.s_w.data_ptr(), 0, N, K,
-                             128, addr[f.y_host.data_ptr()], N, 0, None, 0, st) == 0
 
-    best = [1e9, 1e9]
-    for _ in range(10):
-        for side, run in enumerate((lambda i: fw[i](xh), parts)):
-            t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-            t0.record()
-            for i in range(30):
-                run(i & 1)
-            t1.record()
+@pytest.mark.parametrize("M,N,K", [(1, 1024, 128), (4, 8192, 384), (8, 4096, 896), (3, 2384, 1152), (16, 3600, 1024), (12, 9472, 1024),
+                                   (7, 9488, 2048), (8, 10256, 2048), (13, 4112, 2048), (5, 5136, 2560), (16, 1024, 7168)])
+def test_small_layers_in_bf16_at_the_edges_of_their_rule(M, N, K):
+    # The kernel for small layers stores its own rounding of the sums: small whole numbers and powers of two, so that the
+    # sums are exact in any order and the BF16 result is one rounding of them, bit for bit.
+    rng = np.random.default_rng(M + N + K)
+    tab = e4m3_value_table()
+    ints = np.array([c for v in range(-6, 7) for c in [int(np.flatnonzero(tab == v)[0])]], dtype=np.uint8)
+    x8 = ints[rng.integers(0, 13, size=(M, K))]
+    s_x = 2.0 ** rng.integers(-3, 4, size=M).astype(np.float32)
+    codes = pack_codes(rng.integers(1, 16, size=(N, K)).astype(np.uint8))
+    gs = inputs.f32_to_bf16_bits(np.ones((N, K // 128), dtype=np.float32))
+    gz = rng.integers(4, 12, size=(N, K // 128)).astype(np.uint8)
+    s_w = 2.0 ** rng.integers(-3, 4, size=N).astype(np.float32)
+    xd, sd = dev(x8), dev(s_x)
+    for zero in (gz, None):
+        want = torch.from_numpy(oracle.linear(x8, s_x, oracle.dequant_weight(codes, gs, zero), s_w, want=("y32",))["y32"]).to(torch.bfloat16)
+        wd = weights_to_dev(codes, gs, zero, s_w)
+        tw = binding.prepack_weight(*wd)
+        for run in (lambda y: binding.linear(xd, sd, *wd, out=y), lambda y: binding.linear_tiled(xd, sd, tw, out=y)):
+            buf = torch.full((M + 1, N + 8), -7.5, dtype=torch.bfloat16, device="cuda")
+            run(buf[:M, :N])
             torch.cuda.synchronize()
-            best[side] = min(best[side], t0.elapsed_time(t1) / 30 * 1e3)
-    assert best[0] <= 1.12 * best[1], best
+            assert binding.query_device_status() == 0
+            assert torch.equal(buf[:M, :N].cpu().view(torch.int16), want.view(torch.int16))
+            assert bool((buf[M:] == -7.5).all()) and bool((buf[:, N:] == -7.5).all())
