@@ -115,7 +115,9 @@ int w4a8_dequant_weight(const uint8_t* codes, const void* gscale_bf16, const uin
  * bounded wait gave up (w4a8_query_device_status returns W4A8_ERR_TIMEOUT): zero-fill the
  * workspace again after that.  Calls that share a workspace must not overlap on the device.
  * Calls with M <= 16 on tiled weights place their worker CTAs at run time (at most one per SM and
- * launch, so that consecutive launches can share the SMs).  The bookkeeping (1 KB, cleared by the
+ * launch, so that consecutive launches can share the SMs), unless a CTA has fewer than sixteen k-blocks to
+ * walk or the layer is one of those that, given a workspace, go from global memory to registers (neither has
+ * placement state).  The bookkeeping (1 KB, cleared by the
  * kernel) lives in the workspace when one of the full size is given -- nothing more to observe
  * than the rule above: calls that may overlap on the device need different workspaces; calls
  * issued one after the other on one stream may share one.  Without a workspace it is an entry of a

@@ -550,8 +550,9 @@ static int launch_pair(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, cons
 // 65..128 tokens on a layer with few output channels (at most a quarter as many 128-row tiles as
 // SMs) take the persistent kernel with K cut between a whole number of CTAs per tile and the
 // exchange through the workspace, instead of the split-N kernel, every CTA of which pulls the whole
-// X8 through its L2 port (measured, us: o projection 13.4 against 15.3, down projection 21.5
-// against 27.5; qkv and gate_up stay: 16.9 against 15.4, 33.6 against 27.1).
+// X8 through its L2 port (measured with the expansion through shared memory that this kernel had then, us: o
+// projection 13.4 against 15.3, down projection 21.5 against 27.5; qkv and gate_up stay: 16.9 against 15.4, 33.6 against
+// 27.1.  Since the expansion goes to tensor memory o takes 12.0 and down 17.4; qkv and gate_up have not been measured again).
 static bool streamk_for_128_tokens(int64_t M, int64_t N, int64_t K, int sms) {
     return M > 64 && M <= kSplitNMaxM && K >= 2048 && ((N + 127) / 128) * 4 <= sms;
 }
@@ -797,11 +798,10 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
     }
     if (M > 16) {
         // 17..128 tokens on a layer with few 128-row tiles: K cut between the CTAs of a cluster (measured, us,
-        // against the split-N kernel or the persistent kernel with its exchange through L2:
-        // (32, 4096, 4096) 8.0 / 9.8, (64, 2048, 4096) 7.4 / 12.6, (100, 512, 8192) 9.0 / 15.0,
-        // (128, 4096, 4096) 11.9 / 12.9, (128, 4096, 14336) 19.0 / 21.2, (128, 6144, 4096) 13.5 / 14.5; at
-        // 16 tokens and fewer the split-N kernel, which overlaps its set-up with the launch before, stays
-        // ahead: (8, 4096, 4096) 8.5 / 7.3)
+        // against the split-N kernel or the persistent kernel with its exchange through L2, whichever runs without this
+        // plan: (17, 6144, 4096) 8.0 / 12.8, (32, 4096, 4096) 7.3 / 10.0, (64, 2048, 4096) 6.9 / 12.9, (100, 512, 8192) 7.6 /
+        // 15.1, (128, 4096, 4096) 11.3 / 12.0, (128, 4096, 14336) 16.6 / 17.4, (128, 6144, 4096) 12.1 / 14.8).  Up to 16 tokens
+        // the kernels that overlap their set-up with the launch before are used: (8, 4096, 4096) 6.6.
         const int sms_c = sm_count();
         const int cl0 = sms_c > 0 ? cluster_kcut_ctas(M, N, K, sms_c) : 0;
         for (int cl = cl0; cl >= 2; --cl) {   // the largest cluster size of which all clusters are resident at once

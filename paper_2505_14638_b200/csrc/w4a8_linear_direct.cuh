@@ -7,9 +7,10 @@
 // weights of a 4096 x 4096 layer take to arrive.  Here a warp fetches 16 rows x four k-blocks (4 KB of
 // codes, eight 16-byte loads per lane), expands them in registers (Eq. 10, one table per row and k-block) and
 // feeds them to mma.sync m16n8k32 E4M3 MMAs (FP32 accumulation): no copies, no barriers until the row tile is
-// done.  (1024, 1024) at M = 8: 3.4 us against 6.3.  For larger layers the integer pipe is the bound: this form of
-// the MMA converts its FP8 operands to 16 bits with instructions of that pipe, some 190 per 16 rows x 512 columns
-// beside 250 of expansion, which the tcgen05 kernels are spared: (28672, 4096) at M = 8 22 us against 17.5.
+// done.  (1024, 1024) at M = 8: 3.4 us against 6.3 (the linear layer alone).  For larger layers the integer pipe is taken to be
+// the bound: this form of the MMA has its FP8 operands converted to 16 bits, two conversions for each of the six operand
+// registers of an MMA, 192 per 16 rows x 512 columns and eight tokens, beside some 250 instructions of expansion (both counted
+// from this source, not measured); the tcgen05 kernels are spared the former: (28672, 4096) at M = 8 22 us against 17.5.
 //
 // Fragment layout.  The order of the reduction index is free as long as both operands share it: the four
 // lanes of a row take four different k-blocks (a lane owns all 128 weights of its row and k-block: one table

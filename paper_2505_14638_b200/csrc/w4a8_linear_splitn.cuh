@@ -1,4 +1,4 @@
-// Decode-sized W4A8 linear (M <= 64 tokens) for sm_100a: the weight-bandwidth-bound regime.
+// W4A8 linear for few tokens (M <= 128, tiles of 16, 64 and 128) for sm_100a: the weight-bandwidth-bound regime.
 //
 // The output channels are cut into as many contiguous row ranges as there are SMs (multiples of
 // 8 rows, at most 256, so every SM streams the same share of the packed weights within a few

@@ -336,7 +336,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
             // activations: the weight-only prologue may not be longer than that ring)
             constexpr int kAhead = Cfg::W8 ? (S2 < S1 ? S2 : S1) : S1;
             const int ahead = n_it < kAhead ? n_it : kAhead;
-            // (the activation tiles of the first ring-full are requested by the MMA warp)
+            // (the activation tiles of the first ring-full are requested by the MMA warp; TA: all of them by a warp of their own)
             const int nx = n_it < S1 ? n_it : S1;
             ptx::Ring rx;  // ring position of the next activation tile
             int xkb = kb, xmt = mt;
