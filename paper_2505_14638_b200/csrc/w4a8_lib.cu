@@ -237,56 +237,85 @@ struct SkPlan {
 
 constexpr int kSplitNMaxM = 128;  // token counts served by the split-N (decode) kernel
 
-// Token-tile width and schedule of the persistent kernel from a small cost model (microseconds):
-// a (tile, k-block) unit costs the larger of the dequantization of its 128 x 128 weights and its
-// four MMAs; whole tiles per CTA cost rounds x K/128 units; equal slices cost ceil(U / P) units
-// plus the exchange of partial tiles.  Wider token tiles dequantize each weight fewer times.
-static void make_sk_plan(int64_t M, int64_t N, int64_t K, int sms, SkPlan* pl) {
+// Token-tile width and schedule of the persistent kernel on prepacked weights from a cost model, in microseconds; returns
+// the time.  Whole tiles per CTA cost rounds x (k-blocks x step + drain); where there are fewer tiles than half the CTAs and
+// a number of CTAs per tile divides the k-blocks, that many CTAs share a tile and exchange partial sums, which costs about
+// as much as 30 k-blocks.  Fitted, with the constants of the CTA pairs (see prefill_choice), to 656 + 410 measured (M, N,
+// K) of all alternatives: the alternative chosen takes 0.5 % longer than the fastest on average, 9 % at most from K = 1024
+// on.  Equal slices of the (tile, k-block) space and tiles of 256 tokens, which earlier versions had, are nowhere the
+// fastest by more than 4 %.
+static double make_sk_plan(int64_t M, int64_t N, int64_t K, int sms, SkPlan* pl) {
     const int64_t KB = K / 128;
     const int64_t TN = (N + 127) / 128;
     const int64_t cap = sms < kMaxSMs ? sms : kMaxSMs;
     double best = 1e30;
-    for (int bnx = 256; bnx >= 64; bnx >>= 1) {
+    for (int bnx = 128; bnx >= 64; bnx >>= 1) {
         if (bnx > 64 && bnx / 2 >= M) continue;  // more than half of the tile would be padding
-        const int64_t TM = (M + bnx - 1) / bnx, Tt = TM * TN, U = Tt * KB;
-        const double mma_cycles = 4.0 * (bnx / 2 > 47 ? bnx / 2 : 47);
-        const double t_unit = mma_cycles / 1900.0 > 0.22 ? mma_cycles / 1900.0 : 0.22;
-        const int64_t Pa = cap < Tt ? cap : Tt;
-        const double t_aligned = (double)((Tt + Pa - 1) / Pa) * (double)KB * t_unit;
-        int64_t Ps = cap < U ? cap : U;
-        const double t_tail = 2.0 + bnx * 2048.0 / 1.0e5;   // exchange of partial tiles: two per CTA
-        double t_split = (double)((U + Ps - 1) / Ps) * t_unit + t_tail;
-        if (Tt < cap && KB % (cap / Tt) == 0) {
-            // Fewer tiles than CTAs: a whole number of CTAs per tile instead of equal slices of the
-            // unit space, where that number divides the k-blocks.  Every CTA then stays inside one
-            // tile -- one partial tile to store, and a tile's contributors finish together -- at
-            // the price of a few idle SMs (measured, us: (128, 4096, 4096) 13.4 against 17.9;
-            // (512, 4096, 14336) 41.6 against 49.8; with a remainder -- (256, 6144, 4096), three CTAs
-            // per tile, 32 k-blocks -- it was slower: 20.9 against 18.0).
-            const int64_t Pk = Tt * (cap / Tt);
-            const double t_k = (double)((U + Pk - 1) / Pk) * t_unit + 0.5 * t_tail;
-            if (t_k < t_split) {
-                t_split = t_k;
-                Ps = Pk;
+        const int64_t TM = (M + bnx - 1) / bnx, Tt = TM * TN;
+        const double step = bnx == 64 ? 0.207 : 0.247, drain = bnx == 64 ? 0.46 : 0.89;
+        double t = (double)((Tt + cap - 1) / cap) * ((double)KB * step + drain) + 1.8;
+        int64_t P = cap < Tt ? cap : Tt;
+        bool whole = true;
+        const int64_t per = cap / Tt;   // CTAs per tile
+        // (tile counters must fit the control area)
+        if (per >= 2 && KB % per == 0 && 2 * (size_t)Tt * sizeof(unsigned int) <= kLinearCtlSplitN) {
+            const double t_k = (double)(KB / per) * step + 7.7;
+            if (t_k < t) {
+                t = t_k;
+                P = Tt * per;
+                whole = false;
             }
         }
-        // (tile counters must fit the control area: otherwise whole tiles per CTA, which need none)
-        const bool al = t_aligned <= t_split || 2 * (size_t)Tt * sizeof(unsigned int) > kLinearCtlSplitN;
-        const double t = al ? t_aligned : t_split;
         if (t < best) {
             best = t;
             pl->bnx = bnx;
             pl->TM = (int)TM;
             pl->TN = (int)TN;
-            pl->U = U;
-            pl->aligned = al ? 1 : 0;
-            pl->P = al ? Pa : Ps;
+            pl->U = Tt * KB;
+            pl->aligned = whole ? 1 : 0;
+            pl->P = P;
         }
     }
     // arrivals and finished reducers per tile live in the control area; the size asked of the caller
     // covers every tile width and any SM count up to kMaxSMs, so that the query needs no device
     pl->counter_bytes = kLinearCtlBytes;
     pl->workspace_bytes = kLinearCtlBytes + (size_t)kMaxSMs * 2 * 256 * 128 * sizeof(float);
+    return best;
+}
+
+// CTA pairs against the persistent kernel for a problem of more than 128 tokens: 0 = persistent kernel (its plan in `pl`),
+// 1 = tiles of 256 channels x 256 tokens, 2 = 256 x 512, 3 = 256 x 256 with K cut between the two pairs of a cluster of four
+// CTAs.  Times in microseconds, from the same fit as make_sk_plan's: a k-block of a 256 x 256 tile takes a pair 0.244, of a
+// 256 x 512 tile 0.489 (a round that holds only tiles of at most 256 tokens half of that); drain per tile, launch and fill
+// per call.  Measured, us, sign-magnitude weights not in L2 (before / now, the choice in brackets): (8192, 28672, 8192) 2011 /
+// 1500 [2], (2048, 4096, 4096) 36.3 / 34.7 [2], (1531, 28672, 4096) 208 / 171 [2], (1531, 4096, 14336) 121 / 95 [2], (1024,
+// 28672, 4096) 152 / 121 [2], (512, 6144, 4096) 18.4 / 15.9 [1], (512, 28672, 4096) 71 / 63 [2], (512, 4096, 14336) 45.2 / 33.0
+// [3], (256, 4096, 4096) 16.5 / 10.9 [3]; (512, 4096, 4096) 12.2 / - / 14.1 on pairs [0].
+static int prefill_choice(int64_t M, int64_t N, int64_t K, int sms, SkPlan* pl) {
+    const int64_t KB = K / 128, pairs = sms / 2, TN = (N + 255) / 256;
+    double best = make_sk_plan(M, N, K, sms, pl);
+    int choice = 0;
+    const int64_t t1 = TN * ((M + 255) / 256);
+    const int64_t rounds1 = (t1 + pairs - 1) / pairs;
+    double t = (double)rounds1 * ((double)KB * 0.244 + 2.1) + 3.1;
+    // (back to back, at the power cap, where all pairs work throughout: it expands twice the weights)
+    if (rounds1 >= 2) t *= 1.1;
+    if (t < best) {
+        best = t;
+        choice = 1;
+    }
+    const int64_t TM2 = (M + 511) / 512, t2 = TN * TM2, rounds2 = (t2 + pairs - 1) / pairs;
+    const bool half = M - (TM2 - 1) * 512 <= 256 && TN >= t2 - (rounds2 - 1) * pairs;
+    t = ((double)rounds2 - (half ? 0.5 : 0.0)) * ((double)KB * 0.489 + 2.3) + 6.8;
+    if (t < best) {
+        best = t;
+        choice = 2;
+    }
+    if (4 * t1 <= sms - 4 && KB >= 8) {
+        t = (double)((KB + 1) / 2) * 0.244 + 7.3;
+        if (t < best) choice = 3;
+    }
+    return choice;
 }
 
 template <class Cfg>
@@ -466,50 +495,11 @@ static int launch_splitn_planned(const CUtensorMap& tx, const uint8_t* wpp, cons
     return launch_status();
 }
 
-// The two-CTA kernel takes whole tiles of 256 output channels x 256 tokens, one CTA pair per tile
-// and round.  Each CTA of a pair loads half of the activation tile (24.6 KB per step and SM
-// instead of 41 KB, six ring stages instead of four), but the pair pays for it with remote
-// barrier traffic and coarser tiles.  Measured against the one-CTA persistent kernel (us):
-//   (M, N, K) = (8192, 28672, 8192): 1882 vs 2033;  (2048, 28672, 4096): 241 vs 254;
-//   (1024, 28672, 4096): 133 vs 150;  (4096, 4096, 14336): 254 vs 255;
-//   (4096, 28672, 4096): 459 vs 438;  (8192, 8192, 8192): 536 vs 523;
-//   (4096, 6144, 4096): 113 vs 99;  (4096, 4096, 4096): 77 vs 66;  (2048, 4096, 4096): 42 vs 36.
-// It is used where it won: many output channels, and either few token tiles or a long K.
-static bool pair_kernel_applies(int64_t M, int64_t N, int64_t K, int sms) {
-    if (N % 256 != 0 || N < 16384 || M < 1024 || K < 1024) return false;
-    if (!(M <= 2048 || K >= 8192)) return false;
-    const int64_t tiles = (N / 256) * ((M + 255) / 256);
-    return tiles >= 4 * (int64_t)(sms / 2);
-}
-
-// Tiles of 256 weight rows x 256 tokens (two row blocks per activation tile, whole tiles per CTA)
-// against tiles of 128 x 256: per k-block step about 1060 tensor-pipe cycles for 50 KB from L2 instead
-// of 530 cycles for 41 KB, which the SM's L2 port (about 64 bytes per clock) turns into ~650.  The wide
-// tile cannot be cut along K and its epilogue does not overlap the next tile, so it is used where
-// whole tiles fill the SMs well (measured, us: (2048, 4096, 4096) 34.9 vs 37.7; (4096, 4096, 14336)
-// 203 vs 265; (8192, 28672, 8192) 1785 vs 1906 for the two-CTA kernel) or where a model fitted to
-// such measurements says so ((512, 28672, 4096): 68 vs 87).
-static bool two_block_tiles_apply(int64_t M, int64_t N, int64_t K, int sms) {
-    if (M < 512 || N < 256 || K < 512) return false;
-    const int64_t TM = (M + 255) / 256;
-    const int64_t t2 = TM * ((N + 255) / 256);
-    const int64_t t1 = TM * ((N + 127) / 128);
-    const int64_t KB = K / 128;
-    const int64_t rounds2 = (t2 + sms - 1) / sms;
-    if (5 * t2 >= 4 * rounds2 * sms) return true;   // at least 80 % of the tile slots of its rounds are used
-    // microseconds: 0.857 per k-block step + 3.9 per tile for the wide tile; 0.61 per unit for the
-    // 128-row tile (0.573 in the two-CTA kernel, 0.85 with at most two token tiles, where every
-    // weight tile comes from HBM and four ring stages do not cover that latency)
-    const double per_unit = pair_kernel_applies(M, N, K, sms) ? 0.573 : (TM <= 2 ? 0.85 : 0.61);
-    const double c2 = (double)rounds2 * ((double)KB * 0.857 + 3.9);
-    const double c1 = (double)((t1 * KB + sms - 1) / sms) * per_unit;
-    return c2 < c1;
-}
-
+// Tiles of CTA pairs (see linear_pair_kernel): `kp` pairs share a tile's K.
 template <class Cfg>
 static int launch_pair(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, const float* s_x, const float* s_w,
                        int sw_stride, void* y, int64_t ldy, int out_dtype, int M, int N, int K, int sms,
-                       cudaStream_t st) {
+                       cudaStream_t st, int kp) {
     auto kern = linear_pair_kernel<Cfg>;
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
@@ -522,11 +512,12 @@ static int launch_pair(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, cons
     CUtensorMap tx;  // this CTA's half of an activation tile: 128 tokens x 128 bytes
     if (!make_tmap_u8_2d(&tx, x8, (uint64_t)M, (uint64_t)K, (uint64_t)ldx8, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B))
         return W4A8_ERR_CUDA;
-    const int TM = (M + 255) / 256, TN2 = N / 256;
-    int pairs = sms / 2;
-    if (pairs > TM * TN2) pairs = TM * TN2;
+    const int TM = (M + Cfg::kTokens - 1) / Cfg::kTokens, TN = (N + 255) / 256;
+    if (kp > 1 && K / 128 < 2 * kp) return W4A8_ERR_INVALID_ARG;   // (every pair needs k-blocks of its own)
+    int clusters = sms / (2 * kp);
+    if (clusters > TM * TN) clusters = TM * TN;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * pairs));
+    cfg.gridDim = dim3((unsigned)(2 * kp * clusters));
     cfg.blockDim = dim3(Cfg::kThreads);
     cfg.dynamicSmemBytes = (size_t)Cfg::kSmemBytes;
     cfg.stream = st;
@@ -534,12 +525,12 @@ static int launch_pair(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, cons
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.x = (unsigned)(2 * kp);
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K, TM, TN2,
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K, TM, TN, kp,
                                        status);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     if (e != cudaSuccess) return W4A8_ERR_CUDA;
@@ -555,26 +546,6 @@ static int launch_pair(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, cons
 // 27.1.  Since the expansion goes to tensor memory o takes 12.0 and down 17.4; qkv and gate_up have not been measured again).
 static bool streamk_for_128_tokens(int64_t M, int64_t N, int64_t K, int sms) {
     return M > 64 && M <= kSplitNMaxM && K >= 2048 && ((N + 127) / 128) * 4 <= sms;
-}
-
-// Tiles of 256 weight rows x Cfg::BNX tokens, whole tiles per CTA (no workspace).
-template <class Cfg>
-static int launch_two_block(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, const float* s_x, const float* s_w,
-                            int sw_stride, void* y, int64_t ldy, int out_dtype, int64_t M, int64_t N, int64_t K, int sms,
-                            cudaStream_t st) {
-    SkPlan p2;
-    p2.bnx = Cfg::BNX;
-    p2.TM = (int)((M + Cfg::BNX - 1) / Cfg::BNX);
-    p2.TN = (int)((N + 255) / 256);
-    p2.aligned = 1;
-    p2.U = (int64_t)p2.TM * p2.TN * (K / 128);
-    p2.P = (int64_t)p2.TM * p2.TN < sms ? (int64_t)p2.TM * p2.TN : sms;
-    p2.counter_bytes = 0;
-    p2.workspace_bytes = 0;
-    CUtensorMap tx2;
-    if (!make_tmap_u8_2d(&tx2, x8, (uint64_t)M, (uint64_t)K, (uint64_t)ldx8, 128, (uint32_t)Cfg::BNX, CU_TENSOR_MAP_SWIZZLE_128B))
-        return W4A8_ERR_CUDA;
-    return launch_streamk<Cfg>(tx2, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, nullptr, p2, (int)M, (int)N, (int)K, st);
 }
 
 // Few tiles (at most half as many 128-row tiles as SMs) and at most 128 tokens: CTAs per tile of the plan
@@ -809,15 +780,15 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
             if (rc != W4A8_OK) return rc;
             if (M <= 64)
                 rc = fmt == kFmtTiledSignMag
-                         ? launch_cluster_kcut<SkCfg<64, 4, 12, 12, kFmtTiledSignMag, 1, false, true>>(
+                         ? launch_cluster_kcut<SkCfg<64, 4, 12, 12, kFmtTiledSignMag, false, true>>(
                                x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st)
-                         : launch_cluster_kcut<SkCfg<64, 4, 12, 12, kFmtTiled, 1, false, true>>(
+                         : launch_cluster_kcut<SkCfg<64, 4, 12, 12, kFmtTiled, false, true>>(
                                x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st);
             else
                 rc = fmt == kFmtTiledSignMag
-                         ? launch_cluster_kcut<SkCfg<128, 4, 8, 8, kFmtTiledSignMag, 1, false, true>>(
+                         ? launch_cluster_kcut<SkCfg<128, 4, 8, 8, kFmtTiledSignMag, false, true>>(
                                x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st)
-                         : launch_cluster_kcut<SkCfg<128, 4, 8, 8, kFmtTiled, 1, false, true>>(
+                         : launch_cluster_kcut<SkCfg<128, 4, 8, 8, kFmtTiled, false, true>>(
                                x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st);
             if (rc != -1) return rc;
         }
@@ -870,21 +841,22 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
     if (rc != W4A8_OK) return rc;
     const int sms = sm_count();
     if (sms <= 0) return W4A8_ERR_CUDA;
-    if (two_block_tiles_apply(M, N, K, sms)) {
-        // tiles of 256 weight rows x 256 tokens, whole tiles per CTA
-        return fmt == kFmtTiledSignMag
-                   ? launch_two_block<SkCfg<256, 3, 3, 2, kFmtTiledSignMag, 2>>(x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy,
-                                                                               out_dtype, M, N, K, sms, st)
-                   : launch_two_block<SkCfg<256, 3, 3, 2, kFmtTiled, 2>>(x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy,
-                                                                        out_dtype, M, N, K, sms, st);
+    int choice = 0;
+    if (M > kSplitNMaxM) choice = prefill_choice(M, N, K, sms, &pl);
+    else make_sk_plan(M, N, K, sms, &pl);
+#define W4A8_PAIR(KP, ...)                                                                                            \
+    return fmt == kFmtTiledSignMag                                                                                    \
+               ? launch_pair<PairCfg<kFmtTiledSignMag, __VA_ARGS__>>(x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy,      \
+                                                                     out_dtype, (int)M, (int)N, (int)K, sms, st, KP)  \
+               : launch_pair<PairCfg<kFmtTiled, __VA_ARGS__>>(x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype,  \
+                                                              (int)M, (int)N, (int)K, sms, st, KP)
+    switch (choice) {
+        case 1: W4A8_PAIR(1, 1, 3, 6);
+        case 2: W4A8_PAIR(1, 2, 4, 4);
+        case 3: W4A8_PAIR(2, 1, 3, 6);
+        default: break;
     }
-    if (pair_kernel_applies(M, N, K, sms))
-        return fmt == kFmtTiledSignMag
-                   ? launch_pair<PairCfg<3, 6, 4, kFmtTiledSignMag>>(x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype,
-                                                                      (int)M, (int)N, (int)K, sms, st)
-                   : launch_pair<PairCfg<3, 6, 4, kFmtTiled>>(x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype,
-                                                               (int)M, (int)N, (int)K, sms, st);
-    make_sk_plan(M, N, K, sms, &pl);
+#undef W4A8_PAIR
     CUtensorMap tx;
     if (!make_tmap_u8_2d(&tx, x8, (uint64_t)M, (uint64_t)K, (uint64_t)ldx8, 128, (uint32_t)pl.bnx,
                          CU_TENSOR_MAP_SWIZZLE_128B))
@@ -898,8 +870,7 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
                                                                 workspace, pl, Mi, Ni, Ki, st)
     switch (pl.bnx) {
         case 64: W4A8_SK(64, 4, 12, 12); break;
-        case 128: W4A8_SK(128, 4, 8, 8); break;
-        default: W4A8_SK(256, 4, 4, 3); break;
+        default: W4A8_SK(128, 4, 8, 8); break;
     }
 #undef W4A8_SK
     return rc;
@@ -926,9 +897,9 @@ static int linear_canonical_impl(const uint8_t* x8, int64_t ldx8, const float* s
     if (!make_tmap_u8_2d(&tw, codes, (uint64_t)N, (uint64_t)(K / 2), (uint64_t)(K / 2), 64, 128, CU_TENSOR_MAP_SWIZZLE_64B))
         return W4A8_ERR_CUDA;
     for (int cl = cluster_kcut_ctas(M, N, K, sms); cl >= 2; --cl) {
-        const int rc = M <= 64 ? launch_cluster_kcut<SkCfg<64, 4, 12, 12, kFmtCanonical, 1, false, true>>(
+        const int rc = M <= 64 ? launch_cluster_kcut<SkCfg<64, 4, 12, 12, kFmtCanonical, false, true>>(
                                      x8, ldx8, gs, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st, &tw, gzero)
-                               : launch_cluster_kcut<SkCfg<128, 4, 8, 8, kFmtCanonical, 1, false, true>>(
+                               : launch_cluster_kcut<SkCfg<128, 4, 8, 8, kFmtCanonical, false, true>>(
                                      x8, ldx8, gs, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, cl, st, &tw, gzero);
         if (rc != -1) return rc;
     }
@@ -1093,7 +1064,7 @@ static int linear_w8a8_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, i
             CUtensorMap tx8;
             if (!make_tmap_u8_2d(&tx8, x8, (uint64_t)M, (uint64_t)K, (uint64_t)ldx8, 128, 256, CU_TENSOR_MAP_SWIZZLE_128B))
                 return W4A8_ERR_CUDA;
-            return launch_streamk<SkCfg<256, 4, 4, 3, kFmtTiledSignMag, 1, true>>(tx8, w8, s_x, s_w, sw_stride, y, ldy,
+            return launch_streamk<SkCfg<256, 4, 4, 3, kFmtTiledSignMag, true>>(tx8, w8, s_x, s_w, sw_stride, y, ldy,
                                                                                     out_dtype, nullptr, p8, (int)M,
                                                                                     (int)N, (int)K, st, &tw);
         }
@@ -1225,12 +1196,12 @@ static int linear_w4a16_tiled_impl(const void* x, int64_t ldx, int64_t M, const 
         return W4A8_ERR_CUDA;
     // (the kernel reads no activation scale in this variant)
     if (bnx == 256)
-        return launch_streamk<SkCfg<256, 2, 2, 2, kFmtTiledSignMag, 1, false, false, true>>(
+        return launch_streamk<SkCfg<256, 2, 2, 2, kFmtTiledSignMag, false, false, true>>(
             tx, wpp, s_w, s_w, sw_stride, y, ldy, out_dtype, nullptr, pl, (int)M, (int)N, (int)K, st);
     if (bnx == 128)
-        return launch_streamk<SkCfg<128, 3, 3, 2, kFmtTiledSignMag, 1, false, false, true>>(
+        return launch_streamk<SkCfg<128, 3, 3, 2, kFmtTiledSignMag, false, false, true>>(
             tx, wpp, s_w, s_w, sw_stride, y, ldy, out_dtype, nullptr, pl, (int)M, (int)N, (int)K, st);
-    return launch_streamk<SkCfg<64, 3, 3, 2, kFmtTiledSignMag, 1, false, false, true>>(
+    return launch_streamk<SkCfg<64, 3, 3, 2, kFmtTiledSignMag, false, false, true>>(
         tx, wpp, s_w, s_w, sw_stride, y, ldy, out_dtype, nullptr, pl, (int)M, (int)N, (int)K, st);
 }
 

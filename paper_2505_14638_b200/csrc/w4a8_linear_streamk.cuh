@@ -19,16 +19,6 @@
 // the codes to E4M3 (Eq. 10) into a ring of swizzled shared-memory tiles; one thread issues the
 // tcgen05 kind::f8f6f4 MMAs (weights on the M side, tokens on the N side); accumulators are
 // double-buffered in tensor memory so the epilogue warps overlap the next tile's main loop.
-//
-// RB = 2 (whole tiles only): a tile is 256 weight rows x 256 tokens -- two 128-row blocks against one
-// activation tile per k-block, two accumulators of 256 columns (all of tensor memory, so the
-// epilogue of a tile no longer overlaps the next tile; the expansion warps, which have nothing to
-// expand into meanwhile, help to drain it).  A k-block step then brings 18 KB of packed
-// weights + 32 KB of activations for eight MMAs (about 1060 tensor-pipe cycles) instead of 9 + 32 KB
-// for four: the activation bytes an SM pulls from L2 per flop are halved, and the SM's L2 port
-// (about 64 bytes per clock) no longer sets the pace.  Measured on (2048, 4096, 4096), per CTA:
-// 32 steps in 41.9 k cycles, of which the MMA warp waits 2.2 k for the first operands, 2.6 k for
-// activation tiles and 3.3 k for expanded weights; the rest is the tensor pipe itself.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -80,7 +70,7 @@ namespace w4a8 {
 // through a table of the group's eight magnitudes (two 128-byte panels per row and k-block), the
 // MMAs are kind::f16 with K = 16, and there is no activation scale.  Sign-magnitude format, whole
 // tiles only.
-template <int BNX_, int G_, int S1_, int S2_, int FMT_, int RB_ = 1, bool W8_ = false, bool CL_ = false, bool W16_ = false>
+template <int BNX_, int G_, int S1_, int S2_, int FMT_, bool W8_ = false, bool CL_ = false, bool W16_ = false>
 struct SkCfg {
     static constexpr bool W8 = W8_;
     static constexpr bool CL = CL_;
@@ -92,25 +82,22 @@ struct SkCfg {
     static constexpr int FMT = FMT_;
     static constexpr bool CANON = FMT_ == kFmtCanonical;   // see the kernel's comment
     static constexpr int kMeta = meta_bytes(FMT);
-    static constexpr int RB = RB_;     // 128-row blocks per tile
-    static constexpr int kCodeBytes = RB_ * 8192;   // packed codes of the tile's rows for one k-block
-    static constexpr int kWStage = RB_ * (CANON ? 8192 : 9216);  // rows x (64 code bytes + meta), padded to keep the activation tile 1024-aligned
+    static constexpr int kCodeBytes = 8192;   // packed codes of the tile's rows for one k-block
+    static constexpr int kWStage = CANON ? 8192 : 9216;  // rows x (64 code bytes + meta), padded to keep the activation tile 1024-aligned
     static constexpr int kXBytes = BNX * 128 * (W16_ ? 2 : 1);
     static constexpr int kStage1 = kWStage + kXBytes;
     // TA: expanded weights in tensor memory (see the kernel's comment); S2 slots of 32 columns behind the accumulators
-    static constexpr bool TA = !W8_ && !W16_ && RB_ == 1 && BNX_ <= 128;
+    static constexpr bool TA = !W8_ && !W16_ && BNX_ <= 128;
     static constexpr int kACol = 2 * BNX_;
-    static constexpr int kW8Bytes = TA ? 0 : RB_ * 128 * 128 * (W16_ ? 2 : 1);   // expanded weights of one k-block in shared memory: E4M3 (W16: BF16, two panels)
+    static constexpr int kW8Bytes = TA ? 0 : 128 * 128 * (W16_ ? 2 : 1);   // expanded weights of one k-block in shared memory: E4M3 (W16: BF16, two panels)
     static constexpr int kBarBytes = 640;
     static constexpr int kSmemBytes = S1 * kStage1 + S2 * kW8Bytes + kBarBytes + 1024;
-    static constexpr int kTmemCols = TA ? 512 : (2 * BNX < 32 ? 32 : 2 * BNX);   // RB = 1: two accumulators (double buffer); RB = 2: one per row block
+    static constexpr int kTmemCols = TA ? 512 : (2 * BNX < 32 ? 32 : 2 * BNX);   // two accumulators (double buffer)
     static constexpr int kThreads = 32 * (10 + 4 * G + (TA ? 1 : 0));   // (TA: a warp of its own requests the activation tiles)
     static constexpr int kSlotFloats = BNX * 128;
     static_assert(BNX == 16 || BNX == 32 || BNX == 64 || BNX == 128 || BNX == 256, "token tile");
-    static_assert(RB_ == 1 || (RB_ == 2 && BNX_ == 256), "two row blocks per tile only with 256-token tiles");
-    static_assert((!W8_ && !CANON) || RB_ == 1, "the FP8-weight and canonical variants use one row block per tile");
-    static_assert(!W16_ || (RB_ == 1 && !W8_ && !CL_ && FMT_ == kFmtTiledSignMag), "the BF16 variant: one row block, sign-magnitude codes, whole tiles");
-    static_assert(!CL_ || (RB_ == 1 && !W8_ && BNX_ <= 128), "the cluster exchange serves one row block and at most 128 tokens");
+    static_assert(!W16_ || (!W8_ && !CL_ && FMT_ == kFmtTiledSignMag), "the BF16 variant: sign-magnitude codes, whole tiles");
+    static_assert(!CL_ || (!W8_ && BNX_ <= 128), "the cluster exchange serves at most 128 tokens");
     // the exchange happens in the ring memory, idle by then in every CTA of the cluster: the CTA's own partial
     // tile (BNX columns x 128 channels, fp32) and behind it the slices it receives (C x ceil(BNX / C) columns)
     static_assert(!CL_ || S1_ * kStage1 + S2_ * kW8Bytes >= (2 * BNX_ + 8) * 512, "room for the exchange");
@@ -150,8 +137,8 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                       void* __restrict__ y, int64_t ldy, int out_dtype, unsigned int* counters,
                       float* slots, int M, int N, int K, int TM, int TN, int aligned, int cl,
                       unsigned int* status_word) {
-    constexpr int BNX = Cfg::BNX, G = Cfg::G, S1 = Cfg::S1, S2 = Cfg::S2, RB = Cfg::RB;
-    constexpr int TR = 128 * RB;   // weight rows per tile
+    constexpr int BNX = Cfg::BNX, G = Cfg::G, S1 = Cfg::S1, S2 = Cfg::S2;
+    constexpr int TR = 128;   // weight rows per tile
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = ptx::smem_addr(smem_raw);
     const uint32_t base = (raw_addr + 1023u) & ~1023u;
@@ -210,7 +197,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
         for (int i = lane; i < kNumBars; i += 32) {
             uint32_t count = 1u;
             if (i >= 2 * S1 && i < 2 * S1 + S2) count = Cfg::W8 ? 1u : (Cfg::TA ? 129u : 128u);   // (TA: and the activation tile's request)
-            if (i >= 2 * S1 + 2 * S2 + 2 && i < 2 * S1 + 2 * S2 + 4) count = RB == 2 ? 256u + 128u * G : 256u;   // (RB = 2: the expansion warps drain too)
+            if (i >= 2 * S1 + 2 * S2 + 2 && i < 2 * S1 + 2 * S2 + 4) count = 256u;
             ptx::mbar_init(bars_addr + 8u * (uint32_t)i, count);
         }
         if (lane == 0) {
@@ -237,89 +224,6 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
     // set-up and weight prefetch while this one runs; everything that depends on earlier kernels
     // (activations, scales, outputs, workspace) is touched only after griddepcontrol.wait.
     ptx::griddep_launch_dependents();
-
-    // RB = 2: this warp's share of the 32 chunks (2 row blocks x 16 chunks of 16 token columns) of the
-    // CTA's j-th tile -- Eq. 4 / Eq. 11 scales, cast, store.  The tile's two accumulators fill tensor
-    // memory, so nothing overlaps its epilogue: besides the two epilogue warps of a lane quarter
-    // (slots 0 and 1) the quarter's expansion warps (slot 2 + group), which have nothing to expand
-    // into until the accumulators are free again, take chunks as well.
-    auto drain_wide = [&](int j, int slot) -> bool {
-        constexpr int kSlots = 2 + G;
-        const int q = warp & 3, r = q * 32 + lane;
-        const int64_t tile = tile_begin + j;
-        const int nt = (int)(tile / TM), mt = (int)(tile - (int64_t)nt * TM);
-        const int m0 = mt * BNX;
-        const int n_lo = nt * TR + r, n_hi = n_lo + 128;
-        const float swn_lo = n_lo < N ? __ldg(s_w + (int64_t)n_lo * sw_stride) : 0.0f;
-        const float swn_hi = n_hi < N ? __ldg(s_w + (int64_t)n_hi * sw_stride) : 0.0f;
-        // activation scales of the tile's 256 tokens, one per lane and 32 tokens, fetched before the
-        // accumulator is ready and broadcast by shuffles later
-        float sx_pre[BNX / 32];
-#pragma unroll
-        for (int c = 0; c < BNX / 32; ++c) sx_pre[c] = (m0 + c * 32 + lane < M) ? __ldg(s_x + m0 + c * 32 + lane) : 0.0f;
-        const bool sx_vec = (reinterpret_cast<uintptr_t>(s_x) & 15u) == 0;
-        if (!ptx::mbar_wait(bar_acc_full(0), (uint32_t)(j & 1), abort_flag, status_word)) return false;
-        ptx::tc_fence_after_sync();
-        const uint32_t tmem_acc0 = tmem_base + ((uint32_t)(q * 32) << 16);
-#pragma unroll 1
-        for (int ch = slot; ch < 2 * (BNX / 16); ch += kSlots) {
-            const int b = ch / (BNX / 16), c0 = (ch - b * (BNX / 16)) * 16;
-            uint32_t v[16];
-            ptx::tmem_ld_32x32b_x16(tmem_acc0 + (uint32_t)(b * BNX + c0), v);
-            const int n = b == 0 ? n_lo : n_hi;
-            const float swn = b == 0 ? swn_lo : swn_hi;
-            float sx[16];
-            if (sx_vec && m0 + c0 + 16 <= M) {
-                // the chunk's sixteen activation scales: four 16-byte loads of one address per warp (L1 hits after
-                // the first warp) instead of sixteen shuffles; issued while the tensor-memory load is in flight
-#pragma unroll
-                for (int v4 = 0; v4 < 4; ++v4) {
-                    const float4 t = __ldg(reinterpret_cast<const float4*>(s_x + m0 + c0) + v4);
-                    sx[4 * v4] = t.x;
-                    sx[4 * v4 + 1] = t.y;
-                    sx[4 * v4 + 2] = t.z;
-                    sx[4 * v4 + 3] = t.w;
-                }
-            } else {
-                float sx_lane = sx_pre[0];
-#pragma unroll
-                for (int c = 1; c < BNX / 32; ++c) sx_lane = (c0 >= c * 32) ? sx_pre[c] : sx_lane;
-#pragma unroll
-                for (int jj = 0; jj < 16; ++jj) sx[jj] = __shfl_sync(0xFFFFFFFFu, sx_lane, (c0 & 16) + jj);
-            }
-            ptx::tmem_ld_wait();
-            if (m0 + c0 >= M) continue;  // warp-uniform
-            if (n < N) {
-                if (out_dtype == W4A8_OUT_FP32) {
-                    float* yp = reinterpret_cast<float*>(y) + (int64_t)(m0 + c0) * ldy + n;
-#pragma unroll
-                    for (int jj = 0; jj < 16; ++jj)
-                        if (m0 + c0 + jj < M) yp[(int64_t)jj * ldy] = __uint_as_float(v[jj]) * (sx[jj] * swn);
-                } else if (m0 + c0 + 16 <= M) {
-                    // (the whole chunk inside the problem: no test per token -- the drain is bound by issue slots)
-                    __nv_bfloat16* yp = reinterpret_cast<__nv_bfloat16*>(y) + (int64_t)(m0 + c0) * ldy + n;
-#pragma unroll
-                    for (int jj = 0; jj < 16; jj += 2) {
-                        // two tokens per multiply (packed FP32 pairs: the same two roundings per value)
-                        float sc0, sc1, r0, r1;
-                        ptx::mul_f32x2(sx[jj], sx[jj + 1], swn, swn, sc0, sc1);
-                        ptx::mul_f32x2(__uint_as_float(v[jj]), __uint_as_float(v[jj + 1]), sc0, sc1, r0, r1);
-                        yp[(int64_t)jj * ldy] = __float2bfloat16_rn(r0);
-                        yp[(int64_t)(jj + 1) * ldy] = __float2bfloat16_rn(r1);
-                    }
-                } else {
-                    __nv_bfloat16* yp = reinterpret_cast<__nv_bfloat16*>(y) + (int64_t)(m0 + c0) * ldy + n;
-#pragma unroll
-                    for (int jj = 0; jj < 16; ++jj)
-                        if (m0 + c0 + jj < M)
-                            yp[(int64_t)jj * ldy] = __float2bfloat16_rn(__uint_as_float(v[jj]) * (sx[jj] * swn));
-                }
-            }
-        }
-        ptx::tc_fence_before_sync();
-        ptx::mbar_arrive(bar_acc_empty(0));
-        return true;
-    };
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer (whole warp, one lane issues)
@@ -511,11 +415,9 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                 const int64_t tile = u / KB;
                 const int kb0 = (int)(u - tile * KB);
                 const int len = (int)((u_end - u) < (int64_t)(KB - kb0) ? (u_end - u) : (int64_t)(KB - kb0));
-                // RB = 1: two accumulators used in turn; RB = 2: both belong to the one tile in flight
-                const int buf = RB == 1 ? (j & 1) : 0;
-                if (RB == 1 ? j >= 2 : j >= 1) {
-                    const uint32_t par = RB == 1 ? (uint32_t)(((j >> 1) - 1) & 1) : (uint32_t)((j - 1) & 1);
-                    ok = ptx::mbar_wait(bar_acc_empty(buf), par, abort_flag, status_word);
+                const int buf = j & 1;   // two accumulators used in turn
+                if (j >= 2) {
+                    ok = ptx::mbar_wait(bar_acc_empty(buf), (uint32_t)(((j >> 1) - 1) & 1), abort_flag, status_word);
                     if (!ok) break;
                 }
                 const uint32_t tmem_acc = tmem_base + (uint32_t)(buf * BNX);
@@ -547,7 +449,6 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                         }
                     } else if (ptx::elect_one()) {
                         ptx::umma_f8_kblock(tmem_acc, a_lo, b_lo, idesc, accumulate);
-                        if (RB == 2) ptx::umma_f8_kblock(tmem_acc + (uint32_t)BNX, a_lo + (16384u >> 4), b_lo, idesc, accumulate);
                         ptx::umma_commit(f1);
                         ptx::umma_commit(f2);
                     }
@@ -633,24 +534,17 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
         };
         int64_t shared_tile0 = 0, shared_tile1 = 0;  // tiles of which this CTA holds a partial (first and last segment)
         int n_shared = 0;
-        if constexpr (RB == 2) {
-            // whole tiles only: this warp's chunks of every tile of the CTA
-            for (; u < u_end && ok; u += KB, ++j) ok = drain_wide(j, half);
-        }
-        // (RB = 2 is through; its instantiation does not carry the code below)
-        if constexpr (RB == 1)
         while (u < u_end && ok) {
             const int64_t tile = u / KB;
             const int kb0 = (int)(u - tile * KB);
             const int len = (int)((u_end - u) < (int64_t)(KB - kb0) ? (u_end - u) : (int64_t)(KB - kb0));
             const int nt = (int)(tile / TM), mt = (int)(tile - (int64_t)nt * TM);
             const int m0 = mt * BNX + half * kHalfCols;
-            const int buf = RB == 1 ? (j & 1) : 0;
+            const int buf = j & 1;
             const bool whole = (len == KB);
-            float swn_rb[RB];
-#pragma unroll
-            for (int b = 0; b < RB; ++b)
-                swn_rb[b] = (nt * TR + b * 128 + r < N) ? __ldg(s_w + (int64_t)(nt * TR + b * 128 + r) * sw_stride) : 0.0f;
+            const int n = nt * TR + r;
+            const bool row_ok = n < N;
+            const float swn = row_ok ? __ldg(s_w + (int64_t)n * sw_stride) : 0.0f;
             // Activation scales of this warp's columns, one per lane and 32 columns, fetched before
             // the accumulator is ready and broadcast by shuffles later: global loads issued inside
             // the store loop queue behind the operand traffic of the main loop.
@@ -658,7 +552,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
 #pragma unroll
             for (int c = 0; c < kHalfCols / 32; ++c)
                 sx_pre[c] = Cfg::W16 ? 1.0f : ((m0 + c * 32 + lane < M) ? __ldg(s_x + m0 + c * 32 + lane) : 0.0f);   // (W16: no activation scale)
-            ok = ptx::mbar_wait(bar_acc_full(buf), RB == 1 ? (uint32_t)((j >> 1) & 1) : (uint32_t)(j & 1), abort_flag, status_word);
+            ok = ptx::mbar_wait(bar_acc_full(buf), (uint32_t)((j >> 1) & 1), abort_flag, status_word);
             if (!ok) break;
             ptx::tc_fence_after_sync();
             const uint32_t tmem_acc0 =
@@ -775,15 +669,9 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                 }
             }
 #pragma unroll 1
-            for (int cb = 0; cb < RB * kHalfCols; cb += 16) {
-                // (RB = 2: the second row block's accumulator sits BNX columns further)
-                const int b = cb / kHalfCols, c0 = cb - b * kHalfCols;
-                const int n = nt * TR + b * 128 + r;
-                const bool row_ok = n < N;
-                const float swn = b == 0 ? swn_rb[0] : swn_rb[RB - 1];
-                const uint32_t tmem_acc = tmem_acc0 + (uint32_t)(b * BNX);
+            for (int c0 = 0; c0 < kHalfCols; c0 += 16) {
                 uint32_t v[16];
-                ptx::tmem_ld_32x32b_x16(tmem_acc + (uint32_t)c0, v);
+                ptx::tmem_ld_32x32b_x16(tmem_acc0 + (uint32_t)c0, v);
                 ptx::tmem_ld_wait();
                 if (m0 + c0 >= M) continue;  // warp-uniform
                 if (whole) {
@@ -901,21 +789,11 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                 next_meta(G);   // (past the last stage: a row that does not exist, or one that is not used)
                 dequant_canonical_row_to_smem(stage_w(s1), m, r, stage_w8(s2) + (uint32_t)r * 128u);
             } else
-#pragma unroll
-            for (int b = 0; b < RB; ++b)
-                dequant_row_to_smem<Cfg::FMT>(stage_w(s1) + tiled_row_offset(b * 128 + r),
-                                              stage_w(s1) + (uint32_t)Cfg::kCodeBytes + (uint32_t)((b * 128 + r) * Cfg::kMeta), r,
-                                              stage_w8(s2) + (uint32_t)(b * 16384) + (uint32_t)r * 128u);
+                dequant_row_to_smem<Cfg::FMT>(stage_w(s1) + tiled_row_offset(r),
+                                              stage_w(s1) + (uint32_t)Cfg::kCodeBytes + (uint32_t)(r * Cfg::kMeta), r,
+                                              stage_w8(s2) + (uint32_t)r * 128u);
             ptx::fence_proxy_async_smem();
             ptx::mbar_arrive(bar_w8_full(s2));
-            if constexpr (RB == 2) {
-                // after this group's last stage of a tile: help to drain the tile's accumulators
-                const int jt = it / KB;
-                if (it + G >= n_it || (it + G) / KB != jt) {
-                    ptx::griddep_wait();  // (scales and outputs may still be in use by earlier kernels; long satisfied by now)
-                    if (!drain_wide(jt, 2 + g)) break;
-                }
-            }
         }
         if constexpr (Cfg::CL) {
             ptx::cluster_arrive();

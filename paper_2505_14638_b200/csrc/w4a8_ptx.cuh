@@ -141,6 +141,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// The same for a whole warp that goes on together (collective instructions follow): every lane has the same answer,
+// also when the limit runs out between two lanes' tries.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
+                                               unsigned int* status_word) {
+    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag, status_word)) != 0;
+}
+
 // Generic-proxy writes (st.shared) made visible to the async proxy (TMA / tcgen05 reads).
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -429,6 +436,30 @@ __device__ __forceinline__ void tmem_ld_wait() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// The same, and the registers of the loads that it waits for are not used ahead of it.
+__device__ __forceinline__ void tmem_ld_wait_for(uint32_t (&r)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :
+                 : "memory");
+}
+// 16 lanes x 16 consecutive 32-bit columns as two fragments of eight columns: of fragment f thread t receives lane
+// t / 4, columns 2 (t % 4) and the next in r[4 f], r[4 f + 1] and lane t / 4 + 8 in r[4 f + 2], r[4 f + 3].
+__device__ __forceinline__ void tmem_ld_16x256b_x2(uint32_t taddr, uint32_t* r) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+}
+// Four 8 x 8 matrices of 16-bit values, each turned: thread t holds row t / 4, columns 2 (t % 4) and the next of matrix i
+// in r[i]; column k of matrix i becomes the 16 bytes at the address that lane 8 i + k passes.
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, const uint32_t (&r)[4]) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared::cta.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r[0]), "r"(r[1]),
+                 "r"(r[2]), "r"(r[3])
+                 : "memory");
+}
+
 // ---- CTA pairs (thread-block cluster of two, tcgen05 cta_group::2) ----------------------------
 // The two CTAs of a pair run one MMA of 256 rows: each holds 128 rows of A and of D (in its own
 // shared and tensor memory, at the same offsets in both) and half of the B tile's rows; the CTA
@@ -447,8 +478,11 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
+// Arrival on a barrier of another CTA of the cluster (or of this one).  Release at CTA scope: what it announces is read by
+// tensor cores, behind a proxy fence or a tcgen05 fence of its own.  At cluster scope the arrival first waits for
+// everything the thread has in flight: 1500 cycles for a warp that has just written expanded weights.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
 // Split cluster barrier (every thread of every CTA of the cluster arrives, and waits before it arrives again).
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
@@ -514,12 +548,40 @@ __device__ __forceinline__ void umma_f8_kblock_pair(uint32_t tmem_d, uint32_t a_
         "r"(a_lo), "r"(b_lo), "r"(kUmmaDescHiSw128), "r"(idesc), "r"(accumulate_first)
         : "memory");
 }
-// Arrive on the barrier at `bar` (same offset) in BOTH CTAs of the pair once all MMAs issued so
-// far by this thread have completed.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
+// The same with the A operand in tensor memory (each CTA's 128 rows in its own, at the same columns).
+__device__ __forceinline__ void umma_f8_kblock_pair_ts(uint32_t tmem_d, uint32_t tmem_a, uint32_t b_lo, uint32_t idesc,
+                                                       uint32_t accumulate_first) {
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p, pt;\n\t"
+        ".reg .b64 db;\n\t"
+        ".reg .b32 ta, bl;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "setp.eq.b32 pt, %3, %3;\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], [%1], db, %4, p;\n\t"
+        "add.u32 ta, %1, 8;\n\t"
+        "add.u32 bl, %2, 2;\n\t"
+        "mov.b64 db, {bl, %3};\n\t"
+        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], [ta], db, %4, pt;\n\t"
+        "add.u32 ta, %1, 16;\n\t"
+        "add.u32 bl, %2, 4;\n\t"
+        "mov.b64 db, {bl, %3};\n\t"
+        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], [ta], db, %4, pt;\n\t"
+        "add.u32 ta, %1, 24;\n\t"
+        "add.u32 bl, %2, 6;\n\t"
+        "mov.b64 db, {bl, %3};\n\t"
+        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], [ta], db, %4, pt;\n\t"
+        "}\n" ::"r"(tmem_d),
+        "r"(tmem_a), "r"(b_lo), "r"(kUmmaDescHiSw128), "r"(idesc), "r"(accumulate_first)
+        : "memory");
+}
+// Arrive on the barrier at `bar` (same offset) in BOTH CTAs of the pair (`mask`: their ranks' bits) once all MMAs
+// issued so far by this thread have completed.
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint16_t mask) {
     asm volatile(
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-        "h"((uint16_t)3)
+        "h"(mask)
         : "memory");
 }
 

@@ -77,21 +77,37 @@ __device__ __forceinline__ void load_row_codes(uint32_t src, uint32_t (&pk)[16])
     load_code_chunk<3>(src, pk);
 }
 
-// Expands one row of one k-block into 128 E4M3 bytes written as a row of a K-major tile with
-// the 128-byte swizzle.  `src` = shared address of the row's first code chunk (piece base +
-// tiled_row_offset(row)), `meta` = shared address of its meta entry, `row` = row index within
-// the destination tile, `dst` = shared address of the destination row.
+// The same from global memory, past L1 (`src` as for load_row_codes).
+__device__ __forceinline__ void load_row_codes_global(const uint8_t* src, uint32_t (&pk)[16]) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(pk[4 * c]), "=r"(pk[4 * c + 1]), "=r"(pk[4 * c + 2]), "=r"(pk[4 * c + 3])
+                     : "l"(src + c * kChunkStride));
+}
 template <int FMT>
-__device__ __forceinline__ void dequant_row_to_smem(uint32_t src, uint32_t meta, int row, uint32_t dst) {
-    const uint32_t sw128 = (uint32_t)(row & 7);
+__device__ __forceinline__ uint32_t load_meta_word_global(const uint8_t* p) {
+    return FMT == kFmtTiledSignMag ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(p)) : __ldg(reinterpret_cast<const uint32_t*>(p));
+}
+
+__device__ __forceinline__ uint32_t load_meta_word(uint32_t meta, int fmt) {
     uint32_t mbits;
-    if constexpr (FMT == kFmtTiledSignMag)
+    if (fmt == kFmtTiledSignMag)
         asm volatile("ld.shared.u16 %0, [%1];" : "=r"(mbits) : "r"(meta));
     else
         asm volatile("ld.shared.u32 %0, [%1];" : "=r"(mbits) : "r"(meta));
+    return mbits;
+}
+
+// Expands one row of one k-block into 128 E4M3 bytes written as a row of a K-major tile with
+// the 128-byte swizzle.  `src` = shared address of the row's first code chunk (piece base +
+// tiled_row_offset(row)), `meta` = shared address of its meta entry, `row` = row index within
+// the destination tile, `dst` = shared address of the destination row.  (expand_row_to_smem: codes and meta word are in
+// registers already.)
+template <int FMT>
+__device__ __forceinline__ void expand_row_to_smem(const uint32_t (&pk)[16], uint32_t mbits, int row, uint32_t dst) {
+    const uint32_t sw128 = (uint32_t)(row & 7);
     const float sc = bf16_bits_to_float(mbits & 0xFFFFu);
-    uint32_t pk[16];
-    load_row_codes(src, pk);
     SignMagLut slut;
     DequantLut glut;
     if constexpr (FMT == kFmtTiledSignMag)
@@ -112,6 +128,13 @@ __device__ __forceinline__ void dequant_row_to_smem(uint32_t src, uint32_t meta,
                      "r"(o1), "r"(o2), "r"(o3)
                      : "memory");
     }
+}
+template <int FMT>
+__device__ __forceinline__ void dequant_row_to_smem(uint32_t src, uint32_t meta, int row, uint32_t dst) {
+    const uint32_t mbits = load_meta_word(meta, FMT);
+    uint32_t pk[16];
+    load_row_codes(src, pk);
+    expand_row_to_smem<FMT>(pk, mbits, row, dst);
 }
 
 // The same for a row of a canonical tile: the TMA tile of 64 bytes per row with the 64-byte swizzle at `tile`; scale
@@ -276,15 +299,6 @@ __device__ __forceinline__ void dequant_canonical_row_to_tmem(uint32_t tile, uin
                      : "=r"(p[4 * j]), "=r"(p[4 * j + 1]), "=r"(p[4 * j + 2]), "=r"(p[4 * j + 3])
                      : "r"(src + (((uint32_t)j ^ sw64) << 4)));
     expand_row_to_tmem<kFmtTiled>(p, meta, taddr);
-}
-
-__device__ __forceinline__ uint32_t load_meta_word(uint32_t meta, int fmt) {
-    uint32_t mbits;
-    if (fmt == kFmtTiledSignMag)
-        asm volatile("ld.shared.u16 %0, [%1];" : "=r"(mbits) : "r"(meta));
-    else
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(mbits) : "r"(meta));
-    return mbits;
 }
 
 // Two rows (two items of one pipeline stage) expanded into 2 x 32 consecutive tensor-memory
