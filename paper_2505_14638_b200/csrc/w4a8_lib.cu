@@ -391,11 +391,8 @@ static bool make_sn_plan(int64_t N, int64_t K, int sms, bool may_split_k, SnPlan
     // expansion work then covers 128 useful rows instead of a sliver, and its K walk is shorter;
     // the price is a small fix-up through the workspace.
     const int64_t blocks128 = (N + 127) / 128;
-    // (With 64- and 128-token tiles the partial sums are four and eight times larger: only worth
-    // it for a long K; with 64 tokens also from K = 4096 on when at most a quarter of the SMs would
-    // otherwise get a 128-row block -- o projection at M = 32: 10.9 against 14.6 us.)
-    const int64_t kb_min = Cfg::MT == 16 ? 8 : (Cfg::MT == 64 && blocks128 * 4 <= sms ? 32 : 64);
-    if (may_split_k && blocks128 * 2 <= sms && KB >= kb_min) {
+    // (Up to 16 tokens: with more the partial sums are larger, and such layers take the cluster plan.)
+    if (Cfg::MT == 16 && may_split_k && blocks128 * 2 <= sms && KB >= 8) {
         int64_t ks = sms / blocks128;
         if (ks > KB / 4) ks = KB / 4;  // at least four k-blocks per chunk
         if (ks > 1 && blocks128 <= (int64_t)(kSnCounterBytes / sizeof(unsigned int)) &&
@@ -442,9 +439,11 @@ static int launch_splitn_cfg(const CUtensorMap& tx, const uint8_t* wpp, const fl
     SnPlan pl;
     const bool ws_usable = sn_workspace_usable(workspace, workspace_bytes);
     if (!make_sn_plan<Cfg>(N, K, sms, ws_usable, &pl)) return W4A8_ERR_BAD_SHAPE;
-    if (pl.KSPLIT > 1)
-        return launch_splitn_planned<SnCfg<MT, G, FMT, true>>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K,
-                                                              st, workspace, ws_usable, pl, sms);
+    if constexpr (MT == 16) {
+        if (pl.KSPLIT > 1)
+            return launch_splitn_planned<SnCfg<MT, G, FMT, true>>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K,
+                                                                  st, workspace, ws_usable, pl, sms);
+    }
     return launch_splitn_planned<Cfg>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K, st, workspace,
                                       ws_usable, pl, sms);
 }
@@ -537,15 +536,21 @@ static int launch_pair(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, cons
     return launch_status();
 }
 
-// Where the cluster plan cannot run (not all of its clusters resident at once on this device):
-// 65..128 tokens on a layer with few output channels (at most a quarter as many 128-row tiles as
-// SMs) take the persistent kernel with K cut between a whole number of CTAs per tile and the
-// exchange through the workspace, instead of the split-N kernel, every CTA of which pulls the whole
-// X8 through its L2 port (measured with the expansion through shared memory that this kernel had then, us: o
-// projection 13.4 against 15.3, down projection 21.5 against 27.5; qkv and gate_up stay: 16.9 against 15.4, 33.6 against
-// 27.1.  Since the expansion goes to tensor memory o takes 12.0 and down 17.4; qkv and gate_up have not been measured again).
-static bool streamk_for_128_tokens(int64_t M, int64_t N, int64_t K, int sms) {
-    return M > 64 && M <= kSplitNMaxM && K >= 2048 && ((N + 127) / 128) * 4 <= sms;
+// 17..128 tokens where the cluster plan does not run (more than half as many tiles of 128 channels as SMs): whole tiles of 128 channels x 64 or
+// 128 tokens of the persistent kernel instead of the split-N kernel, whose CTAs each pull all of X8 through their L2
+// port and expand rows that their MMAs then pad.  Split-N / this, us, weights not in L2, K = 1024, 2048, 4096, 8192:
+//   sign-magnitude     (32, 9600)    6.3 / 4.4   8.2 / 6.0    11.3 / 9.2    18.6 / 17.0
+//                      (32, 28672)   8.7 / 7.4   12.0 / 11.4  18.9 / 19.2   34.2 / 37.4
+//                      (64, 19200)   10.1 / 7.3  13.5 / 11.1  20.3 / 19.5   34.1 / 35.7
+//                      (128, 28672)  14.3 / 8.9  17.8 / 12.8  25.4 / 22.2   43.1 / 43.4
+//   generic            (24, 28672)   10.3 / 8.9  15.3 / 14.0  25.4 / 24.4   45.6 / 43.7
+//                      (128, 28672)  15.9 / 10.4 21.4 / 15.4  31.7 / 26.0   56.0 / 52.9
+// Sign-magnitude layers with a long K and more than one round of tiles stay, the more so the fewer the tokens.  Host to host
+// (outputs to pinned host memory) (24, 14336, 2048) 30.2 / 28.0, (128, 28672, 1024) 176 / 168.
+static bool whole_tiles_apply(int64_t M, int64_t N, int64_t K, int fmt, int sms) {
+    const int64_t tiles = (N + 127) / 128;
+    if (M <= 16 || M > kSplitNMaxM) return false;
+    return fmt != kFmtTiledSignMag || tiles <= sms || K < (M <= 32 ? 3072 : 6144);
 }
 
 // Few tiles (at most half as many 128-row tiles as SMs) and at most 128 tokens: CTAs per tile of the plan
@@ -793,17 +798,9 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
             if (rc != -1) return rc;
         }
     }
-    bool split_n = M <= kSplitNMaxM;
-    if (split_n && M > 64) {
-        // (the persistent kernel needs its full workspace; without it the split-N kernel runs)
-        SkPlan plq;
-        make_sk_plan(M, N, K, kNominalSMs, &plq);
-        const int sms_q = sm_count();
-        if (sms_q > 0 && streamk_for_128_tokens(M, N, K, sms_q) && workspace != nullptr &&
-            workspace_bytes >= plq.workspace_bytes && aligned16(workspace))
-            split_n = false;
-    }
-    if (split_n) {
+    const int sms_w = M <= kSplitNMaxM ? sm_count() : 0;
+    const bool whole = whole_tiles_apply(M, N, K, fmt, sms_w);
+    if (M <= kSplitNMaxM && !whole) {
         int rc = check_device();
         if (rc != W4A8_OK) return rc;
         const int mt = M <= 16 ? 16 : (M <= 64 ? 64 : 128);
@@ -812,38 +809,41 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
                              CU_TENSOR_MAP_SWIZZLE_128B))
             return W4A8_ERR_CUDA;
         const int Mi = (int)M, Ni = (int)N, Ki = (int)K;
-        if (mt == 128) {
+        if (mt == 16)
             return fmt == kFmtTiledSignMag
-                       ? launch_splitn_cfg<128, 4, kFmtTiledSignMag>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype,
-                                                                     Mi, Ni, Ki, st, workspace,
-                                                                     workspace_bytes)
-                       : launch_splitn_cfg<128, 4, kFmtTiled>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi, Ni,
-                                                              Ki, st, workspace, workspace_bytes);
-        }
-        if (fmt == kFmtTiledSignMag) {
-            return mt == 16 ? launch_splitn_cfg<16, 2, kFmtTiledSignMag>(tx, wpp, s_x, s_w, sw_stride, y, ldy,
-                                                                            out_dtype, Mi, Ni, Ki, st,
-                                                                            workspace, workspace_bytes)
-                            : launch_splitn_cfg<64, 4, kFmtTiledSignMag>(tx, wpp, s_x, s_w, sw_stride, y, ldy,
-                                                                            out_dtype, Mi, Ni, Ki, st,
-                                                                            workspace, workspace_bytes);
-        }
-        return mt == 16 ? launch_splitn_cfg<16, 2, kFmtTiled>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi,
-                                                                 Ni, Ki, st, workspace, workspace_bytes)
-                        : launch_splitn_cfg<64, 4, kFmtTiled>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi,
-                                                                 Ni, Ki, st, workspace, workspace_bytes);
+                       ? launch_splitn_cfg<16, 2, kFmtTiledSignMag>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi, Ni,
+                                                                    Ki, st, workspace, workspace_bytes)
+                       : launch_splitn_cfg<16, 2, kFmtTiled>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi, Ni, Ki, st,
+                                                             workspace, workspace_bytes);
+        // (more than 16 tokens: sign-magnitude weights only, see whole_tiles_apply)
+        return mt == 64 ? launch_splitn_cfg<64, 4, kFmtTiledSignMag>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi, Ni,
+                                                                     Ki, st)
+                        : launch_splitn_cfg<128, 4, kFmtTiledSignMag>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi, Ni,
+                                                                      Ki, st);
     }
-    if (reinterpret_cast<uintptr_t>(workspace) & 15u) return W4A8_ERR_BAD_ALIGNMENT;
     SkPlan pl;
     make_sk_plan(M, N, K, kNominalSMs, &pl);
-    if (!workspace || workspace_bytes < pl.workspace_bytes) return W4A8_ERR_WORKSPACE_TOO_SMALL;
+    if (!whole) {
+        if (reinterpret_cast<uintptr_t>(workspace) & 15u) return W4A8_ERR_BAD_ALIGNMENT;
+        if (!workspace || workspace_bytes < pl.workspace_bytes) return W4A8_ERR_WORKSPACE_TOO_SMALL;
+    }
     int rc = check_device();
     if (rc != W4A8_OK) return rc;
     const int sms = sm_count();
     if (sms <= 0) return W4A8_ERR_CUDA;
     int choice = 0;
-    if (M > kSplitNMaxM) choice = prefill_choice(M, N, K, sms, &pl);
-    else make_sk_plan(M, N, K, sms, &pl);
+    if (whole) {
+        pl.bnx = M <= 64 ? 64 : 128;
+        pl.TM = 1;
+        pl.TN = (int)((N + 127) / 128);
+        pl.U = (int64_t)pl.TN * (K / 128);
+        pl.aligned = 1;
+        pl.P = pl.TN < sms ? pl.TN : sms;
+        pl.counter_bytes = 0;
+        workspace = nullptr;   // (none is used)
+    } else {
+        choice = prefill_choice(M, N, K, sms, &pl);
+    }
 #define W4A8_PAIR(KP, ...)                                                                                            \
     return fmt == kFmtTiledSignMag                                                                                    \
                ? launch_pair<PairCfg<kFmtTiledSignMag, __VA_ARGS__>>(x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy,      \
