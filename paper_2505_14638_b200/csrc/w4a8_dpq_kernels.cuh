@@ -201,11 +201,24 @@ __device__ __forceinline__ long long row_sum_ll(long long v) {
 }
 
 // Step b of the quantizer, one launch: the first CTAs quantize block b (processing positions
-// [128 b, 128 b + 128), 32 rows per CTA), the others apply the errors of block b - 1 to the columns to
-// the right of block b.  The two touch different columns, so the serial chain of a block (some ten
-// microseconds) runs beside the contraction that fills the chip.  Measured, us per layer, this kernel / a block
-// kernel (57 us: IEEE divisions, half a warp per row) followed by a trailing kernel (scalar FMAs, 8 x 8 per thread):
-// (N, K) = (256, 1024) 221 / 479, (256, 4096) 948 / 2109, (4096, 4096) 2288 / 3525, (4096, 14336) 22264 / 28550.
+// [128 b, 128 b + 128), 32 rows per CTA), after the errors of block b - 1; the others apply the errors of earlier blocks to
+// the columns to the right.  The two touch different columns, so the serial chain of a block (some ten
+// microseconds) runs beside the contraction that fills the chip.
+// The errors of two blocks 2 m, 2 m + 1 are applied together: a tile's weights are read and written, and its
+// CTA started, once per 256 values of q instead of once per 128.  Steps:
+//   2 m + 2: both blocks' errors to the first part of the columns behind block 2 m + 2 (`far`), block 2 m + 3 among them;
+//   2 m + 3: the same for the rest, and (`near`) block 2 m + 2's errors to block 2 m + 4, whose own step then adds those
+//            of block 2 m + 3.
+// Every column sees the errors in ascending order.  (Few tiles in a step: one block's errors at a time, all of them `near`; the
+// launch decides, see there.)  Measured, us per layer, one block at a time / a block kernel (57 us: IEEE divisions, half a warp
+// per row) followed by a trailing kernel (scalar FMAs, 8 x 8 per thread): (N, K) = (256, 1024) 221 / 479, (256, 4096) 948 / 2109,
+// (4096, 4096) 2288 / 3525, (4096, 14336) 22264 / 28550.
+struct DpqTrail {
+    int errors;   // first block whose errors are applied
+    int blocks;   // how many (1 or 2)
+    int first;    // first column block
+    int count;    // column blocks
+};
 constexpr int kDpqThreads = 256;
 constexpr int kDpqRowsPerCta = 32;      // eight lanes per row
 constexpr int kDpqChunk = 32;           // values of q per stage
@@ -256,7 +269,7 @@ __device__ __forceinline__ void dpq_load_errors(float* e_s, uint32_t e_addr, con
     }
 }
 
-// Columns to the right of block b, w[n][v] <- fma(-e[n][q], U[q][v], w[n][v]) for the q of block b - 1 in
+// Columns further to the right, w[n][v] <- fma(-e[n][q], U[q][v], w[n][v]) for the q of one block or of two in
 // ascending order: the chain of fused multiply-adds that the column-by-column algorithm performs for that element.
 // 128 rows x 128 columns per CTA; a warp takes 16 rows and all columns, a lane four columns.  Bound: the FP32 pipes,
 // if shared memory keeps up: per q a warp reads 512 distinct bytes of U and sixteen errors that all lanes share
@@ -267,8 +280,9 @@ __device__ __forceinline__ void dpq_load_errors(float* e_s, uint32_t e_addr, con
 // of the 28-31 T that a loop of FMAs alone reaches.  Errors and rows of U come in double-buffered chunks of 32 q.
 __device__ __forceinline__ void dpq_trailing_tile(uint8_t* sm, uint32_t sm_addr, float* __restrict__ work,
                                                   const float* __restrict__ U, int64_t N, int64_t K, int64_t pprev,
-                                                  int64_t v0, int64_t n0, bool uvec) {
-    constexpr int kChunks = 128 / kDpqChunk;
+                                                  int blocks, int64_t v0, int64_t n0, bool uvec) {
+    constexpr int kPerBlock = 128 / kDpqChunk;
+    const int chunks = blocks * kPerBlock;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const float* usrc = U + (pprev + (tid >> 5)) * K + v0 + 4 * lane;
     auto load_u = [&](int c) {
@@ -278,7 +292,8 @@ __device__ __forceinline__ void dpq_trailing_tile(uint8_t* sm, uint32_t sm_addr,
     };
     auto load_e = [&](int c) {
         const int off = DpqSmem::kTrailErr + (c & 1) * kDpqChunk * 128 * 4;
-        dpq_load_errors<128>(reinterpret_cast<float*>(sm + off), sm_addr + (uint32_t)off, work, N, K, pprev, n0, c);
+        dpq_load_errors<128>(reinterpret_cast<float*>(sm + off), sm_addr + (uint32_t)off, work, N, K, pprev + (int64_t)(c / kPerBlock) * 128, n0,
+                             c % kPerBlock);
     };
     load_u(0);   // (U is the caller's: complete before the first launch of the chain)
     ptx::griddep_wait();
@@ -298,10 +313,10 @@ __device__ __forceinline__ void dpq_trailing_tile(uint8_t* sm, uint32_t sm_addr,
         acc[i][3] = pack_f32x2(a.w, b.w);
     }
 #pragma unroll 1
-    for (int c = 0; c < kChunks; ++c) {
+    for (int c = 0; c < chunks; ++c) {
         dpq_wait<0>();
         __syncthreads();   // chunk c is there; chunk c - 1 has been consumed by everybody
-        if (c + 1 < kChunks) {
+        if (c + 1 < chunks) {
             load_u(c + 1);
             load_e(c + 1);
             dpq_commit();
@@ -367,7 +382,7 @@ __global__ void __launch_bounds__(kDpqThreads, 2)
 dpq_step_kernel(float* __restrict__ work, const float* __restrict__ U, const int32_t* __restrict__ perm,
                 int64_t N, int64_t K, int b, int symmetric, int mse_steps, int per_channel,
                 const float* __restrict__ s_w, uint8_t* __restrict__ codes, uint16_t* __restrict__ gscale,
-                uint8_t* __restrict__ gzero) {
+                uint8_t* __restrict__ gzero, DpqTrail far, DpqTrail near) {
     extern __shared__ __align__(16) uint8_t sm[];
     const uint32_t sm_addr = ptx::smem_addr(sm);
     const int64_t p0 = (int64_t)b * 128;
@@ -377,8 +392,11 @@ dpq_step_kernel(float* __restrict__ work, const float* __restrict__ U, const int
     ptx::griddep_launch_dependents();
     if (blockIdx.x >= block_ctas) {
         const unsigned t = blockIdx.x - block_ctas, row_tiles = (unsigned)((N + 127) / 128);
-        dpq_trailing_tile(sm, sm_addr, work, U, N, K, p0 - 128, p0 + 128 + (int64_t)(t / row_tiles) * 128,
-                          (int64_t)(t % row_tiles) * 128, uvec);
+        const unsigned col = t / row_tiles;
+        const bool is_far = col < (unsigned)far.count;
+        const DpqTrail tr = is_far ? far : near;
+        dpq_trailing_tile(sm, sm_addr, work, U, N, K, (int64_t)tr.errors * 128, tr.blocks,
+                          (int64_t)(tr.first + (int)(is_far ? col : col - (unsigned)far.count)) * 128, (int64_t)(t % row_tiles) * 128, uvec);
         return;
     }
     const float* u_s = reinterpret_cast<const float*>(sm + DpqSmem::kU);

@@ -1816,10 +1816,44 @@ int w4a8_dpq_quantize(const float* W, int64_t N, int64_t K, int group, const flo
     uint64_t launches = 3;
     const int G = (int)(K / kGroup);
     const int64_t block_ctas = (N + kDpqRowsPerCta - 1) / kDpqRowsPerCta, row_tiles = (N + 127) / 128;
+    const int64_t slots = 2 * (int64_t)sm_count();   // CTAs resident at once
+    if (slots <= 0) return W4A8_ERR_CUDA;
+    int rest = 0;         // column blocks that an even step leaves to the next one
+    bool paired = false;  // the columns behind the next block lack the errors of two blocks
     for (int b = 0; b < G; ++b) {
+        DpqTrail far = {0, 2, 0, 0}, near = {0, 1, 0, 0};
+        const int n = G - 1 - b;   // column blocks behind block b
+        // Two blocks' errors at a time pay while a step has tiles for several rounds of CTAs; with fewer, the coarser pieces leave more
+        // of the last round idle.  One block at a time throughout / two throughout / two down to four rounds, us: (4096, 14336)
+        // 22039 / 21260 / 21186, (8192, 8192) 15140 / 14578 / 14529, (4096, 4096) 2371 / 2459 / 2363, (1024, 14336) 6529 / 7020 / 6522.
+        const bool many = row_tiles * n >= 4 * slots;
+        if (b % 2 == 1) {
+            if (paired) far = {b - 3, 2, G - rest, rest};
+            if (b == 1) paired = many;
+            near = {b - 1, 1, b + 1, paired ? (n > 0 ? 1 : 0) : n};
+        } else if (paired) {
+            // the column blocks in two parts, at least two blocks in the first, with as few rounds of CTAs as possible and
+            // otherwise in halves; all of them before the errors of one block at a time follow
+            far = {b - 2, 2, b + 1, n};
+            if (many) {
+                int64_t best = INT64_MAX;
+                for (int h = n < 2 ? n : 2; h <= n; ++h) {
+                    const int64_t rounds = (block_ctas + row_tiles * h + slots - 1) / slots + (block_ctas + row_tiles * (n - h + 1) + slots - 1) / slots;
+                    const int64_t cost = rounds * 2 * G + (2 * h > n ? 2 * h - n : n - 2 * h);
+                    if (cost < best) {
+                        best = cost;
+                        far.count = h;
+                    }
+                }
+            }
+            rest = n - far.count;
+            paired = many;
+        } else if (b > 0) {
+            near = {b - 1, 1, b + 1, n};
+        }
         // (from the second step on the launches overlap: a step's CTAs start, and fetch U, while the one before drains)
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(block_ctas + (b > 0 ? row_tiles * (G - 1 - b) : 0)));
+        cfg.gridDim = dim3((unsigned)(block_ctas + row_tiles * (far.count + near.count)));
         cfg.blockDim = dim3(kDpqThreads);
         cfg.dynamicSmemBytes = (size_t)DpqSmem::kBytes;
         cfg.stream = st;
@@ -1829,7 +1863,7 @@ int w4a8_dpq_quantize(const float* W, int64_t N, int64_t K, int group, const flo
         cfg.attrs = attr;
         cfg.numAttrs = b > 0 ? 1 : 0;
         if (cudaLaunchKernelEx(&cfg, dpq_step_kernel, work, U, perm, N, K, b, symmetric, mse_steps, per_channel,
-                               static_cast<const float*>(s_w), codes, static_cast<uint16_t*>(gscale_bf16), gzero) != cudaSuccess)
+                               static_cast<const float*>(s_w), codes, static_cast<uint16_t*>(gscale_bf16), gzero, far, near) != cudaSuccess)
             return W4A8_ERR_CUDA;
         ++launches;
     }
