@@ -232,7 +232,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
                         if (ptx::elect_one()) {
                             if (Cfg::TS) ptx::umma_f8_kblock_pair_ts(acc0, a_lo, b_lo, idesc, (uint32_t)i);
                             else ptx::umma_f8_kblock_pair(acc0, a_lo, b_lo, idesc, (uint32_t)i);
-                            ptx::umma_commit_pair(fr, pair_mask);
+                            if (left >= S) ptx::umma_commit_pair(fr, pair_mask);   // (the slot is used again: see the closing barrier)
                         }
                     }
                     if (ok && ptx::elect_one()) ptx::umma_commit_pair(bar_acc_full(0), pair_mask);
@@ -263,12 +263,13 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
                             free1 = true;
                         }
                         for (int k = 0; k < d; ++k) {
+                            const bool again = left + (d - 1 - k) >= S;   // the slot is used again
                             const uint32_t a_lo = ptx::umma_desc_lo(stage_w8(r1.idx));
                             const uint32_t b_lo = ptx::umma_desc_lo(stage_x(r1.idx) + (uint32_t)Cfg::kXHalf);
                             const uint32_t fr = bar_free(r1.idx);
                             if (ptx::elect_one()) {
                                 ptx::umma_f8_kblock_pair(acc1, a_lo, b_lo, idesc, (uint32_t)(i + k));
-                                ptx::umma_commit_pair(fr, pair_mask);
+                                if (again) ptx::umma_commit_pair(fr, pair_mask);
                             }
                             r1.advance(S);
                         }
@@ -280,7 +281,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
             }
             if (!ok && lane == 0) {
                 // Gave up: let the MMAs already issued finish before tensor memory is freed.
-                ptx::umma_commit_pair(bar_drain, pair_mask);
+                ptx::umma_commit_pair(bar_drain, (uint16_t)(1u << pair_leader));
                 const uint64_t t0 = ptx::globaltimer_ns();
                 while (!ptx::mbar_try_wait(bar_drain, 0u) && ptx::globaltimer_ns() - t0 < ptx::kWaitLimitNs) {
                 }
@@ -296,6 +297,12 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
         const bool vec_ok = out_dtype != W4A8_OUT_FP32 && (ldy & 7) == 0;   // (the base is 16-byte aligned)
         bool ok = true;
         int used1 = 0;   // H = 2: tiles so far that used the second accumulator
+        int last1 = n_tiles - 1;   // H = 2: last tile that uses it
+        for (; H == 2 && last1 >= 0; --last1) {
+            int nt, mt;
+            pair_tile(c + last1 * C, TM, TN, nt, mt);
+            if (halves_of(mt) == 2) break;
+        }
         ptx::griddep_wait();  // scales come from, outputs may still be in use by, earlier kernels
         for (int j = 0; j < n_tiles && ok; ++j) {
             int nt, mt;
@@ -457,7 +464,8 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
                 }
                 ptx::tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive_cluster(ptx::map_to_cta(bar_acc_empty(h), pair_leader));
+                // (a later tile uses the accumulator: see the closing barrier)
+                if (lane == 0 && j < (h == 0 ? n_tiles - 1 : last1)) ptx::mbar_arrive_cluster(ptx::map_to_cta(bar_acc_empty(h), pair_leader));
             }
         }
     } else {
@@ -534,14 +542,27 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
 
     ptx::tc_fence_before_sync();
     __syncthreads();
-    // Nothing of the cluster touches another CTA's barriers, shared or tensor memory any more.  (Execution order only: a
-    // releasing arrival would first wait for this thread's output stores.)
-    ptx::cluster_arrive_relaxed();
+    // Closing barrier: no CTA of the cluster leaves while another may still reach into its shared memory or barriers.  It
+    // orders execution only (a releasing arrival would first wait for this thread's output stores), so nothing may be sent to
+    // another CTA that no thread of that CTA has waited for by now:
+    //   stage complete (leader: the peer's expanding warps, both CTAs' activation tiles)   by the issuer, before the stage's MMAs
+    //   stage free (both: the leader's commits)               by the warps that fill the slot again; not sent for the last S stages
+    //   accumulator complete (both: the leader's commits)     by the epilogue warps
+    //   accumulator drained (leader: the peer's epilogue warps)   by the issuer, before the next tile in it; not sent after the last
+    //   partial sums (KP = 2: the other pair's copies)        by the epilogue warps
+    // (Sent always and waited for behind the loops, (2048, 4096, 4096) took 29.3 us in place of 28.6, (8192, 28672, 8192) 1332 in place of 1301.)
+    const bool gave_up = *abort_flag != 0u;   // (the same for all threads: nobody of this CTA waits any more)
+    if (gave_up) ptx::cluster_arrive();
+    else ptx::cluster_arrive_relaxed();
     ptx::cluster_wait();
-    // gave up: partial sums that the other pair has sent all the same land before this CTA's shared memory goes away
-    if (Cfg::TS && KP == 2 && *abort_flag != 0u && threadIdx.x < 8) {
+    if (gave_up) {
+        // Not all of it has been waited for: partial sums that the other pair has sent all the same land before this CTA's
+        // shared memory goes away, and a late arrival of a CTA that has not given up has 2 ms.
         const uint64_t t0 = ptx::globaltimer_ns();
-        while (!ptx::mbar_try_wait(bar_red((int)threadIdx.x), 0u) && ptx::globaltimer_ns() - t0 < ptx::kWaitLimitNs / 20) {
+        if (Cfg::TS && KP == 2 && threadIdx.x < 8)
+            while (!ptx::mbar_try_wait(bar_red((int)threadIdx.x), 0u) && ptx::globaltimer_ns() - t0 < ptx::kWaitLimitNs / 20) {
+            }
+        while (ptx::globaltimer_ns() - t0 < ptx::kWaitLimitNs / 1000) {
         }
     }
     __syncwarp();
