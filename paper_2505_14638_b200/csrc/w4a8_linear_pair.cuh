@@ -40,6 +40,7 @@
 #include <cuda_bf16.h>
 
 #include "w4a8_common.cuh"
+#include "w4a8_prefill_plan.h"
 #include "w4a8_ptx.cuh"
 #include "w4a8_tiled_format.cuh"
 
@@ -73,18 +74,6 @@ struct PairCfg {
     static_assert(H == 2 || (256 + 32 * S <= 512 && S * kXBytes >= 8 * 8192), "tensor memory columns; room for the partial sums to send");
     static_assert(kSmemBytes <= 232448, "shared memory per CTA");
 };
-
-// Tile t -> channel tile and token tile.  Token tiles are taken in bands of kPairBand: the tiles in flight at a time
-// then cover a few token tiles and a few channel tiles, and what they read fits L2 (with token tiles running through
-// (8192, 28672, 8192) reads all 67 MB of X8 again for every four channel tiles).
-constexpr int kPairBand = 8;
-__host__ __device__ __forceinline__ void pair_tile(int t, int TM, int TN, int& nt, int& mt) {
-    const int per = kPairBand * TN, band = t / per, first = band * kPairBand;
-    const int width = TM - first < kPairBand ? TM - first : kPairBand;
-    const int u = t - band * per;
-    nt = u / width;
-    mt = first + (u - nt * width);
-}
 
 template <class Cfg>
 __global__ void __launch_bounds__(Cfg::kThreads)
@@ -124,7 +113,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
     const int kb0 = KP == 1 ? 0 : kp * KBall / KP, KB = KP == 1 ? KBall : (kp + 1) * KBall / KP - kb0;
     const uint8_t* meta_base = wpp + (int64_t)KBall * N * kRowCodeBytes;
     const int C = (int)gridDim.x / (2 * KP), c = (int)blockIdx.x / (2 * KP);
-    const int Tt = TM * TN;
+    const int Tt = TM * TN, full_tiles = pair_full_tiles(M, Cfg::kTokens, TM);
     const int n_tiles = c < Tt ? (Tt - c + C - 1) / C : 0;  // tiles c, c + C, ...
     const int n_it = n_tiles * KB;
     // accumulators of 256 tokens that a token tile needs
@@ -161,10 +150,10 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
         bool ok = true;
         ptx::Ring r;
         int issued = 0, nt, mt = 0;
-        if (n_tiles > 0) pair_tile(c, TM, TN, nt, mt);   // (ahead of the wait: nothing is between it and the first request)
+        if (n_tiles > 0) pair_tile(c, full_tiles, TN, nt, mt);   // (ahead of the wait: nothing is between it and the first request)
         ptx::griddep_wait();
         for (int j = 0; j < n_tiles && ok; ++j) {
-            if (j > 0) pair_tile(c + j * C, TM, TN, nt, mt);
+            if (j > 0) pair_tile(c + j * C, full_tiles, TN, nt, mt);
             const int halves = halves_of(mt);
             const int y0 = mt * Cfg::kTokens + (int)rank * 128;
             for (int kb = 0; kb < KB; ++kb) {
@@ -214,7 +203,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
             int used1 = 0;   // H = 2: tiles so far that used the second accumulator
             for (int j = 0; j < n_tiles && ok; ++j) {
                 int nt, mt;
-                pair_tile(c + j * C, TM, TN, nt, mt);
+                pair_tile(c + j * C, full_tiles, TN, nt, mt);
                 const int halves = halves_of(mt);
                 if (j >= 1) {
                     ok = ptx::mbar_wait_warp(bar_acc_empty(0), (uint32_t)((j - 1) & 1), abort_flag, status_word);
@@ -297,16 +286,11 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
         const bool vec_ok = out_dtype != W4A8_OUT_FP32 && (ldy & 7) == 0;   // (the base is 16-byte aligned)
         bool ok = true;
         int used1 = 0;   // H = 2: tiles so far that used the second accumulator
-        int last1 = n_tiles - 1;   // H = 2: last tile that uses it
-        for (; H == 2 && last1 >= 0; --last1) {
-            int nt, mt;
-            pair_tile(c + last1 * C, TM, TN, nt, mt);
-            if (halves_of(mt) == 2) break;
-        }
+        const int last1 = c < full_tiles * TN ? (full_tiles * TN - c + C - 1) / C - 1 : -1;   // H = 2: last tile that uses it
         ptx::griddep_wait();  // scales come from, outputs may still be in use by, earlier kernels
         for (int j = 0; j < n_tiles && ok; ++j) {
             int nt, mt;
-            pair_tile(c + j * C, TM, TN, nt, mt);
+            pair_tile(c + j * C, full_tiles, TN, nt, mt);
             const int halves = halves_of(mt);
             const int n0 = nt * 256 + (int)rank * 128 + q * 32;   // this warp's first channel
             // Eq. 11 scales: of the fragment's channels (rows lane / 4 + 8 g), or of this lane's channel
@@ -485,7 +469,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
                 at.kb -= KB;
                 if (++at.j < n_tiles) {
                     int nt, mt;
-                    pair_tile(c + at.j * C, TM, TN, nt, mt);
+                    pair_tile(c + at.j * C, full_tiles, TN, nt, mt);
                     at.n0 = nt * 256 + (int)rank * 128;
                 }
             }
