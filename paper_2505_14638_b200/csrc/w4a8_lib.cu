@@ -393,6 +393,45 @@ static int launch_splitn_planned(const CUtensorMap& tx, const uint8_t* wpp, cons
     return launch_status();
 }
 
+// Clusters of `size` CTAs (at most 8) of a kernel that the device holds at once, asked of the device once per kernel and size; -1
+// where it cannot tell.
+template <class Cfg, class Kernel>
+static int clusters_resident(Kernel kern, int size) {
+    static std::atomic<int> fits[9];   // (0: not asked yet)
+    int have = fits[size].load(std::memory_order_relaxed);
+    if (have != 0) return have;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(size * 64));
+    cfg.blockDim = dim3(Cfg::kThreads);
+    cfg.dynamicSmemBytes = (size_t)Cfg::kSmemBytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&have, kern, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        have = -1;
+    }
+    if (have <= 0) have = -1;
+    fits[size].store(have, std::memory_order_relaxed);
+    return have;
+}
+
+// Tiles of 256 channels x 256 tokens, also with K cut between two pairs.
+template <int FMT>
+using PairKCut = PairCfg<FMT, 1, 3, 6>;
+
+// Clusters of two pairs that the device holds at once (33 on 148 SMs: a cluster's SMs lie in one group of SMs, and the groups'
+// sizes are no multiples of four).
+template <int FMT>
+static int pair_quads() {
+    return clusters_resident<PairKCut<FMT>>(linear_pair_kernel<PairKCut<FMT>>, 4);
+}
+
 // Tiles of CTA pairs (see linear_pair_kernel): `kp` pairs share a tile's K.
 template <class Cfg>
 static int launch_pair(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, const float* s_x, const float* s_w,
@@ -413,6 +452,7 @@ static int launch_pair(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, cons
     const int TM = (M + Cfg::kTokens - 1) / Cfg::kTokens, TN = (N + 255) / 256;
     if (kp > 1 && K / 128 < 2 * kp) return W4A8_ERR_INVALID_ARG;   // (every pair needs k-blocks of its own)
     int clusters = sms / (2 * kp);
+    if (kp > 1 && clusters < TM * TN) return W4A8_ERR_INVALID_ARG;   // (one tile per cluster)
     if (clusters > TM * TN) clusters = TM * TN;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * kp * clusters));
@@ -471,32 +511,7 @@ static int launch_cluster_kcut(const uint8_t* x8, int64_t ldx8, const uint8_t* w
                                int sw_stride, void* y, int64_t ldy, int out_dtype, int M, int N, int K, int cl,
                                cudaStream_t st, const CUtensorMap* tw = nullptr, const uint8_t* gzero = nullptr) {
     const int TN = (N + 127) / 128;
-    static std::atomic<int> fits[9];   // clusters of size cl resident at once (0: not asked yet)
-    int have = fits[cl].load(std::memory_order_relaxed);
-    if (have == 0) {
-        auto kern = linear_streamk_kernel<Cfg>;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes) != cudaSuccess)
-            return W4A8_ERR_CUDA;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(cl * 64));
-        cfg.blockDim = dim3(Cfg::kThreads);
-        cfg.dynamicSmemBytes = (size_t)Cfg::kSmemBytes;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)cl;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            n = -1;
-        }
-        have = n > 0 ? n : -1;
-        fits[cl].store(have, std::memory_order_relaxed);
-    }
-    if (have < TN) return -1;
+    if (clusters_resident<Cfg>(linear_streamk_kernel<Cfg>, cl) < TN) return -1;
     CUtensorMap tx;
     if (!make_tmap_u8_2d(&tx, x8, (uint64_t)M, (uint64_t)K, (uint64_t)ldx8, 128, (uint32_t)Cfg::BNX,
                          CU_TENSOR_MAP_SWIZZLE_128B))
@@ -741,7 +756,8 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
         pl.counter_bytes = 0;
         workspace = nullptr;   // (none is used)
     } else {
-        choice = prefill_choice(M, N, K, sms, &pl);
+        const int quads = fmt == kFmtTiledSignMag ? pair_quads<kFmtTiledSignMag>() : pair_quads<kFmtTiled>();
+        choice = prefill_choice(M, N, K, sms, quads, &pl);
     }
 #define W4A8_PAIR(KP, ...)                                                                                            \
     return fmt == kFmtTiledSignMag                                                                                    \

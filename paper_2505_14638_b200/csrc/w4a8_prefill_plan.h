@@ -116,7 +116,7 @@ inline double make_sk_plan(int64_t M, int64_t N, int64_t K, int sms, SkPlan* pl)
 // 1500 [2], (2048, 4096, 4096) 36.3 / 34.7 [2], (1531, 28672, 4096) 208 / 171 [2], (1531, 4096, 14336) 121 / 95 [2], (1024,
 // 28672, 4096) 152 / 121 [2], (512, 6144, 4096) 18.4 / 15.9 [1], (512, 28672, 4096) 71 / 63 [2], (512, 4096, 14336) 45.2 / 33.0
 // [3], (256, 4096, 4096) 16.5 / 10.9 [3]; (512, 4096, 4096) 12.2 / - / 14.1 on pairs [0].
-inline int prefill_choice(int64_t M, int64_t N, int64_t K, int sms, SkPlan* pl) {
+inline int prefill_choice(int64_t M, int64_t N, int64_t K, int sms, int quads, SkPlan* pl) {
     const int64_t KB = K / 128, pairs = sms / 2, TN = (N + 255) / 256;
     double best = make_sk_plan(M, N, K, sms, pl);
     int choice = 0;
@@ -134,7 +134,7 @@ inline int prefill_choice(int64_t M, int64_t N, int64_t K, int sms, SkPlan* pl) 
         best = t;
         choice = 2;
     }
-    if (4 * t1 <= sms - 4 && KB >= 8) {
+    if (t1 <= quads && KB >= 8) {   // (a second round of them would cost more than the cut saves)
         t = (double)((KB + 1) / 2) * 0.244 + 7.3;
         if (t < best) choice = 3;
     }

@@ -19,6 +19,10 @@ extern "C" void tiles(long long M, long long N, int tokens, int* nt, int* mt) {
     const int TM = (int)((M + tokens - 1) / tokens), TN = (int)((N + 255) / 256);
     for (int t = 0; t < TM * TN; ++t) pair_tile(t, pair_full_tiles(M, tokens, TM), TN, nt[t], mt[t]);
 }
+extern "C" int choice(long long M, long long N, long long K, int sms, int quads) {
+    SkPlan pl;
+    return prefill_choice(M, N, K, sms, quads, &pl);
+}
 """
 
 
@@ -31,6 +35,7 @@ def plan(tmp_path_factory):
                    check=True, capture_output=True)
     lib = ctypes.CDLL(str(so))
     lib.half_rounds.argtypes, lib.half_rounds.restype = [ctypes.c_longlong] * 3, ctypes.c_longlong
+    lib.choice.argtypes = [ctypes.c_longlong] * 3 + [ctypes.c_int] * 2
     lib.tiles.argtypes = [ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p]
     return lib
 
@@ -60,3 +65,14 @@ def test_rounds_of_the_model_are_those_of_the_schedule(plan, pairs):
     for M, N in _shapes():
         cost = [2 if M - 512 * m > 256 else 1 for _, m in _tiles(plan, M, N, 512)]
         assert plan.half_rounds(M, N, pairs) == max(sum(cost[c::pairs]) for c in range(min(pairs, len(cost)))), (M, N)
+
+
+@pytest.mark.parametrize("quads", [37, 33, 4, -1])
+def test_k_is_cut_between_pairs_in_one_round_only(plan, quads):
+    # a cluster of four CTAs works on one tile: no more tiles than clusters that the device holds at once
+    rng = random.Random(quads)
+    named = [(374, 4608, 11904), (1488, 1376, 10496), (1557, 1280, 7296), (512, 4096, 14336), (300, 2064, 8320), (257, 256, 14336)]
+    shapes = named + [(rng.randint(129, 2000), 16 * rng.randint(16, 600), 128 * rng.randint(8, 112)) for _ in range(2000)]
+    cut = [(M, N) for M, N, K in shapes if plan.choice(M, N, K, 148, quads) == 3]
+    assert all(-(-M // 256) * -(-N // 256) <= quads for M, N in cut)
+    assert bool(cut) == (quads > 0)
