@@ -468,8 +468,8 @@ static int launch_pair(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, cons
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K, TM, TN, kp,
-                                       status);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K, TM, TN,
+                                       pair_full_tiles(M, Cfg::kTokens, TM), kp, status);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     if (e != cudaSuccess) return W4A8_ERR_CUDA;
     return launch_status();

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(Cfg::kThreads)
 linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K], box 128 x 128, 128B swizzle
                    const uint8_t* __restrict__ wpp, const float* __restrict__ s_x,
                    const float* __restrict__ s_w, int sw_stride, void* __restrict__ y, int64_t ldy, int out_dtype,
-                   int M, int N, int K, int TM, int TN, int KP, unsigned int* status_word) {
+                   int M, int N, int K, int TM, int TN, int full_tiles, int KP, unsigned int* status_word) {
     constexpr int H = Cfg::H, G = Cfg::G, S = Cfg::S;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = ptx::smem_addr(smem_raw);
@@ -113,7 +113,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
     const int kb0 = KP == 1 ? 0 : kp * KBall / KP, KB = KP == 1 ? KBall : (kp + 1) * KBall / KP - kb0;
     const uint8_t* meta_base = wpp + (int64_t)KBall * N * kRowCodeBytes;
     const int C = (int)gridDim.x / (2 * KP), c = (int)blockIdx.x / (2 * KP);
-    const int Tt = TM * TN, full_tiles = pair_full_tiles(M, Cfg::kTokens, TM);
+    const int Tt = TM * TN;
     const int n_tiles = c < Tt ? (Tt - c + C - 1) / C : 0;  // tiles c, c + C, ...
     const int n_it = n_tiles * KB;
     // accumulators of 256 tokens that a token tile needs

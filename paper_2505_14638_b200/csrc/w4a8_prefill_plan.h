@@ -39,17 +39,18 @@ struct SkPlan {
 // through (8192, 28672, 8192) reads all 67 MB of X8 again for every four channel tiles).  A last token tile that takes half as
 // long as the others (256 x 512 tiles, at most 256 tokens in it) is a band of its own: `full` token tiles come first, so that
 // the last round of tiles holds short ones where it can.  (1152, 7648, 2560) 32.9 -> 27.3 us, (526, 14128, 2560) 33.0 -> 27.3.
+// (`full` is the host's: worked out in the kernel, the same loops took 3 % longer, (2048, 4096, 4096) 41.2 -> 42.2 us.)
 constexpr int kPairBand = 8;
 W4A8_HOST_DEVICE int pair_full_tiles(int64_t M, int tokens, int TM) { return tokens > 256 && M - (int64_t)(TM - 1) * tokens <= 256 ? TM - 1 : TM; }
 W4A8_HOST_DEVICE void pair_tile(int t, int full, int TN, int& nt, int& mt) {
+    const int per = kPairBand * TN, band = t / per;
+    int first = band * kPairBand, u = t - band * per;
+    int width = full - first < kPairBand ? full - first : kPairBand;
     if (t >= full * TN) {
-        nt = t - full * TN;
-        mt = full;
-        return;
+        first = full;
+        u = t - full * TN;
+        width = 1;
     }
-    const int per = kPairBand * TN, band = t / per, first = band * kPairBand;
-    const int width = full - first < kPairBand ? full - first : kPairBand;
-    const int u = t - band * per;
     nt = u / width;
     mt = first + (u - nt * width);
 }
