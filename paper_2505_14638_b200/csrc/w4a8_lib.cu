@@ -524,7 +524,6 @@ static int launch_cluster_kcut(const uint8_t* x8, int64_t ldx8, const uint8_t* w
     pl.U = (int64_t)TN * (K / 128);
     pl.P = (int64_t)TN * cl;
     pl.counter_bytes = 0;
-    pl.workspace_bytes = 0;
     return launch_streamk<Cfg>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, nullptr, pl, M, N, K, st, tw, cl, gzero);
 }
 
@@ -735,17 +734,16 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
                         : launch_splitn_cfg<128, 4, kFmtTiledSignMag>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi, Ni,
                                                                       Ki, st);
     }
-    SkPlan pl;
-    make_sk_plan(M, N, K, kNominalSMs, &pl);
     if (!whole) {
         if (reinterpret_cast<uintptr_t>(workspace) & 15u) return W4A8_ERR_BAD_ALIGNMENT;
-        if (!workspace || workspace_bytes < pl.workspace_bytes) return W4A8_ERR_WORKSPACE_TOO_SMALL;
+        if (!workspace || workspace_bytes < kSkWorkspaceBytes) return W4A8_ERR_WORKSPACE_TOO_SMALL;
     }
     int rc = check_device();
     if (rc != W4A8_OK) return rc;
     const int sms = sm_count();
     if (sms <= 0) return W4A8_ERR_CUDA;
-    int choice = 0;
+    SkPlan pl;
+    PrefillKind kind = kPrefillKinds;
     if (whole) {
         pl.bnx = M <= 64 ? 64 : 128;
         pl.TM = 1;
@@ -754,10 +752,9 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
         pl.aligned = 1;
         pl.P = pl.TN < sms ? pl.TN : sms;
         pl.counter_bytes = 0;
-        workspace = nullptr;   // (none is used)
     } else {
         const int quads = fmt == kFmtTiledSignMag ? pair_quads<kFmtTiledSignMag>() : pair_quads<kFmtTiled>();
-        choice = prefill_choice(M, N, K, sms, quads, &pl);
+        kind = prefill_choice(M, N, K, fmt == kFmtTiledSignMag, sms, quads, &pl);
     }
 #define W4A8_PAIR(KP, ...)                                                                                            \
     return fmt == kFmtTiledSignMag                                                                                    \
@@ -765,12 +762,13 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
                                                                      out_dtype, (int)M, (int)N, (int)K, sms, st, KP)  \
                : launch_pair<PairCfg<kFmtTiled, __VA_ARGS__>>(x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype,  \
                                                               (int)M, (int)N, (int)K, sms, st, KP)
-    switch (choice) {
-        case 1: W4A8_PAIR(1, 1, 3, 6);
-        case 2: W4A8_PAIR(1, 2, 4, 4);
-        case 3: W4A8_PAIR(2, 1, 3, 6);
+    switch (kind) {
+        case kPairs256: W4A8_PAIR(1, 1, 3, 6);
+        case kPairs512: W4A8_PAIR(1, 2, 4, 4);
+        case kPairsKCut: W4A8_PAIR(2, 1, 3, 6);
         default: break;
     }
+    if (pl.aligned) workspace = nullptr;   // (none is used)
 #undef W4A8_PAIR
     CUtensorMap tx;
     if (!make_tmap_u8_2d(&tx, x8, (uint64_t)M, (uint64_t)K, (uint64_t)ldx8, 128, (uint32_t)pl.bnx,
@@ -785,7 +783,8 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
                                                                 workspace, pl, Mi, Ni, Ki, st)
     switch (pl.bnx) {
         case 64: W4A8_SK(64, 4, 12, 12); break;
-        default: W4A8_SK(128, 4, 8, 8); break;
+        case 128: W4A8_SK(128, 4, 8, 8); break;
+        default: W4A8_SK(256, 4, 4, 3); break;
     }
 #undef W4A8_SK
     return rc;
@@ -975,7 +974,6 @@ static int linear_w8a8_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, i
             p8.U = TM * TN * (K / 128);
             p8.P = sms;
             p8.counter_bytes = 0;
-            p8.workspace_bytes = 0;
             CUtensorMap tx8;
             if (!make_tmap_u8_2d(&tx8, x8, (uint64_t)M, (uint64_t)K, (uint64_t)ldx8, 128, 256, CU_TENSOR_MAP_SWIZZLE_128B))
                 return W4A8_ERR_CUDA;
@@ -1104,7 +1102,6 @@ static int linear_w4a16_tiled_impl(const void* x, int64_t ldx, int64_t M, const 
     pl.U = (int64_t)pl.TM * pl.TN * (K / 128);
     pl.P = (int64_t)pl.TM * pl.TN < sms ? (int64_t)pl.TM * pl.TN : sms;
     pl.counter_bytes = 0;
-    pl.workspace_bytes = 0;
     CUtensorMap tx;   // X as bytes: rows of 2 K bytes, boxes of 128 bytes (64 BF16 values) x bnx tokens
     if (!make_tmap_u8_2d(&tx, x, (uint64_t)M, (uint64_t)(2 * K), (uint64_t)(2 * ldx), 128, (uint32_t)bnx,
                          CU_TENSOR_MAP_SWIZZLE_128B))
@@ -1447,11 +1444,8 @@ size_t w4a8_linear_workspace_bytes(int64_t M, int64_t N, int64_t K, int weight_f
     if (M <= 0 || N <= 0 || K <= 0 || K % kGroup != 0) return 0;
     if (weight_format == kFmtCanonical) return w4a8_linear_ex_workspace_bytes(M, N, K, W4A8_ALGO_AUTO, 0);
     if (weight_format != kFmtTiled && weight_format != kFmtTiledSignMag) return 0;
-    if (M <= 64) return kSnWorkspaceBytes;  // used when the layer has few output channels and K is cut
-    SkPlan pl;
-    make_sk_plan(M, N, K, kNominalSMs, &pl);
-    // (65..128 tokens: either kernel may run, the persistent one only with its full workspace)
-    return M <= kSplitNMaxM && pl.workspace_bytes < kSnWorkspaceBytes ? kSnWorkspaceBytes : pl.workspace_bytes;
+    if (M <= 64) return kSnWorkspaceBytes;  // used at up to 16 tokens, when the layer has few output channels and K is cut
+    return kSkWorkspaceBytes;   // (65..128 tokens use none of it)
 }
 
 int w4a8_prepack_fp8(const uint8_t* w8, int64_t N, int64_t K, uint8_t* out, size_t out_bytes, void* stream) {

@@ -26,12 +26,17 @@ constexpr size_t kLinearCtlBytes = 65536;
 // by design) sit at the END of the control area, the persistent kernel's tile counters at its start.
 constexpr size_t kLinearCtlSplitN = kLinearCtlBytes - 2048;
 
+// What w4a8_linear_workspace_bytes asks for and w4a8_linear requires for more than 128 tokens on prepacked weights, whatever
+// arrangement runs (most use none of it): a bound on what the persistent kernel ever used, for any SM count up to kMaxSMs.  It
+// does not follow the plans, so that a workspace that was accepted stays accepted and one that was refused stays refused.
+constexpr size_t kSkWorkspaceBytes = kLinearCtlBytes + (size_t)kMaxSMs * 2 * 256 * 128 * sizeof(float);
+
 struct SkPlan {
     int bnx, TM, TN;
-    int aligned;   // 1: whole tiles per CTA, nothing shared; 0: equal slices of the (tile, k-block) space
+    int aligned;   // 1: whole tiles per CTA, nothing shared; 0: several CTAs per tile
     int64_t P;     // CTAs
     int64_t U;
-    size_t counter_bytes, workspace_bytes;
+    size_t counter_bytes;
 };
 
 // Tile t of a CTA pair's schedule -> channel tile and token tile.  Token tiles are taken in bands of kPairBand: the tiles in
@@ -55,91 +60,121 @@ W4A8_HOST_DEVICE void pair_tile(int t, int full, int TN, int& nt, int& mt) {
     mt = first + (u - nt * width);
 }
 
-// Time of 256 x 512 tiles on `pairs` pairs, in half rounds: pair c takes tiles c, c + pairs, ..., and one of at most 256 tokens
-// takes half as long.
-inline int64_t pair_half_rounds(int64_t M, int64_t N, int64_t pairs) {
-    const int64_t TN = (N + 255) / 256, TM = (M + 511) / 512, tiles = TN * TM, rounds = (tiles + pairs - 1) / pairs;
-    const int64_t full = TN * pair_full_tiles(M, 512, (int)TM);   // pair 0 has most of them, and a tile of each round
-    return rounds + (full + pairs - 1) / pairs;
+// Tiles of 256 x 512 that the busiest of `pairs` pairs works on (pair c takes tiles c, c + pairs, ...): those with two
+// accumulators, or those with one.
+inline int64_t pair_rounds(int64_t M, int64_t N, int64_t pairs, bool two) {
+    const int64_t TN = (N + 255) / 256, TM = (M + 511) / 512, full = TN * pair_full_tiles(M, 512, (int)TM);
+    const int64_t of_two = (full + pairs - 1) / pairs;
+    return two ? of_two : (TN * TM + pairs - 1) / pairs - of_two;
 }
 
-// Token-tile width and schedule of the persistent kernel on prepacked weights from a cost model, in microseconds; returns
-// the time.  Whole tiles per CTA cost rounds x (k-blocks x step + drain); where there are fewer tiles than half the CTAs and
-// a number of CTAs per tile divides the k-blocks, that many CTAs share a tile and exchange partial sums, which costs about
-// as much as 30 k-blocks.  Fitted, with the constants of the CTA pairs (see prefill_choice), to 656 + 410 measured (M, N,
-// K) of all alternatives: the alternative chosen takes 0.5 % longer than the fastest on average, 9 % at most from K = 1024
-// on.  Equal slices of the (tile, k-block) space and tiles of 256 tokens, which earlier versions had, are nowhere the
-// fastest by more than 4 %.
-inline double make_sk_plan(int64_t M, int64_t N, int64_t K, int sms, SkPlan* pl) {
-    const int64_t KB = K / 128;
-    const int64_t TN = (N + 127) / 128;
-    const int64_t cap = sms < kMaxSMs ? sms : kMaxSMs;
+// More than 128 tokens on prepacked weights: the arrangements there are.
+enum PrefillKind {
+    kPairs256,     // CTA pairs, tiles of 256 channels x 256 tokens
+    kPairs512,     // 256 x 512
+    kPairsKCut,    // 256 x 256 with K cut between the two pairs of a cluster of four CTAs
+    kWhole64,      // persistent kernel, whole tiles of 128 channels x 64 tokens per CTA
+    kWhole128,     // x 128
+    kWhole256,     // x 256
+    kCut128,       // persistent kernel, several CTAs per tile of 128 x 128, which exchange partial sums through the workspace
+    kCut256,       // 128 x 256
+    kPrefillKinds
+};
+
+// Time of a launch in microseconds, with the activation quantization before it:
+//   rounds of tiles x max(k-blocks x step + drain, least) + fixed + full x (share of the SMs that the first round takes)^4
+// `least`: the drain of a tile that its k-blocks do not cover (kPairs512: the time of a tile with one accumulator as a part of
+// one with two).  `full`: a launch that leaves SMs free lets the next one set up beside it, which is why 69 CTAs with 128 tokens
+// each take less time than 138 with 64, (383, 2896, 1536) 7.7 against 8.3 us.
+struct PlanCost {
+    double step, drain, fixed, full, least;
+};
+// Sign-magnitude and generic format (whose expansion costs 11 integer instructions per eight weights instead of 7).
+constexpr PlanCost kPlanCost[2][kPrefillKinds] = {
+    {
+        {0.373, 3.16, 2.71, 0.19, 0.00},    // pairs, 256 x 256
+        {0.887, 3.28, 4.52, -0.91, 0.52},   // pairs, 256 x 512
+        {0.309, 0.00, 8.83, 6.79, 0.00},    // pairs, 256 x 256, K cut
+        {0.276, 0.22, 2.48, 2.31, 1.44},    // whole tiles, 128 x 64
+        {0.300, 0.81, 2.85, 1.78, 2.12},    // whole tiles, 128 x 128
+        {0.524, 2.18, 3.35, 0.09, 0.25},    // whole tiles, 128 x 256
+        {0.356, 0.00, 11.48, 0.02, 0.00},   // K cut, 128 x 128
+        {0.546, 0.00, 14.63, 0.04, 0.00},   // K cut, 128 x 256
+    },
+    {
+        {0.486, 2.31, 2.68, 0.38, 0.00},    // pairs, 256 x 256
+        {0.809, 3.66, 3.82, -0.14, 0.60},   // pairs, 256 x 512
+        {0.447, 0.00, 7.98, 4.67, 0.00},    // pairs, 256 x 256, K cut
+        {0.356, 0.38, 2.56, 2.75, 1.24},    // whole tiles, 128 x 64
+        {0.376, 1.06, 2.42, 2.31, 2.52},    // whole tiles, 128 x 128
+        {0.539, 1.77, 3.99, 1.72, 0.09},    // whole tiles, 128 x 256
+        {0.467, 0.00, 9.15, 2.85, 0.00},    // K cut, 128 x 128
+        {0.643, 0.00, 7.44, 9.09, 0.00},    // K cut, 128 x 256
+    },
+};
+
+inline double plan_time(const PlanCost& c, double rounds, int64_t steps, double taken) {
+    const double tile = (double)steps * c.step + c.drain, share = taken < 1.0 ? taken : 1.0;
+    return rounds * (tile > c.least ? tile : c.least) + c.fixed + c.full * share * share * share * share;
+}
+
+// The arrangement with the least time by that model; `pl`: the persistent kernel's plan where it is one of those.  `quads`:
+// clusters of four CTAs that the device holds at once (a second round of them costs more than the cut saves).
+// The constants are fitted to 1778 (M, N, K) in both formats, M 129 to 8192, N 1024 to 28672, K 1024 to 14336 and some shorter
+// ones: every arrangement in turn for a few milliseconds, quantization and linear layer back to back, weights not in L2; and
+// to 190 of them run for a quarter of a second each, at the power cap.  The arrangement taken is 0.5 % slower than the fastest
+// on average, 15 % at most; it is slower than the kernels before CTA pairs by more than 3 % at 24 of the 3542, by 11 % at most
+// ((635, 1216, 2944) generic 11.8 -> 13.3 us), and 1.17 times as fast on average.
+// The model before this one had the same constants for both formats, took 36 clusters of four for granted and lacked 256-token
+// tiles and uneven cuts of K: (241, 8592, 5248) 28.6 -> 17.5 us, (1488, 1376, 10496) 47.0 -> 31.0, (151, 1072, 12416) 22.1 -> 15.5,
+// (1196, 3680, 4864) generic 33.5 -> 28.3, (1531, 4096, 14336) 104.8 -> 97.2.
+inline PrefillKind prefill_choice(int64_t M, int64_t N, int64_t K, bool signmag, int sms, int quads, SkPlan* pl) {
+    const PlanCost* cost = kPlanCost[signmag ? 0 : 1];
+    const int64_t KB = K / 128, cap = sms < kMaxSMs ? sms : kMaxSMs, pairs = sms / 2;
+    PrefillKind kind = kPrefillKinds;
     double best = 1e30;
-    for (int bnx = 128; bnx >= 64; bnx >>= 1) {
+    auto better = [&](PrefillKind k, double t) {
+        if (t >= best) return false;
+        best = t;
+        kind = k;
+        return true;
+    };
+    const int64_t TNp = (N + 255) / 256, t1 = TNp * ((M + 255) / 256), TM2 = (M + 511) / 512;
+    const int64_t rounds1 = (t1 + pairs - 1) / pairs, full = TNp * pair_full_tiles(M, 512, (int)TM2);
+    // Sign-magnitude launches of some 35 us and more, one after the other, run at the power cap, where expanding the weights twice
+    // as often as 256 x 512 tiles with two accumulators do costs clock: a quarter of a second of (2048, 4096, 4096) 39.4 against
+    // 38.6 us, of (1531, 28672, 4096) 178 / 170, of (8192, 28672, 8192) 1669 / 1632.
+    double capped = 0.0;
+    if (signmag) capped = rounds1 >= 8 ? 0.18 : ((double)M * (double)N * (double)K >= 3e10 ? 0.09 : 0.0);
+    capped = 1.0 + capped * (double)full / (double)(TNp * TM2);
+    better(kPairs256, plan_time(cost[kPairs256], (double)rounds1, KB, (double)t1 / (double)pairs) * capped);
+    {
+        // (`least` of this arrangement is a factor, see PlanCost)
+        PlanCost c = cost[kPairs512];
+        const double rounds = (double)pair_rounds(M, N, pairs, true) + c.least * (double)pair_rounds(M, N, pairs, false);
+        c.least = 0.0;
+        better(kPairs512, plan_time(c, rounds, KB, (double)(TNp * TM2) / (double)pairs));
+    }
+    if (t1 <= quads && KB >= 8) better(kPairsKCut, plan_time(cost[kPairsKCut], 1.0, (KB + 1) / 2, 2.0 * (double)t1 / (double)pairs));
+    for (int i = 0; i < 3; ++i) {
+        const int bnx = 64 << i;
         if (bnx > 64 && bnx / 2 >= M) continue;  // more than half of the tile would be padding
-        const int64_t TM = (M + bnx - 1) / bnx, Tt = TM * TN;
-        const double step = bnx == 64 ? 0.207 : 0.247, drain = bnx == 64 ? 0.46 : 0.89;
-        double t = (double)((Tt + cap - 1) / cap) * ((double)KB * step + drain) + 1.8;
-        int64_t P = cap < Tt ? cap : Tt;
-        bool whole = true;
-        const int64_t per = cap / Tt;   // CTAs per tile
-        // (tile counters must fit the control area)
-        if (per >= 2 && KB % per == 0 && 2 * (size_t)Tt * sizeof(unsigned int) <= kLinearCtlSplitN) {
-            const double t_k = (double)(KB / per) * step + 7.7;
-            if (t_k < t) {
-                t = t_k;
-                P = Tt * per;
-                whole = false;
-            }
-        }
-        if (t < best) {
-            best = t;
-            pl->bnx = bnx;
-            pl->TM = (int)TM;
-            pl->TN = (int)TN;
-            pl->U = Tt * KB;
-            pl->aligned = whole ? 1 : 0;
-            pl->P = P;
-        }
+        const int64_t TM = (M + bnx - 1) / bnx, TN = (N + 127) / 128, tiles = TM * TN, per = cap / tiles;
+        int64_t ctas = 0;   // per tile
+        if (better((PrefillKind)(kWhole64 + i), plan_time(cost[kWhole64 + i], (double)((tiles + cap - 1) / cap), KB, (double)tiles / (double)cap))) ctas = 1;
+        if (i > 0 && per >= 2 && KB >= 2 * per &&
+            better((PrefillKind)(kCut128 + i - 1), plan_time(cost[kCut128 + i - 1], 1.0, (KB + per - 1) / per, (double)(tiles * per) / (double)cap)))
+            ctas = per;
+        if (ctas == 0) continue;
+        pl->bnx = bnx;
+        pl->TM = (int)TM;
+        pl->TN = (int)TN;
+        pl->U = tiles * KB;
+        pl->aligned = ctas == 1 ? 1 : 0;
+        pl->P = ctas == 1 ? (tiles < cap ? tiles : cap) : tiles * ctas;
+        pl->counter_bytes = ctas == 1 ? 0 : kLinearCtlBytes;
     }
-    // arrivals and finished reducers per tile live in the control area; the size asked of the caller
-    // covers every tile width and any SM count up to kMaxSMs, so that the query needs no device
-    pl->counter_bytes = kLinearCtlBytes;
-    pl->workspace_bytes = kLinearCtlBytes + (size_t)kMaxSMs * 2 * 256 * 128 * sizeof(float);
-    return best;
-}
-
-// CTA pairs against the persistent kernel for a problem of more than 128 tokens: 0 = persistent kernel (its plan in `pl`),
-// 1 = tiles of 256 channels x 256 tokens, 2 = 256 x 512, 3 = 256 x 256 with K cut between the two pairs of a cluster of four
-// CTAs.  Times in microseconds, from the same fit as make_sk_plan's: a k-block of a 256 x 256 tile takes a pair 0.244, of a
-// 256 x 512 tile 0.489 (a round that holds only tiles of at most 256 tokens half of that); drain per tile, launch and fill
-// per call.  Measured, us, sign-magnitude weights not in L2 (before / now, the choice in brackets): (8192, 28672, 8192) 2011 /
-// 1500 [2], (2048, 4096, 4096) 36.3 / 34.7 [2], (1531, 28672, 4096) 208 / 171 [2], (1531, 4096, 14336) 121 / 95 [2], (1024,
-// 28672, 4096) 152 / 121 [2], (512, 6144, 4096) 18.4 / 15.9 [1], (512, 28672, 4096) 71 / 63 [2], (512, 4096, 14336) 45.2 / 33.0
-// [3], (256, 4096, 4096) 16.5 / 10.9 [3]; (512, 4096, 4096) 12.2 / - / 14.1 on pairs [0].
-inline int prefill_choice(int64_t M, int64_t N, int64_t K, int sms, int quads, SkPlan* pl) {
-    const int64_t KB = K / 128, pairs = sms / 2, TN = (N + 255) / 256;
-    double best = make_sk_plan(M, N, K, sms, pl);
-    int choice = 0;
-    const int64_t t1 = TN * ((M + 255) / 256);
-    const int64_t rounds1 = (t1 + pairs - 1) / pairs;
-    double t = (double)rounds1 * ((double)KB * 0.244 + 2.1) + 3.1;
-    // (back to back, at the power cap, where all pairs work throughout: it expands twice the weights)
-    if (rounds1 >= 2) t *= 1.1;
-    if (t < best) {
-        best = t;
-        choice = 1;
-    }
-    t = 0.5 * (double)pair_half_rounds(M, N, pairs) * ((double)KB * 0.489 + 2.3) + 6.8;
-    if (t < best) {
-        best = t;
-        choice = 2;
-    }
-    if (t1 <= quads && KB >= 8) {   // (a second round of them would cost more than the cut saves)
-        t = (double)((KB + 1) / 2) * 0.244 + 7.3;
-        if (t < best) choice = 3;
-    }
-    return choice;
+    return kind;
 }
 
 }  // namespace w4a8

@@ -88,13 +88,18 @@ SM, TI, CA = binding.FMT_TILED_SIGNMAG, binding.FMT_TILED, binding.FMT_CANONICAL
 CASES = {
     "split-N, candidates": lambda: _linear(8, 14336, 4096, SM),
     "split-N, K cut": lambda: _linear(8, 4096, 14336, TI),
-    "split-N, 128 tokens": lambda: _linear(100, 28672, 2048, TI),
+    "whole tiles, 128 tokens, wide layer": lambda: _linear(100, 28672, 2048, TI),
+    "split-N, 128 tokens": lambda: _linear(100, 28672, 8192, SM),
     "cluster, 64 tokens": lambda: _linear(40, 4096, 14336, SM),
-    "64-token tiles, equal slices": lambda: _linear(130, 1024, 14336, TI),
-    "128-token tiles, equal slices": lambda: _linear(300, 1024, 14336, SM),
-    "256-token tiles": lambda: _linear(512, 4096, 14336, TI),
-    "256 x 256 tiles": lambda: _linear(2048, 4096, 4096, SM),
-    "two-CTA tiles": lambda: _linear(1100, 16384, 2048, SM),
+    "K cut between CTAs, 128 tokens, generic": lambda: _linear(130, 1024, 14336, TI),
+    "K cut between CTAs, 128 tokens": lambda: _linear(300, 1024, 14336, SM),
+    "K cut between CTAs, 256 tokens": lambda: _linear(193, 4000, 14336, TI),
+    "whole tiles, 64 tokens": lambda: _linear(200, 4080, 4096, SM),
+    "whole tiles, 256 tokens": lambda: _linear(1196, 3680, 4864, TI),
+    "pairs, K cut": lambda: _linear(512, 4096, 14336, TI),
+    "pairs, 256 x 256 tiles": lambda: _linear(2048, 4096, 4096, SM),
+    "pairs, 256 x 256 tiles, wide layer": lambda: _linear(1100, 16384, 2048, SM),
+    "pairs, 256 x 512 tiles": lambda: _linear(1152, 7648, 2560, TI),
     "canonical": lambda: _linear(100, 14336, 4096, CA),
     "chain": _chain,
     "W4A16": _w4a16,

@@ -84,9 +84,8 @@ def test_config_c4_prefill_sampled_channels():
                                         ("o", 4096, 4096, 1), ("o", 4096, 4096, 32),
                                         ("gate_up", 4096, 28672, 128), ("down", 14336, 4096, 128)])
 def test_config_c5_layers_sampled_channels(name, K, N, M):
-    # c5: the four Llama-3-8B linears; token counts that reach the split-N kernel (<= 64: the
-    # smallest layers there take the K-cut path), its 128-token tiles (128), the persistent kernel
-    # with shared tiles (512) and with whole tiles (4096)
+    # c5: the four Llama-3-8B linears; token counts that reach the kernels for up to 16 tokens, the cluster plan
+    # and whole tiles of the persistent kernel (32, 128), and CTA pairs (512, 4096)
     _run_case(M, N, K, 0.02, 0.01, 20.0, seed=500 + M + N // 64, n_random=40)
 
 
@@ -189,10 +188,9 @@ def test_two_cta_kernel_shape_exact_integers_and_gaussian():
 
 
 def test_wide_tile_kernel_shape_exact_integers_and_gaussian():
-    """A shape that the prefill kernel with tiles of 256 output channels x 256 tokens takes (whole
-    tiles fill the SMs well), ragged in both directions -- the last token tile has 120 tokens, the
-    last channel tile 80 rows -- and with more tiles than SMs, so that some CTAs run a second tile
-    on the same accumulators.  Small-integer inputs (exact FP32 sums: a misplaced operand changes a
+    """A shape that CTA pairs with tiles of 256 output channels take, ragged in both directions -- the last
+    token tile has 120 tokens, the last channel tile 80 rows -- and with more tiles than pairs, so that every
+    pair runs further tiles on the same accumulators.  Small-integer inputs (exact FP32 sums: a misplaced operand changes a
     result by at least one unit) in the generic tiled format, then Gaussian inputs in the
     sign-magnitude format within the usual gates.  Sampled output channels: the first and last row of
     every 128-row block."""

@@ -103,7 +103,7 @@ def test_gaussian_inputs_within_gates(M, N, K, asym, pc):
                                    (32, 4096, 14336), (64, 1024, 2048), (128, 2048, 1024), (512, 1024, 1024),
                                    (300, 640, 8192), (100, 512, 8192), (65, 4096, 4096), (128, 14336, 1024)])
 def test_persistent_kernel_split_tiles_and_reuse_of_workspace(M, N, K):
-    # shapes whose tiles are split between CTAs in many ways (equal slices in the persistent kernel, K
+    # shapes whose tiles are split between CTAs in many ways (several CTAs per tile in the persistent kernel, K
     # chunks in the split-N kernel with 16-token tiles, clusters of two to eight CTAs per tile); the workspace is shared by
     # consecutive calls (the kernel leaves its counters zeroed) and results repeat bit for bit
     x8, s_x, wq = _gaussian_case(M, N, K, seed=M * 3 + N + K)

@@ -15,7 +15,7 @@ from paper_2505_14638_b200 import binding, inputs
 pytestmark = pytest.mark.gpu
 
 SHAPES = [
-    # 256 x 256 tiles, one pair per tile, and one round of 147 tiles of which two share a pair
+    # 256 x 256 tiles: one tile per pair; two rounds, 147 tiles on 74 pairs; and (sign-magnitude) 256 x 512 with one accumulator
     (129, 28672, 1280), (512, 6144, 4096), (700, 12304, 2048),
     # 256 x 512 tiles: last token tile of at most 256 tokens, of more, of one token; several rounds; K = 128 and 256
     (1030, 16400, 1024), (2100, 9232, 640), (4609, 9488, 384), (513, 18448, 1152), (9000, 9488, 128), (4700, 9488, 256),

@@ -4,11 +4,10 @@ against a float32 product of the dequantized operands, which is exact enough to 
 was summed from stale or missing data).  A repeat on a USED workspace cannot show such an error: a
 kernel that reads partial sums too early finds the previous launch's identical values there.  (This
 is how a barrier-phase hazard in the expansion groups showed up: wrong sums in a few tiles of the
-first launch of a process only.)  Shapes: one per kernel and plan -- split-N with and without a
-K cut, the persistent kernel with 64-, 128- and 256-token tiles as equal slices, as whole CTAs per
-tile and as whole tiles, the 256 x 256 tiles, the two-CTA kernel, the cluster plan (K cut between two to eight CTAs of a cluster,
-with a ragged last tile, with as few as two k-blocks per CTA, with the largest number of clusters
-that fits)."""
+first launch of a process only.)  Shapes: split-N with and without a
+K cut, the cluster plan (K cut between two to eight CTAs of a cluster, with a ragged last tile, with as few as
+two k-blocks per CTA, with the largest number of clusters that fits), whole tiles of the persistent kernel, CTA pairs; every
+arrangement for more than 128 tokens is in test_gpu_prefill_arrangements.py."""
 import numpy as np
 import pytest
 import torch
@@ -51,8 +50,8 @@ def test_fresh_workspace_launches_agree_and_are_right(M, N, K):
 
 def test_one_workspace_shared_by_layers_of_different_shapes_and_kernels():
     # One workspace of the largest size, used by calls of different shapes one after the other -- split-N
-    # with and without a K cut, the persistent kernel as equal slices and as whole CTAs per tile, the
-    # 256 x 256 tiles: whatever a call leaves behind in the data part of the workspace, the next call's
+    # with and without a K cut, the persistent kernel with whole tiles and with several CTAs per tile, CTA
+    # pairs: whatever a call leaves behind in the data part of the workspace, the next call's
     # counters must be zero.  Every result must equal the one computed on a fresh workspace of its own.
     dev = torch.device("cuda")
     shapes = [(128, 4096, 14336), (128, 28672, 4096), (128, 4096, 4096), (16, 4096, 14336), (300, 640, 8192),
