@@ -220,7 +220,7 @@ constexpr int kSplitNMaxM = 128;  // token counts served by the split-N (decode)
 template <class Cfg>
 static int launch_streamk(const CUtensorMap& tx, const uint8_t* wpp, const float* s_x, const float* s_w,
                           int sw_stride, void* y, int64_t ldy, int out_dtype, void* workspace, const SkPlan& pl,
-                          int M, int N, int K, cudaStream_t st, const CUtensorMap* tw8 = nullptr, int cl = 0,
+                          int M, int N, int K, cudaStream_t st, const CUtensorMap* tw8 = nullptr,
                           const uint8_t* gzero = nullptr) {
     auto kern = linear_streamk_kernel<Cfg>;
     static std::once_flag once;
@@ -232,7 +232,7 @@ static int launch_streamk(const CUtensorMap& tx, const uint8_t* wpp, const float
     unsigned int* status = status_word_ptr();
     if (!status) return W4A8_ERR_CUDA;
     const int64_t P = pl.P;
-    const int aligned = pl.aligned;
+    if (!Cfg::CL && !Cfg::kCut && pl.per != 1) return W4A8_ERR_INVALID_ARG;
     unsigned int* counters = static_cast<unsigned int*>(workspace);
     float* slots = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + pl.counter_bytes);
     cudaLaunchConfig_t cfg = {};
@@ -246,24 +246,25 @@ static int launch_streamk(const CUtensorMap& tx, const uint8_t* wpp, const float
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (Cfg::CL) {
-        // the cl CTAs of a tile as one thread-block cluster (P = tiles x cl)
-        if (cl < 2 || cl > 8 || P % cl != 0) return W4A8_ERR_INVALID_ARG;
+        // the CTAs of a tile as one thread-block cluster
+        if (pl.per < 2 || pl.per > 8) return W4A8_ERR_INVALID_ARG;
         attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = (unsigned)cl;
+        attr[1].val.clusterDim.x = (unsigned)pl.per;
         attr[1].val.clusterDim.y = 1;
         attr[1].val.clusterDim.z = 1;
         cfg.numAttrs = 2;
     }
     // (the second tensor map is read only by the FP8-weight and canonical variants)
     cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tx, tw8 ? *tw8 : tx, wpp, gzero, s_x, s_w, sw_stride, y, ldy, out_dtype,
-                                       counters, slots, M, N, K, pl.TM, pl.TN, aligned, cl, status);
+                                       counters, slots, M, N, K, pl.TM, pl.TN, Cfg::kCut && pl.per > 1 ? 1 : 0, pl.per, status);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     if (e != cudaSuccess) return W4A8_ERR_CUDA;
     return launch_status();
 }
 
 // Row partition and ring sizes of the split-N kernel for the current device.
-// Workspace of the split-N kernel when it cuts K (bytes; fits any SM count up to kMaxSMs and 128 tokens).
+// Workspace of the split-N kernel when it cuts K, which it does at up to 16 tokens (bytes; room for any SM count up to kMaxSMs and,
+// from earlier versions, 128 tokens: the size that calls are refused or accepted by stays).
 // Layout: split-K counters (1 KB) and placement state of the launch (1 KB) at the end of the common
 // control area, partial tiles behind that area.
 constexpr size_t kSnCounterBytes = 1024;
@@ -520,11 +521,10 @@ static int launch_cluster_kcut(const uint8_t* x8, int64_t ldx8, const uint8_t* w
     pl.bnx = Cfg::BNX;
     pl.TM = 1;
     pl.TN = TN;
-    pl.aligned = 1;
-    pl.U = (int64_t)TN * (K / 128);
+    pl.per = cl;
     pl.P = (int64_t)TN * cl;
     pl.counter_bytes = 0;
-    return launch_streamk<Cfg>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, nullptr, pl, M, N, K, st, tw, cl, gzero);
+    return launch_streamk<Cfg>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, nullptr, pl, M, N, K, st, tw, gzero);
 }
 
 // ------------------------------------------------------------------------------ few tokens, weights to registers
@@ -748,8 +748,7 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
         pl.bnx = M <= 64 ? 64 : 128;
         pl.TM = 1;
         pl.TN = (int)((N + 127) / 128);
-        pl.U = (int64_t)pl.TN * (K / 128);
-        pl.aligned = 1;
+        pl.per = 1;
         pl.P = pl.TN < sms ? pl.TN : sms;
         pl.counter_bytes = 0;
     } else {
@@ -768,7 +767,7 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
         case kPairsKCut: W4A8_PAIR(2, 1, 3, 6);
         default: break;
     }
-    if (pl.aligned) workspace = nullptr;   // (none is used)
+    if (pl.per == 1) workspace = nullptr;   // (none is used)
 #undef W4A8_PAIR
     CUtensorMap tx;
     if (!make_tmap_u8_2d(&tx, x8, (uint64_t)M, (uint64_t)K, (uint64_t)ldx8, 128, (uint32_t)pl.bnx,
@@ -833,8 +832,7 @@ static int linear_canonical_impl(const uint8_t* x8, int64_t ldx8, const float* s
             pl.bnx = bnx;
             pl.TM = (int)TM;
             pl.TN = (int)TN;
-            pl.aligned = 1;
-            pl.U = tiles * (K / 128);
+            pl.per = 1;
             pl.P = tiles < sms ? tiles : sms;
         }
     }
@@ -843,7 +841,7 @@ static int linear_canonical_impl(const uint8_t* x8, int64_t ldx8, const float* s
         return W4A8_ERR_CUDA;
 #define W4A8_SKC(BNX, G, S1, S2)                                                                                       \
     return launch_streamk<SkCfg<BNX, G, S1, S2, kFmtCanonical>>(tx, gs, s_x, s_w, sw_stride, y, ldy, out_dtype, nullptr, \
-                                                                pl, (int)M, (int)N, (int)K, st, &tw, 0, gzero)
+                                                                pl, (int)M, (int)N, (int)K, st, &tw, gzero)
     switch (pl.bnx) {
         case 64: W4A8_SKC(64, 4, 12, 12);
         case 128: W4A8_SKC(128, 4, 8, 8);
@@ -970,8 +968,7 @@ static int linear_w8a8_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, i
             p8.bnx = 256;
             p8.TM = (int)TM;
             p8.TN = (int)TN;
-            p8.aligned = 1;
-            p8.U = TM * TN * (K / 128);
+            p8.per = 1;
             p8.P = sms;
             p8.counter_bytes = 0;
             CUtensorMap tx8;
@@ -1098,8 +1095,7 @@ static int linear_w4a16_tiled_impl(const void* x, int64_t ldx, int64_t M, const 
     pl.bnx = bnx;
     pl.TM = (int)((M + bnx - 1) / bnx);
     pl.TN = (int)((N + 127) / 128);
-    pl.aligned = 1;
-    pl.U = (int64_t)pl.TM * pl.TN * (K / 128);
+    pl.per = 1;
     pl.P = (int64_t)pl.TM * pl.TN < sms ? (int64_t)pl.TM * pl.TN : sms;
     pl.counter_bytes = 0;
     CUtensorMap tx;   // X as bytes: rows of 2 K bytes, boxes of 128 bytes (64 BF16 values) x bnx tokens

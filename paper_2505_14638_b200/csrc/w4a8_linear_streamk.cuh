@@ -1,18 +1,15 @@
-// Persistent, load-balanced W4A8 linear for sm_100a on the tiled ("prepacked") weight layout.
+// Persistent W4A8 linear for sm_100a on the tiled ("prepacked") weight layout.
 //
-// Work is the flattened space (weight tile of 128 rows, token tile of BNX rows, k-block of 128):
-// every CTA takes an equal, contiguous share of it, so the SMs stay evenly loaded whatever the
-// layer shape (decode-sized problems have fewer tiles than SMs).  A CTA whose share covers only
-// part of a tile's K range stores an fp32 partial tile and bumps the tile's arrival counter.  When
-// a CTA has finished its whole share it turns to the (at most two) tiles it shares with others:
-// it waits (bounded) until all of that tile's partials have arrived and then reduces ITS columns
-// of the tile -- contributor i of C takes the i-th slice of the token columns, adds the C partials
-// in ascending CTA order, applies the Eq. 4 / Eq. 11 scales and stores the outputs.  The
-// reduction is thus spread over all contributors with many independent loads in flight (one CTA
-// adding whole partial tiles one after another spent tens of microseconds on L2 round trips), it
-// needs no second kernel, and results are bit-identical from run to run.  The waits cannot
-// deadlock: publishing a partial never waits for anything, and the grid is no larger than what
-// is resident at once.
+// Work is cut into tiles of 128 weight rows x BNX tokens, and every CTA takes a run of whole tiles.  With fewer tiles than half the
+// SMs and a long K (cut = 1), `per` CTAs share a tile, each with a part of its k-blocks: a CTA stores an fp32
+// partial tile, bumps the tile's arrival counter, waits (bounded) until all partials of the tile have arrived and then
+// reduces ITS columns of the tile -- contributor i takes the i-th slice of the token columns, adds the `per` partials in
+// ascending CTA order, applies the Eq. 4 / Eq. 11 scales and stores the outputs.  The reduction is thus spread over all
+// contributors with many independent loads in flight (one CTA adding whole partial tiles one after another spent tens
+// of microseconds on L2 round trips), it needs no second kernel, and results are bit-identical from run to run.  The
+// waits cannot deadlock: publishing a partial never waits for anything, and the grid is no larger than what is resident
+// at once.  (Equal slices of the flattened space of tiles and k-blocks, in which a CTA could hold parts of two tiles, were the
+// fastest arrangement at none of 772 shapes.)
 //
 // Per k-block one bulk copy brings the tile's packed INT4 codes, BF16 group scales (and
 // zero-points) and one TMA tile load brings the FP8 activations.  G groups of four warps expand
@@ -81,6 +78,7 @@ struct SkCfg {
     static constexpr int S2 = S2_;     // ring of dequantized E4M3 weight tiles
     static constexpr int FMT = FMT_;
     static constexpr bool CANON = FMT_ == kFmtCanonical;   // see the kernel's comment
+    static constexpr bool kCut = !CL_ && !W8_ && !W16_ && !CANON;   // a tile may be shared through the workspace
     static constexpr int kMeta = meta_bytes(FMT);
     static constexpr int kCodeBytes = 8192;   // packed codes of the tile's rows for one k-block
     static constexpr int kWStage = CANON ? 8192 : 9216;  // rows x (64 code bytes + meta), padded to keep the activation tile 1024-aligned
@@ -135,7 +133,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                       const uint8_t* __restrict__ gzero,           // canonical only: zero-points u8 [N][K/128] or NULL
                       const float* __restrict__ s_x, const float* __restrict__ s_w, int sw_stride,
                       void* __restrict__ y, int64_t ldy, int out_dtype, unsigned int* counters,
-                      float* slots, int M, int N, int K, int TM, int TN, int aligned, int cl,
+                      float* slots, int M, int N, int K, int TM, int TN, int cut, int per,
                       unsigned int* status_word) {
     constexpr int BNX = Cfg::BNX, G = Cfg::G, S1 = Cfg::S1, S2 = Cfg::S2;
     constexpr int TR = 128;   // weight rows per tile
@@ -160,7 +158,6 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
     constexpr int kNumBars = 3 * S1 + 2 * S2 + 6;
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bars + kNumBars);
     volatile uint32_t* abort_flag = tmem_slot + 1;
-    volatile uint32_t* share_slot = tmem_slot + 2;  // [3] number of shared tiles and their indices
 
     auto stage_w = [&](int s) { return base + (uint32_t)(s * Cfg::kStage1); };
     auto stage_x = [&](int s) { return base + (uint32_t)(s * Cfg::kStage1 + Cfg::kWStage); };
@@ -169,26 +166,22 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int KB = K >> 7;
     const uint8_t* meta_base = wpp + (int64_t)KB * N * kRowCodeBytes;
-    const int64_t U = (int64_t)TM * TN * KB;
-    const int64_t P = gridDim.x, p = blockIdx.x;
-    // Share of this CTA: an equal slice of the unit space, or -- when there are enough tiles
-    // for whole tiles to balance -- a run of whole tiles (then no partial tile is ever produced).
+    // Share of this CTA: a run of whole tiles, or (cut; CL) part p % per of the k-blocks of tile p / per.
     const int64_t Tt = (int64_t)TM * TN;
     int64_t u_begin, u_end;
-    if constexpr (Cfg::CL) {
-        // CTA p is member p % cl of the cluster of tile p / cl and takes that share of the tile's k-blocks
-        // (32-bit arithmetic: the 64-bit divisions of the general case cost a good part of a microsecond
-        // at the head of a launch that lasts ten)
-        const int pi = (int)blockIdx.x, tl = pi / cl, me = pi - tl * cl;
-        u_begin = (int64_t)tl * KB + me * KB / cl;
-        u_end = (int64_t)tl * KB + (me + 1) * KB / cl;
+    if (Cfg::CL || cut) {
+        // (32-bit arithmetic: 64-bit divisions cost a good part of a microsecond at the head of a launch that lasts ten)
+        const int pi = (int)blockIdx.x, tl = pi / per, me = pi - tl * per;
+        u_begin = (int64_t)tl * KB + me * KB / per;
+        u_end = (int64_t)tl * KB + (me + 1) * KB / per;
     } else {
-        u_begin = aligned ? (p * Tt / P) * KB : p * U / P;
-        u_end = aligned ? ((p + 1) * Tt / P) * KB : (p + 1) * U / P;
+        const int64_t P = gridDim.x, p = blockIdx.x;
+        u_begin = (p * Tt / P) * KB;
+        u_end = ((p + 1) * Tt / P) * KB;
     }
     const int n_it = (int)(u_end - u_begin);
     // first tile and k-block of the share
-    const int64_t tile_begin = Cfg::CL ? (int64_t)((int)blockIdx.x / cl) : u_begin / KB;
+    const int64_t tile_begin = Cfg::CL ? (int64_t)((int)blockIdx.x / per) : u_begin / KB;
     const int kb_begin = (int)(u_begin - tile_begin * KB);
 
     if (warp == 0) {
@@ -532,8 +525,6 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
             else
                 reinterpret_cast<__nv_bfloat16*>(y)[(int64_t)m * ldy + n] = __float2bfloat16_rn(res);
         };
-        int64_t shared_tile0 = 0, shared_tile1 = 0;  // tiles of which this CTA holds a partial (first and last segment)
-        int n_shared = 0;
         while (u < u_end && ok) {
             const int64_t tile = u / KB;
             const int kb0 = (int)(u - tile * KB);
@@ -557,9 +548,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
             ptx::tc_fence_after_sync();
             const uint32_t tmem_acc0 =
                 tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BNX + half * kHalfCols);
-            // The CTA's first segment uses slot 0, a later (necessarily last) one slot 1.
-            float* my_slot = slots + ((int64_t)p * 2 + (j == 0 ? 0 : 1)) * Cfg::kSlotFloats +
-                             (int64_t)half * kHalfCols * 128;
+            float* my_slot = slots + (int64_t)blockIdx.x * Cfg::kSlotFloats + (int64_t)half * kHalfCols * 128;
             if constexpr (Cfg::CL) {
                 if (!whole) {
                     // ---- exchange inside the cluster ----
@@ -568,10 +557,10 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                     const uint32_t red_local = base + (uint32_t)(BNX * 512);   // [source rank][column of my slice][128 channels]
                     const int me = (int)ptx::cluster_ctarank();
                     const int ncol = (M - mt * BNX) < BNX ? (M - mt * BNX) : BNX;   // valid token columns of the tile
-                    const int w = (ncol + cl - 1) / cl;                             // columns per slice
+                    const int w = (ncol + per - 1) / per;                             // columns per slice
                     int wn = ncol - me * w;                                         // valid columns of my slice
                     wn = wn < 0 ? 0 : (wn > w ? w : wn);
-                    if (leader) ptx::mbar_arrive_expect_tx(bar_red, (uint32_t)(cl * wn * 512));
+                    if (leader) ptx::mbar_arrive_expect_tx(bar_red, (uint32_t)(per * wn * 512));
                     // this thread's outputs as the owner of slice `me`: channels c4 .. c4 + 3 of the slice's
                     // columns te / 32, te / 32 + 8, ...; their scales are fetched before the wait
                     const int te = (warp - 2) * 32 + lane, c4 = (te & 31) * 4;
@@ -604,7 +593,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                     ptx::cluster_wait();   // the rings of every CTA of the cluster are idle
                     cl_waited = true;
                     asm volatile("bar.sync 1, 256;" ::: "memory");
-                    if (te < cl) {
+                    if (te < per) {
                         // one bulk copy per owner: my partial sums of its slice into its staging area,
                         // completion counted on its barrier
                         int cols = ncol - te * w;
@@ -622,7 +611,10 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                         const int tl = (te >> 5) + 8 * k;
                         if (tl >= wn) break;
                         float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
-                        for (int sr = 0; sr < cl; ++sr) {   // ascending rank order: the same sum on every launch
+                        // (unrolled: left to the compiler, (40, 4096, 4096) took 7.3 us in place of 6.8, (77, 4096, 14336) 15.4 in
+                        // place of 14.9)
+#pragma unroll 4
+                        for (int sr = 0; sr < per; ++sr) {   // ascending rank order: the same sum on every launch
                             float4 pv;
                             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
                                          : "=f"(pv.x), "=f"(pv.y), "=f"(pv.z), "=f"(pv.w)
@@ -717,20 +709,13 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
             ptx::tc_fence_before_sync();
             ptx::mbar_arrive(bar_acc_empty(buf));
             if (!whole) {
-                // Publish the partial tile and remember the tile for the reduction at the end.
+                // Publish the partial tile.
                 __threadfence();
                 asm volatile("bar.sync 1, 256;" ::: "memory");
                 if (leader) atomicAdd(counters + tile, 1u);
-                if (n_shared++ == 0) shared_tile0 = tile;
-                else shared_tile1 = tile;
             }
             u += len;
             ++j;
-        }
-        if (leader) {
-            share_slot[0] = (uint32_t)n_shared;
-            share_slot[1] = (uint32_t)shared_tile0;
-            share_slot[2] = (uint32_t)shared_tile1;
         }
     } else {
         // ------------------------------------------------------------------ dequantization groups
@@ -818,84 +803,68 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
         ptx::cluster_wait();
     }
 
-    // ---- reduction of the shared tiles, by every thread of the CTA: this CTA's slice of the token
-    // columns of each tile it holds a partial of ----
-    if (aligned) return;
+    // ---- reduction of a shared tile, by every thread of the CTA: this CTA's slice of the token columns ----
+    if (!cut) return;
     ptx::griddep_wait();
-    const int n_shared = (int)share_slot[0];
+    const int tile = (int)blockIdx.x / per, me = (int)blockIdx.x - tile * per;
     unsigned int* done = counters + (int64_t)TM * TN;  // second counter per tile: finished reducers
-    // Slot index of every contributor of the tile, worked out once (64-bit divisions: left inside
-    // the adding loop they cost every thread more than the loads did).  The rings are idle by now.
-    int* slot_of = reinterpret_cast<int*>(sm);
-    for (int k = 0; k < n_shared; ++k) {
-        const int64_t tile = (int64_t)share_slot[1 + k];
-        const int64_t p_lo = ((tile * KB + 1) * P - 1) / U;  // first and last contributor
-        const int64_t p_hi = (((tile + 1) * KB) * P - 1) / U;
-        const int C = (int)(p_hi - p_lo) + 1, me = (int)(p - p_lo);
-        __syncthreads();  // readers of the previous tile's table are done
-        for (int i = (int)threadIdx.x; i < C; i += Cfg::kThreads) {
-            // contributor q's slot for this tile: its first slot if the tile is where its share begins, else its second
-            const int64_t q = p_lo + i;
-            const int64_t first_tile = (q * U / P) / KB;
-            slot_of[i] = (int)(q * 2 + (tile == first_tile ? 0 : 1));
-        }
-        if (threadIdx.x == 0 && *abort_flag == 0u) {
-            // bounded wait for the C arrivals
-            uint64_t t0 = 0;
-            uint32_t spins = 0;
-            while (ptx::ld_acquire_gpu(counters + tile) < (uint32_t)C) {
-                if ((++spins & 63u) == 0u) {
-                    const uint64_t now = ptx::globaltimer_ns();
-                    if (t0 == 0) {
-                        t0 = now;
-                    } else if (now - t0 > ptx::kWaitLimitNs) {
-                        *abort_flag = 1u;
-                        atomicOr(status_word, kStatusTimeout);
-                        break;
-                    }
+    if (threadIdx.x == 0 && *abort_flag == 0u) {
+        // bounded wait for the arrivals
+        uint64_t t0 = 0;
+        uint32_t spins = 0;
+        while (ptx::ld_acquire_gpu(counters + tile) < (uint32_t)per) {
+            if ((++spins & 63u) == 0u) {
+                const uint64_t now = ptx::globaltimer_ns();
+                if (t0 == 0) {
+                    t0 = now;
+                } else if (now - t0 > ptx::kWaitLimitNs) {
+                    *abort_flag = 1u;
+                    atomicOr(status_word, kStatusTimeout);
+                    break;
                 }
             }
         }
-        __syncthreads();
-        if (*abort_flag != 0u) break;
-        __threadfence();
-        const int nt = (int)(tile / TM), mt = (int)(tile - (int64_t)nt * TM);
-        const int nrow = (N - nt * 128) < 128 ? (N - nt * 128) : 128;
-        const int ncol = (M - mt * BNX) < BNX ? (M - mt * BNX) : BNX;  // valid token columns of the tile
-        const int c_lo = (int)((int64_t)me * ncol / C), c_hi = (int)((int64_t)(me + 1) * ncol / C);
-        // element e of the slice: row e % 128 (consecutive threads, consecutive addresses), column c_lo + e / 128
-        const int total = (c_hi - c_lo) * 128;
-        for (int e0 = (int)threadIdx.x; e0 < total; e0 += 4 * Cfg::kThreads) {
-            float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    }
+    __syncthreads();
+    if (*abort_flag != 0u) return;
+    __threadfence();
+    const int nt = tile / TM, mt = tile - nt * TM;
+    const int nrow = (N - nt * 128) < 128 ? (N - nt * 128) : 128;
+    const int ncol = (M - mt * BNX) < BNX ? (M - mt * BNX) : BNX;  // valid token columns of the tile
+    const int c_lo = me * ncol / per, c_hi = (me + 1) * ncol / per;
+    const float* first = slots + (int64_t)tile * per * Cfg::kSlotFloats + c_lo * 128;   // the first contributor's partial sums
+    // element e of the slice: row e % 128 (consecutive threads, consecutive addresses), column c_lo + e / 128
+    const int total = (c_hi - c_lo) * 128;
+    for (int e0 = (int)threadIdx.x; e0 < total; e0 += 4 * Cfg::kThreads) {
+        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 4
-            for (int i = 0; i < C; ++i) {
-                const float* sl = slots + (int64_t)slot_of[i] * Cfg::kSlotFloats + c_lo * 128;
-#pragma unroll
-                for (int jj = 0; jj < 4; ++jj) {
-                    const int e = e0 + jj * Cfg::kThreads;
-                    if (e < total && (e & 127) < nrow) acc[jj] += __ldcg(sl + e);
-                }
-            }
+        for (int i = 0; i < per; ++i) {
+            const float* sl = first + (int64_t)i * Cfg::kSlotFloats;
 #pragma unroll
             for (int jj = 0; jj < 4; ++jj) {
                 const int e = e0 + jj * Cfg::kThreads;
-                if (e < total && (e & 127) < nrow) {
-                    const int n = nt * 128 + (e & 127), m = mt * BNX + c_lo + (e >> 7);
-                    const float res = acc[jj] * (__ldg(s_x + m) * __ldg(s_w + (int64_t)n * sw_stride));
-                    if (out_dtype == W4A8_OUT_FP32)
-                        reinterpret_cast<float*>(y)[(int64_t)m * ldy + n] = res;
-                    else
-                        reinterpret_cast<__nv_bfloat16*>(y)[(int64_t)m * ldy + n] = __float2bfloat16_rn(res);
-                }
+                if (e < total && (e & 127) < nrow) acc[jj] += __ldcg(sl + e);
             }
         }
-        // the last reducer to finish re-arms the tile's counters for the next launch
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            if (atomicAdd(done + tile, 1u) == (uint32_t)(C - 1)) {
-                counters[tile] = 0u;
-                done[tile] = 0u;
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+            const int e = e0 + jj * Cfg::kThreads;
+            if (e < total && (e & 127) < nrow) {
+                const int n = nt * 128 + (e & 127), m = mt * BNX + c_lo + (e >> 7);
+                const float res = acc[jj] * (__ldg(s_x + m) * __ldg(s_w + (int64_t)n * sw_stride));
+                if (out_dtype == W4A8_OUT_FP32)
+                    reinterpret_cast<float*>(y)[(int64_t)m * ldy + n] = res;
+                else
+                    reinterpret_cast<__nv_bfloat16*>(y)[(int64_t)m * ldy + n] = __float2bfloat16_rn(res);
             }
+        }
+    }
+    // the last reducer to finish re-arms the tile's counters for the next launch
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (atomicAdd(done + tile, 1u) == (uint32_t)(per - 1)) {
+            counters[tile] = 0u;
+            done[tile] = 0u;
         }
     }
 }

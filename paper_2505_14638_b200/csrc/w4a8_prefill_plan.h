@@ -33,9 +33,8 @@ constexpr size_t kSkWorkspaceBytes = kLinearCtlBytes + (size_t)kMaxSMs * 2 * 256
 
 struct SkPlan {
     int bnx, TM, TN;
-    int aligned;   // 1: whole tiles per CTA, nothing shared; 0: several CTAs per tile
+    int per;       // CTAs per tile (1: whole tiles, a run of them per CTA)
     int64_t P;     // CTAs
-    int64_t U;
     size_t counter_bytes;
 };
 
@@ -169,8 +168,7 @@ inline PrefillKind prefill_choice(int64_t M, int64_t N, int64_t K, bool signmag,
         pl->bnx = bnx;
         pl->TM = (int)TM;
         pl->TN = (int)TN;
-        pl->U = tiles * KB;
-        pl->aligned = ctas == 1 ? 1 : 0;
+        pl->per = (int)ctas;
         pl->P = ctas == 1 ? (tiles < cap ? tiles : cap) : tiles * ctas;
         pl->counter_bytes = ctas == 1 ? 0 : kLinearCtlBytes;
     }

@@ -29,8 +29,8 @@ extern "C" int choice(long long M, long long N, long long K, int signmag, int sm
 
 
 class SkPlan(ctypes.Structure):
-    _fields_ = [("bnx", ctypes.c_int), ("TM", ctypes.c_int), ("TN", ctypes.c_int), ("aligned", ctypes.c_int), ("P", ctypes.c_int64),
-                ("U", ctypes.c_int64), ("counter_bytes", ctypes.c_size_t)]
+    _fields_ = [("bnx", ctypes.c_int), ("TM", ctypes.c_int), ("TN", ctypes.c_int), ("per", ctypes.c_int), ("P", ctypes.c_int64),
+                ("counter_bytes", ctypes.c_size_t)]
 
 
 @pytest.fixture(scope="module")
@@ -105,10 +105,9 @@ def test_plans_of_the_persistent_kernel(plan, sms):
         if kind.startswith("pairs"):
             continue
         bnx, tiles = int(kind.lstrip("wholecut")), pl.TM * pl.TN
-        assert (pl.bnx, pl.TM, pl.TN, pl.U) == (bnx, -(-M // bnx), -(-N // 128), tiles * K // 128)
+        assert (pl.bnx, pl.TM, pl.TN) == (bnx, -(-M // bnx), -(-N // 128))
         if kind.startswith("whole"):
-            assert pl.aligned == 1 and pl.P == min(tiles, sms)
+            assert pl.per == 1 and pl.P == min(tiles, sms)
         else:
-            # a whole number of CTAs per tile, resident at once, each with k-blocks of its own
-            per = pl.P // tiles
-            assert pl.aligned == 0 and pl.P == per * tiles and 2 <= per <= K // 128 // 2 and pl.P <= sms
+            # resident at once, each with k-blocks of its own
+            assert pl.P == pl.per * tiles <= sms and 2 <= pl.per <= K // 128 // 2
