@@ -8,7 +8,8 @@
 // to shared memory and has 64 KB read by its MMAs, 1024 tensor-pipe cycles; one CTA on its own with a 256 x 256 tile, the
 // kernel before this one, expanded 256 rows, wrote 32 + 49 KB and had 96 KB read, which is more than the 128 bytes a
 // clock of shared memory allow.  (8192, 28672, 8192): 2011 -> 1500 us back to back (1180-1230 MHz, 1000 W; the library's FP8
-// GEMM on FP8 weights 1460), 84 % of the tensor pipe at that clock; (2048, 4096, 4096): 1130-1170 cycles per k-block of the 1024.
+// GEMM on FP8 weights 1460), 86-90 % of the tensor pipe at that clock by the cycles of its MMAs; (2048, 4096, 4096): 1130-1170 cycles
+// per k-block of the 1024.
 //
 //   H = 2  both accumulators belong to the tile in flight, expanded weights in shared memory.  The MMAs of a tile's first and
 //          last kSkew k-blocks are issued for one accumulator first and then for the other: the second accumulator is
