@@ -99,7 +99,7 @@ linear_direct_kernel(const uint8_t* __restrict__ x8, int64_t ldx8, const uint8_t
     // 8-row unit does not exist, the last or first one is read in its place and its scale is taken as zero: zero weights.
     const uint8_t* meta0 = weights + (int64_t)KB * N * kRowCodeBytes;
     uint4 lo[4], hi[4];
-    uint32_t mlo = 0u, mhi = 0u;   // scale (BF16 bits), zero-point above it
+    uint32_t mlo = kZeroMeta<FMT>, mhi = kZeroMeta<FMT>;   // scale (BF16 bits), zero-point above it
     struct Unit {
         const uint8_t* lo;
         const uint8_t* hi;
@@ -129,8 +129,7 @@ linear_direct_kernel(const uint8_t* __restrict__ x8, int64_t ldx8, const uint8_t
     auto load_meta = [&](int t, int q, uint32_t& a, uint32_t& b) {
         const int kb = 4 * q + tig, n = (u0 + 2 * t) * 8 + gid;
         const bool in = kb < KB, in_hi = in && u0 + 2 * t + 1 < u1;
-        a = 0u;
-        b = 0u;
+        a = b = kZeroMeta<FMT>;
         if constexpr (kCanonical) {
             const int64_t i = (int64_t)n * KB + kb, j = i + (int64_t)8 * KB;
             if (in) a = (uint32_t)__ldg(gscale + i) | (gzero ? (uint32_t)__ldg(gzero + i) : 8u) << 16;
@@ -190,15 +189,9 @@ linear_direct_kernel(const uint8_t* __restrict__ x8, int64_t ldx8, const uint8_t
         }
         const bool more = tn < T;
         const uint32_t xoff = (uint32_t)(min(4 * q + tig, KB - 1) * 144);
-        using Lut = typename std::conditional<kSignMag, SignMagLut, DequantLut>::type;
-        Lut llo, lhi;
-        if constexpr (kSignMag) {
-            llo.build(bf16_bits_to_float(mlo));
-            lhi.build(bf16_bits_to_float(mhi));
-        } else {
-            llo.build(bf16_bits_to_float(mlo & 0xFFFFu), (int)((mlo >> 16) & 0xFFu));
-            lhi.build(bf16_bits_to_float(mhi & 0xFFFFu), (int)((mhi >> 16) & 0xFFu));
-        }
+        typename LutOf<FMT>::type llo, lhi;
+        llo.build_meta(mlo);
+        lhi.build_meta(mhi);
         if (more) load_meta(tn, qn, mlo, mhi);
         const bool has_hi = u0 + 2 * t + 1 < u1;
         const Unit next = unit(more ? tn : t, more ? qn : q);

@@ -9,8 +9,9 @@
 //                 chunks at a fixed 128-byte stride (no per-chunk address arithmetic), and eight
 //                 consecutive rows read with 128-bit loads touch every shared-memory bank once.
 //   meta region   [KB][N][MB bytes]   starts at KB * N * 64; MB = 2 (BF16 group scale) in the
-//                 sign-magnitude format, 4 (BF16 scale, zero-point byte, one byte of padding) in
-//                 the generic format
+//                 sign-magnitude format, 4 in the generic format (BF16 scale >= 0, then the zero-point
+//                 as BF16 with the bits 0x7FC0 flipped: see PairLut)
+// Codes are kept in the form that the expansion takes least instructions for: SignMagLut, PairLut.
 // Any run of consecutive eight-row units of one k-block is therefore one contiguous, 128-byte
 // aligned piece of codes plus one contiguous piece of meta data: two bulk copies bring it into
 // shared memory, whatever row partition the kernel picks at launch.
@@ -44,24 +45,90 @@ __host__ __device__ constexpr uint32_t row_offset(int fmt, int row) {
     return fmt == kFmtTiledFp8 ? (uint32_t)(row >> 3) * 1024u + (uint32_t)(row & 7) * 16u : tiled_row_offset(row);
 }
 
+// The expansion is bound by the integer pipe (a warp's instruction every other cycle: logic, shifts, byte permutes), so what
+// can is done beside it on the multipliers: shifts as multiplications, sums as multiply-adds.  The factors are read from
+// here because ptxas turns constants back into shifts and plain sums.
+__constant__ uint32_t kExpandOne = 1u;
+__constant__ uint32_t kExpandHigh = 0x0100u;   // two-way dot product: 0 * low half + 1 * high half
+
+// Selector of the upper four nibbles (a byte permute reads the low half only).
+__device__ __forceinline__ uint32_t high_half(uint32_t w) {
+    uint32_t d;
+    asm("dp2a.lo.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(kExpandHigh), "r"(0u));
+    return d;
+}
+
 // Sign-magnitude table of a symmetric group (z = 8): entry d = nearest_E4M3(d * s), d = 0..7.
 // A stored nibble carries |u - 8| in its low three bits; the sign travels separately and is
 // applied by flipping the E4M3 sign bit (the format is sign-magnitude and the rounding is
 // symmetric, so nearest_E4M3(-d s) and nearest_E4M3(d s) differ in that bit only).
+// Eight weights take 5 instructions of the integer pipe and 2 of the multipliers: 10.3 cycles of a sub-partition, against
+// 12.1 with the shift on the integer pipe (registers to registers, four warps, one more multiply-add in both).
 struct SignMagLut {
     uint32_t t0, t1;
     __device__ __forceinline__ void build(float s) {
         t0 = cvt_e4m3x4(__fmul_rn(0.0f, s), s, __fmul_rn(2.0f, s), __fmul_rn(3.0f, s));
         t1 = cvt_e4m3x4(__fmul_rn(4.0f, s), __fmul_rn(5.0f, s), __fmul_rn(6.0f, s), __fmul_rn(7.0f, s));
     }
+    __device__ __forceinline__ void build_meta(uint32_t meta) { build(bf16_bits_to_float(meta & 0xFFFFu)); }
     // Word layout: nibble i (i = 0..3) = magnitude of element i, nibble 4+i = magnitude of
     // element 4+i; sign of element i in bit 8i+7, sign of element 4+i in bit 8i+3.
     __device__ __forceinline__ void dequant8(uint32_t w, uint32_t& out0, uint32_t& out1) const {
         const uint32_t sel = w & 0x77777777u;
         out0 = prmt(t0, t1, sel) ^ (w & 0x80808080u);
-        out1 = prmt(t0, t1, sel >> 16) ^ ((w << 4) & 0x80808080u);
+        out1 = prmt(t0, t1, high_half(sel)) ^ ((w << 4) & 0x80808080u);
     }
 };
+
+// Table of a group with a zero-point.  The sixteen values nearest_E4M3((u - z) s) of a group are eight pairs (2i, 2i + 1) of
+// one sign each (the value 0 takes the sign of the pair it is in: -0 beside a negative value).  A stored nibble is the pair in
+// its low three bits and a bit that is SET for the value of smaller magnitude; the word keeps the element order.  a = the
+// smaller value's byte, d = what the larger one's is more (0..127).  A byte permute by the nibble as it is gives d where the
+// top bit is clear and, since that bit asks for copies of the selected byte's sign bit, 0 where it is set: the expanded byte is
+// the sum a + d of two look-ups, without a carry, on the multipliers.  Eight weights take 5 instructions of the integer pipe
+// and 4 of the multipliers: 11.9 cycles (see SignMagLut), against 24.2 for the sixteen-entry table of DequantLut.
+// s >= 0 in this format (prepack mirrors groups of negative scale).  The zero-point is stored as BF16 with the bits 0x7FC0
+// flipped: one instruction restores it, and the integer zero-points of a buffer written before this form existed become NaN
+// and so do all outputs, instead of being read wrongly.
+constexpr uint32_t kPairZeroFlip = 0x7FC0u;
+struct PairLut {
+    uint32_t a0, a1, d0, d1;
+    static __device__ __forceinline__ void pairs(uint32_t even, uint32_t odd, uint32_t& a, uint32_t& d) {
+        const uint32_t neg = prmt(even, 0u, 0xBA98u);   // 0xFF where the pair is negative: there the even code is the larger one
+        const uint32_t large = (even & neg) | (odd & ~neg), small = (odd & neg) | (even & ~neg);
+        a = small | (large & 0x80808080u);
+        d = large - a;   // (rounding is monotonic: no byte borrows)
+    }
+    __device__ __forceinline__ void build_meta(uint32_t meta) {
+        const float s = __uint_as_float(meta << 16), z = __uint_as_float((meta ^ (kPairZeroFlip << 16)) & 0xFFFF0000u);
+        float v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = __fmul_rn((float)u - z, s);
+        pairs(cvt_e4m3x4(v[0], v[2], v[4], v[6]), cvt_e4m3x4(v[1], v[3], v[5], v[7]), a0, d0);
+        pairs(cvt_e4m3x4(v[8], v[10], v[12], v[14]), cvt_e4m3x4(v[9], v[11], v[13], v[15]), a1, d1);
+    }
+    __device__ __forceinline__ void dequant8(uint32_t w, uint32_t& out0, uint32_t& out1) const {
+        const uint32_t sel = w & 0x77777777u;
+        out0 = prmt(a0, a1, sel) * kExpandOne + prmt(d0, d1, w);
+        out1 = prmt(a0, a1, high_half(sel)) * kExpandOne + prmt(d0, d1, high_half(w));
+    }
+};
+
+// The look-up table of a format, built from a row's meta word (scale; canonical weights: zero-point from bit 16 on).
+struct CanonicalLut : DequantLut {
+    __device__ __forceinline__ void build_meta(uint32_t meta) { build(bf16_bits_to_float(meta & 0xFFFFu), (int)(meta >> 16)); }
+};
+template <int FMT>
+struct LutOf;
+template <>
+struct LutOf<kFmtCanonical> { using type = CanonicalLut; };
+template <>
+struct LutOf<kFmtTiled> { using type = PairLut; };
+template <>
+struct LutOf<kFmtTiledSignMag> { using type = SignMagLut; };
+// Meta word whose weights are all zero, for rows and k-blocks that do not exist.
+template <int FMT>
+constexpr uint32_t kZeroMeta = FMT == kFmtTiled ? kPairZeroFlip << 16 : 0u;
 
 // The four code chunks of one row (constant address offsets: no arithmetic per chunk).
 template <int C>
@@ -107,23 +174,13 @@ __device__ __forceinline__ uint32_t load_meta_word(uint32_t meta, int fmt) {
 template <int FMT>
 __device__ __forceinline__ void expand_row_to_smem(const uint32_t (&pk)[16], uint32_t mbits, int row, uint32_t dst) {
     const uint32_t sw128 = (uint32_t)(row & 7);
-    const float sc = bf16_bits_to_float(mbits & 0xFFFFu);
-    SignMagLut slut;
-    DequantLut glut;
-    if constexpr (FMT == kFmtTiledSignMag)
-        slut.build(sc);
-    else
-        glut.build(sc, (int)((mbits >> 16) & 0xFFu));
+    typename LutOf<FMT>::type lut;
+    lut.build_meta(mbits);
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
         uint32_t o0, o1, o2, o3;
-        if constexpr (FMT == kFmtTiledSignMag) {
-            slut.dequant8(pk[2 * c], o0, o1);
-            slut.dequant8(pk[2 * c + 1], o2, o3);
-        } else {
-            glut.dequant8(pk[2 * c], o0, o1);
-            glut.dequant8(pk[2 * c + 1], o2, o3);
-        }
+        lut.dequant8(pk[2 * c], o0, o1);
+        lut.dequant8(pk[2 * c + 1], o2, o3);
         asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (((uint32_t)c ^ sw128) << 4)), "r"(o0),
                      "r"(o1), "r"(o2), "r"(o3)
                      : "memory");
@@ -141,8 +198,8 @@ __device__ __forceinline__ void dequant_row_to_smem(uint32_t src, uint32_t meta,
 // (BF16 bits) and zero-point (from bit 16 on) in `meta`.
 __device__ __forceinline__ void dequant_canonical_row_to_smem(uint32_t tile, uint32_t meta, int row, uint32_t dst) {
     const uint32_t sw64 = (uint32_t)((row >> 1) & 3), sw128 = (uint32_t)(row & 7), src = tile + (uint32_t)row * 64u;
-    DequantLut lut;
-    lut.build(bf16_bits_to_float(meta & 0xFFFFu), (int)(meta >> 16));
+    CanonicalLut lut;
+    lut.build_meta(meta);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         uint32_t p[4];
@@ -204,37 +261,25 @@ __device__ __forceinline__ void dequant_row_to_smem_bf16(uint32_t src, uint32_t 
 // warp's lane quarter), written as two 16-column stores to keep the live register count low.
 // Warp-collective: every lane of the warp must call it with a readable row (a lane without a
 // row of its own repeats another one; its tensor-memory lane is then never read out).
+// (expand_row_to_tmem: codes and meta word are in registers already.)
+template <int FMT>
+__device__ __forceinline__ void expand_row_to_tmem(const uint32_t (&pk)[16], uint32_t mbits, uint32_t taddr) {
+    typename LutOf<FMT>::type lut;
+    lut.build_meta(mbits);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t out[16];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) lut.dequant8(pk[8 * h + w], out[2 * w], out[2 * w + 1]);
+        ptx::tmem_st_32x32b_x16(taddr + 16u * h, out);
+    }
+}
 template <int FMT>
 __device__ __forceinline__ void dequant_row_to_tmem(uint32_t src, uint32_t meta, uint32_t taddr) {
-    uint32_t mbits;
+    const uint32_t mbits = load_meta_word(meta, FMT);
     uint32_t pk[16];
-    if constexpr (FMT == kFmtTiledSignMag)
-        asm volatile("ld.shared.u16 %0, [%1];" : "=r"(mbits) : "r"(meta));
-    else
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(mbits) : "r"(meta));
     load_row_codes(src, pk);
-    const float sc = bf16_bits_to_float(mbits & 0xFFFFu);
-    if constexpr (FMT == kFmtTiledSignMag) {
-        SignMagLut lut;
-        lut.build(sc);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            uint32_t out[16];
-#pragma unroll
-            for (int w = 0; w < 8; ++w) lut.dequant8(pk[8 * h + w], out[2 * w], out[2 * w + 1]);
-            ptx::tmem_st_32x32b_x16(taddr + 16u * h, out);
-        }
-    } else {
-        DequantLut lut;
-        lut.build(sc, (int)((mbits >> 16) & 0xFFu));
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            uint32_t out[16];
-#pragma unroll
-            for (int w = 0; w < 8; ++w) lut.dequant8(pk[8 * h + w], out[2 * w], out[2 * w + 1]);
-            ptx::tmem_st_32x32b_x16(taddr + 16u * h, out);
-        }
-    }
+    expand_row_to_tmem<FMT>(pk, mbits, taddr);
 }
 
 // FP8 weights (W8A8 comparison scheme): the row's 128 bytes of the k-block go to tensor memory as they are.
@@ -262,33 +307,6 @@ __global__ void prepack_fp8_kernel(const uint8_t* __restrict__ w8, int64_t N, in
     *reinterpret_cast<uint4*>(out + (kb * N + (n & ~(int64_t)7)) * 128 + c * 128 + (n & 7) * 16) = v;
 }
 
-// The expansion of one row whose codes and meta word are already in registers.
-template <int FMT>
-__device__ __forceinline__ void expand_row_to_tmem(const uint32_t (&pk)[16], uint32_t mbits, uint32_t taddr) {
-    const float sc = bf16_bits_to_float(mbits & 0xFFFFu);
-    if constexpr (FMT == kFmtTiledSignMag) {
-        SignMagLut lut;
-        lut.build(sc);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            uint32_t out[16];
-#pragma unroll
-            for (int w = 0; w < 8; ++w) lut.dequant8(pk[8 * h + w], out[2 * w], out[2 * w + 1]);
-            ptx::tmem_st_32x32b_x16(taddr + 16u * h, out);
-        }
-    } else {
-        DequantLut lut;
-        lut.build(sc, (int)((mbits >> 16) & 0xFFu));
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            uint32_t out[16];
-#pragma unroll
-            for (int w = 0; w < 8; ++w) lut.dequant8(pk[8 * h + w], out[2 * w], out[2 * w + 1]);
-            ptx::tmem_st_32x32b_x16(taddr + 16u * h, out);
-        }
-    }
-}
-
 // A row of a canonical tile (see dequant_canonical_row_to_smem) to tensor memory.
 __device__ __forceinline__ void dequant_canonical_row_to_tmem(uint32_t tile, uint32_t meta, int row, uint32_t taddr) {
     const uint32_t sw64 = (uint32_t)((row >> 1) & 3), src = tile + (uint32_t)row * 64u;
@@ -298,7 +316,7 @@ __device__ __forceinline__ void dequant_canonical_row_to_tmem(uint32_t tile, uin
         asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
                      : "=r"(p[4 * j]), "=r"(p[4 * j + 1]), "=r"(p[4 * j + 2]), "=r"(p[4 * j + 3])
                      : "r"(src + (((uint32_t)j ^ sw64) << 4)));
-    expand_row_to_tmem<kFmtTiled>(p, meta, taddr);
+    expand_row_to_tmem<kFmtCanonical>(p, meta, taddr);
 }
 
 // Two rows (two items of one pipeline stage) expanded into 2 x 32 consecutive tensor-memory
@@ -340,6 +358,18 @@ __device__ __forceinline__ uint32_t to_signmag_word(uint32_t w, bool& bad) {
     return out;
 }
 
+// Codes of a group with zero-point z as PairLut reads them.
+__device__ __forceinline__ uint32_t to_pair_word(uint32_t w, int z) {
+    uint32_t out = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int u = (int)((w >> (4 * i)) & 15u);
+        const bool negative = (u & ~1) < z, odd = u & 1;
+        out |= (uint32_t)((u >> 1) | (negative == odd ? 8 : 0)) << (4 * i);
+    }
+    return out;
+}
+
 __global__ void __launch_bounds__(128)
 prepack_kernel(const uint8_t* __restrict__ codes, const uint16_t* __restrict__ gscale,
                const uint8_t* __restrict__ gzero, int64_t N, int64_t K, int fmt, uint8_t* __restrict__ out,
@@ -352,6 +382,8 @@ prepack_kernel(const uint8_t* __restrict__ codes, const uint16_t* __restrict__ g
     uint4 w[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) w[c] = src[c];
+    uint32_t sc = gscale[n * KB + kb];
+    int z = gzero ? (int)gzero[n * KB + kb] : 8;
     if (fmt == kFmtTiledSignMag) {
         bool bad = false;
 #pragma unroll
@@ -362,18 +394,26 @@ prepack_kernel(const uint8_t* __restrict__ codes, const uint16_t* __restrict__ g
             w[c].w = to_signmag_word(w[c].w, bad);
         }
         if (bad) atomicOr(status_word, kStatusBadCode);
+    } else {
+        // (u - z) s = ((15 - u) - (15 - z)) (-s)
+        if (sc & 0x8000u) {
+            sc ^= 0x8000u;
+            z = 15 - z;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) w[c] = make_uint4(~w[c].x, ~w[c].y, ~w[c].z, ~w[c].w);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            w[c] = make_uint4(to_pair_word(w[c].x, z), to_pair_word(w[c].y, z), to_pair_word(w[c].z, z), to_pair_word(w[c].w, z));
     }
     uint8_t* dst = out + (kb * N + (n & ~(int64_t)7)) * kRowCodeBytes + (n & 7) * 16;
 #pragma unroll
     for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(dst + c * kChunkStride) = w[c];
     uint8_t* meta = out + KB * N * kRowCodeBytes + (kb * N + n) * meta_bytes(fmt);
-    const uint16_t sc = gscale[n * KB + kb];
-    if (fmt == kFmtTiledSignMag) {
-        *reinterpret_cast<uint16_t*>(meta) = sc;
-    } else {
-        const uint32_t z = gzero ? (uint32_t)gzero[n * KB + kb] : 8u;
-        *reinterpret_cast<uint32_t*>(meta) = (uint32_t)sc | (z << 16);
-    }
+    if (fmt == kFmtTiledSignMag)
+        *reinterpret_cast<uint16_t*>(meta) = (uint16_t)sc;
+    else   // (a zero-point is a byte, 15 - z no less than -240: exact in BF16)
+        *reinterpret_cast<uint32_t*>(meta) = sc | ((__float_as_uint((float)z) ^ (kPairZeroFlip << 16)) & 0xFFFF0000u);
 }
 
 }  // namespace w4a8
