@@ -30,15 +30,63 @@ __device__ __forceinline__ uint32_t cvt_e4m3x2(float hi, float lo) {
     return (uint32_t)r;
 }
 
-// Four fp32 values -> four E4M3 bytes, v0 in the lowest byte.
+// Four fp32 values -> four E4M3 bytes, v0 in the lowest byte.  (Both halves in one asm block: the second conversion then
+// merges the first one's result, 5 cycles of a sub-partition; a shift and an OR behind them made it 8.)
 __device__ __forceinline__ uint32_t cvt_e4m3x4(float v0, float v1, float v2, float v3) {
-    return cvt_e4m3x2(v1, v0) | (cvt_e4m3x2(v3, v2) << 16);
+    uint32_t r;
+    asm("{\n\t"
+        ".reg .b16 lo, hi;\n\t"
+        "cvt.rn.satfinite.e4m3x2.f32 lo, %2, %1;\n\t"
+        "cvt.rn.satfinite.e4m3x2.f32 hi, %4, %3;\n\t"
+        "mov.b32 %0, {lo, hi};\n\t"
+        "}\n"
+        : "=r"(r)
+        : "f"(v0), "f"(v1), "f"(v2), "f"(v3));
+    return r;
 }
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     uint32_t d;
     asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
     return d;
+}
+
+// The expansion is bound by the integer pipe (a warp's instruction every other cycle: logic, shifts, byte permutes), so what
+// can is done beside it on the multipliers: shifts as multiplications, sums as multiply-adds.  The factors are read from
+// here because ptxas turns constants back into shifts and plain sums.
+__constant__ uint32_t kExpandOne = 1u;
+__constant__ uint32_t kExpandHigh = 0x0100u;   // two-way dot product: 0 * low half + 1 * high half
+
+// Selector of the upper four nibbles (a byte permute reads the low half only).
+__device__ __forceinline__ uint32_t high_half(uint32_t w) {
+    uint32_t d;
+    asm("dp2a.lo.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(kExpandHigh), "r"(0u));
+    return d;
+}
+
+// Two fp32 lanes per instruction.
+__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long mul_f32x2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ void unpack_f32x2(unsigned long long v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
 }
 
 // Two BF16 lanes: (x - off) * sc, the subtraction exact for the small integers it is used on, the
@@ -80,7 +128,7 @@ struct DequantLut {
         uint32_t a0 = prmt(t[0], t[1], lo3);
         uint32_t b0 = prmt(t[2], t[3], lo3);
         out0 = prmt(a0, b0, pick);
-        uint32_t lo3h = lo3 >> 16, pickh = pick >> 16;
+        uint32_t lo3h = high_half(lo3), pickh = high_half(pick);
         uint32_t a1 = prmt(t[0], t[1], lo3h);
         uint32_t b1 = prmt(t[2], t[3], lo3h);
         out1 = prmt(a1, b1, pickh);

@@ -113,30 +113,6 @@ __device__ __forceinline__ float div_recip(float a, const Recip& r) {
 __device__ __forceinline__ bool recip_range(float b) { return fabsf(b) >= 0x1p-40f && fabsf(b) <= 0x1p40f; }
 
 // Two FP32 operations in one instruction (each rounded once, as two scalar ones).
-__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ unsigned long long mul_f32x2(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
-    unsigned long long d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-    return d;
-}
-__device__ __forceinline__ void unpack_f32x2(unsigned long long v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-
 __device__ __forceinline__ unsigned long long div_recip_f32x2(unsigned long long a, const Recip& r) {
     const unsigned long long h = pack_f32x2(r.h, r.h);
     const unsigned long long q = fma_f32x2(a, h, mul_f32x2(a, pack_f32x2(r.l, r.l)));

@@ -45,19 +45,6 @@ __host__ __device__ constexpr uint32_t row_offset(int fmt, int row) {
     return fmt == kFmtTiledFp8 ? (uint32_t)(row >> 3) * 1024u + (uint32_t)(row & 7) * 16u : tiled_row_offset(row);
 }
 
-// The expansion is bound by the integer pipe (a warp's instruction every other cycle: logic, shifts, byte permutes), so what
-// can is done beside it on the multipliers: shifts as multiplications, sums as multiply-adds.  The factors are read from
-// here because ptxas turns constants back into shifts and plain sums.
-__constant__ uint32_t kExpandOne = 1u;
-__constant__ uint32_t kExpandHigh = 0x0100u;   // two-way dot product: 0 * low half + 1 * high half
-
-// Selector of the upper four nibbles (a byte permute reads the low half only).
-__device__ __forceinline__ uint32_t high_half(uint32_t w) {
-    uint32_t d;
-    asm("dp2a.lo.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(kExpandHigh), "r"(0u));
-    return d;
-}
-
 // Sign-magnitude table of a symmetric group (z = 8): entry d = nearest_E4M3(d * s), d = 0..7.
 // A stored nibble carries |u - 8| in its low three bits; the sign travels separately and is
 // applied by flipping the E4M3 sign bit (the format is sign-magnitude and the rounding is
@@ -87,12 +74,18 @@ struct SignMagLut {
 // top bit is clear and, since that bit asks for copies of the selected byte's sign bit, 0 where it is set: the expanded byte is
 // the sum a + d of two look-ups, without a carry, on the multipliers.  Eight weights take 5 instructions of the integer pipe
 // and 4 of the multipliers: 11.9 cycles (see SignMagLut), against 24.2 for the sixteen-entry table of DequantLut.
-// s >= 0 in this format (prepack mirrors groups of negative scale).  The zero-point is stored as BF16 with the bits 0x7FC0
+// 0 <= s <= 448 in this format (prepack mirrors groups of negative scale; a larger one gives the same table as 448).  The zero-point is stored as BF16 with the bits 0x7FC0
 // flipped: one instruction restores it, and the integer zero-points of a buffer written before this form existed become NaN
 // and so do all outputs, instead of being read wrongly.
 constexpr uint32_t kPairZeroFlip = 0x7FC0u;
 struct PairLut {
     uint32_t a0, a1, d0, d1;
+    static __device__ __forceinline__ uint32_t cvt_two(unsigned long long x, unsigned long long y) {
+        float x0, x1, y0, y1;
+        unpack_f32x2(x, x0, x1);
+        unpack_f32x2(y, y0, y1);
+        return cvt_e4m3x4(x0, x1, y0, y1);
+    }
     static __device__ __forceinline__ void pairs(uint32_t even, uint32_t odd, uint32_t& a, uint32_t& d) {
         const uint32_t neg = prmt(even, 0u, 0xBA98u);   // 0xFF where the pair is negative: there the even code is the larger one
         const uint32_t large = (even & neg) | (odd & ~neg), small = (odd & neg) | (even & ~neg);
@@ -101,11 +94,18 @@ struct PairLut {
     }
     __device__ __forceinline__ void build_meta(uint32_t meta) {
         const float s = __uint_as_float(meta << 16), z = __uint_as_float((meta ^ (kPairZeroFlip << 16)) & 0xFFFF0000u);
-        float v[16];
+        // (u - z) s for u = {0, 2} and {1, 3}, then four codes further at a time: multiples of s below 2^17 times its unit, so every
+        // sum is exact (and u = z gives +0).  22 cycles of a sub-partition fewer than sixteen differences and products.
+        const float e = __fmaf_rn(-z, s, 0.0f), o = __fmaf_rn(-z, s, s), step = 4.0f * s;
+        const unsigned long long step2 = pack_f32x2(step, step);
+        unsigned long long even[4] = {pack_f32x2(e, __fmaf_rn(2.0f, s, e))}, odd[4] = {pack_f32x2(o, __fmaf_rn(2.0f, s, o))};
 #pragma unroll
-        for (int u = 0; u < 16; ++u) v[u] = __fmul_rn((float)u - z, s);
-        pairs(cvt_e4m3x4(v[0], v[2], v[4], v[6]), cvt_e4m3x4(v[1], v[3], v[5], v[7]), a0, d0);
-        pairs(cvt_e4m3x4(v[8], v[10], v[12], v[14]), cvt_e4m3x4(v[9], v[11], v[13], v[15]), a1, d1);
+        for (int i = 1; i < 4; ++i) {
+            even[i] = add_f32x2(even[i - 1], step2);
+            odd[i] = add_f32x2(odd[i - 1], step2);
+        }
+        pairs(cvt_two(even[0], even[1]), cvt_two(odd[0], odd[1]), a0, d0);
+        pairs(cvt_two(even[2], even[3]), cvt_two(odd[2], odd[3]), a1, d1);
     }
     __device__ __forceinline__ void dequant8(uint32_t w, uint32_t& out0, uint32_t& out1) const {
         const uint32_t sel = w & 0x77777777u;
@@ -395,13 +395,14 @@ prepack_kernel(const uint8_t* __restrict__ codes, const uint16_t* __restrict__ g
         }
         if (bad) atomicOr(status_word, kStatusBadCode);
     } else {
-        // (u - z) s = ((15 - u) - (15 - z)) (-s)
+        // (u - z) s = ((15 - u) - (15 - z)) (-s); from 448 on every value that is not zero saturates
         if (sc & 0x8000u) {
             sc ^= 0x8000u;
             z = 15 - z;
 #pragma unroll
             for (int c = 0; c < 4; ++c) w[c] = make_uint4(~w[c].x, ~w[c].y, ~w[c].z, ~w[c].w);
         }
+        sc = sc > 0x43E0u && sc <= 0x7F80u ? 0x43E0u : sc;   // BF16 of 448
 #pragma unroll
         for (int c = 0; c < 4; ++c)
             w[c] = make_uint4(to_pair_word(w[c].x, z), to_pair_word(w[c].y, z), to_pair_word(w[c].z, z), to_pair_word(w[c].w, z));
