@@ -114,16 +114,6 @@ int w4a8_dequant_weight(const uint8_t* codes, const void* gscale_bf16, const uin
  * workspace of the largest size may serve all layers of a model) -- except a call during which a
  * bounded wait gave up (w4a8_query_device_status returns W4A8_ERR_TIMEOUT): zero-fill the
  * workspace again after that.  Calls that share a workspace must not overlap on the device.
- * Calls with M <= 16 on tiled weights place their worker CTAs at run time (at most one per SM and
- * launch, so that consecutive launches can share the SMs), unless a CTA has fewer than sixteen k-blocks to
- * walk or the layer is one of those that, given a workspace, go from global memory to registers (neither has
- * placement state).  The bookkeeping (1 KB, cleared by the
- * kernel) lives in the workspace when one of the full size is given -- nothing more to observe
- * than the rule above: calls that may overlap on the device need different workspaces; calls
- * issued one after the other on one stream may share one.  Without a workspace it is an entry of a
- * 64-entry table in the library image, handed out round-robin over all such calls of the process
- * (a captured call keeps the entry it drew at capture): then no more than 64 such launches may be
- * in flight on a device at a time, replays of graphs captured far apart included.
  */
 int w4a8_linear(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* weights,
                 const void* gscale_bf16, const uint8_t* gzero, int weight_format, const float* s_w,
@@ -139,7 +129,9 @@ size_t w4a8_linear_workspace_bytes(int64_t M, int64_t N, int64_t K, int weight_f
  * aligned) for weight_format W4A8_FMT_TILED or W4A8_FMT_TILED_SIGNMAG.  The dequantized weights
  * the linear layer sees are bit-identical to Eq. 10 on the canonical arrays.  If a code 0 is met
  * while writing W4A8_FMT_TILED_SIGNMAG, bit 1 of the device status word is raised
- * (w4a8_query_device_status) and the buffer must not be used.
+ * (w4a8_query_device_status) and the buffer must not be used.  A buffer is read by the library that wrote it: the
+ * order of bits inside it may change between versions, so what a program keeps in files is the canonical arrays.  (W4A8_FMT_TILED
+ * buffers of a version before codes were stored as pairs give NaN in every output.)
  */
 size_t w4a8_prepack_bytes(int64_t N, int64_t K, int weight_format);
 

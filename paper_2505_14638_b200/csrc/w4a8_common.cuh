@@ -52,15 +52,15 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 }
 
 // The expansion is bound by the integer pipe (a warp's instruction every other cycle: logic, shifts, byte permutes), so what
-// can is done beside it on the multipliers: shifts as multiplications, sums as multiply-adds.  The factors are read from
-// here because ptxas turns constants back into shifts and plain sums.
-__constant__ uint32_t kExpandOne = 1u;
-__constant__ uint32_t kExpandHigh = 0x0100u;   // two-way dot product: 0 * low half + 1 * high half
+// can is done beside it on the multipliers: shifts as multiplications, sums as multiply-adds.  The factors must not be known to
+// ptxas, which turns constants back into shifts and plain sums: they come from the block's z extent, 1 in every launch here, which
+// is read where a launch's parameters are.  (From __constant__ variables each launch waited half a microsecond for the first one.)
+__device__ __forceinline__ uint32_t expand_one() { return blockDim.z; }
 
-// Selector of the upper four nibbles (a byte permute reads the low half only).
+// Selector of the upper four nibbles (a byte permute reads the low half only): 0 * low half + 1 * high half.
 __device__ __forceinline__ uint32_t high_half(uint32_t w) {
     uint32_t d;
-    asm("dp2a.lo.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(kExpandHigh), "r"(0u));
+    asm("dp2a.lo.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(blockDim.z << 8), "r"(0u));
     return d;
 }
 
@@ -122,6 +122,7 @@ struct DequantLut {
     }
     // w holds eight codes, element i in bits [4i+3 : 4i].  out0 = E4M3 bytes of elements 0..3,
     // out1 = elements 4..7 (element order = byte order).
+    template <bool = false>
     __device__ __forceinline__ void dequant8(uint32_t w, uint32_t& out0, uint32_t& out1) const {
         uint32_t lo3 = w & 0x77777777u;                               // low three bits: entry within a half table
         uint32_t pick = ((w >> 1) & 0x44444444u) | 0x32103210u;      // bit 3 chooses the half table

@@ -12,7 +12,7 @@
 #include "w4a8_dpq_kernels.cuh"
 #include "w4a8_linear_chain.cuh"
 #include "w4a8_linear_direct.cuh"
-#include "w4a8_linear_splitn.cuh"
+#include "w4a8_linear_rows.cuh"
 #include "w4a8_linear_pair.cuh"
 #include "w4a8_linear_streamk.cuh"
 #include "w4a8_linear_umma.cuh"
@@ -215,7 +215,8 @@ static int sm_count() {
 
 constexpr int kNominalSMs = 148;  // for size queries made without a device
 
-constexpr int kSplitNMaxM = 128;  // token counts served by the split-N (decode) kernel
+constexpr int64_t kHostFewOutputs = 40000;   // outputs in host memory up to which the kernels for small layers write them
+constexpr int kRowsMaxM = 128;    // token counts served by linear_rows_kernel (and what runs beside it up to there)
 
 template <class Cfg>
 static int launch_streamk(const CUtensorMap& tx, const uint8_t* wpp, const float* s_x, const float* s_w,
@@ -262,136 +263,17 @@ static int launch_streamk(const CUtensorMap& tx, const uint8_t* wpp, const float
     return launch_status();
 }
 
-// Row partition and ring sizes of the split-N kernel for the current device.
-// Workspace of the split-N kernel when it cuts K, which it does at up to 16 tokens (bytes; room for any SM count up to kMaxSMs and,
-// from earlier versions, 128 tokens: the size that calls are refused or accepted by stays).
-// Layout: split-K counters (1 KB) and placement state of the launch (1 KB) at the end of the common
-// control area, partial tiles behind that area.
-constexpr size_t kSnCounterBytes = 1024;
-constexpr size_t kSnSchedBytes = 1024;
-static_assert(kSnCounterBytes == (size_t)kSchedWsOffset, "the kernel finds the placement state behind the counters");
-static_assert(kLinearCtlSplitN + kSnCounterBytes + kSnSchedBytes == kLinearCtlBytes, "split-N control data at the end of the common control area");
-constexpr size_t kSnWorkspaceBytes = kLinearCtlBytes + (size_t)kMaxSMs * 128 * 128 * sizeof(float);
+// Workspace of linear_rows_kernel when it cuts K, which it does at up to 16 tokens (bytes; room for any SM count up to kMaxSMs and,
+// from earlier versions, 128 tokens: the size that calls are refused or accepted by stays).  Layout: arrival counters (1 KB) in
+// the last 2 KB of the common control area, partial tiles behind that area.
+constexpr size_t kRowsCounterBytes = 1024;
+constexpr size_t kRowsWorkspaceBytes = kLinearCtlBytes + (size_t)kMaxSMs * 128 * 128 * sizeof(float);
+static_assert(kMaxSMs * sizeof(unsigned int) <= kRowsCounterBytes && kLinearCtlRows + kRowsCounterBytes <= kLinearCtlBytes,
+              "a counter per run of rows");
 
 // K is cut only when the caller gave the (zero-initialised) workspace for the partial sums.
-static bool sn_workspace_usable(const void* workspace, size_t bytes) {
-    return workspace != nullptr && bytes >= kSnWorkspaceBytes && aligned16(workspace);
-}
-
-template <class Cfg>
-static bool make_sn_plan(int64_t N, int64_t K, int sms, bool may_split_k, SnPlan* pl) {
-    const int64_t NU = N / 8;
-    const int64_t KB = K / 128;
-    int64_t P = sms < NU ? sms : NU;
-    int64_t per = (NU + 32 * P - 1) / (32 * P);  // ranges per CTA so that none exceeds 256 rows
-    pl->T = (int)(P * per);
-    pl->KSPLIT = 1;
-    // Few output channels (at most half as many 128-row blocks as SMs): ranges of whole 128-row
-    // blocks, and the K range cut in chunks so that every SM gets a tile.  A CTA's MMA and
-    // expansion work then covers 128 useful rows instead of a sliver, and its K walk is shorter;
-    // the price is a small fix-up through the workspace.
-    const int64_t blocks128 = (N + 127) / 128;
-    // (Up to 16 tokens: with more the partial sums are larger, and such layers take the cluster plan.)
-    if (Cfg::MT == 16 && may_split_k && blocks128 * 2 <= sms && KB >= 8) {
-        int64_t ks = sms / blocks128;
-        if (ks > KB / 4) ks = KB / 4;  // at least four k-blocks per chunk
-        if (ks > 1 && blocks128 <= (int64_t)(kSnCounterBytes / sizeof(unsigned int)) &&
-            blocks128 * ks <= kMaxSMs) {
-            pl->KSPLIT = (int)ks;
-            pl->T = (int)(blocks128 * ks);
-        }
-    }
-    const int64_t TR = pl->T / pl->KSPLIT;
-    const int rmax = (int)((NU + TR - 1) / TR) * 8;
-    pl->MBLK = rmax > 128 ? 2 : 1;
-    pl->KS = Cfg::kItems / pl->MBLK;
-    if ((int64_t)pl->KS > K / 128) pl->KS = 1;
-    pl->meta_off = pl->KS * rmax * kRowCodeBytes;
-    pl->wstage = (pl->KS * rmax * (kRowCodeBytes + Cfg::kMeta) + 127) / 128 * 128;
-    pl->xstage = pl->KS * Cfg::MT * 128;
-    const int fixed = Cfg::kBarBytes + Cfg::kOutBytes + 1024;
-    int s1 = (Cfg::kSmemBudget - fixed) / (pl->wstage + pl->xstage);
-    if (s1 > Cfg::kS1Max) s1 = Cfg::kS1Max;
-    if (s1 < Cfg::kS2 || s1 < Cfg::G) return false;  // the tensor-memory ring may not be deeper than the TMA ring, nor may there be more groups than slots
-    pl->S1 = s1;
-    pl->smem = s1 * (pl->wstage + pl->xstage) + fixed;
-    return true;
-}
-
-// Launches without a workspace draw their placement slot round-robin over ALL decode launches of
-// the process: one counter for every instantiation of the launcher (a counter per instantiation
-// gave two kernels of a chain, e.g. a gate/up and a down projection, the same slot while both were
-// in flight).  Launches with a workspace keep the state there and need no slot.
-static std::atomic<unsigned int> g_sched_seq{0};
-
-template <class Cfg>
-static int launch_splitn_planned(const CUtensorMap& tx, const uint8_t* wpp, const float* s_x, const float* s_w,
-                                 int sw_stride, void* y, int64_t ldy, int out_dtype, int M, int N, int K,
-                                 cudaStream_t st, void* workspace, bool ws_usable, const SnPlan& pl, int sms);
-
-template <int MT, int G, int FMT>
-static int launch_splitn_cfg(const CUtensorMap& tx, const uint8_t* wpp, const float* s_x, const float* s_w,
-                             int sw_stride, void* y, int64_t ldy, int out_dtype, int M, int N, int K, cudaStream_t st,
-                             void* workspace = nullptr, size_t workspace_bytes = 0) {
-    using Cfg = SnCfg<MT, G, FMT, false>;
-    const int sms = sm_count();
-    if (sms <= 0) return W4A8_ERR_CUDA;
-    SnPlan pl;
-    const bool ws_usable = sn_workspace_usable(workspace, workspace_bytes);
-    if (!make_sn_plan<Cfg>(N, K, sms, ws_usable, &pl)) return W4A8_ERR_BAD_SHAPE;
-    if constexpr (MT == 16) {
-        if (pl.KSPLIT > 1)
-            return launch_splitn_planned<SnCfg<MT, G, FMT, true>>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K,
-                                                                  st, workspace, ws_usable, pl, sms);
-    }
-    return launch_splitn_planned<Cfg>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K, st, workspace,
-                                      ws_usable, pl, sms);
-}
-
-template <class Cfg>
-static int launch_splitn_planned(const CUtensorMap& tx, const uint8_t* wpp, const float* s_x, const float* s_w,
-                                 int sw_stride, void* y, int64_t ldy, int out_dtype, int M, int N, int K,
-                                 cudaStream_t st, void* workspace, bool ws_usable, const SnPlan& pl, int sms) {
-    auto kern = linear_splitn_kernel<Cfg>;
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [&] {
-        attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBudget);
-    });
-    if (attr_err != cudaSuccess) return W4A8_ERR_CUDA;
-    unsigned int* status = status_word_ptr();
-    if (!status) return W4A8_ERR_CUDA;
-    const int P = pl.T < sms ? pl.T : sms;
-    SnPlan plan = pl;
-    plan.P = P;
-    plan.sched = -1;
-    unsigned grid = (unsigned)P;
-    if (Cfg::MT == 16 && sms <= kSchedMaxSMs && (K / 128) / pl.KSPLIT >= 16) {
-        // two CTAs of this variant fit on an SM: launch twice the workers and let the kernel keep
-        // one worker per SM (see the placement notes beside SchedSlot).  Not for short K walks
-        // (under 16 k-blocks per tile): there the extra microsecond at the start of a launch costs
-        // more than an occasional SM with two workers (o projection at M = 1: 8.4 against 6.6 us).
-        plan.sched = ws_usable ? kSchedInWorkspace
-                               : (int)(g_sched_seq.fetch_add(1, std::memory_order_relaxed) % (unsigned)kSchedSlots);
-        grid = 2u * (unsigned)P;
-    }
-    unsigned int* counters = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(workspace) + kLinearCtlSplitN);
-    float* partials = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + kLinearCtlBytes);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(Cfg::kThreads);
-    cfg.dynamicSmemBytes = (size_t)pl.smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K, plan,
-                                       counters, partials, status);
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    if (e != cudaSuccess) return W4A8_ERR_CUDA;
-    return launch_status();
+static bool rows_workspace_usable(const void* workspace, size_t bytes) {
+    return workspace != nullptr && bytes >= kRowsWorkspaceBytes && aligned16(workspace);
 }
 
 // Clusters of `size` CTAs (at most 8) of a kernel that the device holds at once, asked of the device once per kernel and size; -1
@@ -476,22 +358,32 @@ static int launch_pair(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, cons
     return launch_status();
 }
 
-// 17..128 tokens where the cluster plan does not run (more than half as many tiles of 128 channels as SMs): whole tiles of 128 channels x 64 or
-// 128 tokens of the persistent kernel instead of the split-N kernel, whose CTAs each pull all of X8 through their L2
-// port and expand rows that their MMAs then pad.  Split-N / this, us, weights not in L2, K = 1024, 2048, 4096, 8192:
-//   sign-magnitude     (32, 9600)    6.3 / 4.4   8.2 / 6.0    11.3 / 9.2    18.6 / 17.0
-//                      (32, 28672)   8.7 / 7.4   12.0 / 11.4  18.9 / 19.2   34.2 / 37.4
-//                      (64, 19200)   10.1 / 7.3  13.5 / 11.1  20.3 / 19.5   34.1 / 35.7
-//                      (128, 28672)  14.3 / 8.9  17.8 / 12.8  25.4 / 22.2   43.1 / 43.4
-//   generic            (24, 28672)   10.3 / 8.9  15.3 / 14.0  25.4 / 24.4   45.6 / 43.7
-//                      (128, 28672)  15.9 / 10.4 21.4 / 15.4  31.7 / 26.0   56.0 / 52.9
-// Sign-magnitude layers with a long K and more than one round of tiles stay, the more so the fewer the tokens.  Host to host
-// (outputs to pinned host memory) (24, 14336, 2048) 30.2 / 28.0, (128, 28672, 1024) 176 / 168.
-static bool whole_tiles_apply(int64_t M, int64_t N, int64_t K, int fmt, int sms) {
+// Up to 128 tokens: whole tiles of the persistent kernel, at most one per SM, where K is so short that start and end of a launch
+// count more than its main loop: its roles are fewer and set up faster than linear_rows_kernel's, nothing is exchanged, no cluster
+// has to be placed.  Time, quantization and linear layer back to back, weights not in L2, this / linear_rows_kernel / the other
+// candidate (up to sixteen tokens linear_direct_kernel, above K cut in clusters), us:
+//   M <= 8   (8064, 256) 4.0 / 4.4 / 4.2, (992, 640) 4.4 / 4.6 / -, (672, 1792) 6.0 / 7.0 / -, (8656, 2560) 7.9 / 8.5 / 8.9
+//   M <= 16  (4672, 896) 4.8 / 5.5 / 5.9, (5312, 1408) 5.4 / 7.2 / 6.5, (8048, 2176) 6.9 / 8.5 / 10.0, (1344, 3456) 9.3 / 7.4 / 7.6
+//   above    (57, 11776, 640) 5.3 / 5.8 / -, (126, 7360, 512) 5.6 / 6.2 / 9.6, (46, 7872, 1024) 5.4 / 5.7 / 7.1, (29, 800, 1920) 6.4 / 6.8 / 5.5
+// The limits follow 1000 shapes of 512..20000 channels; the kernel taken is 0.4 % slower than the fastest on average.  With more
+// tiles than half the SMs the rows of linear_rows_kernel fill all SMs as well: there K up to 512 (up to sixteen tokens), 1024
+// or 2048 (more than 32), this over that 0.95, 0.99, 0.97.
+// Outputs in host memory: always where there are more tiles than half the SMs and more than sixteen tokens; the bus takes its
+// stores better, (77, 28672, 4096) 119 us host to host against 128.  Up to sixteen tokens not for more than kHostFewOutputs, like
+// linear_direct_kernel.
+static bool whole_tiles_apply(int64_t M, int64_t N, int64_t K, int fmt, int sms, bool y_on_host) {
     const int64_t tiles = (N + 127) / 128;
-    if (M <= 16 || M > kSplitNMaxM) return false;
-    return fmt != kFmtTiledSignMag || tiles <= sms || K < (M <= 32 ? 3072 : 6144);
+    if (y_on_host && M <= 16 && M * N > kHostFewOutputs) return false;
+    if (2 * tiles > sms) return (tiles <= sms && K <= (M > 32 ? 2048 : (M > 16 ? 1024 : 512))) || (y_on_host && M > 16);
+    if (M > 16) return 100 * (K / 128) <= 800 + 12 * M;
+    return K <= (N < 1024 ? 2304 : (fmt == kFmtTiledSignMag ? 2944 : 2688));
 }
+
+// 17..128 tokens: whether cutting the tiles' K between the CTAs of clusters of `cl` pays for the exchange of the partial sums: the
+// k-blocks that a CTA is spared against what grows with the tokens.  Fitted to 400 shapes of up to 9472 channels (see whole_tiles_apply);
+// against linear_rows_kernel, us: (124, 7328, 512) 10.0 / 6.7, (112, 5600, 3584) 12.3 / 10.2, (20, 4096, 4096) 7.5 / 9.7, (20, 4096,
+// 14336) 12.6 / 24.9.
+static bool cluster_kcut_pays(int64_t M, int64_t K, int cl) { return 50 * (K / 128) * (cl - 1) >= cl * (120 + 7 * M); }
 
 // Few tiles (at most half as many 128-row tiles as SMs) and at most 128 tokens: CTAs per tile of the plan
 // that cuts K between the CTAs of a thread-block cluster (0: the plan does not apply).  Every CTA keeps
@@ -582,65 +474,30 @@ static int64_t make_direct_plan(int64_t N, int64_t K, int sms, DirPlan* plan) {
     return best;
 }
 
-// Layers at up to sixteen tokens for which the kernel above is the faster one: by and large those whose K the split-N
-// kernel would cut (see make_sn_plan), which costs it an exchange, up to a number of weights that this kernel's
-// expansion keeps up with (its FP8 fragments are converted to 16 bits for the MMA on the pipe that expands).  Time of
-// this kernel over that of the split-N kernel, activation quantization and linear layer back to back, weights not in L2,
-// sign-magnitude (generic) format; at M = 8 (1024, 1024) takes 7.5 us there and 4.3 here, (4096, 4096) 9.2 and 8.8:
-//   (N, K)          M = 4          M = 8          M = 9          M = 16
-//   (2048, 128)     0.96 (0.98)    1.05 (1.03)    1.05 (1.19)    1.17 (1.29)    K not cut
-//   (2048, 512)     0.91 (0.97)    1.04 (1.03)    1.13 (1.20)    1.25 (1.30)    K not cut
-//   (2048, 896)     0.81 (0.90)    0.91 (0.90)    1.01 (1.03)    1.10 (1.14)    K not cut
-//   (6144, 896)     0.93 (0.98)    0.97 (1.03)    1.08 (1.17)    1.19 (1.26)    K not cut
-//   (9472, 1536)    0.86 (0.94)    0.82 (0.91)    0.88 (0.98)    0.82 (0.89)
-//   (8192, 2048)    0.87 (0.91)    0.87 (0.91)    0.96 (1.01)    0.97 (1.00)
-//   (9472, 2048)    1.00 (1.06)    0.95 (1.01)    1.05           0.94
-//   (8192, 2560)    0.90 (0.95)    0.91 (0.94)    1.00           1.00
-//   (5120, 2560)    0.86 (0.94)    0.82 (0.88)    0.89 (0.97)    0.90 (0.96)
-//   (4096, 3072)    0.82 (0.91)    0.86 (0.93)    0.96 (1.02)    1.02 (1.08)
-//   (6144, 3072)    1.02 (1.13)    1.00 (1.09)    1.11           1.06
-//   (4096, 4096)    0.96 (0.99)    0.96 (1.02)    1.07 (1.13)    1.04 (1.13)
-//   (5120, 4096)    0.91 (0.88)    0.90 (0.88)    1.03           1.02
-//   (1552, 7168)    0.88 (0.96)    0.85 (0.96)    0.94 (1.04)    0.84 (0.89)
-//   (2048, 7168)    0.96 (1.04)    0.90 (1.00)    1.01 (1.08)    0.96 (1.03)
-//   (3072, 7168)    1.05 (1.09)    1.01 (1.06)    1.12           1.04
-//   (1552, 8192)    0.92 (1.02)    0.91 (0.98)    1.01 (1.11)    0.91 (0.97)
-//   (1296, 11008)   1.04 (1.17)    1.04 (1.11)    1.16 (1.27)
-//   (12288, 1024)   1.21 (1.30)    1.26 (1.28)    1.38 (1.46)    1.42 (1.46)    K not cut
-//   (12288, 1536)   1.33 (1.37)    1.43 (1.41)    1.61           1.64           K not cut
-//   (10240, 2048)   0.82 (0.89)    0.87 (0.95)    1.02           1.00           K not cut, candidates placed at run time
-//   (12288, 2048)   0.87 (1.00)    0.92 (1.05)    1.06           1.12           the same
-// M = 1: (2048, 512) 0.89 (0.93), (1024, 7168) 0.84 (0.90).  Canonical, against the kernel of one tile per CTA: M = 8
-// (1024, 1024) 0.46, (6144, 4096) 0.87, (12288, 2048) 0.81; M = 16 (6144, 4096) 0.98, (2048, 8192) 1.05; (1552, 14336) M = 4
-// 1.01, M = 8 1.05, M = 9 1.15; (4096, 6144) M = 12 1.06.  24 tokens: level at (1024, 1024), slower everywhere else.
-// Prepacked layers with a 96-row block for every SM keep the kernel that walks all of K in one chain of MMAs: a chain launch
-// gives the same bits there.
+// Layers at up to sixteen tokens for which the kernel above is the faster one: those of few weights, where its short start and
+// end count; its expansion does not keep up with larger ones (the FP8 fragments of its MMA are converted to 16 bits on the pipe that
+// expands), and a short K is better walked by one CTA per tile (whole_tiles_apply, with the same 1000 shapes).  Time, quantization
+// and linear layer back to back, weights not in L2, this kernel / whole tiles / linear_rows_kernel, us:
+//   M <= 8   (1616, 512) 4.1 / 4.1 / 4.5, (1104, 1408) 4.4 / 5.4 / 7.1, (2160, 3328) 5.2 / 9.0 / 6.9, (7488, 2048) 7.5 / 6.7 / 7.7,
+//            (5968, 3968) 8.8 / 9.3 / 8.1, (4960, 8192) 15.4 / 20.0 / 11.2
+//   M <= 16  (2752, 512) 5.4 / 4.1 / 4.7, (1072, 1920) 5.3 / 6.4 / 7.5, (3472, 1280) 6.1 / 5.2 / 6.9, (2352, 8064) 10.9 / 19.8 / 9.0
+// (Up to 2.2 million weights from nine tokens on: launched one by one such a layer is bound by the host's calls, of which the tensor map
+// of the other kernels takes 0.3 us: (16, 1024, 1024) 5.8 against 6.1 us; replayed from a graph it takes 5.3 against 4.8.)
+// Layers of more 128-channel tiles than half the SMs keep the kernels that walk all of K in one chain of MMAs: a chain launch gives
+// the same bits there, and this one is the slower by (14352, 512) 4.6 / 4.6 to (16640, 512) 6.3 / 4.9.
+// Canonical, against the kernel of one tile per CTA: M = 8 (1024, 1024) 0.46, (6144, 4096) 0.87, (12288, 2048) 0.81; M = 16 (6144,
+// 4096) 0.98, (2048, 8192) 1.05; (1552, 14336) M = 4 1.01, M = 8 1.05, M = 9 1.15; (4096, 6144) M = 12 1.06.  24 tokens: level at
+// (1024, 1024), slower everywhere else.
 static bool direct_applies(int64_t M, int64_t N, int64_t K, int fmt, int sms, DirPlan* plan) {
     if (M > 16 || N < 1024 || direct_smem(M, K, M <= 8 ? 1 : 2) > (size_t)kDirMaxSmem) return false;
-    if (make_direct_plan(N, K, sms, plan) > 2) return false;
-    const int64_t weights = N * K;
-    const bool sm = fmt == kFmtTiledSignMag, few = M <= 8;
-    if (fmt == kFmtCanonical) return weights <= (few || K <= 4096 || K > 8192 ? 26 : 16) * (int64_t)1000000 && (K <= 11008 || M <= 4);
-    const int64_t blocks = (N + 127) / 128;
-    int64_t most;   // million weights
-    if (K < 1024) {                       // the split-N kernel does not cut K
-        if (M <= 4 ? !(sm ? N <= 8192 : K >= 512 && N <= 4096) : !(few && K > 512 && N <= (sm ? 6144 : 4096))) return false;
-        most = 8;
-    } else if (2 * blocks > sms) {        // nor here
-        if (K < 2048 || M < 4 || !few || N >= (int64_t)96 * sms) return false;
-        most = sm ? 26 : 24;
-    } else if (M < 4) {
-        most = 8;
-    } else if (K <= 2048) {
-        most = sm ? 20 : (few ? 17 : 15);
-    } else if (sm) {
-        if (K <= 4096) most = few ? 26 : (K <= 2560 ? 21 : 13);
-        else most = K <= 7168 ? 15 : (K <= 8192 ? 13 : 0);
-    } else {
-        if (few && K <= 6144 && blocks * (sms / blocks) < sms * 7 / 8) most = 26;   // the cut leaves an eighth of the SMs idle
-        else most = K <= 7168 ? (few ? 13 : (K <= 3072 ? 12 : 14)) : 0;
-    }
-    return weights <= most * 1000000;
+    const int64_t rounds = make_direct_plan(N, K, sms, plan), weights = N * K;
+    const bool few = M <= 8;
+    if (fmt == kFmtCanonical)
+        return rounds <= 2 && weights <= (few || K <= 4096 || K > 8192 ? 26 : 16) * (int64_t)1000000 && (K <= 11008 || M <= 4);
+    if (2 * ((N + 127) / 128) > sms) return false;
+    const bool sm = fmt == kFmtTiledSignMag;
+    return few ? weights <= 8000 * K - (sm ? 2000000 : 3000000) && weights <= (sm ? 12000000 : 10000000)
+               : K >= 1024 && weights <= 8000000 && (weights <= 5000 * K - 5000000 || weights <= 2200000);
 }
 
 // Canonical weights, kernel chosen by the library: whether linear_umma_kernel runs, whose K cut needs the caller's
@@ -670,14 +527,92 @@ static int launch_direct(const uint8_t* x8, int64_t ldx8, const float* s_x, int6
 #undef W4A8_DIR
 }
 
+// Up to 128 tokens: the plan of linear_rows_kernel.  K is cut (may_cut: up to sixteen tokens, with a workspace) where the
+// channels make less than half as many runs of 128 rows as there are SMs.
+template <class Cfg>
+static void make_rows_plan(int64_t M, int64_t N, int64_t K, int sms, bool may_cut, RowsPlan* pl) {
+    const int64_t NU = N / 8, P = sms < NU ? sms : NU, blocks = (N + 127) / 128;
+    int64_t cut = 1, runs;
+    if (may_cut && blocks * 2 <= sms) {
+        cut = sms / blocks;
+        if (cut > K / 512) cut = K / 512;   // at least four k-blocks per part
+        if (cut < 1) cut = 1;
+    }
+    if (cut > 1) {
+        runs = sms / cut;
+        if (runs > NU) runs = NU;
+    } else {
+        runs = P * ((NU + 32 * P - 1) / (32 * P));   // none exceeds 256 rows
+    }
+    pl->cut = (int)cut;
+    pl->T = (int)(runs * cut);
+    pl->units = (int)(NU / runs);
+    pl->more = (int)(NU % runs);
+    const int rmax = (pl->units + (pl->more > 0)) * 8;
+    pl->RB = rmax > 128 ? 2 : 1;
+    pl->MN = (int)((M + 15) / 16) * 16;
+    const int acols = (pl->RB * pl->MN + 31) & ~31;
+    pl->S2 = (Cfg::kTmemCols - acols) / 64;
+    if (pl->S2 > Cfg::kS2Max) pl->S2 = Cfg::kS2Max;
+    pl->whalf = (rmax * (kRowCodeBytes + Cfg::kMeta) + 127) / 128 * 128;
+    const int ks = 2 / pl->RB, x = ks * pl->MN * 128, slot = ks * pl->whalf, room = Cfg::kSmemBudget - Cfg::kFixed;
+    while (pl->S2 > Cfg::G && room - pl->S2 * x < (pl->S2 + 2) * slot) --pl->S2;
+    pl->S1 = (room - pl->S2 * x) / slot;
+    if (pl->S1 > Cfg::kS1Max) pl->S1 = Cfg::kS1Max;
+    pl->smem = Cfg::kFixed + pl->S2 * x + pl->S1 * slot;
+}
+
+template <class Cfg>
+static int launch_rows(const uint8_t* x8, int64_t ldx8, const uint8_t* wpp, const float* s_x, const float* s_w, int sw_stride, void* y,
+                       int64_t ldy, int out_dtype, int M, int N, int K, void* workspace, bool may_cut, int sms, cudaStream_t st) {
+    RowsPlan plan;
+    make_rows_plan<Cfg>(M, N, K, sms, may_cut, &plan);
+    if (plan.S2 < Cfg::G || plan.S1 < plan.S2) return W4A8_ERR_BAD_SHAPE;   // (what the kernel's waits rely on; holds for every plan)
+    CUtensorMap tx;
+    if (!make_tmap_u8_2d(&tx, x8, (uint64_t)M, (uint64_t)K, (uint64_t)ldx8, 128, (uint32_t)plan.MN, CU_TENSOR_MAP_SWIZZLE_128B))
+        return W4A8_ERR_CUDA;
+    auto kern = linear_rows_kernel<Cfg>;
+    static std::once_flag once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(once, [&] {
+        attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBudget);
+    });
+    if (attr_err != cudaSuccess) return W4A8_ERR_CUDA;
+    unsigned int* status = status_word_ptr();
+    if (!status) return W4A8_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(plan.T < sms ? plan.T : sms));
+    cfg.blockDim = dim3(Cfg::kThreads);
+    cfg.dynamicSmemBytes = (size_t)plan.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    unsigned int* counters = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(workspace) + kLinearCtlRows);
+    float* partials = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + kLinearCtlBytes);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, M, N, K, plan, counters, partials, status);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    if (e != cudaSuccess) return W4A8_ERR_CUDA;
+    return launch_status();
+}
+
+// Up to sixteen tokens on layers of more 128-channel tiles than half the SMs, short K: CTAs of half an SM, so that the next launch's set up,
+// fetch and expand beside this one's.  Against the better of whole tiles and full-SM rows, 55 shapes: K up to 512 1.03 times the
+// time, to 896 0.95, to 1664 0.96, to 2304 1.02, to 3072 1.18; with fewer tiles slower throughout.
+static bool half_rows_apply(int64_t M, int64_t N, int64_t K, int sms) {
+    return M <= 16 && 2 * ((N + 127) / 128) > sms && K <= 1664;
+}
+
 static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* wpp,
                              int fmt, const float* s_w, int sw_stride, int64_t N, int64_t K, void* y, int64_t ldy,
                              int out_dtype, void* workspace, size_t workspace_bytes, cudaStream_t st, bool y_on_host) {
-    if (M <= 16 && sn_workspace_usable(workspace, workspace_bytes) && (!y_on_host || M * N <= 40000)) {
+    if (M <= 16 && rows_workspace_usable(workspace, workspace_bytes) && (!y_on_host || M * N <= kHostFewOutputs)) {
         // (linear_direct_kernel cuts K between the warps of a CTA.  Without a workspace K is never cut, which is how a
         // caller asks for the bits of a chain launch.  An output in host memory it writes in pieces of 32 bytes, which the
-        // bus takes more slowly than the split-N kernel's rows: host to host, us, split-N / this, (4, 8192, 2048) 15.6 / 14.8,
-        // (8, 4096, 3072) 17.1 / 16.8, (8, 6144, 2048) 15.9 / 17.2, (16, 6144, 2048) 19.1 / 24.1, (16, 8192, 1024) 19.3 / 24.0.)
+        // bus takes more slowly than rows: host to host, us, a kernel that writes rows / this, (4, 8192, 2048) 15.6 / 14.8, (8, 4096,
+        // 3072) 17.1 / 16.8, (8, 6144, 2048) 15.9 / 17.2, (16, 6144, 2048) 19.1 / 24.1, (16, 8192, 1024) 19.3 / 24.0.)
         const int rc = check_device();
         if (rc != W4A8_OK) return rc;
         const int sms_d = sm_count();
@@ -685,15 +620,14 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
         if (sms_d > 0 && direct_applies(M, N, K, fmt, sms_d, &plan))
             return launch_direct(x8, ldx8, s_x, M, wpp, nullptr, nullptr, fmt, s_w, sw_stride, N, K, y, ldy, out_dtype, plan, st);
     }
-    if (M > 16) {
-        // 17..128 tokens on a layer with few 128-row tiles: K cut between the CTAs of a cluster (measured, us,
-        // against the split-N kernel or the persistent kernel with its exchange through L2, whichever runs without this
-        // plan: (17, 6144, 4096) 8.0 / 12.8, (32, 4096, 4096) 7.3 / 10.0, (64, 2048, 4096) 6.9 / 12.9, (100, 512, 8192) 7.6 /
-        // 15.1, (128, 4096, 4096) 11.3 / 12.0, (128, 4096, 14336) 16.6 / 17.4, (128, 6144, 4096) 12.1 / 14.8).  Up to 16 tokens
-        // the kernels that overlap their set-up with the launch before are used: (8, 4096, 4096) 6.6.
+    const bool whole = M <= kRowsMaxM && whole_tiles_apply(M, N, K, fmt, sm_count(), y_on_host);
+    if (M > 16 && !whole) {
+        // 17..128 tokens on a layer with few 128-row tiles and a long K: K cut between the CTAs of a cluster (cluster_kcut_pays;
+        // us against the exchange through L2: (64, 2048, 4096) 6.9 / 12.9, (100, 512, 8192) 7.6 / 15.1).
         const int sms_c = sm_count();
         const int cl0 = sms_c > 0 ? cluster_kcut_ctas(M, N, K, sms_c) : 0;
         for (int cl = cl0; cl >= 2; --cl) {   // the largest cluster size of which all clusters are resident at once
+            if (!cluster_kcut_pays(M, K, cl)) break;
             int rc = check_device();
             if (rc != W4A8_OK) return rc;
             if (M <= 64)
@@ -711,28 +645,22 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
             if (rc != -1) return rc;
         }
     }
-    const int sms_w = M <= kSplitNMaxM ? sm_count() : 0;
-    const bool whole = whole_tiles_apply(M, N, K, fmt, sms_w);
-    if (M <= kSplitNMaxM && !whole) {
-        int rc = check_device();
+    if (M <= kRowsMaxM && !whole) {
+        const int rc = check_device();
         if (rc != W4A8_OK) return rc;
-        const int mt = M <= 16 ? 16 : (M <= 64 ? 64 : 128);
-        CUtensorMap tx;
-        if (!make_tmap_u8_2d(&tx, x8, (uint64_t)M, (uint64_t)K, (uint64_t)ldx8, 128, (uint32_t)mt,
-                             CU_TENSOR_MAP_SWIZZLE_128B))
-            return W4A8_ERR_CUDA;
-        const int Mi = (int)M, Ni = (int)N, Ki = (int)K;
-        if (mt == 16)
-            return fmt == kFmtTiledSignMag
-                       ? launch_splitn_cfg<16, 2, kFmtTiledSignMag>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi, Ni,
-                                                                    Ki, st, workspace, workspace_bytes)
-                       : launch_splitn_cfg<16, 2, kFmtTiled>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi, Ni, Ki, st,
-                                                             workspace, workspace_bytes);
-        // (more than 16 tokens: sign-magnitude weights only, see whole_tiles_apply)
-        return mt == 64 ? launch_splitn_cfg<64, 4, kFmtTiledSignMag>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi, Ni,
-                                                                     Ki, st)
-                        : launch_splitn_cfg<128, 4, kFmtTiledSignMag>(tx, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, Mi, Ni,
-                                                                      Ki, st);
+        const int sms_r = sm_count();
+        const bool may_cut = M <= 16 && rows_workspace_usable(workspace, workspace_bytes);
+        const bool half = half_rows_apply(M, N, K, sms_r);
+#define W4A8_ROWS(...)                                                                                                     \
+    return launch_rows<RowsCfg<__VA_ARGS__>>(x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, \
+                                             workspace, may_cut, sms_r, st)
+        if (fmt == kFmtTiledSignMag) {
+            if (half) W4A8_ROWS(kFmtTiledSignMag, true);
+            W4A8_ROWS(kFmtTiledSignMag);
+        }
+        if (half) W4A8_ROWS(kFmtTiled, true);
+        W4A8_ROWS(kFmtTiled);
+#undef W4A8_ROWS
     }
     if (!whole) {
         if (reinterpret_cast<uintptr_t>(workspace) & 15u) return W4A8_ERR_BAD_ALIGNMENT;
@@ -1440,7 +1368,7 @@ size_t w4a8_linear_workspace_bytes(int64_t M, int64_t N, int64_t K, int weight_f
     if (M <= 0 || N <= 0 || K <= 0 || K % kGroup != 0) return 0;
     if (weight_format == kFmtCanonical) return w4a8_linear_ex_workspace_bytes(M, N, K, W4A8_ALGO_AUTO, 0);
     if (weight_format != kFmtTiled && weight_format != kFmtTiledSignMag) return 0;
-    if (M <= 64) return kSnWorkspaceBytes;  // used at up to 16 tokens, when the layer has few output channels and K is cut
+    if (M <= 64) return kRowsWorkspaceBytes;  // used at up to 16 tokens, when the layer has few output channels and K is cut
     return kSkWorkspaceBytes;   // (65..128 tokens use none of it)
 }
 
@@ -1799,7 +1727,7 @@ int w4a8_forward_host(const void* x_host_bf16, int64_t M, const uint8_t* weights
     // result to, the host buffers themselves (they are mapped into the device's address space), which
     // moves the same bytes over the bus without two copy-engine operations and their hand-overs to
     // and from the compute engine (about 20 of the 37 us such a call took on the device).
-    if (M <= kSplitNMaxM) {
+    if (M <= kRowsMaxM) {
         const void* xh = host_buffer_as_device_pointer(x_host_bf16);
         void* yh = const_cast<void*>(host_buffer_as_device_pointer(y_host_bf16));
         if (xh && yh && aligned16(xh) && aligned16(yh)) {

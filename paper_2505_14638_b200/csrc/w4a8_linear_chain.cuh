@@ -31,7 +31,7 @@
 // a dependent chain waits for it.  Every CTA expands the same number of weights within one item,
 // whatever N is.
 //
-// Data path of one (k-block, 96-row block) item: as in the split-N kernel --
+// Data path of one (k-block, 96-row block) item: as in linear_rows_kernel --
 //   HBM --bulk copy--> shared memory (INT4 codes + group scales [+ zero-points])
 //       --one thread per row: look-up-table expansion to E4M3 (Eq. 10)--> tensor memory (A operand)
 //       --tcgen05.mma kind::f8f6f4, B = FP8 activation tile from shared memory--> accumulator.

@@ -513,11 +513,11 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][K],
             }
             if constexpr (Cfg::TS) {
                 ptx::tc_fence_after_sync();
-                expand_row_to_tmem<Cfg::FMT>(now, m, tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(256 + 32 * s));
+                expand_row_to_tmem<Cfg::FMT, true>(now, m, tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(256 + 32 * s));
                 ptx::tmem_st_wait();
                 ptx::tc_fence_before_sync();
             } else {
-                expand_row_to_smem<Cfg::FMT>(now, m, r, stage_w8(s) + (uint32_t)r * 128u);
+                expand_row_to_smem<Cfg::FMT, true>(now, m, r, stage_w8(s) + (uint32_t)r * 128u);
                 ptx::fence_proxy_async_smem();
             }
             __syncwarp();

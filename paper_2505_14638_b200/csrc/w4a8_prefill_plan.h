@@ -16,15 +16,15 @@ namespace w4a8 {
 constexpr int kMaxSMs = 160;  // upper bound used to size workspaces without touching a device
 
 // Layout of every w4a8_linear workspace, whatever kernel and shape use it: a control area of fixed
-// size at the start (tile counters of the persistent kernel; K-cut counters and placement state
-// of the split-N kernel), which every launch leaves zero-filled, and behind it the data (partial
+// size at the start (tile counters of the persistent kernel; K-cut counters of
+// linear_rows_kernel), which every launch leaves zero-filled, and behind it the data (partial
 // sums), which may be left in any state.  With the control area at a shape-dependent size, one
 // call's left-over partial sums could sit where the next call -- another layer, another kernel
 // -- expects zeroed counters; callers do share one workspace between the layers of a model.
 constexpr size_t kLinearCtlBytes = 65536;
-// The split-N kernel's 2 KB (K-cut counters, placement state -- whose generation word stays non-zero
-// by design) sit at the END of the control area, the persistent kernel's tile counters at its start.
-constexpr size_t kLinearCtlSplitN = kLinearCtlBytes - 2048;
+// The K-cut counters of linear_rows_kernel sit in the last 2 KB of the control area, the persistent kernel's tile counters at
+// its start.
+constexpr size_t kLinearCtlRows = kLinearCtlBytes - 2048;
 
 // What w4a8_linear_workspace_bytes asks for and w4a8_linear requires for more than 128 tokens on prepacked weights, whatever
 // arrangement runs (most use none of it): a bound on what the persistent kernel ever used, for any SM count up to kMaxSMs.  It

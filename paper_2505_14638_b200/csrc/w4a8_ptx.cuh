@@ -113,7 +113,7 @@ __device__ __forceinline__ void griddep_launch_dependents() {
 // A wait may be for something that only follows the kernels this one depends on, and the time they take must
 // not count: after kWaitAlone tries (some microseconds at least: before the dependency there is work to
 // overlap) it is continued behind them, and the limit counts from there.  Waiting for earlier kernels ahead of
-// every such wait instead made the split-N kernel on layers whose K it cuts 1.6 % slower.
+// every such wait instead cost a decode kernel on layers whose K it cut 1.6 %.
 constexpr uint32_t kWaitAlone = 256u;   // a multiple of 64
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
                                           unsigned int* status_word) {

@@ -51,6 +51,8 @@ __host__ __device__ constexpr uint32_t row_offset(int fmt, int row) {
 // symmetric, so nearest_E4M3(-d s) and nearest_E4M3(d s) differ in that bit only).
 // Eight weights take 5 instructions of the integer pipe and 2 of the multipliers: 10.3 cycles of a sub-partition, against
 // 12.1 with the shift on the integer pipe (registers to registers, four warps, one more multiply-add in both).
+// PLAIN: shifts and sums where they belong, for kernels that the power cap bounds and not the integer pipe: CTA pairs take (8192,
+// 28672, 8192) 1500 us so and 1514 the other way, with zero-points 1567 and 1572.
 struct SignMagLut {
     uint32_t t0, t1;
     __device__ __forceinline__ void build(float s) {
@@ -60,10 +62,11 @@ struct SignMagLut {
     __device__ __forceinline__ void build_meta(uint32_t meta) { build(bf16_bits_to_float(meta & 0xFFFFu)); }
     // Word layout: nibble i (i = 0..3) = magnitude of element i, nibble 4+i = magnitude of
     // element 4+i; sign of element i in bit 8i+7, sign of element 4+i in bit 8i+3.
+    template <bool PLAIN = false>
     __device__ __forceinline__ void dequant8(uint32_t w, uint32_t& out0, uint32_t& out1) const {
         const uint32_t sel = w & 0x77777777u;
         out0 = prmt(t0, t1, sel) ^ (w & 0x80808080u);
-        out1 = prmt(t0, t1, high_half(sel)) ^ ((w << 4) & 0x80808080u);
+        out1 = prmt(t0, t1, PLAIN ? sel >> 16 : high_half(sel)) ^ ((w << 4) & 0x80808080u);
     }
 };
 
@@ -107,10 +110,16 @@ struct PairLut {
         pairs(cvt_two(even[0], even[1]), cvt_two(odd[0], odd[1]), a0, d0);
         pairs(cvt_two(even[2], even[3]), cvt_two(odd[2], odd[3]), a1, d1);
     }
+    template <bool PLAIN = false>
     __device__ __forceinline__ void dequant8(uint32_t w, uint32_t& out0, uint32_t& out1) const {
         const uint32_t sel = w & 0x77777777u;
-        out0 = prmt(a0, a1, sel) * kExpandOne + prmt(d0, d1, w);
-        out1 = prmt(a0, a1, high_half(sel)) * kExpandOne + prmt(d0, d1, high_half(w));
+        if constexpr (PLAIN) {
+            out0 = prmt(a0, a1, sel) + prmt(d0, d1, w);
+            out1 = prmt(a0, a1, sel >> 16) + prmt(d0, d1, w >> 16);
+            return;
+        }
+        out0 = prmt(a0, a1, sel) * expand_one() + prmt(d0, d1, w);
+        out1 = prmt(a0, a1, high_half(sel)) * expand_one() + prmt(d0, d1, high_half(w));
     }
 };
 
@@ -171,7 +180,7 @@ __device__ __forceinline__ uint32_t load_meta_word(uint32_t meta, int fmt) {
 // tiled_row_offset(row)), `meta` = shared address of its meta entry, `row` = row index within
 // the destination tile, `dst` = shared address of the destination row.  (expand_row_to_smem: codes and meta word are in
 // registers already.)
-template <int FMT>
+template <int FMT, bool PLAIN = false>
 __device__ __forceinline__ void expand_row_to_smem(const uint32_t (&pk)[16], uint32_t mbits, int row, uint32_t dst) {
     const uint32_t sw128 = (uint32_t)(row & 7);
     typename LutOf<FMT>::type lut;
@@ -179,8 +188,8 @@ __device__ __forceinline__ void expand_row_to_smem(const uint32_t (&pk)[16], uin
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
         uint32_t o0, o1, o2, o3;
-        lut.dequant8(pk[2 * c], o0, o1);
-        lut.dequant8(pk[2 * c + 1], o2, o3);
+        lut.template dequant8<PLAIN>(pk[2 * c], o0, o1);
+        lut.template dequant8<PLAIN>(pk[2 * c + 1], o2, o3);
         asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (((uint32_t)c ^ sw128) << 4)), "r"(o0),
                      "r"(o1), "r"(o2), "r"(o3)
                      : "memory");
@@ -262,7 +271,7 @@ __device__ __forceinline__ void dequant_row_to_smem_bf16(uint32_t src, uint32_t 
 // Warp-collective: every lane of the warp must call it with a readable row (a lane without a
 // row of its own repeats another one; its tensor-memory lane is then never read out).
 // (expand_row_to_tmem: codes and meta word are in registers already.)
-template <int FMT>
+template <int FMT, bool PLAIN = false>
 __device__ __forceinline__ void expand_row_to_tmem(const uint32_t (&pk)[16], uint32_t mbits, uint32_t taddr) {
     typename LutOf<FMT>::type lut;
     lut.build_meta(mbits);
@@ -270,7 +279,7 @@ __device__ __forceinline__ void expand_row_to_tmem(const uint32_t (&pk)[16], uin
     for (int h = 0; h < 2; ++h) {
         uint32_t out[16];
 #pragma unroll
-        for (int w = 0; w < 8; ++w) lut.dequant8(pk[8 * h + w], out[2 * w], out[2 * w + 1]);
+        for (int w = 0; w < 8; ++w) lut.template dequant8<PLAIN>(pk[8 * h + w], out[2 * w], out[2 * w + 1]);
         ptx::tmem_st_32x32b_x16(taddr + 16u * h, out);
     }
 }

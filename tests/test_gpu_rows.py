@@ -1,0 +1,71 @@
+"""GPU: up to 128 tokens on layers whose rows are dealt out to the SMs in contiguous runs (linear_rows_kernel): one and two blocks
+of 128 rows per run, more runs than SMs, an odd number of k-blocks, K cut through the workspace, CTAs of half an SM, rows of Y that
+16-byte stores do not fit.
+
+Tolerance: FP32 sums of K exact products against float64, 4 K 2^-24 of the root of the summed squares."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_utils import Guarded, bf16_dev
+from paper_2505_14638_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _layer(M, N, K, asym):
+    W = torch.from_numpy(inputs.make_weight(N, K, 0.02, seed=M + N + K)).cuda()
+    codes, gs, gz, sw = binding.quantize_weight_rtn(W, symmetric=not asym, per_channel=asym)
+    w64 = binding.dequant_weight(codes, gs, gz).view(torch.float8_e4m3fn).double()
+    x8, s_x = binding.quantize_act(bf16_dev(inputs.make_activation(M, K, M + K, 0.01, 20.0)))
+    x64 = x8.view(torch.float8_e4m3fn).double()
+    scale = s_x.double()[:, None] * (sw.double() if sw.numel() > 1 else sw.double().reshape(1))[None, :]
+    ref, mag = (x64 @ w64.t()) * scale, (x64.square() @ w64.square().t()).sqrt() * scale
+    return x8, s_x, binding.prepack_weight(codes, gs, gz, sw), ref, mag
+
+
+@pytest.mark.parametrize("asym", [False, True])
+@pytest.mark.parametrize("M,N,K", [
+    (1, 18944, 2176), (16, 18960, 2304), (8, 37888, 1792), (3, 37904, 1920),      # 128 / 136 / 256 rows a run, two runs a CTA
+    (17, 9488, 4224), (64, 19216, 2176), (65, 18944, 2304), (128, 28688, 2176), (100, 37904, 2304),
+    (128, 9472, 2944), (40, 8720, 2176),                                          # few tiles, K not cut
+    (16, 1552, 14336), (9, 1024, 8320), (1, 4096, 5760), (12, 9472, 3456), (2, 128, 4096), (4, 16, 4224),   # K cut
+    (1, 9488, 640), (16, 18960, 1408), (5, 37904, 896)])                          # half an SM
+def test_rows_in_runs(M, N, K, asym):
+    x8, s_x, tw, ref, mag = _layer(M, N, K, asym)
+    ws = binding.new_workspace(M, N, K, tw.fmt, "cuda")
+    outs = []
+    for rep in range(2):
+        y = Guarded((M, N), torch.float32, 777.0)
+        binding.linear_tiled(x8, s_x, tw, out_dtype=binding.OUT_FP32, out=y.t, workspace=ws)
+        y.check()
+        outs.append(y.t)
+        assert not bool(ws[:65536].any())          # counters left at zero
+    assert binding.query_device_status() == 0
+    assert bool(((outs[0].double() - ref).abs() <= 4.0 * K * 2.0 ** -24 * mag + 1e-30).all())
+    assert torch.equal(outs[0], outs[1])
+    yb = binding.linear_tiled(x8, s_x, tw, workspace=ws)
+    assert torch.equal(yb, outs[0].to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("M,N,K", [(5, 18944, 2176), (40, 28688, 2304), (16, 1552, 14336), (7, 18960, 896)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_rows_of_y_that_wide_stores_do_not_fit(M, N, K, dtype):
+    x8, s_x, tw, ref, _ = _layer(M, N, K, True)
+    ws = binding.new_workspace(M, N, K, tw.fmt, "cuda")
+    out_dtype = binding.OUT_FP32 if dtype == torch.float32 else binding.OUT_BF16
+    want = binding.linear_tiled(x8, s_x, tw, out_dtype=out_dtype, workspace=ws)
+    wide = Guarded((M, N + 3), dtype, 7.0)
+    binding.linear_tiled(x8, s_x, tw, out_dtype=out_dtype, out=wide.t[:, :N], workspace=ws)
+    wide.check()
+    assert torch.equal(wide.t[:, :N], want) and bool((wide.t[:, N:] == 7.0).all())
+
+
+@pytest.mark.parametrize("M,N,K", [(4, 1552, 8320), (16, 4096, 4096), (3, 18960, 2176)])
+def test_without_a_workspace_k_is_not_cut(M, N, K):
+    # the bits of one chain of sums over K, which is what a chain launch computes where it does not cut K
+    x8, s_x, tw, ref, mag = _layer(M, N, K, False)
+    tiny = torch.zeros(16, dtype=torch.uint8, device="cuda")
+    y = [binding.linear_tiled(x8, s_x, tw, out_dtype=binding.OUT_FP32, workspace=tiny) for _ in range(3)]
+    assert torch.equal(y[0], y[1]) and torch.equal(y[0], y[2])
+    assert bool(((y[0].double() - ref).abs() <= 4.0 * K * 2.0 ** -24 * mag + 1e-30).all())
