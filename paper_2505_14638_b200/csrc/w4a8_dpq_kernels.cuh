@@ -5,11 +5,11 @@
 // The rows of W are independent; the columns of a row are quantized one after the other, each
 // sending its scaled error e to the columns on its right (Eq. 12): w_v <- fma(-e, U_qv, w_v),
 // U = upper Cholesky factor of the inverse Hessian in processing order.  Work is cut the way
-// GPTQ cuts it, in blocks of one group (128 columns), one launch of dpq_step_kernel per block: its
-// first CTAs bring the block's columns up to date and quantize them (group scale / zero-point,
-// Eq. 8, optional search; the 128 columns in sequence), the others apply the errors of the block
-// before to all later columns, q ascending -- the same chain of fused multiply-adds, in the same
-// order, that the column-by-column algorithm performs for each element.
+// GPTQ cuts it, in blocks of one group (128 columns).  Tasks of two kinds: 32 rows of a block are brought up to
+// date and quantized (group scale / zero-point, Eq. 8, optional search; the 128 columns in sequence); the errors
+// of a block or two are applied to 128 rows of a later column block, q ascending -- the same chain of fused
+// multiply-adds, in the same order, that the column-by-column algorithm performs for each element.  One persistent
+// launch (dpq_kernel) takes the tasks in an order in which each follows those it waits for.
 // Every floating-point step that decides an integer is one explicitly rounded fp32 operation
 // (__fmul_rn, __fmaf_rn ...: never contracted; quotients correctly rounded), and the search compares exact integer
 // sums, so the codes do not depend on how the work is spread over threads.
@@ -19,6 +19,7 @@
 #include <cuda_fp16.h>
 
 #include "w4a8_common.cuh"
+#include "w4a8_dpq_plan.h"
 #include "w4a8_ptx.cuh"
 #include "w4a8_simple_kernels.cuh"
 
@@ -57,14 +58,25 @@ gar_order_kernel(const int32_t* __restrict__ within, const float* __restrict__ g
     perm[(int64_t)rank * 128 + threadIdx.x] = within[(int64_t)g * 128 + threadIdx.x];
 }
 
-// work[n][p] = W[n][perm[p]]: the rows in processing order.
+// work[n][p] = W[n][perm[p]]: the rows in processing order; the marks of dpq_kernel (see DpqMarks); and, once the kernel before has found
+// the largest magnitudes, Eq. 6.
 __global__ void __launch_bounds__(256)
 dpq_gather_kernel(const float* __restrict__ W, const int32_t* __restrict__ perm, int64_t N, int64_t K,
-                  float* __restrict__ work) {
+                  float* __restrict__ work, uint8_t* __restrict__ codes, uint16_t* __restrict__ gscale, float* s_w, int64_t scales) {
+    ptx::griddep_launch_dependents();
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= N * K) return;
     const int64_t n = i / K, p = i - n * K;
     work[i] = W[n * K + (perm ? perm[p] : (int32_t)p)];
+    if (n % 32 == 0 && (p & 127) == 0) {   // (the first row's hold control words too)
+        uint4* c = reinterpret_cast<uint4*>(codes + n * (K >> 1) + (p >> 1));
+        c[0] = c[3] = make_uint4(0u, 0u, 0u, 0u);
+        gscale[n * (K >> 7) + (p >> 7)] = 0xFFFFu;
+    }
+    if (i < scales) {
+        ptx::griddep_wait();
+        amax_to_scale(s_w + i);
+    }
 }
 
 // ---- Eq. 8 / Eq. 9 / Eq. 10 on one FP8-valued weight ------------------------------------------
@@ -176,25 +188,67 @@ __device__ __forceinline__ long long row_sum_ll(long long v) {
     return v;
 }
 
-// Step b of the quantizer, one launch: the first CTAs quantize block b (processing positions
-// [128 b, 128 b + 128), 32 rows per CTA), after the errors of block b - 1; the others apply the errors of earlier blocks to
-// the columns to the right.  The two touch different columns, so the serial chain of a block (some ten
-// microseconds) runs beside the contraction that fills the chip.
-// The errors of two blocks 2 m, 2 m + 1 are applied together: a tile's weights are read and written, and its
-// CTA started, once per 256 values of q instead of once per 128.  Steps:
-//   2 m + 2: both blocks' errors to the first part of the columns behind block 2 m + 2 (`far`), block 2 m + 3 among them;
-//   2 m + 3: the same for the rest, and (`near`) block 2 m + 2's errors to block 2 m + 4, whose own step then adds those
-//            of block 2 m + 3.
-// Every column sees the errors in ascending order.  (Few tiles in a step: one block's errors at a time, all of them `near`; the
-// launch decides, see there.)  Measured, us per layer, one block at a time / a block kernel (57 us: IEEE divisions, half a warp
-// per row) followed by a trailing kernel (scalar FMAs, 8 x 8 per thread): (N, K) = (256, 1024) 221 / 479, (256, 4096) 948 / 2109,
-// (4096, 4096) 2288 / 3525, (4096, 14336) 22264 / 28550.
-struct DpqTrail {
-    int errors;   // first block whose errors are applied
-    int blocks;   // how many (1 or 2)
-    int first;    // first column block
-    int count;    // column blocks
+// Progress is marked in the outputs, where these are not written yet, so that a call needs no memory beside its work array:
+//   * gscale of the first of 32 rows and a block: 0xFFFF until the block's errors for those rows are in place (no scale has these
+//     bits: a NaN is rounded to 0x7FFF);
+//   * the last word of that row's codes of a column block: how many blocks' errors its 32 rows have taken (of no use, and
+//     overwritten with codes, once the block itself is done);
+//   * the word before it: not 0 once the block's first 96 columns are done, whose errors the next block's task can take
+//     beside the rest of the chain (and of no use when the block is done);
+//   * the first words of the first row's codes of the last block: tickets handed out, CTAs that have left, abort.  What belongs
+//     there waits in the work array until the last CTA leaves.
+struct DpqMarks {
+    uint8_t* codes;
+    uint16_t* gscale;
+    const int32_t* perm;
+    int64_t K;
+    __device__ __forceinline__ int64_t group(int b) const { return perm ? (int64_t)(__ldg(perm + (int64_t)b * 128) >> 7) : (int64_t)b; }
+    __device__ __forceinline__ uint16_t* done(int64_t rows32, int b) const { return gscale + rows32 * 32 * (K >> 7) + group(b); }
+    __device__ __forceinline__ unsigned int* applied(int64_t rows32, int c) const {
+        return reinterpret_cast<unsigned int*>(codes + rows32 * 32 * (K >> 1) + group(c) * 64 + 60);
+    }
+    __device__ __forceinline__ unsigned int* early(int64_t rows32, int b) const { return applied(rows32, b) - 1; }
+    __device__ __forceinline__ unsigned int* control() const { return reinterpret_cast<unsigned int*>(codes + group((int)(K >> 7) - 1) * 64); }
 };
+struct DpqWait {   // bounded polls by single threads
+    unsigned int* control;
+    unsigned int* status_word;
+    template <class Test>
+    __device__ __forceinline__ bool until(Test test) const {
+        uint64_t t0 = 0;
+        uint32_t spins = 0;
+        while (!test()) {
+            if (spins > 32u) __nanosleep(64);
+            if ((++spins & 15u) == 0u) {
+                if (*reinterpret_cast<volatile unsigned int*>(control + 2)) return false;
+                const uint64_t now = ptx::globaltimer_ns();
+                if (t0 == 0) {
+                    t0 = now;
+                } else if (now - t0 > ptx::kWaitLimitNs) {
+                    atomicExch(control + 2, 1u);
+                    atomicOr(status_word, kStatusTimeout);
+                    return false;
+                }
+            }
+        }
+        return true;
+    }
+};
+// A copy that is still on its way when a CTA gives up.
+__device__ __forceinline__ void dpq_land(uint32_t bar, uint32_t parity) {
+    const uint64_t t0 = ptx::globaltimer_ns();
+    while (!ptx::mbar_try_wait(bar, parity) && ptx::globaltimer_ns() - t0 < ptx::kWaitLimitNs / 20) {
+    }
+}
+struct DpqMaps {
+    CUtensorMap u;        // U [K][K], box 128 x 32 (only used where U is 16-byte aligned)
+    CUtensorMap errors;   // the work array as [N / 4][4][K], box 128 x 1 x 32: where errors are kept, see dpq_load_errors
+};
+__device__ __forceinline__ uint16_t dpq_ld_acquire_u16(const uint16_t* p) {
+    uint16_t v;
+    asm volatile("ld.acquire.gpu.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
+    return v;
+}
 constexpr int kDpqThreads = 256;
 constexpr int kDpqRowsPerCta = 32;      // eight lanes per row
 constexpr int kDpqChunk = 32;           // values of q per stage
@@ -212,10 +266,11 @@ struct DpqSmem {
     static constexpr int kLut = kPanel;
     static constexpr int kLutU = kLut + kDpqRowsPerCta * kLutPitch * 4;
     static_assert(kLutU + kDpqRowsPerCta * 256 <= kCodes, "tables");
-    // trailing CTAs
-    static constexpr int kTrailU = 0;                              // 2 x [32][128]
-    static constexpr int kTrailErr = 2 * kDpqChunk * 128 * 4;      // 2 x [32][128 rows]
-    static constexpr int kTrailBytes = 2 * kTrailErr;
+    // applications: a stage is 32 q of U [32][128] and of the errors [32 groups of four rows][32 q][4]
+    static constexpr int kStages = 3;
+    static constexpr int kStageU = kDpqChunk * 128 * 4;
+    static constexpr int kStage = 2 * kStageU;
+    static constexpr int kTrailBytes = kStages * kStage;
     static constexpr int kBytes = kBlockBytes > kTrailBytes ? kBlockBytes : kTrailBytes;
     static_assert(2 * (kBytes + 1024) <= 228 * 1024, "two CTAs per SM");
 };
@@ -240,7 +295,7 @@ __device__ __forceinline__ void dpq_load_errors(float* e_s, uint32_t e_addr, con
             dpq_copy16(e_addr + (uint32_t)at * 4u, work + (n + c) * K + p + 4 * q, true);
         } else {
 #pragma unroll
-            for (int r = 0; r < 4; ++r) e_s[at + r] = n + r < N ? work[(n + r) * K + p + c * kDpqChunk + q] : 0.0f;
+            for (int r = 0; r < 4; ++r) e_s[at + r] = n + r < N ? __ldcg(work + (n + r) * K + p + c * kDpqChunk + q) : 0.0f;
         }
     }
 }
@@ -252,37 +307,74 @@ __device__ __forceinline__ void dpq_load_errors(float* e_s, uint32_t e_addr, con
 // (five 16-byte loads, eight 128-byte passes), half of what an 8 x 8 tile per thread takes, whose lanes read the
 // same words from different quarters of the warp; the operands of the next q are fetched ahead (waiting for them
 // was the largest stall with four warps per scheduler).  Packed pairs of rows: the pipe takes a packed FMA every other
-// cycle, which leaves issue slots for the loads (scalar: 23.7 ms against 21.9 for (4096, 14336)); 19 T FMA/s in all,
-// of the 28-31 T that a loop of FMAs alone reaches.  Errors and rows of U come in double-buffered chunks of 32 q.
-__device__ __forceinline__ void dpq_trailing_tile(uint8_t* sm, uint32_t sm_addr, float* __restrict__ work,
-                                                  const float* __restrict__ U, int64_t N, int64_t K, int64_t pprev,
-                                                  int blocks, int64_t v0, int64_t n0, bool uvec) {
+// cycle, which leaves issue slots for the loads; this loop on its own runs at 30 T FMA/s (16 x 8 per thread and one CTA per
+// SM: 32; operands that are repeated in shared memory instead of registers: 25-27).  Errors and rows of U come by tile loads,
+// 32 q a stage, two stages ahead.
+__device__ __forceinline__ bool dpq_trailing_tile(uint8_t* sm, uint32_t sm_addr, float* work, const float* __restrict__ U,
+                                                  int64_t N, int64_t K, int e0, int blocks, int col, int64_t n0, bool uvec,
+                                                  const DpqMarks& marks, const DpqWait& wait, const DpqMaps& maps, uint32_t bars,
+                                                  volatile uint32_t* abort_s, uint32_t& ring) {
+    const int64_t pprev = (int64_t)e0 * 128, v0 = (int64_t)col * 128;
     constexpr int kPerBlock = 128 / kDpqChunk;
     const int chunks = blocks * kPerBlock;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const float* usrc = U + (pprev + (tid >> 5)) * K + v0 + 4 * lane;
+    const int groups = (int)(N - n0 >= 128 ? 32 : (N - n0) >> 2);   // complete groups of four rows
+    const bool tail = groups < 32 && n0 + 4 * groups < N;           // up to three rows behind the last one
+    // Stage of chunk c, counted over all tasks in `ring`: one tile load for 32 rows of U, one for the errors of 32 groups.
+    auto stage = [&](int c) { return (int)((ring + (uint32_t)c) % DpqSmem::kStages); };
+    auto parity = [&](int c) { return ((ring + (uint32_t)c) / DpqSmem::kStages) & 1u; };
     auto load_u = [&](int c) {
-        const uint32_t dst = sm_addr + DpqSmem::kTrailU + (uint32_t)((c & 1) * kDpqChunk * 128 * 4) + (uint32_t)tid * 16u;
+        const uint32_t dst = sm_addr + (uint32_t)(stage(c) * DpqSmem::kStage), bar = bars + 8u * (uint32_t)stage(c);
+        const int q = (int)pprev + c * kDpqChunk;
+        if (warp == 0 && ptx::elect_one()) {
+            ptx::mbar_arrive_expect_tx(bar, (uint32_t)(uvec ? DpqSmem::kStage : DpqSmem::kStageU));
+            if (uvec) ptx::tma_load_2d(dst, &maps.u, (int)v0, q, bar);
+        }
+        if (!uvec) {
 #pragma unroll
-        for (int i = 0; i < kDpqChunk / 8; ++i) dpq_copy16(dst + (uint32_t)(i * 8 * 512), usrc + (int64_t)(c * kDpqChunk + 8 * i) * K, uvec);
+            for (int i = 0; i < kDpqChunk / 8; ++i)
+                dpq_copy16(dst + (uint32_t)(i * 8 * 512 + tid * 16), U + (int64_t)(q + 8 * i + warp) * K + v0 + 4 * lane, false);
+            dpq_commit();
+        }
     };
     auto load_e = [&](int c) {
-        const int off = DpqSmem::kTrailErr + (c & 1) * kDpqChunk * 128 * 4;
-        dpq_load_errors<128>(reinterpret_cast<float*>(sm + off), sm_addr + (uint32_t)off, work, N, K, pprev + (int64_t)(c / kPerBlock) * 128, n0,
-                             c % kPerBlock);
+        const uint32_t dst = sm_addr + (uint32_t)(stage(c) * DpqSmem::kStage + DpqSmem::kStageU), bar = bars + 8u * (uint32_t)stage(c);
+        const int x = (int)pprev + (c / kPerBlock) * 128, y = c % kPerBlock, z = (int)(n0 >> 2);
+        if (warp == 0 && ptx::elect_one()) ptx::tma_load_3d(dst, &maps.errors, x, y, z, bar);
     };
-    load_u(0);   // (U is the caller's: complete before the first launch of the chain)
-    ptx::griddep_wait();
+    // (the marks' addresses come from perm: looked up while U, which is the caller's, is requested)
+    const int64_t r32 = n0 / 32 + (tid & 3);
+    const uint16_t* done = nullptr;
+    const unsigned int* applied = nullptr;
+    if (tid < 4 && r32 * 32 < N) done = marks.done(r32, e0 + blocks - 1);
+    if (tid == 32 && e0 > 0) applied = marks.applied(n0 / 32, col);
+    load_u(0);
+    load_u(1);
+    {   // the errors of these rows are there, and those before them have been applied to this tile
+        bool ok = true;
+        if (done) ok = wait.until([&] { return dpq_ld_acquire_u16(done) != 0xFFFFu; });
+        else if (applied) ok = wait.until([&] { return ptx::ld_acquire_gpu(applied) >= (unsigned)e0; });
+        if (!__syncthreads_and(ok)) {   // given up: what is on its way lands first
+            load_e(0);
+            load_e(1);
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            dpq_land(bars + 8u * (uint32_t)stage(0), parity(0));
+            dpq_land(bars + 8u * (uint32_t)stage(1), parity(1));
+            return false;
+        }
+    }
+    // (what was seen of the other CTAs' writes holds for the tile loads too)
+    asm volatile("fence.proxy.async.global;" ::: "memory");
     load_e(0);
-    dpq_commit();
+    load_e(1);
     float* wp = work + (n0 + 16 * warp) * K + v0 + 4 * lane;
     const int rows = (int)min((int64_t)16, N - (n0 + 16 * warp));   // (may be negative: a warp without rows)
     unsigned long long acc[8][4];   // rows 2 i and 2 i + 1, four columns
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
-        if (2 * i < rows) a = *reinterpret_cast<const float4*>(wp + (int64_t)(2 * i) * K);
-        if (2 * i + 1 < rows) b = *reinterpret_cast<const float4*>(wp + (int64_t)(2 * i + 1) * K);
+        if (2 * i < rows) a = __ldcg(reinterpret_cast<const float4*>(wp + (int64_t)(2 * i) * K));
+        if (2 * i + 1 < rows) b = __ldcg(reinterpret_cast<const float4*>(wp + (int64_t)(2 * i + 1) * K));
         acc[i][0] = pack_f32x2(a.x, b.x);
         acc[i][1] = pack_f32x2(a.y, b.y);
         acc[i][2] = pack_f32x2(a.z, b.z);
@@ -290,17 +382,29 @@ __device__ __forceinline__ void dpq_trailing_tile(uint8_t* sm, uint32_t sm_addr,
     }
 #pragma unroll 1
     for (int c = 0; c < chunks; ++c) {
-        dpq_wait<0>();
-        __syncthreads();   // chunk c is there; chunk c - 1 has been consumed by everybody
-        if (c + 1 < chunks) {
-            load_u(c + 1);
-            load_e(c + 1);
-            dpq_commit();
+        if (!uvec) {
+            if (c + 1 < chunks) dpq_wait<1>();
+            else dpq_wait<0>();
         }
-        // group 4 warp + g of row q is at 4 ((4 warp + g) ^ (q & 7)) = 4 (4 warp ^ (q & 4)) + 4 (g ^ (q & 3)): two bases
-        const uint8_t* us = sm + DpqSmem::kTrailU + (c & 1) * kDpqChunk * 512 + 16 * lane;
-        const uint8_t* e0 = sm + DpqSmem::kTrailErr + (c & 1) * kDpqChunk * 512 + 64 * warp;
-        const uint8_t* e1 = sm + DpqSmem::kTrailErr + (c & 1) * kDpqChunk * 512 + 64 * (warp ^ 1);
+        const bool ok = ptx::mbar_wait(bars + 8u * (uint32_t)stage(c), parity(c), abort_s, wait.status_word);
+        if (!__syncthreads_and(ok)) {   // chunk c is there; chunk c - 1 has been consumed by everybody
+            if (c + 1 < chunks) dpq_land(bars + 8u * (uint32_t)stage(c + 1), parity(c + 1));
+            return false;
+        }
+        if (c + 2 < chunks) {
+            load_u(c + 2);
+            load_e(c + 2);
+        }
+        if (tail) {   // (the tile load has put zeros there)
+            if (warp == 0) {
+                float* e = reinterpret_cast<float*>(sm + stage(c) * DpqSmem::kStage + DpqSmem::kStageU) + groups * 128 + 4 * lane;
+                for (int64_t n = n0 + 4 * groups; n < N; ++n)
+                    e[n & 3] = __ldcg(work + n * K + pprev + c * kDpqChunk + lane);
+            }
+            __syncthreads();
+        }
+        const uint8_t* us = sm + stage(c) * DpqSmem::kStage + 16 * lane;
+        const uint8_t* es = sm + stage(c) * DpqSmem::kStage + DpqSmem::kStageU + 4 * warp * 512;
         struct Q {
             ulonglong2 e[4];
             float4 u;
@@ -308,8 +412,7 @@ __device__ __forceinline__ void dpq_trailing_tile(uint8_t* sm, uint32_t sm_addr,
         auto fetch = [&](Q& t, int q8, int j) {   // q = q8 + j, j = 0..7 known at compile time
             t.u = *reinterpret_cast<const float4*>(us + (q8 + j) * 512);
 #pragma unroll
-            for (int g = 0; g < 4; ++g)
-                t.e[g] = *reinterpret_cast<const ulonglong2*>(((j & 4) ? e1 : e0) + (q8 + j) * 512 + 16 * (g ^ (j & 3)));
+            for (int g = 0; g < 4; ++g) t.e[g] = *reinterpret_cast<const ulonglong2*>(es + g * 512 + (q8 + j) * 16);
         };
         auto apply = [&](const Q& t) {
             const float uv[4] = {t.u.x, t.u.y, t.u.z, t.u.w};
@@ -346,6 +449,13 @@ __device__ __forceinline__ void dpq_trailing_tile(uint8_t* sm, uint32_t sm_addr,
         if (2 * i < rows) *reinterpret_cast<float4*>(wp + (int64_t)(2 * i) * K) = a;
         if (2 * i + 1 < rows) *reinterpret_cast<float4*>(wp + (int64_t)(2 * i + 1) * K) = b;
     }
+    ring += (uint32_t)chunks;
+    __syncthreads();
+    if (tid < 4 && n0 + 32 * tid < N) {
+        __threadfence();
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(marks.applied(n0 / 32 + tid, col)), "r"((uint32_t)(e0 + blocks)) : "memory");
+    }
+    return true;
 }
 
 // Block b of 32 rows, eight lanes per row.  Lane sl of a row keeps columns 32 k + 4 sl + {0..3}, k = 0..3.
@@ -354,33 +464,19 @@ __device__ __forceinline__ void dpq_trailing_tile(uint8_t* sm, uint32_t sm_addr,
 // instead of one per column), follows the same scalar computation through all four, and then applies
 // the four errors to its own columns, in ascending order.  Columns that are finished are updated along
 // with the others; nothing reads them again.
-__global__ void __launch_bounds__(kDpqThreads, 2)
-dpq_step_kernel(float* __restrict__ work, const float* __restrict__ U, const int32_t* __restrict__ perm,
-                int64_t N, int64_t K, int b, int symmetric, int mse_steps, int per_channel,
-                const float* __restrict__ s_w, uint8_t* __restrict__ codes, uint16_t* __restrict__ gscale,
-                uint8_t* __restrict__ gzero, DpqTrail far, DpqTrail near) {
-    extern __shared__ __align__(16) uint8_t sm[];
-    const uint32_t sm_addr = ptx::smem_addr(sm);
+__device__ __forceinline__ bool dpq_block_rows(uint8_t* sm, uint32_t sm_addr, float* work, const float* __restrict__ U,
+                                               const int32_t* __restrict__ perm, int64_t N, int64_t K, int b, int64_t rows32,
+                                               int symmetric, int mse_steps, int per_channel, const float* __restrict__ s_w,
+                                               uint8_t* codes, uint16_t* gscale, uint8_t* __restrict__ gzero, bool uvec,
+                                               const DpqMarks& marks, const DpqWait& wait) {
     const int64_t p0 = (int64_t)b * 128;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, sl = lane & 7;
-    const bool uvec = (reinterpret_cast<uintptr_t>(U) & 15u) == 0;
-    const unsigned block_ctas = (unsigned)((N + kDpqRowsPerCta - 1) / kDpqRowsPerCta);
-    ptx::griddep_launch_dependents();
-    if (blockIdx.x >= block_ctas) {
-        const unsigned t = blockIdx.x - block_ctas, row_tiles = (unsigned)((N + 127) / 128);
-        const unsigned col = t / row_tiles;
-        const bool is_far = col < (unsigned)far.count;
-        const DpqTrail tr = is_far ? far : near;
-        dpq_trailing_tile(sm, sm_addr, work, U, N, K, (int64_t)tr.errors * 128, tr.blocks,
-                          (int64_t)(tr.first + (int)(is_far ? col : col - (unsigned)far.count)) * 128, (int64_t)(t % row_tiles) * 128, uvec);
-        return;
-    }
     const float* u_s = reinterpret_cast<const float*>(sm + DpqSmem::kU);
     uint8_t* code_s = sm + DpqSmem::kCodes;
     float4* diag_s = reinterpret_cast<float4*>(sm + DpqSmem::kDiag);
     uint8_t* perm_s = sm + DpqSmem::kPerm;
     const int rl = 4 * warp + (lane >> 3);                        // row within the CTA
-    const int64_t n_raw = (int64_t)blockIdx.x * kDpqRowsPerCta + rl;
+    const int64_t n_raw = rows32 * kDpqRowsPerCta + rl;
     const bool valid = n_raw < N;                                 // (lanes without a row repeat the last one and store nothing)
     const int64_t n = valid ? n_raw : N - 1;
     const int64_t G = K >> 7;
@@ -397,32 +493,49 @@ dpq_step_kernel(float* __restrict__ work, const float* __restrict__ U, const int
     auto load_err = [&](int c) {
         const int off = DpqSmem::kErr + (c & 1) * kDpqChunk * kDpqRowsPerCta * 4;
         dpq_load_errors<kDpqRowsPerCta>(reinterpret_cast<float*>(sm + off), sm_addr + (uint32_t)off, work, N, K, p0 - 128,
-                                        (int64_t)blockIdx.x * kDpqRowsPerCta, c);
+                                        rows32 * kDpqRowsPerCta, c);
     };
+    // U is the caller's: what is wanted of it first is requested ahead of the wait
     if (b > 0) {
-        load_panel(0);   // (U is the caller's: complete before the first launch of the chain)
-        ptx::griddep_wait();
-        load_err(0);
-        dpq_commit();
+        load_panel(0);
         load_panel(1);
-        load_err(1);
-        dpq_commit();
     }
 #pragma unroll
     for (int i = 0; i < 128 * 32 / kDpqThreads; ++i) {
         const int idx = i * kDpqThreads + tid, q = idx >> 5, c4 = (idx & 31) * 4;
         dpq_copy16(sm_addr + DpqSmem::kU + (uint32_t)((q * 128 + c4) * 4), U + (p0 + q) * K + p0 + c4, uvec);
     }
-    dpq_commit();
     if (tid < 128) perm_s[tid] = (uint8_t)(perm ? (perm[p0 + tid] & 127) : tid);
+    if (b == 0) {
+        dpq_commit();
+    } else {
+        // the block before is done but for its last 32 columns, and the errors before its have been applied to this one
+        bool ok = true;
+        if (tid == 0) {
+            const uint16_t* d = marks.done(rows32, b - 1);
+            const unsigned int* early = marks.early(rows32, b - 1);
+            ok = wait.until([&] { return ptx::ld_acquire_gpu(early) != 0u || dpq_ld_acquire_u16(d) != 0xFFFFu; });
+        } else if (tid == 32 && b > 1) {
+            const unsigned int* d = marks.applied(rows32, b);
+            ok = wait.until([&] { return ptx::ld_acquire_gpu(d) >= (unsigned)(b - 1); });
+        }
+        if (!__syncthreads_and(ok)) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            return false;
+        }
+        load_err(0);
+        dpq_commit();
+        load_err(1);
+        dpq_commit();
+    }
     // The errors of the previous block first (the trailing CTAs of the previous launch left this block out): a
     // warp takes its four rows, a lane four consecutive columns of each, so that U is read once per four rows.
     {
-        const int64_t r0 = (int64_t)blockIdx.x * kDpqRowsPerCta + 4 * warp;
+        const int64_t r0 = rows32 * kDpqRowsPerCta + 4 * warp;
         float a[4][4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            const float4 t = *reinterpret_cast<const float4*>(work + (r0 + r < N ? r0 + r : N - 1) * K + p0 + 4 * lane);
+            const float4 t = __ldcg(reinterpret_cast<const float4*>(work + (r0 + r < N ? r0 + r : N - 1) * K + p0 + 4 * lane));
             a[r][0] = t.x;
             a[r][1] = t.y;
             a[r][2] = t.z;
@@ -431,9 +544,9 @@ dpq_step_kernel(float* __restrict__ work, const float* __restrict__ U, const int
         if (b > 0) {
 #pragma unroll 1
             for (int c = 0; c < 128 / kDpqChunk; ++c) {
-                // groups in flight, in order: chunks 0 and 1, U of the block, chunks 2 and 3
-                if (c < 2) dpq_wait<2>();
-                else if (c == 2) dpq_wait<1>();
+                // groups in flight, in order: chunk 0 (and all that was requested ahead of the wait), chunk 1, chunk 2, U of chunk 3,
+                // errors of chunk 3
+                if (c < 3) dpq_wait<1>();
                 else dpq_wait<0>();
                 __syncthreads();
                 const float* us = reinterpret_cast<const float*>(sm + DpqSmem::kPanel) + (c & 1) * kDpqChunk * 128 + 4 * lane;
@@ -451,12 +564,18 @@ dpq_step_kernel(float* __restrict__ work, const float* __restrict__ U, const int
                         a[r][3] = __fmaf_rn(ev[r], u4.w, a[r][3]);
                     }
                 }
-                __syncthreads();
-                if (c + 2 < 128 / kDpqChunk) {
-                    load_panel(c + 2);
-                    load_err(c + 2);
-                    dpq_commit();
+                bool ok = true;
+                if (c == 2 && tid == 0) {   // the last 32 columns of the block before
+                    const uint16_t* d = marks.done(rows32, b - 1);
+                    ok = wait.until([&] { return dpq_ld_acquire_u16(d) != 0xFFFFu; });
                 }
+                if (!__syncthreads_and(ok)) {
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    return false;
+                }
+                if (c < 2) load_panel(c + 2);
+                if (c == 0 || c == 2) load_err(c == 0 ? 2 : 3);
+                dpq_commit();
             }
         } else {
             dpq_wait<0>();
@@ -639,16 +758,29 @@ dpq_step_kernel(float* __restrict__ work, const float* __restrict__ U, const int
             if (sl == o && valid) {
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
-                    ew[whole ? (int64_t)k * K + 16 * o + 4 * c : (int64_t)(q0 + c)] = ne[c];
+                    if (p0 + 128 < K) ew[whole ? (int64_t)k * K + 16 * o + 4 * c : (int64_t)(q0 + c)] = ne[c];
                     code_s[rl * 128 + perm_s[q0 + c]] = lut_u[code[c]];
                 }
             }
         }
+        if (k == 2) {
+            __syncthreads();
+            if (tid == 0) {
+                __threadfence();
+                asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(marks.early(rows32, b)), "r"(1u) : "memory");
+            }
+        }
     }
-    __syncwarp();
-    if (!valid) return;
-    // codes of the group, original order, two per byte (even column in the low nibble)
-    {
+    // The scale of the first row marks that the errors are in place; the codes need not be for that.
+    const uint16_t scale = __bfloat16_as_ushort(__float2bfloat16_rn(grp.s));
+    __syncthreads();
+    if (tid == 0) {   // (row 0 of the 32)
+        __threadfence();
+        asm volatile("st.release.gpu.global.u16 [%0], %1;" ::"l"(gscale + n * G + og), "h"(scale) : "memory");
+    }
+    // codes of the group, original order, two per byte (even column in the low nibble); the first row's of the last block wait in the
+    // work array (see DpqMarks)
+    if (valid) {
         const uint32_t* cs = reinterpret_cast<const uint32_t*>(code_s + rl * 128 + sl * 16);
         uint32_t packed[2];
 #pragma unroll
@@ -657,11 +789,99 @@ dpq_step_kernel(float* __restrict__ work, const float* __restrict__ U, const int
             packed[i] = (a & 15u) | ((a >> 4) & 0xF0u) | ((a >> 8) & 0xF00u) | ((a >> 12) & 0xF000u) |
                         ((c & 15u) << 16) | ((c << 12) & 0xF00000u) | ((c << 8) & 0xF000000u) | ((c << 4) & 0xF0000000u);
         }
-        *reinterpret_cast<uint2*>(codes + n * (K >> 1) + og * 64 + sl * 8) = make_uint2(packed[0], packed[1]);
+        uint8_t* to = n == 0 && p0 + 128 == K ? reinterpret_cast<uint8_t*>(work + p0) : codes + n * (K >> 1) + og * 64;
+        *reinterpret_cast<uint2*>(to + sl * 8) = make_uint2(packed[0], packed[1]);
     }
-    if (sl == 0) {
-        gscale[n * G + og] = __bfloat16_as_ushort(__float2bfloat16_rn(grp.s));
+    if (sl == 0 && valid) {
+        if (rl > 0) gscale[n * G + og] = scale;
         if (gzero) gzero[n * G + og] = (uint8_t)grp.z;
+    }
+    return true;
+}
+
+// Bound by the FP32 pipes for large layers, by the chain of a block for small ones.  No CTA has to be resident for another to make
+// progress: a task waits for tasks of earlier tickets only, which running CTAs hold; any number of calls can share the device.
+// Measured, us per layer, a launch per step (whose CTAs start and drain together, with cp.async by all threads and two blocks' errors
+// at a time) / this: (N, K) = (256, 1024) 264 / 263, (256, 4096) 880 / 840, (1024, 2048) 552 / 487, (2048, 2048) 616 / 505, (4096,
+// 4096) 2390 / 2070, (8192, 8192) 14560 / 11950, (4096, 14336) 21200 / 16900 = 25 T FMA/s.  Of the last: order and waits 21200 -> 19800, tile
+// loads three stages ahead -> 17850, panels of up to eight blocks -> 16870.  A tile's loop runs at 85 % of the pipe; what is left is
+// the start and the end of tiles (13000 cycles of some 95000 at two blocks, 4 % at eight) and the tasks of the blocks, 14 % of the places.
+__global__ void __launch_bounds__(kDpqThreads, 2)
+dpq_kernel(const __grid_constant__ DpqMaps maps, float* work, const float* __restrict__ U, const int32_t* __restrict__ perm, int64_t N, int64_t K, int symmetric,
+           int mse_steps, int per_channel, const float* __restrict__ s_w, uint8_t* codes, uint16_t* gscale,
+           uint8_t* __restrict__ gzero, const DpqSteps first_step, unsigned int* status_word) {
+    extern __shared__ __align__(128) uint8_t sm[];
+    __shared__ int task[6];   // kind (0: end, 1: block, 2: errors), then what it is about
+    __shared__ DpqSteps steps;                        // (thread 0's)
+    __shared__ unsigned long long begin, end;         // tickets of the current step
+    __shared__ uint64_t stage_bars[DpqSmem::kStages];
+    __shared__ uint32_t abort_flag;
+    const uint32_t bars = ptx::smem_addr(stage_bars);
+    uint32_t ring = 0;                                // stages that this CTA has used
+    const uint32_t sm_addr = ptx::smem_addr(sm);
+    ptx::griddep_wait();
+    const bool uvec = (reinterpret_cast<uintptr_t>(U) & 15u) == 0;
+    const DpqMarks marks = {codes, gscale, perm, K};
+    unsigned int* const control = marks.control();
+    const DpqWait wait = {control, status_word};
+    const unsigned int blocks32 = (unsigned)((N + kDpqRowsPerCta - 1) / kDpqRowsPerCta);
+    if (threadIdx.x == 0) {
+        steps = first_step;
+        begin = end = 0;
+        abort_flag = 0u;
+        for (int i = 0; i < DpqSmem::kStages; ++i) ptx::mbar_init(bars + 8u * i, 1);
+        ptx::fence_mbar_init();
+    }
+    while (true) {
+        if (threadIdx.x == 0) {
+            const unsigned int ticket = atomicAdd(control, 1u);
+            while (ticket >= end && steps.b < steps.G) {
+                begin = end;
+                steps.next();
+                if (steps.b < steps.G)
+                    end = begin + blocks32 + (unsigned long long)steps.row_tiles * (unsigned)(steps.far.count + steps.near.count);
+            }
+            task[0] = 0;
+            if (steps.b < steps.G) {
+                unsigned int i = (unsigned int)(ticket - begin);
+                if (i < blocks32) {
+                    task[0] = 1;
+                    task[1] = steps.b;
+                    task[2] = (int)i;
+                } else {
+                    i -= blocks32;
+                    const unsigned int col = i / (unsigned)steps.row_tiles;
+                    const bool is_far = col < (unsigned)steps.far.count;
+                    const DpqTrail tr = is_far ? steps.far : steps.near;
+                    task[0] = 2;
+                    task[1] = tr.errors;
+                    task[2] = tr.blocks;
+                    task[3] = tr.first + (int)(is_far ? col : col - (unsigned)steps.far.count);
+                    task[4] = (int)(i % (unsigned)steps.row_tiles);
+                }
+            }
+        }
+        __syncthreads();
+        const int kind = task[0], t1 = task[1], t2 = task[2], t3 = task[3], t4 = task[4];
+        __syncthreads();
+        if (kind == 0) break;
+        const bool ok = kind == 1 ? dpq_block_rows(sm, sm_addr, work, U, perm, N, K, t1, t2, symmetric, mse_steps, per_channel, s_w, codes,
+                                                   gscale, gzero, uvec, marks, wait)
+                                  : dpq_trailing_tile(sm, sm_addr, work, U, N, K, t1, t2, t3, (int64_t)t4 * 128, uvec, marks, wait, maps, bars,
+                                                     &abort_flag, ring);
+        if (!ok) break;   // (the whole CTA)
+        ptx::fence_proxy_async_smem();   // (the next task's bulk copies go where this one read and wrote)
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(control + 1, 1u) == gridDim.x - 1u) {   // the last one puts the codes where the control words were
+            __threadfence();
+            const uint4* from = reinterpret_cast<const uint4*>(work + K - 128);
+            uint4* to = reinterpret_cast<uint4*>(control);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) to[i] = __ldcg(from + i);
+        }
     }
 }
 

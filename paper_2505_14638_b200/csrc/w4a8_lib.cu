@@ -129,6 +129,26 @@ static bool make_tmap_u8_2d(CUtensorMap* m, const void* ptr, uint64_t rows, uint
     return r == CUDA_SUCCESS;
 }
 
+// What dpq_kernel's tile loads read: U [K][K] (nothing there where it is not 16-byte aligned) and the work array [N][K] in groups of
+// four rows (up to three rows behind the last complete group lie outside).
+static bool make_dpq_maps(DpqMaps* maps, const float* U, const float* work, int64_t N, int64_t K) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    auto encode = [&](CUtensorMap* m, const float* ptr, cuuint32_t rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
+        const cuuint32_t step[3] = {1, 1, 1};
+        return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, rank, const_cast<float*>(ptr), dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    const cuuint64_t k = (cuuint64_t)K, n = (cuuint64_t)N;
+    const cuuint64_t edims[3] = {k, n < 4 ? n : 4, n < 4 ? 1 : n / 4}, estrides[2] = {k * 4, k * 16};
+    const cuuint32_t ebox[3] = {128, 1, 32};
+    if (!encode(&maps->errors, work, 3, edims, estrides, ebox)) return false;
+    maps->u = maps->errors;
+    const cuuint64_t udims[2] = {k, k}, ustrides[1] = {k * 4};
+    const cuuint32_t ubox[2] = {128, kDpqChunk};
+    return (reinterpret_cast<uintptr_t>(U) & 15u) != 0 || encode(&maps->u, U, 2, udims, ustrides, ubox);
+}
+
 // ------------------------------------------------------------------------------ linear plan
 struct LinearPlan {
     int algo;      // W4A8_ALGO_SIMT or W4A8_ALGO_UMMA
@@ -1629,7 +1649,7 @@ int w4a8_dpq_quantize(const float* W, int64_t N, int64_t K, int group, const flo
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(once, [&] {
-        attr_err = cudaFuncSetAttribute(dpq_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DpqSmem::kBytes);
+        attr_err = cudaFuncSetAttribute(dpq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DpqSmem::kBytes);
     });
     if (attr_err != cudaSuccess) return W4A8_ERR_CUDA;
     // Eq. 6
@@ -1642,64 +1662,42 @@ int w4a8_dpq_quantize(const float* W, int64_t N, int64_t K, int group, const flo
         unsigned blocks = (unsigned)((total + 255) / 256 < 148 * 8 ? (total + 255) / 256 : 148 * 8);
         absmax_f32_kernel<<<blocks, 256, 0, st>>>(W, N, K, 0, amax_bits);
     }
-    int64_t ns = per_channel ? N : 1;
-    amax_to_scale_kernel<<<(unsigned)((ns + 255) / 256), 256, 0, st>>>(s_w, ns);
+    // (this kernel starts beside the one before, and the next while this one drains)
     float* work = static_cast<float*>(workspace);
-    dpq_gather_kernel<<<(unsigned)((N * K + 255) / 256), 256, 0, st>>>(W, perm, N, K, work);
-    uint64_t launches = 3;
-    const int G = (int)(K / kGroup);
-    const int64_t block_ctas = (N + kDpqRowsPerCta - 1) / kDpqRowsPerCta, row_tiles = (N + 127) / 128;
-    const int64_t slots = 2 * (int64_t)sm_count();   // CTAs resident at once
+    uint16_t* gscale = static_cast<uint16_t*>(gscale_bf16);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((N * K + 255) / 256));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, dpq_gather_kernel, W, perm, N, K, work, codes, gscale, s_w, per_channel ? N : (int64_t)1) != cudaSuccess)
+        return W4A8_ERR_CUDA;
+    unsigned int* status = status_word_ptr();
+    if (!status) return W4A8_ERR_CUDA;
+    const int64_t slots = 2 * (int64_t)sm_count(), row_tiles = (N + 127) / 128;   // CTAs resident at once
     if (slots <= 0) return W4A8_ERR_CUDA;
-    int rest = 0;         // column blocks that an even step leaves to the next one
-    bool paired = false;  // the columns behind the next block lack the errors of two blocks
-    for (int b = 0; b < G; ++b) {
-        DpqTrail far = {0, 2, 0, 0}, near = {0, 1, 0, 0};
-        const int n = G - 1 - b;   // column blocks behind block b
-        // Two blocks' errors at a time pay while a step has tiles for several rounds of CTAs; with fewer, the coarser pieces leave more
-        // of the last round idle.  One block at a time throughout / two throughout / two down to four rounds, us: (4096, 14336)
-        // 22039 / 21260 / 21186, (8192, 8192) 15140 / 14578 / 14529, (4096, 4096) 2371 / 2459 / 2363, (1024, 14336) 6529 / 7020 / 6522.
-        const bool many = row_tiles * n >= 4 * slots;
-        if (b % 2 == 1) {
-            if (paired) far = {b - 3, 2, G - rest, rest};
-            if (b == 1) paired = many;
-            near = {b - 1, 1, b + 1, paired ? (n > 0 ? 1 : 0) : n};
-        } else if (paired) {
-            // the column blocks in two parts, at least two blocks in the first, with as few rounds of CTAs as possible and
-            // otherwise in halves; all of them before the errors of one block at a time follow
-            far = {b - 2, 2, b + 1, n};
-            if (many) {
-                int64_t best = INT64_MAX;
-                for (int h = n < 2 ? n : 2; h <= n; ++h) {
-                    const int64_t rounds = (block_ctas + row_tiles * h + slots - 1) / slots + (block_ctas + row_tiles * (n - h + 1) + slots - 1) / slots;
-                    const int64_t cost = rounds * 2 * G + (2 * h > n ? 2 * h - n : n - 2 * h);
-                    if (cost < best) {
-                        best = cost;
-                        far.count = h;
-                    }
-                }
-            }
-            rest = n - far.count;
-            paired = many;
-        } else if (b > 0) {
-            near = {b - 1, 1, b + 1, n};
-        }
-        // (from the second step on the launches overlap: a step's CTAs start, and fetch U, while the one before drains)
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(block_ctas + row_tiles * (far.count + near.count)));
-        cfg.blockDim = dim3(kDpqThreads);
-        cfg.dynamicSmemBytes = (size_t)DpqSmem::kBytes;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = b > 0 ? 1 : 0;
-        if (cudaLaunchKernelEx(&cfg, dpq_step_kernel, work, U, perm, N, K, b, symmetric, mse_steps, per_channel,
-                               static_cast<const float*>(s_w), codes, static_cast<uint16_t*>(gscale_bf16), gzero, far, near) != cudaSuccess)
-            return W4A8_ERR_CUDA;
-        ++launches;
-    }
+    DpqMaps maps;
+    if (!make_dpq_maps(&maps, U, work, N, K)) return W4A8_ERR_CUDA;
+    DpqSteps steps = {};
+    steps.G = (int)(K / kGroup);
+    steps.row_tiles = (int)row_tiles;
+    steps.slots = (int)slots;
+    steps.b = -1;
+    // One CTA per SM where a step's tiles do not keep two busy: the chain of a block, which is what counts then, has the SM for itself.
+    // (2048, 2048) 597 us with two, 539 with one; (1024, 2048) 592 and 514.
+    const int64_t nb = (N + kDpqRowsPerCta - 1) / kDpqRowsPerCta, tiles = row_tiles * steps.G;
+    const int64_t most = tiles <= slots ? slots / 2 : slots, useful = nb + (tiles <= slots ? tiles / 2 : tiles);
+    cfg.gridDim = dim3((unsigned)(useful < most ? useful : most));
+    cfg.blockDim = dim3(kDpqThreads);
+    cfg.dynamicSmemBytes = (size_t)DpqSmem::kBytes;
+    if (cudaLaunchKernelEx(&cfg, dpq_kernel, maps, work, U, perm, N, K, symmetric, mse_steps, per_channel, static_cast<const float*>(s_w), codes,
+                           gscale, gzero, steps, status) != cudaSuccess)
+        return W4A8_ERR_CUDA;
+    const uint64_t launches = 3;
     g_launches.fetch_add(launches, std::memory_order_relaxed);
     return launch_status();
 }

@@ -301,6 +301,7 @@ absmax_f32_kernel(const float* __restrict__ W, int64_t rows, int64_t cols, int p
     // per_row: one CTA per row writes out_bits[row]; else grid-stride with an atomic max on the
     // bit pattern (non-negative floats order like unsigned integers).
     __shared__ float red[32];
+    ptx::griddep_launch_dependents();
     float m = 0.0f;
     if (per_row) {
         const float* r = W + (int64_t)blockIdx.x * cols;
@@ -317,12 +318,13 @@ absmax_f32_kernel(const float* __restrict__ W, int64_t rows, int64_t cols, int p
     }
 }
 
+__device__ __forceinline__ void amax_to_scale(float* s_w) {
+    const float a = *s_w;  // holds the absmax written by absmax_f32_kernel
+    *s_w = (a > 0.0f) ? __fdiv_rn(a, kE4M3Max) : 1.0f;  // Eq. 6
+}
 __global__ void amax_to_scale_kernel(float* s_w, int64_t n) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        float a = s_w[i];  // holds the absmax written by absmax_f32_kernel
-        s_w[i] = (a > 0.0f) ? __fdiv_rn(a, kE4M3Max) : 1.0f;  // Eq. 6
-    }
+    if (i < n) amax_to_scale(s_w + i);
 }
 
 __device__ __forceinline__ float e4m3_roundtrip(float q) {
