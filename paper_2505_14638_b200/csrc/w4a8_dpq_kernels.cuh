@@ -896,169 +896,208 @@ dpq_kernel(const __grid_constant__ DpqMaps maps, float* work, const float* __res
 // loads for 32 packed FMAs, with (8, 2) three for 8, against 8 for 16 scalar ones before.  Tokens come
 // in double-buffered chunks of 16, through registers (BF16 -> FP32 on the way).  Measured, us, against the 64 x 64
 // tiles of 4 x 4 scalar FMAs per thread: (T, K) = (2000, 1024) 212 -> 76, (1024, 4096) 799 -> 367 (24 T FMA/s,
-// of the 28-31 T that a loop of FMAs alone reaches), (2048, 8192) 5820 -> 2586.
+// of the 28-31 T that a loop of FMAs alone reaches), (2048, 8192) 5820 -> 2586.  Where whole tiles would leave a last round that is not
+// full, some are shared by their tokens between two launches (hessian_split, with figures).
 // ---------------------------------------------------------------------------------------------
 constexpr int kHessTok = 16;
-template <int TILE>
+// PART: 0, whole tiles only; 1, the first launch of a split; 2, the second.
+template <int TILE, int PART>
 __global__ void __launch_bounds__(256, TILE == 128 ? 2 : 4)
-hessian_xtx_kernel(const uint16_t* __restrict__ x, int64_t T, int64_t K, int64_t ldx, float* __restrict__ H,
-                   int accumulate) {
+hessian_xtx_kernel(const uint16_t* __restrict__ x, int64_t tokens, int64_t K, int64_t ldx, float* __restrict__ H,
+                   int accumulate, HessianSplit split) {
     constexpr int R = TILE / 8, C = TILE / 32;             // rows of a warp, columns of a lane
     constexpr int kLoads = 2 * kHessTok * TILE / 8 / 256;  // groups of eight features a thread fetches per chunk
     __shared__ __align__(16) float x_s[2][2][kHessTok][TILE];   // [buffer][rows | columns of the tile][token][feature]
-    // row bi of the upper triangle starts at tile bi nb - bi (bi - 1) / 2: the root of that, corrected by steps
-    const int nb = (int)((K + TILE - 1) / TILE), t = (int)blockIdx.x;
-    const float b2 = 2.0f * (float)nb + 1.0f;
-    int bi = (int)((b2 - sqrtf(fmaxf(b2 * b2 - 8.0f * (float)t, 0.0f))) * 0.5f);
-    bi = min(max(bi, 0), nb - 1);
-    while (bi > 0 && bi * nb - bi * (bi - 1) / 2 > t) --bi;
-    while ((bi + 1) * nb - (bi + 1) * bi / 2 <= t) ++bi;
-    const int bj = bi + t - (bi * nb - bi * (bi - 1) / 2);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // eight features at once where every row of X starts on a 16-byte boundary
-    const bool vec = (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && ldx % 8 == 0;
+    if (PART == 1) ptx::griddep_launch_dependents();
+    // Whole tiles only: the upper triangle by rows; else the diagonal first, then the strict triangle by rows.
+    const int nb = (int)((K + TILE - 1) / TILE), off = PART ? 1 : 0, n = nb - off;
+    const bool bundle = PART == 1 && (int)blockIdx.x >= split.whole;
+    int t = bundle ? split.whole + ((int)blockIdx.x - split.whole) * split.bundle : (PART == 2 ? split.whole : 0) + (int)blockIdx.x;
+    const int end = bundle ? min(t + split.bundle, nb * (nb + 1) / 2) : t + 1;
+    const int64_t T = bundle ? (int64_t)split.cut : tokens;
+    do {
+        // Row r of a triangle with n rows starts at r n - r (r - 1) / 2: the root of that, corrected by steps.
+        const float b2 = 2.0f * (float)n + 1.0f;
+        const int u = t - off * nb;
+        int bi = (int)((b2 - sqrtf(fmaxf(b2 * b2 - 8.0f * (float)u, 0.0f))) * 0.5f);
+        bi = min(max(bi, 0), n - 1);
+        while (bi > 0 && bi * n - bi * (bi - 1) / 2 > u) --bi;
+        while ((bi + 1) * n - (bi + 1) * bi / 2 <= u) ++bi;
+        int bj = bi + u - (bi * n - bi * (bi - 1) / 2) + off;
+        if (PART && t < nb) bi = bj = t;
+        const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+        // eight features at once where every row of X starts on a 16-byte boundary
+        const bool vec = (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && ldx % 8 == 0;
 
-    uint4 in[kLoads];
-    auto fetch = [&](int64_t t0) {
+        uint4 in[kLoads];
+        auto fetch = [&](int64_t t0) {
 #pragma unroll
-        for (int l = 0; l < kLoads; ++l) {
-            const int i = tid + 256 * l, op = i / (kHessTok * TILE / 8), rest = i % (kHessTok * TILE / 8);
-            const int64_t tok = t0 + rest / (TILE / 8), f = (int64_t)(op ? bj : bi) * TILE + rest % (TILE / 8) * 8;
-            const uint16_t* src = x + tok * ldx + f;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (tok < T) {
-                if (vec && f + 8 <= K) {
-                    v = __ldg(reinterpret_cast<const uint4*>(src));
-                } else {
-                    uint32_t h[8];
+            for (int l = 0; l < kLoads; ++l) {
+                const int i = tid + 256 * l, op = i / (kHessTok * TILE / 8), rest = i % (kHessTok * TILE / 8);
+                const int64_t tok = t0 + rest / (TILE / 8), f = (int64_t)(op ? bj : bi) * TILE + rest % (TILE / 8) * 8;
+                const uint16_t* src = x + tok * ldx + f;
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (tok < T) {
+                    if (vec && f + 8 <= K) {
+                        v = __ldg(reinterpret_cast<const uint4*>(src));
+                    } else {
+                        uint32_t h[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) h[j] = f + j < K ? (uint32_t)__ldg(src + j) : 0u;
-                    v = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
-                }
-            }
-            in[l] = v;
-        }
-    };
-    auto put = [&](int buf) {
-#pragma unroll
-        for (int l = 0; l < kLoads; ++l) {
-            const int i = tid + 256 * l, op = i / (kHessTok * TILE / 8), rest = i % (kHessTok * TILE / 8);
-            float4* d = reinterpret_cast<float4*>(&x_s[buf][op][rest / (TILE / 8)][rest % (TILE / 8) * 8]);
-            const uint4 v = in[l];
-            d[0] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16),
-                               __uint_as_float(v.y & 0xFFFF0000u));
-            d[1] = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xFFFF0000u), __uint_as_float(v.w << 16),
-                               __uint_as_float(v.w & 0xFFFF0000u));
-        }
-    };
-    unsigned long long acc[R / 2][C];   // rows 2 i and 2 i + 1
-#pragma unroll
-    for (int i = 0; i < R / 2; ++i)
-#pragma unroll
-        for (int j = 0; j < C; ++j) acc[i][j] = 0ull;
-    struct Tok {
-        ulonglong2 a[R / 4];
-        float b[C];
-    } k0, k1;
-    fetch(0);
-    int buf = 0;
-#pragma unroll 1
-    for (int64_t t0 = 0; t0 < T; t0 += kHessTok, buf ^= 1) {
-        put(buf);
-        __syncthreads();   // this chunk is there; the one before has been consumed by everybody
-        if (t0 + kHessTok < T) fetch(t0 + kHessTok);
-        const float* as = &x_s[buf][0][0][R * warp];
-        const float* bs = &x_s[buf][1][0][C * lane];
-        auto get = [&](Tok& k, int r) {
-#pragma unroll
-            for (int g = 0; g < R / 4; ++g) k.a[g] = *reinterpret_cast<const ulonglong2*>(as + r * TILE + 4 * g);
-            if (C == 4) {
-                const float4 v = *reinterpret_cast<const float4*>(bs + r * TILE);
-                k.b[0] = v.x;
-                k.b[1] = v.y;
-                k.b[C - 2] = v.z;
-                k.b[C - 1] = v.w;
-            } else {
-                const float2 v = *reinterpret_cast<const float2*>(bs + r * TILE);
-                k.b[0] = v.x;
-                k.b[1] = v.y;
-            }
-        };
-        auto apply = [&](const Tok& k) {
-#pragma unroll
-            for (int j = 0; j < C; ++j) {
-                const unsigned long long b = pack_f32x2(k.b[j], k.b[j]);
-#pragma unroll
-                for (int g = 0; g < R / 4; ++g) {
-                    acc[2 * g][j] = fma_f32x2(k.a[g].x, b, acc[2 * g][j]);
-                    acc[2 * g + 1][j] = fma_f32x2(k.a[g].y, b, acc[2 * g + 1][j]);
-                }
-            }
-        };
-        get(k0, 0);
-#pragma unroll
-        for (int r = 0; r < kHessTok; r += 2) {
-            get(k1, r + 1);
-            apply(k0);
-            if (r + 2 < kHessTok) get(k0, r + 2);
-            apply(k1);
-        }
-    }
-    // On a diagonal tile the 64 x 64 blocks below the diagonal are written as mirrors of those above.
-    const int64_t gi0 = (int64_t)bi * TILE + R * warp, gj0 = (int64_t)bj * TILE + C * lane;
-    const bool skip_row = bi == bj && TILE == 128 && warp >= 4 && lane < 16, mirror = bi != bj || (TILE == 128 && warp < 4 && lane >= 16);
-    const bool wide = C == 4 && K % 4 == 0 && (reinterpret_cast<uintptr_t>(H) & 15u) == 0;   // (then gj0 < K covers the lane's four columns)
-#pragma unroll
-    for (int i = 0; i < R / 2; ++i) {
-        float lo[C], hi[C];
-#pragma unroll
-        for (int j = 0; j < C; ++j) unpack_f32x2(acc[i][j], lo[j], hi[j]);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float* v = h == 0 ? lo : hi;
-            const int64_t gi = gi0 + 2 * i + h;
-            if (gi >= K || gj0 >= K || skip_row) continue;
-            float* hr = H + gi * K + gj0;
-            if (wide) {
-                if (accumulate) {
-                    const float4 o = *reinterpret_cast<const float4*>(hr);
-                    v[0] = __fadd_rn(v[0], o.x);
-                    v[1] = __fadd_rn(v[1], o.y);
-                    v[C - 2] = __fadd_rn(v[C - 2], o.z);
-                    v[C - 1] = __fadd_rn(v[C - 1], o.w);
-                }
-                *reinterpret_cast<float4*>(hr) = make_float4(v[0], v[1], v[C - 2], v[C - 1]);
-            } else {
-#pragma unroll
-                for (int j = 0; j < C; ++j)
-                    if (gj0 + j < K) {
-                        if (accumulate) v[j] = __fadd_rn(v[j], hr[j]);
-                        hr[j] = v[j];
+                        for (int j = 0; j < 8; ++j) h[j] = f + j < K ? (uint32_t)__ldg(src + j) : 0u;
+                        v = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
                     }
+                }
+                in[l] = v;
+            }
+        };
+        auto put = [&](int buf) {
+#pragma unroll
+            for (int l = 0; l < kLoads; ++l) {
+                const int i = tid + 256 * l, op = i / (kHessTok * TILE / 8), rest = i % (kHessTok * TILE / 8);
+                float4* d = reinterpret_cast<float4*>(&x_s[buf][op][rest / (TILE / 8)][rest % (TILE / 8) * 8]);
+                const uint4 v = in[l];
+                d[0] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16),
+                                   __uint_as_float(v.y & 0xFFFF0000u));
+                d[1] = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xFFFF0000u), __uint_as_float(v.w << 16),
+                                   __uint_as_float(v.w & 0xFFFF0000u));
+            }
+        };
+        unsigned long long acc[R / 2][C];   // rows 2 i and 2 i + 1
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i)
+#pragma unroll
+            for (int j = 0; j < C; ++j) acc[i][j] = 0ull;
+        struct Tok {
+            ulonglong2 a[R / 4];
+            float b[C];
+        } k0, k1;
+        // What the first launch hands to the second stands where the tile's mirror image goes in the end.
+        float4* hand = reinterpret_cast<float4*>(H + ((int64_t)bj * TILE + R * warp) * K + (int64_t)bi * TILE) + lane;
+        const int64_t from = PART == 2 ? split.cut : 0;
+        fetch(from);
+        if (PART == 2) {
+            ptx::griddep_wait();
+#pragma unroll
+            for (int i = 0; i < R / 2; ++i)
+#pragma unroll
+                for (int j = 0; j < C; j += 2) {
+                    const float4 v = __ldcg(hand + (int64_t)(i * C / 2 + j / 2) * (K / 4));
+                    acc[i][j] = pack_f32x2(v.x, v.y);
+                    acc[i][j + 1] = pack_f32x2(v.z, v.w);
+                }
+        }
+        int buf = 0;
+#pragma unroll 1
+        for (int64_t t0 = from; t0 < T; t0 += kHessTok, buf ^= 1) {
+            put(buf);
+            __syncthreads();   // this chunk is there; the one before has been consumed by everybody
+            if (t0 + kHessTok < T) fetch(t0 + kHessTok);
+            const float* as = &x_s[buf][0][0][R * warp];
+            const float* bs = &x_s[buf][1][0][C * lane];
+            auto get = [&](Tok& k, int r) {
+#pragma unroll
+                for (int g = 0; g < R / 4; ++g) k.a[g] = *reinterpret_cast<const ulonglong2*>(as + r * TILE + 4 * g);
+                if (C == 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(bs + r * TILE);
+                    k.b[0] = v.x;
+                    k.b[1] = v.y;
+                    k.b[C - 2] = v.z;
+                    k.b[C - 1] = v.w;
+                } else {
+                    const float2 v = *reinterpret_cast<const float2*>(bs + r * TILE);
+                    k.b[0] = v.x;
+                    k.b[1] = v.y;
+                }
+            };
+            auto apply = [&](const Tok& k) {
+#pragma unroll
+                for (int j = 0; j < C; ++j) {
+                    const unsigned long long b = pack_f32x2(k.b[j], k.b[j]);
+#pragma unroll
+                    for (int g = 0; g < R / 4; ++g) {
+                        acc[2 * g][j] = fma_f32x2(k.a[g].x, b, acc[2 * g][j]);
+                        acc[2 * g + 1][j] = fma_f32x2(k.a[g].y, b, acc[2 * g + 1][j]);
+                    }
+                }
+            };
+            get(k0, 0);
+#pragma unroll
+            for (int r = 0; r < kHessTok; r += 2) {
+                get(k1, r + 1);
+                apply(k0);
+                if (r + 2 < kHessTok) get(k0, r + 2);
+                apply(k1);
             }
         }
+        if (bundle) {
 #pragma unroll
-        for (int j = 0; j < C; ++j) acc[i][j] = pack_f32x2(lo[j], hi[j]);
-    }
-    if (!mirror) return;
+            for (int i = 0; i < R / 2; ++i)
 #pragma unroll
-    for (int j = 0; j < C; ++j) {
-        if (gj0 + j >= K) continue;
-        float* hc = H + (gj0 + j) * K + gi0;
+                for (int j = 0; j < C; j += 2) {
+                    float4 v;
+                    unpack_f32x2(acc[i][j], v.x, v.y);
+                    unpack_f32x2(acc[i][j + 1], v.z, v.w);
+                    hand[(int64_t)(i * C / 2 + j / 2) * (K / 4)] = v;
+                }
+            __syncthreads();   // (the last chunk has been read by everybody)
+            continue;
+        }
+        // On a diagonal tile the 64 x 64 blocks below the diagonal are written as mirrors of those above.
+        const int64_t gi0 = (int64_t)bi * TILE + R * warp, gj0 = (int64_t)bj * TILE + C * lane;
+        const bool skip_row = bi == bj && TILE == 128 && warp >= 4 && lane < 16, mirror = bi != bj || (TILE == 128 && warp < 4 && lane >= 16);
+        const bool wide = C == 4 && K % 4 == 0 && (reinterpret_cast<uintptr_t>(H) & 15u) == 0;   // (then gj0 < K covers the lane's four columns)
 #pragma unroll
-        for (int i = 0; i < R / 2; i += 2) {
-            float v[4];
-            unpack_f32x2(acc[i][j], v[0], v[1]);
-            unpack_f32x2(acc[i + 1][j], v[2], v[3]);
-            if (wide) {
-                if (gi0 + 2 * i < K) *reinterpret_cast<float4*>(hc + 2 * i) = make_float4(v[0], v[1], v[2], v[3]);
-            } else {
+        for (int i = 0; i < R / 2; ++i) {
+            float lo[C], hi[C];
 #pragma unroll
-                for (int h = 0; h < 4; ++h)
-                    if (gi0 + 2 * i + h < K) hc[2 * i + h] = v[h];
+            for (int j = 0; j < C; ++j) unpack_f32x2(acc[i][j], lo[j], hi[j]);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float* v = h == 0 ? lo : hi;
+                const int64_t gi = gi0 + 2 * i + h;
+                if (gi >= K || gj0 >= K || skip_row) continue;
+                float* hr = H + gi * K + gj0;
+                if (wide) {
+                    if (accumulate) {
+                        const float4 o = *reinterpret_cast<const float4*>(hr);
+                        v[0] = __fadd_rn(v[0], o.x);
+                        v[1] = __fadd_rn(v[1], o.y);
+                        v[C - 2] = __fadd_rn(v[C - 2], o.z);
+                        v[C - 1] = __fadd_rn(v[C - 1], o.w);
+                    }
+                    *reinterpret_cast<float4*>(hr) = make_float4(v[0], v[1], v[C - 2], v[C - 1]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < C; ++j)
+                        if (gj0 + j < K) {
+                            if (accumulate) v[j] = __fadd_rn(v[j], hr[j]);
+                            hr[j] = v[j];
+                        }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < C; ++j) acc[i][j] = pack_f32x2(lo[j], hi[j]);
+        }
+        if (!mirror) return;
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            if (gj0 + j >= K) continue;
+            float* hc = H + (gj0 + j) * K + gi0;
+#pragma unroll
+            for (int i = 0; i < R / 2; i += 2) {
+                float v[4];
+                unpack_f32x2(acc[i][j], v[0], v[1]);
+                unpack_f32x2(acc[i + 1][j], v[2], v[3]);
+                if (wide) {
+                    if (gi0 + 2 * i < K) *reinterpret_cast<float4*>(hc + 2 * i) = make_float4(v[0], v[1], v[2], v[3]);
+                } else {
+#pragma unroll
+                    for (int h = 0; h < 4; ++h)
+                        if (gi0 + 2 * i + h < K) hc[2 * i + h] = v[h];
+                }
             }
         }
-    }
+    } while (++t < end && PART == 1);
 }
 
 // Sec. 3.3 (as in GPTQ): the Hessian in processing order, a unit diagonal for input features that

@@ -1601,10 +1601,35 @@ int w4a8_hessian_accumulate(const void* x_bf16, int64_t T, int64_t K, int64_t ld
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // Tiles of 128 features once there are half as many as SMs, of 64 below (measured with 128 / 64, us:
     // (T, K) = (2000, 1024) 191 / 76, (1024, 1536) 105 / 113, (1024, 2560) 193 / 217, (1024, 4096) 367 / 507).
-    if (n128 * (n128 + 1) / 2 >= kNominalSMs / 2)
-        hessian_xtx_kernel<128><<<(unsigned)(n128 * (n128 + 1) / 2), 256, 0, st>>>(xb, T, K, ldx, H, accumulate ? 1 : 0);
-    else
-        hessian_xtx_kernel<64><<<(unsigned)(n64 * (n64 + 1) / 2), 256, 0, st>>>(xb, T, K, ldx, H, accumulate ? 1 : 0);
+    // Those of 128 are shared by tokens where whole ones leave a last round that is not full (hessian_split).
+    HessianSplit split = {0, 0, 0};
+    if (n128 * (n128 + 1) / 2 >= kNominalSMs / 2) {
+        const int n = (int)(n128 * (n128 + 1) / 2);
+        if (K % 128 == 0 && (reinterpret_cast<uintptr_t>(H) & 15u) == 0) split = hessian_split(n128, sm_count(), T, kHessTok);
+        else split.whole = n;
+        const int acc = accumulate ? 1 : 0;
+        if (split.cut) {
+            const int rest = n - split.whole, bundles = (rest + split.bundle - 1) / split.bundle;
+            hessian_xtx_kernel<128, 1><<<(unsigned)(split.whole + bundles), 256, 0, st>>>(xb, T, K, ldx, H, acc, split);
+            // The second is set up beside the end of the first and waits for its sums; but not where it has one CTA per SM, which would
+            // come to sit two to an SM where the first is through: K = 3584 281.9 us whole, 274.2 one after the other, 338.9 beside.
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = rest > sm_count() ? 1 : 0;
+            cfg.gridDim = dim3((unsigned)rest);
+            cfg.blockDim = dim3(256);
+            cfg.stream = st;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            cudaLaunchKernelEx(&cfg, hessian_xtx_kernel<128, 2>, xb, T, K, ldx, H, acc, split);
+            g_launches.fetch_add(1, std::memory_order_relaxed);
+        } else {
+            hessian_xtx_kernel<128, 0><<<(unsigned)n, 256, 0, st>>>(xb, T, K, ldx, H, acc, split);
+        }
+    } else {
+        hessian_xtx_kernel<64, 0><<<(unsigned)(n64 * (n64 + 1) / 2), 256, 0, st>>>(xb, T, K, ldx, H, accumulate ? 1 : 0, split);
+    }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return launch_status();
 }
