@@ -628,6 +628,7 @@ static bool half_rows_apply(int64_t M, int64_t N, int64_t K, int sms) {
 static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, int64_t M, const uint8_t* wpp,
                              int fmt, const float* s_w, int sw_stride, int64_t N, int64_t K, void* y, int64_t ldy,
                              int out_dtype, void* workspace, size_t workspace_bytes, cudaStream_t st, bool y_on_host) {
+    const int sms = sm_count();   // (once: a call of a small layer is bound by the host)
     if (M <= 16 && rows_workspace_usable(workspace, workspace_bytes) && (!y_on_host || M * N <= kHostFewOutputs)) {
         // (linear_direct_kernel cuts K between the warps of a CTA.  Without a workspace K is never cut, which is how a
         // caller asks for the bits of a chain launch.  An output in host memory it writes in pieces of 32 bytes, which the
@@ -635,17 +636,15 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
         // 3072) 17.1 / 16.8, (8, 6144, 2048) 15.9 / 17.2, (16, 6144, 2048) 19.1 / 24.1, (16, 8192, 1024) 19.3 / 24.0.)
         const int rc = check_device();
         if (rc != W4A8_OK) return rc;
-        const int sms_d = sm_count();
         DirPlan plan;
-        if (sms_d > 0 && direct_applies(M, N, K, fmt, sms_d, &plan))
+        if (sms > 0 && direct_applies(M, N, K, fmt, sms, &plan))
             return launch_direct(x8, ldx8, s_x, M, wpp, nullptr, nullptr, fmt, s_w, sw_stride, N, K, y, ldy, out_dtype, plan, st);
     }
-    const bool whole = M <= kRowsMaxM && whole_tiles_apply(M, N, K, fmt, sm_count(), y_on_host);
+    const bool whole = M <= kRowsMaxM && whole_tiles_apply(M, N, K, fmt, sms, y_on_host);
     if (M > 16 && !whole) {
         // 17..128 tokens on a layer with few 128-row tiles and a long K: K cut between the CTAs of a cluster (cluster_kcut_pays;
         // us against the exchange through L2: (64, 2048, 4096) 6.9 / 12.9, (100, 512, 8192) 7.6 / 15.1).
-        const int sms_c = sm_count();
-        const int cl0 = sms_c > 0 ? cluster_kcut_ctas(M, N, K, sms_c) : 0;
+        const int cl0 = sms > 0 ? cluster_kcut_ctas(M, N, K, sms) : 0;
         for (int cl = cl0; cl >= 2; --cl) {   // the largest cluster size of which all clusters are resident at once
             if (!cluster_kcut_pays(M, K, cl)) break;
             int rc = check_device();
@@ -668,12 +667,11 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
     if (M <= kRowsMaxM && !whole) {
         const int rc = check_device();
         if (rc != W4A8_OK) return rc;
-        const int sms_r = sm_count();
         const bool may_cut = M <= 16 && rows_workspace_usable(workspace, workspace_bytes);
-        const bool half = half_rows_apply(M, N, K, sms_r);
+        const bool half = half_rows_apply(M, N, K, sms);
 #define W4A8_ROWS(...)                                                                                                     \
     return launch_rows<RowsCfg<__VA_ARGS__>>(x8, ldx8, wpp, s_x, s_w, sw_stride, y, ldy, out_dtype, (int)M, (int)N, (int)K, \
-                                             workspace, may_cut, sms_r, st)
+                                             workspace, may_cut, sms, st)
         if (fmt == kFmtTiledSignMag) {
             if (half) W4A8_ROWS(kFmtTiledSignMag, true);
             W4A8_ROWS(kFmtTiledSignMag);
@@ -688,7 +686,6 @@ static int linear_tiled_impl(const uint8_t* x8, int64_t ldx8, const float* s_x, 
     }
     int rc = check_device();
     if (rc != W4A8_OK) return rc;
-    const int sms = sm_count();
     if (sms <= 0) return W4A8_ERR_CUDA;
     SkPlan pl;
     PrefillKind kind = kPrefillKinds;
