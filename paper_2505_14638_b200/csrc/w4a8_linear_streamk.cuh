@@ -79,6 +79,11 @@ struct SkCfg {
     static constexpr int FMT = FMT_;
     static constexpr bool CANON = FMT_ == kFmtCanonical;   // see the kernel's comment
     static constexpr bool kCut = !CL_ && !W8_ && !W16_ && !CANON;   // a tile may be shared through the workspace
+    // Expansion with ordinary shifts and sums instead of the multipliers (see SignMagLut): a step is paced by its MMAs, barriers and the
+    // latency of a row's expansion, not by the integer pipe.  us with the multipliers / so, zero-points: (256, 1584, 2432) 8.59 / 8.17,
+    // (512, 4096, 4096) 16.4 / 15.5, (1100, 2048, 6016) 22.0 / 20.7, 17..128 tokens 0.6 % less on average; sign-magnitude: (384,
+    // 4096, 4096) 13.8 / 13.2, (250, 6144, 4096) 13.1 / 12.8, but clusters 0.3 % more on average.
+    static constexpr bool kPlain = FMT_ == kFmtTiled || (FMT_ == kFmtTiledSignMag && !CL_);
     static constexpr int kMeta = meta_bytes(FMT);
     static constexpr int kCodeBytes = 8192;   // packed codes of the tile's rows for one k-block
     static constexpr int kWStage = CANON ? 8192 : 9216;  // rows x (64 code bytes + meta), padded to keep the activation tile 1024-aligned
@@ -758,7 +763,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                     next_meta(G);   // (past the last stage: a row that does not exist, or one that is not used)
                     dequant_canonical_row_to_tmem(stage_w(s1), m, r, a_col);
                 } else {
-                    dequant_row_to_tmem<Cfg::FMT>(stage_w(s1) + tiled_row_offset(r),
+                    dequant_row_to_tmem<Cfg::FMT, Cfg::kPlain>(stage_w(s1) + tiled_row_offset(r),
                                                   stage_w(s1) + (uint32_t)Cfg::kCodeBytes + (uint32_t)(r * Cfg::kMeta), a_col);
                 }
                 ptx::tmem_st_wait();
@@ -774,7 +779,7 @@ linear_streamk_kernel(const __grid_constant__ CUtensorMap tmap_x,  // X8 u8 [M][
                 next_meta(G);   // (past the last stage: a row that does not exist, or one that is not used)
                 dequant_canonical_row_to_smem(stage_w(s1), m, r, stage_w8(s2) + (uint32_t)r * 128u);
             } else
-                dequant_row_to_smem<Cfg::FMT>(stage_w(s1) + tiled_row_offset(r),
+                dequant_row_to_smem<Cfg::FMT, Cfg::kPlain>(stage_w(s1) + tiled_row_offset(r),
                                               stage_w(s1) + (uint32_t)Cfg::kCodeBytes + (uint32_t)(r * Cfg::kMeta), r,
                                               stage_w8(s2) + (uint32_t)r * 128u);
             ptx::fence_proxy_async_smem();

@@ -53,6 +53,7 @@ __host__ __device__ constexpr uint32_t row_offset(int fmt, int row) {
 // 12.1 with the shift on the integer pipe (registers to registers, four warps, one more multiply-add in both).
 // PLAIN: shifts and sums where they belong, for kernels that the power cap bounds and not the integer pipe: CTA pairs take (8192,
 // 28672, 8192) 1500 us so and 1514 the other way, with zero-points 1567 and 1572.
+// The persistent kernel: SkCfg::kPlain; linear_rows_kernel 6 % more so, (8, 28672, 4096) 16.3 and 15.3.
 struct SignMagLut {
     uint32_t t0, t1;
     __device__ __forceinline__ void build(float s) {
@@ -195,12 +196,12 @@ __device__ __forceinline__ void expand_row_to_smem(const uint32_t (&pk)[16], uin
                      : "memory");
     }
 }
-template <int FMT>
+template <int FMT, bool PLAIN = false>
 __device__ __forceinline__ void dequant_row_to_smem(uint32_t src, uint32_t meta, int row, uint32_t dst) {
     const uint32_t mbits = load_meta_word(meta, FMT);
     uint32_t pk[16];
     load_row_codes(src, pk);
-    expand_row_to_smem<FMT>(pk, mbits, row, dst);
+    expand_row_to_smem<FMT, PLAIN>(pk, mbits, row, dst);
 }
 
 // The same for a row of a canonical tile: the TMA tile of 64 bytes per row with the 64-byte swizzle at `tile`; scale
@@ -283,12 +284,12 @@ __device__ __forceinline__ void expand_row_to_tmem(const uint32_t (&pk)[16], uin
         ptx::tmem_st_32x32b_x16(taddr + 16u * h, out);
     }
 }
-template <int FMT>
+template <int FMT, bool PLAIN = false>
 __device__ __forceinline__ void dequant_row_to_tmem(uint32_t src, uint32_t meta, uint32_t taddr) {
     const uint32_t mbits = load_meta_word(meta, FMT);
     uint32_t pk[16];
     load_row_codes(src, pk);
-    expand_row_to_tmem<FMT>(pk, mbits, taddr);
+    expand_row_to_tmem<FMT, PLAIN>(pk, mbits, taddr);
 }
 
 // FP8 weights (W8A8 comparison scheme): the row's 128 bytes of the k-block go to tensor memory as they are.
