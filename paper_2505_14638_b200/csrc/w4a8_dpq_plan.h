@@ -55,8 +55,8 @@ struct DpqSteps {
 // Two CTAs to an SM share its FMA pipes, and one alone has nearly all of them, so that the time in tiles per SM is ceil(n / sms) where
 // all tiles are whole, 4 for 528 tiles on 148 SMs, which 3.57 would do.  With bundles of k tiles, each a k-th of its tokens, a bundle
 // takes as long as a tile, and the second launch (k - 1) / k of that for each CTA that an SM has of it.  The least of these is taken
-// where it spares a tenth of a tile and what 110 tokens of a tile take (10 us: the sums go out and come back, (256, 4480) 138.8 whole,
-// 140.7 shared).  Measured, us per call, whole / shared: (T, K) = (1024, 3072) 282 / 238, (1024, 3584) 282 / 274,
+// where it spares 1.5 % of the time (the loop over a bundle's tiles), a twelfth of a tile and what 110 tokens of a tile take (10 us: the
+// sums go out and come back): (256, 4480) 138.8 whole, 140.7 shared, (823, 4736) 372 and 375.  Measured, us per call, whole / shared: (T, K) = (1024, 3072) 282 / 238, (1024, 3584) 282 / 274,
 // (640, 4096) 240 / 230, (1024, 4096) 368 / 353, (2048, 4096) 711 / 670, (1024, 4480) 458 / 422, (2048, 5120) 1059 / 1027, (1024, 8192)
 // 1329 / 1309.
 struct HessianSplit {
@@ -66,7 +66,8 @@ inline HessianSplit hessian_split(long long nb, long long sms, long long tokens,
     const long long n = nb * (nb + 1) / 2, chunks = tokens / chunk;
     HessianSplit s = {(int)n, 0, 0};
     if (sms <= 0) return s;
-    double best = (double)((n + sms - 1) / sms) - 0.1 - 110.0 / (double)tokens;
+    const double whole = (double)((n + sms - 1) / sms);
+    double best = 0.985 * whole - 0.08 - 110.0 / (double)tokens;
     for (int k = 2; k <= 8 && chunks >= 8 * k; ++k)
         for (int rounds = 1; rounds <= 2; ++rounds) {
             const long long split = rounds * sms < n - nb ? rounds * sms : n - nb;
