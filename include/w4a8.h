@@ -127,7 +127,9 @@ size_t w4a8_linear_workspace_bytes(int64_t M, int64_t N, int64_t K, int weight_f
  * Offline re-layout of the stored weights (no arithmetic on values): canonical codes, scales and
  * zero-points -> a tiled buffer of w4a8_prepack_bytes(N, K, weight_format) bytes (128-byte
  * aligned) for weight_format W4A8_FMT_TILED or W4A8_FMT_TILED_SIGNMAG.  The dequantized weights
- * the linear layer sees are bit-identical to Eq. 10 on the canonical arrays.  If a code 0 is met
+ * the linear layer sees have the values of Eq. 10 on the canonical arrays (W4A8_FMT_TILED holds some
+ * zeros as -0, and a group of infinite scale with a code at its zero-point, where Eq. 10 is NaN, as NaN
+ * throughout: the row's outputs are NaN either way).  If a code 0 is met
  * while writing W4A8_FMT_TILED_SIGNMAG, bit 1 of the device status word is raised
  * (w4a8_query_device_status) and the buffer must not be used.  A buffer is read by the library that wrote it: the
  * order of bits inside it may change between versions, so what a program keeps in files is the canonical arrays.  (W4A8_FMT_TILED

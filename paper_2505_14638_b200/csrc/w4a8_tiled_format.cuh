@@ -78,9 +78,9 @@ struct SignMagLut {
 // top bit is clear and, since that bit asks for copies of the selected byte's sign bit, 0 where it is set: the expanded byte is
 // the sum a + d of two look-ups, without a carry, on the multipliers.  Eight weights take 5 instructions of the integer pipe
 // and 4 of the multipliers: 11.9 cycles (see SignMagLut), against 24.2 for the sixteen-entry table of DequantLut.
-// 0 <= s <= 448 in this format (prepack mirrors groups of negative scale; a larger one gives the same table as 448).  The zero-point is stored as BF16 with the bits 0x7FC0
-// flipped: one instruction restores it, and the integer zero-points of a buffer written before this form existed become NaN
-// and so do all outputs, instead of being read wrongly.
+// In this format s is 0..448 or NaN (prepack mirrors groups of negative scale; a larger finite one gives the same table as 448, for
+// an infinite one see there).  The zero-point is stored as BF16 with the bits 0x7FC0 flipped: one instruction restores it, and the
+// integer zero-points of a buffer written before this form existed become NaN and so do all outputs, instead of being read wrongly.
 constexpr uint32_t kPairZeroFlip = 0x7FC0u;
 struct PairLut {
     uint32_t a0, a1, d0, d1;
@@ -380,6 +380,13 @@ __device__ __forceinline__ uint32_t to_pair_word(uint32_t w, int z) {
     return out;
 }
 
+__device__ __forceinline__ bool has_code(uint32_t w, int z) {
+    bool has = false;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) has |= (int)((w >> (4 * i)) & 15u) == z;
+    return has;
+}
+
 __global__ void __launch_bounds__(128)
 prepack_kernel(const uint8_t* __restrict__ codes, const uint16_t* __restrict__ gscale,
                const uint8_t* __restrict__ gzero, int64_t N, int64_t K, int fmt, uint8_t* __restrict__ out,
@@ -405,6 +412,14 @@ prepack_kernel(const uint8_t* __restrict__ codes, const uint16_t* __restrict__ g
         }
         if (bad) atomicOr(status_word, kStatusBadCode);
     } else {
+        // An infinite scale: 0 x s is NaN, and one such weight makes all outputs of the row NaN, as a NaN scale does; a group
+        // without one has the values of 448.
+        if ((sc & 0x7FFFu) == 0x7F80u) {
+            bool zero = false;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) zero |= has_code(w[c].x, z) | has_code(w[c].y, z) | has_code(w[c].z, z) | has_code(w[c].w, z);
+            sc = zero ? 0x7FFFu : (sc & 0x8000u) | 0x43E0u;
+        }
         // (u - z) s = ((15 - u) - (15 - z)) (-s); from 448 on every value that is not zero saturates
         if (sc & 0x8000u) {
             sc ^= 0x8000u;
@@ -412,7 +427,7 @@ prepack_kernel(const uint8_t* __restrict__ codes, const uint16_t* __restrict__ g
 #pragma unroll
             for (int c = 0; c < 4; ++c) w[c] = make_uint4(~w[c].x, ~w[c].y, ~w[c].z, ~w[c].w);
         }
-        sc = sc > 0x43E0u && sc <= 0x7F80u ? 0x43E0u : sc;   // BF16 of 448
+        sc = sc > 0x43E0u && sc < 0x7F80u ? 0x43E0u : sc;   // BF16 of 448
 #pragma unroll
         for (int c = 0; c < 4; ++c)
             w[c] = make_uint4(to_pair_word(w[c].x, z), to_pair_word(w[c].y, z), to_pair_word(w[c].z, z), to_pair_word(w[c].w, z));

@@ -58,3 +58,27 @@ def test_a_buffer_of_integer_zero_points_reads_as_nan():
     meta.copy_(torch.arange(meta.numel(), device="cuda", dtype=torch.int32) % 16 << 16 | 0x3F80)
     x8, s_x = binding.quantize_act(torch.ones((4, K), dtype=torch.bfloat16, device="cuda"))
     assert bool(binding.linear_tiled(x8, s_x, tw).isnan().all())
+
+
+@pytest.mark.parametrize("M,N,K", [(4, 2048, 896), (16, 1024, 384), (64, 1040, 256), (256, 1040, 256)])
+def test_scales_that_are_not_finite(M, N, K):
+    # 0 x infinity is NaN, so an infinite scale gives NaN for the codes at the zero-point and +-448 for the others; one such
+    # weight, or a NaN scale, makes the row's outputs NaN.  Every other row has no code at the zero-point.
+    codes, gs, gz = _weights(N, K, 5)
+    u = torch.stack((codes & 15, codes >> 4), -1).reshape(N, K // 128, 128).int()
+    z = gz.int()[:, :, None]
+    u[::2] = torch.where(u[::2] == z[::2], (u[::2] + 1) % 16, u[::2])
+    u = u.reshape(N, K // 2, 2)
+    codes = (u[:, :, 0] | u[:, :, 1] << 4).to(torch.uint8).contiguous()
+    odd = bf16_dev(np.array([0x7F80, 0xFF80, 0x7F80, 0xFF80, 0x7FC0, 0xFFFF], dtype=np.uint16))
+    gs[:, K // 128 - 1] = odd[torch.arange(N, device="cuda") // 2 % 6]
+    one = torch.ones(1, device="cuda")
+    w = binding.dequant_weight(codes, gs, gz).view(torch.float8_e4m3fn).double()
+    x = torch.zeros((M, K), dtype=torch.bfloat16, device="cuda")
+    x[torch.arange(M, device="cuda"), torch.arange(M, device="cuda") * (K - 1) // (M - 1)] = 1.0
+    x8, s_x = binding.quantize_act(x, static_scale=one)
+    want = x.double() @ w.t()
+    assert bool(want.isnan().any()) and bool((want.abs() == 448).any())
+    y = binding.linear_tiled(x8, s_x, binding.prepack_weight(codes, gs, gz, one), out_dtype=binding.OUT_FP32).double()
+    assert binding.query_device_status() == 0
+    assert torch.equal(y.isnan(), want.isnan()) and torch.equal(y.nan_to_num(), want.nan_to_num())
