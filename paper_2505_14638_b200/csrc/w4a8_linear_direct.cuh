@@ -44,14 +44,6 @@ struct DirCfg {
     static_assert(NT == 1 || NT == 2, "up to sixteen tokens");
 };
 
-// Launch-time plan.
-struct DirPlan {
-    int P;    // CTAs; CTA p takes units [p NU / P, (p + 1) NU / P)
-    int Wq;   // warps that share a row tile's k-block quads
-    int Tc;   // row tiles in progress at once (Wq * Tc <= 16)
-    int xpitch;   // bytes between two tokens in shared memory
-};
-
 namespace direct {
 __device__ __forceinline__ void mma_e4m3(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                          uint32_t b1) {

@@ -37,40 +37,19 @@
 
 #include <cuda_bf16.h>
 
+#include "w4a8_decode_plan.h"
 #include "w4a8_ptx.cuh"
 #include "w4a8_tiled_format.cuh"
 
 namespace w4a8 {
 
-struct RowsPlan {
-    int T;       // runs of rows x parts of K; CTA p takes tiles p, p + gridDim.x, ... (cut: one tile each)
-    int cut;     // parts of K (1: none; above, the partial sums meet in the workspace)
-    int units, more;   // units of eight rows in a run; the first `more` runs have one more
-    int RB;      // blocks of 128 rows in a run (1 or 2)
-    int MN;      // tokens rounded up to sixteen
-    int S1;      // ring of packed stages
-    int S2;      // ring of expanded stages and their activation tiles
-    int whalf;   // bytes of a k-block in a slot of the first
-    int smem;
-};
-
 template <int FMT_, bool HALF_ = false>
-struct RowsCfg {
+struct RowsCfg : RowsSizes<FMT_, HALF_> {
     static constexpr int FMT = FMT_;
     static constexpr bool HALF = HALF_;         // half an SM per CTA (see the kernel's comment)
-    static constexpr int G = HALF_ ? 2 : 4;     // expansion groups
-    static constexpr int kMeta = meta_bytes(FMT_);
-    static constexpr int kS1Max = 16, kS2Max = 8;
-    static constexpr int kThreads = 128 + 128 * G;
+    static constexpr int kThreads = 128 + 128 * RowsSizes<FMT_, HALF_>::G;
     // (registers: 80 a thread, 640 threads of them leave room for the quantization kernel's CTA beside them; so do 2 x 384)
     static constexpr int kBoundThreads = HALF_ ? kThreads : 768, kBoundCtas = HALF_ ? 2 : 1;
-    static constexpr int kTmemCols = HALF_ ? 256 : 512;
-    static constexpr int kStageBytes = 1024;                    // per warp: 16 tokens x 32 rows of outputs (FP32: 8 tokens)
-    static constexpr int kOutBytes = 4 * G * kStageBytes;
-    static constexpr int kBarBytes = 512;
-    static constexpr int kSmemBudget = (HALF_ ? 110 : 224) * 1024;
-    static constexpr int kFixed = kOutBytes + kBarBytes + 1024;
-    static_assert((2 * kS1Max + 2 * kS2Max + 3) * 8 + 16 <= kBarBytes, "barrier area");
 };
 
 template <class Cfg>

@@ -20,23 +20,15 @@
 #include <cuda_bf16.h>
 
 #include "w4a8_common.cuh"
+#include "w4a8_decode_plan.h"
 #include "w4a8_ptx.cuh"
 
 namespace w4a8 {
 
-constexpr int kFmtCanonical = W4A8_FMT_CANONICAL;
-constexpr int kFmtTiled = W4A8_FMT_TILED;
-constexpr int kFmtTiledSignMag = W4A8_FMT_TILED_SIGNMAG;
-constexpr int kFmtTiledFp8 = W4A8_FMT_TILED_FP8;   // FP8 weights (W8A8 comparison scheme): 128 bytes per row and k-block, no meta data
-
-constexpr int kRowCodeBytes = 64;  // one row of one k-block: 128 INT4 codes
 constexpr uint32_t kChunkStride = 128;  // bytes between two chunks of one row
 // Offset of a row's first chunk within a piece of codes that starts on a multiple of eight rows.
 __host__ __device__ constexpr uint32_t tiled_row_offset(int row) {
     return (uint32_t)(row >> 3) * 512u + (uint32_t)(row & 7) * 16u;
-}
-__host__ __device__ constexpr int meta_bytes(int fmt) {
-    return fmt == kFmtTiledSignMag ? 2 : (fmt == kFmtTiled ? 4 : 0);   // (FP8: none; canonical: in arrays of their own)
 }
 // Bytes of one row of one k-block, and the offset of a row's first 16-byte chunk within a piece that
 // starts on a multiple of eight rows (chunk c of the row sits c * 128 bytes further), per format.
