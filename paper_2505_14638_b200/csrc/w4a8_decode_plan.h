@@ -65,18 +65,28 @@ struct RowsSizes {
 //   M <= 8   (8064, 256) 4.0 / 4.4 / 4.2, (992, 640) 4.4 / 4.6 / -, (672, 1792) 6.0 / 7.0 / -, (8656, 2560) 7.9 / 8.5 / 8.9
 //   M <= 16  (4672, 896) 4.8 / 5.5 / 5.9, (5312, 1408) 5.4 / 7.2 / 6.5, (8048, 2176) 6.9 / 8.5 / 10.0, (1344, 3456) 9.3 / 7.4 / 7.6
 //   above    (57, 11776, 640) 5.3 / 5.8 / -, (126, 7360, 512) 5.6 / 6.2 / 9.6, (46, 7872, 1024) 5.4 / 5.7 / 7.1, (29, 800, 1920) 6.4 / 6.8 / 5.5
-// The limits follow 1000 shapes of 512..20000 channels; the kernel taken is 0.4 % slower than the fastest on average.  With more
-// tiles than half the SMs the rows of linear_rows_kernel fill all SMs as well: there K up to 512 (up to sixteen tokens), 1024
-// or 2048 (more than 32), this over that 0.95, 0.99, 0.97.
+// The limits follow 1050 shapes of up to 16 tokens and 560 of 17..128, timed that way and as linear layers alone, back to back, as a
+// caller has it that runs several on one X8.  With more tiles than half the SMs linear_rows_kernel fills all SMs as well: there
+// K up to 512 for so many tiles (up to sixteen tokens; CTAs of half an SM above, us with quantization, alone: (8, 14384, 512) 4.7, 4.2
+// here and 4.6, 3.5 there, (6, 11104, 512) 4.3, 3.6 and 4.5, 3.1, (12, 18128, 256) 4.2, 3.7 and 4.2, 2.8), or K up to 1024, above 32 tokens
+// 2432 or 3072 ((106, 9616, 2176) 8.6, 7.4 and 8.6, 8.2; with zero-points (101, 16080, 2304) 9.7, 8.7 and 10.3, 9.8).  More tiles than
+// SMs: two k-blocks with zero-points ((108, 24032, 256) 6.9, 6.6 and 7.4, 6.8), and where a run of rows would exceed 256 and a second round comes to be all
+// but empty ((124, 39040, 1024) 14.1, 11.8 and 15.9, 15.3).
 // Outputs in host memory: always where there are more tiles than half the SMs and more than sixteen tokens; the bus takes its
 // stores better, (77, 28672, 4096) 119 us host to host against 128.  Up to sixteen tokens not for more than kHostFewOutputs, like
 // linear_direct_kernel.
 inline bool whole_tiles_apply(int64_t M, int64_t N, int64_t K, int fmt, int sms, bool y_on_host) {
     const int64_t tiles = (N + 127) / 128;
+    const bool sm = fmt == kFmtTiledSignMag;
     if (y_on_host && M <= 16 && M * N > kHostFewOutputs) return false;
-    if (2 * tiles > sms) return (tiles <= sms && K <= (M > 32 ? 2048 : (M > 16 ? 1024 : 512))) || (y_on_host && M > 16);
+    if (2 * tiles > sms) {
+        if (M <= 16) return K <= 512 && 20 * tiles <= sms * (K > 384 ? 14 : 17);
+        if (y_on_host) return true;
+        if (tiles > sms) return N > (int64_t)256 * sms ? K <= 2048 : !sm && K <= 256 && 2 * tiles <= 3 * sms;
+        return K <= (M <= 32 ? 1024 : (sm ? 2432 : 3072));
+    }
     if (M > 16) return 100 * (K / 128) <= 800 + 12 * M;
-    return K <= (N < 1024 ? 2304 : (fmt == kFmtTiledSignMag ? 2944 : 2688));
+    return K <= (N < 1024 ? 2304 : (4 * tiles > sms ? 3072 : (sm ? 2944 : 2688)));
 }
 
 // 17..128 tokens: whether cutting the tiles' K between the CTAs of clusters of `cl` pays for the exchange of the partial sums: the
@@ -132,6 +142,9 @@ inline int64_t make_direct_plan(int64_t N, int64_t K, int sms, DirPlan* plan) {
 //   M <= 16  (2752, 512) 5.4 / 4.1 / 4.7, (1072, 1920) 5.3 / 6.4 / 7.5, (3472, 1280) 6.1 / 5.2 / 6.9, (2352, 8064) 10.9 / 19.8 / 9.0
 // (Up to 2.2 million weights from nine tokens on: launched one by one such a layer is bound by the host's calls, of which the tensor map
 // of the other kernels takes 0.3 us: (16, 1024, 1024) 5.8 against 6.1 us; replayed from a graph it takes 5.3 against 4.8.)
+// And layers of which every warp has one unit of work, up to four tokens with a longer K, nine to twelve of up to 4 million weights
+// (with quantization, alone; this / linear_rows_kernel with CTAs of half an SM): (1, 2048, 7168) 7.0, 5.4 / 7.6, 6.4, (4, 3888, 3456) 7.0, 5.3 / 7.3,
+// 5.8, (1, 4096, 4096) 7.3, 6.0 / 7.5, 5.9; (12, 2304, 1664) 5.4, 3.5 / whole tiles 5.8, 4.3.
 // Layers of more 128-channel tiles than half the SMs keep the kernels that walk all of K in one chain of MMAs: a chain launch gives
 // the same bits there, and this one is the slower by (14352, 512) 4.6 / 4.6 to (16640, 512) 6.3 / 4.9.
 // Canonical, against the kernel of one tile per CTA: M = 8 (1024, 1024) 0.46, (6144, 4096) 0.87, (12288, 2048) 0.81; M = 16 (6144,
@@ -144,6 +157,7 @@ inline bool direct_applies(int64_t M, int64_t N, int64_t K, int fmt, int sms, Di
     if (fmt == kFmtCanonical)
         return rounds <= 2 && weights <= (few || K <= 4096 || K > 8192 ? 26 : 16) * (int64_t)1000000 && (K <= 11008 || M <= 4);
     if (2 * ((N + 127) / 128) > sms) return false;
+    if (rounds == 1 && (M <= 4 ? K >= 2304 : (M > 8 && M <= 12 && K >= 1408 && weights <= 4000000))) return true;
     const bool sm = fmt == kFmtTiledSignMag;
     return few ? weights <= 8000 * K - (sm ? 2000000 : 3000000) && weights <= (sm ? 12000000 : 10000000)
                : K >= 1024 && weights <= 8000000 && (weights <= 5000 * K - 5000000 || weights <= 2200000);
@@ -151,15 +165,17 @@ inline bool direct_applies(int64_t M, int64_t N, int64_t K, int fmt, int sms, Di
 
 // Up to 128 tokens: the plan of linear_rows_kernel.  K is cut (may_cut: up to sixteen tokens, with a workspace) where the
 // channels make less than half as many runs of 128 rows as there are SMs.
+inline int64_t rows_cut(int64_t N, int64_t K, int sms, bool may_cut) {
+    const int64_t blocks = (N + 127) / 128;
+    if (!may_cut || blocks * 2 > sms) return 1;
+    int64_t cut = sms / blocks;
+    if (cut > K / 512) cut = K / 512;   // at least four k-blocks per part
+    return cut < 1 ? 1 : cut;
+}
 template <class Cfg>
 inline void make_rows_plan(int64_t M, int64_t N, int64_t K, int sms, bool may_cut, RowsPlan* pl) {
-    const int64_t NU = N / 8, P = sms < NU ? sms : NU, blocks = (N + 127) / 128;
-    int64_t cut = 1, runs;
-    if (may_cut && blocks * 2 <= sms) {
-        cut = sms / blocks;
-        if (cut > K / 512) cut = K / 512;   // at least four k-blocks per part
-        if (cut < 1) cut = 1;
-    }
+    const int64_t NU = N / 8, P = sms < NU ? sms : NU, cut = rows_cut(N, K, sms, may_cut);
+    int64_t runs;
     if (cut > 1) {
         runs = sms / cut;
         if (runs > NU) runs = NU;
@@ -184,11 +200,23 @@ inline void make_rows_plan(int64_t M, int64_t N, int64_t K, int sms, bool may_cu
     pl->smem = Cfg::kFixed + pl->S2 * x + pl->S1 * slot;
 }
 
-// Up to sixteen tokens on layers of more 128-channel tiles than half the SMs, short K: CTAs of half an SM, so that the next launch's set up,
-// fetch and expand beside this one's.  Against the better of whole tiles and full-SM rows, 55 shapes: K up to 512 1.03 times the
-// time, to 896 0.95, to 1664 0.96, to 2304 1.02, to 3072 1.18; with fewer tiles slower throughout.
-inline bool half_rows_apply(int64_t M, int64_t N, int64_t K, int sms) {
-    return M <= 16 && 2 * ((N + 127) / 128) > sms && K <= 1664;
+// Up to sixteen tokens: CTAs of half an SM, so that the next launch's set up, fetch and expand beside this one's, where their main loop
+// is short, since a CTA that has the SM to itself expands with half its warps.  Time of these over that of whole SMs, with quantization and
+// alone, all of 1050 shapes but those that other kernels take:
+//   more 128-channel tiles than half the SMs, K up to 1664 0.94, 0.73, to 2048 0.97, 0.80, to 3072 1.22, 0.88, to 6144 1.43, 0.93
+//   K cut, k-blocks of a part: up to 8, M <= 12 0.98, 0.91; 13..16 1.08, 1.05
+//                              9 or 10, M <= 4 1.00, 0.90; 5..12 1.05, 0.89
+//                              11 to 14, M <= 4 1.03, 0.90 (11 of K up to 4352 0.95, 0.92); 5..12 1.14, 0.92
+//                              more, M <= 4 1.22, 0.93; 5..12 1.26, 0.92
+// us: (8, 4096, 4096) 7.6, 6.0 / 7.7, 7.6, (9, 4400, 3072) 7.2, 5.6 / 7.5, 7.5, (1, 5344, 3328) 7.3, 6.5 / 8.0, 7.4, (2, 13712, 1920) 6.7,
+// 5.0 / 7.1, 6.6; (8, 6144, 4096), 11 k-blocks, 8.9, 7.3 / 8.5, 7.9, (8, 4096, 14336), 28, 16.2, 10.2 / 12.5, 11.9.  With many parts of a
+// very long K more than four tokens lose as well, (8, 1296, 12288) 8.8, 7.1 / 8.3, 7.3.  (Between launches that take whole SMs nothing
+// starts beside these either: a block of qkv, o, gate_up and down with 8 tokens, o here, takes 51.2 us, o on whole SMs 50.7.)
+inline bool half_rows_apply(int64_t M, int64_t N, int64_t K, int sms, bool may_cut) {
+    if (M > 16) return false;
+    if (2 * ((N + 127) / 128) > sms) return K <= 2048;
+    const int64_t cut = rows_cut(N, K, sms, may_cut), blocks = (K / 128 + cut - 1) / cut;
+    return cut > 1 && (M <= 4 ? blocks <= (K <= 4352 ? 11 : 10) : (M <= 12 && blocks <= 8 && K <= 12000));
 }
 
 enum DecodeKind {
@@ -206,7 +234,7 @@ struct DecodePlan {
 };
 template <int FMT>
 inline DecodeKind decode_rows_choice(int64_t M, int64_t N, int64_t K, int sms, bool may_cut, DecodePlan* plan) {
-    if (half_rows_apply(M, N, K, sms)) {
+    if (half_rows_apply(M, N, K, sms, may_cut)) {
         make_rows_plan<RowsSizes<FMT, true>>(M, N, K, sms, may_cut, &plan->rows);
         return kDecodeRowsHalf;
     }
@@ -235,6 +263,9 @@ inline DecodeKind decode_choice(int64_t M, int64_t N, int64_t K, int fmt, int sm
                 plan->cluster = cl;
                 return kDecodeCluster;
             }
+        // (With zero-points whole tiles are the better ones where clusters do not pay, us against rows: (120, 2048, 2944) 9.6 / 10.9, (54,
+        // 6336, 2304) 7.5 / 8.3, (126, 7776, 4864) 14.6 / 15.0; sign-magnitude level, (98, 3488, 2688) 9.0 / 9.0.)
+        if (fmt == kFmtTiled && 2 * ((N + 127) / 128) <= sms && K <= 5120) return kDecodeWhole;
     }
     const bool may_cut = M <= 16 && workspace;
     return fmt == kFmtTiledSignMag ? decode_rows_choice<kFmtTiledSignMag>(M, N, K, sms, may_cut, plan)

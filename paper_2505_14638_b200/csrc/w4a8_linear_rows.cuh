@@ -23,7 +23,8 @@
 // K cut (up to sixteen tokens, few channels): each CTA takes part of a run's k-blocks and leaves its sums in the workspace; the CTA
 // that arrives last adds them in ascending order of the parts.  HALF: two expansion groups, half the shared and tensor
 // memory, so that the CTAs of two launches share an SM and the second is set up and has expanded its first stages when its
-// activations come: better only for a short K, where the main loop does not hide that (half_rows_apply).
+// activations come, or the launch before is through: better only where a CTA walks a short K and the main loop does not hide
+// that (half_rows_apply).
 //
 // Each accumulator is one chain of MMAs over K in ascending order: where K is not cut, the bits of a chain launch.
 //

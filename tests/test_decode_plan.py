@@ -1,5 +1,6 @@
 """Host-side checks of csrc/w4a8_decode_plan.h, compiled here with the host compiler: what linear_rows_kernel's waits and memory
-rely on holds for every plan, every row and k-block is taken once, and without a number of SMs there is no plan."""
+rely on holds for every plan, every row and k-block is taken once, without a number of SMs there is no plan, and the shapes of the
+GPU tests take the kernels they stand for."""
 import ctypes
 import os
 import random
@@ -8,10 +9,10 @@ import subprocess
 import pytest
 
 from paper_2505_14638_b200 import build
+from decode_shapes import KINDS, RESIDENT, SHAPES, SMS
 
 NONE, DIRECT, WHOLE, CLUSTER, ROWS, HALF = range(6)
 TILED, SIGNMAG = 1, 2
-SMS = 148
 
 SHIM = r"""
 #include "w4a8_decode_plan.h"
@@ -55,10 +56,9 @@ def lib(tmp_path_factory):
     return lib
 
 
-def _route(lib, M, N, K, fmt, sms=SMS, workspace=True, on_host=False, clusters=True):
+def _route(lib, M, N, K, fmt, sms=SMS, workspace=True, on_host=False, resident=RESIDENT):
     plan = DecodePlan()
-    resident = (ctypes.c_int * 9)(*[sms // max(s, 1) if clusters else -1 for s in range(9)])
-    return lib.route(M, N, K, fmt, sms, workspace, on_host, resident, ctypes.byref(plan)), plan
+    return lib.route(M, N, K, fmt, sms, workspace, on_host, (ctypes.c_int * 9)(*resident), ctypes.byref(plan)), plan
 
 
 def _shapes():
@@ -71,8 +71,8 @@ def _shapes():
 def test_plans_of_rows_hold_what_the_kernel_relies_on(lib):
     seen = set()
     for M, N, K, fmt, workspace in _shapes():
-        for clusters in (True, False):
-            kind, plan = _route(lib, M, N, K, fmt, workspace=workspace, clusters=clusters)
+        for resident in (RESIDENT, [-1] * 9):
+            kind, plan = _route(lib, M, N, K, fmt, workspace=workspace, resident=resident)
             assert kind != NONE
             if kind not in (ROWS, HALF):
                 continue
@@ -93,7 +93,8 @@ def test_plans_of_rows_hold_what_the_kernel_relies_on(lib):
             if p.cut > 1:   # a CTA per part; counters per run and partial sums in the workspace
                 assert M <= 16 and workspace and p.T <= SMS and p.RB == 1 and K // 128 >= 4 * p.cut, what
             seen.add((kind, p.cut > 1, p.RB, p.T > SMS))
-    assert {(ROWS, True, 1, False), (ROWS, False, 2, False), (ROWS, False, 2, True), (HALF, False, 1, False)} <= seen
+    assert {(ROWS, True, 1, False), (ROWS, False, 2, False), (ROWS, False, 2, True), (HALF, False, 1, False),
+            (HALF, True, 1, False)} <= seen
 
 
 @pytest.mark.parametrize("M,N,K", [(1, 4096, 4096), (8, 1024, 1024), (16, 28672, 4096), (32, 4096, 4096), (128, 28672, 4096)])
@@ -101,3 +102,22 @@ def test_no_number_of_sms_is_an_error_and_not_a_division(lib, M, N, K):
     for sms in (0, -1):
         for workspace in (True, False):
             assert _route(lib, M, N, K, SIGNMAG, sms=sms, workspace=workspace)[0] == NONE
+
+
+@pytest.mark.parametrize("kind", sorted(SHAPES))
+def test_shapes_of_the_gpu_tests_take_the_kernels_they_stand_for(lib, kind):
+    rings = set()
+    for M, N, K, symmetric in SHAPES[kind]:
+        got, plan = _route(lib, M, N, K, SIGNMAG if symmetric else TILED, resident=RESIDENT)
+        assert KINDS[got] == kind, (M, N, K, symmetric, KINDS[got])
+        rings.add((plan.rows.RB, plan.rows.S1, plan.rows.S2, plan.rows.cut > 1, plan.rows.T > SMS))
+    if kind == "rows":
+        assert (1, 4, 4, False, False) in rings and {r[3:] for r in rings} == {(True, False), (False, False), (False, True)}
+    if kind == "rows_half":
+        assert {r[3:] for r in rings} == {(True, False), (False, False), (False, True)}
+
+
+def test_without_a_workspace_k_is_not_cut(lib):
+    for M, N, K, fmt, _ in _shapes():
+        kind, plan = _route(lib, M, N, K, fmt, workspace=False)
+        assert M > 16 or kind == WHOLE or plan.rows.cut == 1

@@ -380,7 +380,10 @@ def test_host_forward_on_pinned_buffers_leaves_large_outputs_to_the_split_n_kern
 
 
 @pytest.mark.parametrize("M,N,K", [(1, 1024, 128), (4, 8192, 384), (8, 4096, 896), (3, 2384, 1152), (16, 3600, 1024), (12, 9472, 1024),
-                                   (7, 9488, 2048), (8, 10256, 2048), (13, 4112, 2048), (5, 5136, 2560), (16, 1024, 7168)])
+                                   (7, 9488, 2048), (8, 10256, 2048), (13, 4112, 2048), (5, 5136, 2560), (16, 1024, 7168),
+                                   # both sides of the limits on prepacked layers: the kernel for small layers, another one
+                                   (8, 4864, 640), (8, 4880, 640), (8, 4256, 2816), (8, 4272, 2816), (4, 2048, 7168), (12, 2304, 1664),
+                                   (13, 2304, 1664), (9, 2112, 1024), (9, 2160, 1024), (16, 3040, 2560), (16, 3088, 2560)])
 def test_small_layers_in_bf16_at_the_edges_of_their_rule(M, N, K):
     # The kernel for small layers stores its own rounding of the sums: small whole numbers and powers of two, so that the
     # sums are exact in any order and the BF16 result is one rounding of them, bit for bit.

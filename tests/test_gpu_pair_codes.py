@@ -25,7 +25,9 @@ def _weights(N, K, seed):
 
 
 @pytest.mark.parametrize("M,N,K", [(1, 1024, 256), (16, 1024, 384), (8, 19216, 256), (64, 1040, 256), (100, 19216, 128),
-                                   (256, 1040, 256), (640, 9616, 640)])
+                                   (256, 1040, 256), (640, 9616, 640),
+                                   # weights to registers: also an odd number of units per CTA, k-blocks that are no multiple of four
+                                   (8, 2048, 896), (16, 1024, 2048), (5, 2384, 640), (16, 1216, 1792)])
 @pytest.mark.parametrize("chain", [False, True])
 def test_every_zero_point_expands_to_the_dequantized_weights(M, N, K, chain):
     if chain and M > 16:

@@ -28,7 +28,8 @@ def _layer(M, N, K, asym):
 @pytest.mark.parametrize("M,N,K", [
     (1, 18944, 2176), (16, 18960, 2304), (8, 37888, 1792), (3, 37904, 1920),      # 128 / 136 / 256 rows a run, two runs a CTA
     (17, 9488, 4224), (64, 19216, 2176), (65, 18944, 2304), (128, 28688, 2176), (100, 37904, 2304),
-    (128, 9472, 2944), (40, 8720, 2176),                                          # few tiles, K not cut
+    (128, 7664, 3072), (44, 6384, 1792),                   # few tiles, K not cut (sign-magnitude; with zero-points whole tiles)
+    (128, 18944, 3200),                                    # with zero-points as many stages as groups in both rings
     (16, 1552, 14336), (9, 1024, 8320), (1, 4096, 5760), (12, 9472, 3456), (2, 128, 4096), (4, 16, 4224),   # K cut
     (1, 9488, 640), (16, 18960, 1408), (5, 37904, 896)])                          # half an SM
 def test_rows_in_runs(M, N, K, asym):
@@ -61,11 +62,23 @@ def test_rows_of_y_that_wide_stores_do_not_fit(M, N, K, dtype):
     assert torch.equal(wide.t[:, :N], want) and bool((wide.t[:, N:] == 7.0).all())
 
 
+@pytest.mark.parametrize("asym", [False, True])
 @pytest.mark.parametrize("M,N,K", [(4, 1552, 8320), (16, 4096, 4096), (3, 18960, 2176)])
-def test_without_a_workspace_k_is_not_cut(M, N, K):
-    # the bits of one chain of sums over K, which is what a chain launch computes where it does not cut K
-    x8, s_x, tw, ref, mag = _layer(M, N, K, False)
+def test_without_a_workspace_k_is_not_cut(M, N, K, asym):
+    # The bits of one chain of sums over K: of a chain launch on the layer's rows, repeated until every SM has a whole block of 96 of
+    # them, whose K it does not cut.
+    W = torch.from_numpy(inputs.make_weight(N, K, 0.02, seed=M + N + K)).cuda()
+    q = binding.quantize_weight_rtn(W, symmetric=not asym, per_channel=False)
+    x = bf16_dev(inputs.make_activation(M, K, M + K, 0.01, 20.0))
+    x8, s_x = binding.quantize_act(x)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    whole = 96 * sms
+    rows = torch.arange(max(whole, N) // 16 * 16, device="cuda") % N
+    many = binding.prepack_weight(*[None if t is None else t[rows].contiguous() for t in q[:3]], q[3])
+    chain = torch.zeros((M, rows.numel()), dtype=torch.float32, device="cuda")
+    binding.LinearChain([dict(x=x, weight=many, y=chain)])()
     tiny = torch.zeros(16, dtype=torch.uint8, device="cuda")
-    y = [binding.linear_tiled(x8, s_x, tw, out_dtype=binding.OUT_FP32, workspace=tiny) for _ in range(3)]
-    assert torch.equal(y[0], y[1]) and torch.equal(y[0], y[2])
-    assert bool(((y[0].double() - ref).abs() <= 4.0 * K * 2.0 ** -24 * mag + 1e-30).all())
+    y = binding.linear_tiled(x8, s_x, binding.prepack_weight(*q), out_dtype=binding.OUT_FP32, workspace=tiny)
+    assert binding.query_device_status() == 0
+    n = min(N, whole)
+    assert torch.equal(y[:, :n], chain[:, :n])
