@@ -476,12 +476,11 @@ int w4a8_forward_host(const void* x_host_bf16, int64_t M, const uint8_t* weights
 /*
  * Reads and clears the device-side status word (synchronises the device).  *flags receives a
  * bit mask: bit 0 = a bounded wait inside a kernel gave up; bit 1 = w4a8_prepack_weight met a
- * code its target format cannot hold; bit 2 = the run-time placement of a decode launch
- * (w4a8_linear, M <= 16 on tiled weights) ended with a worker index unissued.  Bits 0 and 2 mean
- * that the outputs of some launch are incomplete: returns W4A8_ERR_TIMEOUT; W4A8_ERR_BAD_SHAPE when
+ * code its target format cannot hold; the others are unused.  Bit 0 means that the outputs of some
+ * launch are incomplete: returns W4A8_ERR_TIMEOUT; W4A8_ERR_BAD_SHAPE when
  * only bit 1 was set, W4A8_OK otherwise.  After W4A8_ERR_TIMEOUT the workspaces of w4a8_linear
  * calls that were in flight must be zero-filled again before they are reused (their split-K
- * counters and placement state may have been left part-way); the workspace of w4a8_linear_chain
+ * counters may have been left part-way); the workspace of w4a8_linear_chain
  * needs no such care (its last CTA clears it after an aborted launch too).
  */
 int w4a8_query_device_status(unsigned int* flags_host);

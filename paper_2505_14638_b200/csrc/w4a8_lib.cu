@@ -1667,7 +1667,7 @@ int w4a8_query_device_status(unsigned int* flags_host) {
     if (cudaMemcpyFromSymbol(&v, g_status_word, sizeof v) != cudaSuccess) return W4A8_ERR_CUDA;
     if (v != 0 && cudaMemcpyToSymbol(g_status_word, &zero, sizeof zero) != cudaSuccess) return W4A8_ERR_CUDA;
     *flags_host = v;
-    if (v & (kStatusTimeout | kStatusPlacement)) return W4A8_ERR_TIMEOUT;   // outputs of some launch are incomplete
+    if (v & kStatusTimeout) return W4A8_ERR_TIMEOUT;   // outputs of some launch are incomplete
     return (v != 0) ? W4A8_ERR_BAD_SHAPE : W4A8_OK;
 }
 

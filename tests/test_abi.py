@@ -39,7 +39,7 @@ def test_workspace_and_prepack_size_queries_are_host_only(L):
     assert L.w4a8_prepack_bytes(14336, 4096, binding.FMT_TILED_SIGNMAG) == 14336 * 32 * 66
     assert L.w4a8_prepack_bytes(14336 + 16, 4096, binding.FMT_TILED) == (14336 + 16) * 32 * 68
     assert L.w4a8_prepack_bytes(14336, 4096, binding.FMT_CANONICAL) == 0
-    assert binding.linear_workspace_bytes(16, 14336, 4096, weight_format=binding.FMT_TILED_SIGNMAG) == 65536 + 160 * 128 * 128 * 4   # control area of fixed size (counters, placement state), partial tiles
+    assert binding.linear_workspace_bytes(16, 14336, 4096, weight_format=binding.FMT_TILED_SIGNMAG) == 65536 + 160 * 128 * 128 * 4   # control area of fixed size (counters), partial tiles
     ws = binding.linear_workspace_bytes(2048, 4096, 4096, weight_format=binding.FMT_TILED_SIGNMAG)
     assert ws >= 2 * 8 * 32 * 4 + 2 * 148 * 256 * 128 * 4
     assert binding.linear_workspace_bytes(2048, 4096, 4096) == 0          # large M: no split

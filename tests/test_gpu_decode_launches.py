@@ -1,10 +1,6 @@
-"""GPU: the decode-sized launches hand out their worker indices at run time (twice as many CTAs
-as workers, at most one worker per SM and launch).  The state of a launch lives in the caller's
-workspace, behind the split-K counters, and is cleared by the last CTA to enter; launches without
-a workspace use an entry of a 64-entry table in the library image.  Whatever the placement, every
-row range must be computed exactly once: long runs of launches -- more than the table has entries,
-eager and replayed from one CUDA graph, alternating shapes, from two streams -- must reproduce the
-first result bit for bit, and that result must match the oracle."""
+"""GPU: long runs of decode-sized launches, whose starts overlap the launches before -- eager and replayed from one CUDA graph,
+alternating shapes and kernels, from two streams, with and without a workspace -- must reproduce the first result bit for bit,
+and that result must match the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -30,8 +26,7 @@ def _case(M, N, K, seed):
 
 
 def test_many_launches_repeat_the_first_result():
-    # K = 2048 and K = 4096 walk 16 and 32 k-blocks per tile (run-time worker indices);
-    # N = 18960 gives ragged ranges, N = 37904 two tiles per worker
+    # CTAs of half an SM and of a whole one; N = 18960 gives runs of two lengths, N = 37904 two runs per CTA
     cases = [_case(16, 18960, 2048, 5), _case(3, 37904, 4096, 7)]
     outs = [torch.empty((c[1].shape[0], c[0].N), dtype=torch.float32, device="cuda") for c in cases]
     first = []
@@ -41,7 +36,7 @@ def test_many_launches_repeat_the_first_result():
         worst, _ = fp32_gate(out.cpu().numpy(), y64, rel=2e-3)
         assert worst <= 2e-3, worst
         first.append(out.clone())
-    # eager: 150 launches (more than two rounds of the 64 slots), alternating the two shapes
+    # eager: 150 launches, alternating the two shapes
     for i in range(150):
         tw, x8, s_x, _, ws = cases[i & 1]
         outs[i & 1].fill_(float("nan"))
@@ -50,7 +45,7 @@ def test_many_launches_repeat_the_first_result():
             assert torch.equal(outs[i & 1], first[i & 1]), i
     torch.cuda.synchronize()
     assert binding.query_device_status() == 0
-    # one graph with 70 launches (slots repeat inside the graph), replayed several times
+    # one graph with 70 launches, replayed several times
     side = torch.cuda.Stream()
     side.wait_stream(torch.cuda.current_stream())
     g = torch.cuda.CUDAGraph()
@@ -71,7 +66,7 @@ def test_many_launches_repeat_the_first_result():
 
 
 def test_two_streams_issue_decode_launches_concurrently():
-    # launches of two streams overlap on the device and share the placement table (different slots)
+    # launches of two streams overlap on the device
     a = _case(8, 14336, 4096, 11)
     b = _case(16, 18960, 2048, 13)
     outs = [torch.empty((c[1].shape[0], c[0].N), dtype=torch.float32, device="cuda") for c in (a, b)]
@@ -99,12 +94,9 @@ def test_two_streams_issue_decode_launches_concurrently():
 
 
 @pytest.mark.parametrize("shared_workspace", [False, True])
-def test_chain_of_two_kernel_variants_never_waits_out_a_placement_hold(shared_workspace):
+def test_alternating_launches_with_and_without_a_k_cut(shared_workspace):
     # A chain that alternates a launch without a K cut (many output channels) and one with K cut
-    # into chunks (few output channels) runs two instantiations of the decode kernel back to back,
-    # each launch overlapping the next one's start.  Their placement slots must differ: when both
-    # drew the same slot, candidates of one launch counted into the other's table and now and then
-    # sat out the full hold limit (200 us), and worker indices could go missing.
+    # into parts (few output channels), each launch overlapping the next one's start.
     H, F, M = 4096, 14336, 1
     mk = lambda N, K, seed: binding.prepack_weight(
         *binding.quantize_weight_rtn(torch.from_numpy(inputs.make_weight(N, K, 0.02, seed)).cuda(), symmetric=True))
@@ -138,8 +130,7 @@ def test_chain_of_two_kernel_variants_never_waits_out_a_placement_hold(shared_wo
     for _ in range(60):
         g.replay()
     torch.cuda.synchronize()
-    # what must hold whatever the placement did: no bounded wait ran out, every row range of every
-    # launch was computed exactly once (a lost worker index leaves stale rows behind)
+    # no bounded wait ran out, every row of every launch was computed
     assert binding.query_device_status() == 0
     ya2, yb2 = ya.clone(), yb.clone()
     ya.fill_(7.0)
@@ -150,9 +141,8 @@ def test_chain_of_two_kernel_variants_never_waits_out_a_placement_hold(shared_wo
     assert torch.equal(ya2, first[0]) and torch.equal(yb2, first[1])
 
 
-def test_launches_without_a_workspace_use_the_library_table_and_agree():
-    # No (or too small a) workspace: the placement state is an entry of the library's own table and K
-    # is never cut.  Results: equal bit for bit to the workspace path where that does not cut K
+def test_launches_without_a_workspace_agree():
+    # No (or too small a) workspace: K is never cut.  Results: equal bit for bit to the workspace path where that does not cut K
     # either (many output channels), within the output gate where it does (few output channels).
     tiny = torch.zeros((16,), dtype=torch.uint8, device="cuda")
     for M, N, K, cuts_k in ((4, 14336, 4096, False), (2, 4096, 14336, True)):

@@ -86,10 +86,12 @@ def _w8a8():
 
 SM, TI, CA = binding.FMT_TILED_SIGNMAG, binding.FMT_TILED, binding.FMT_CANONICAL
 CASES = {
-    "split-N, candidates": lambda: _linear(8, 14336, 4096, SM),
-    "split-N, K cut": lambda: _linear(8, 4096, 14336, TI),
+    "runs of rows": lambda: _linear(8, 14336, 4096, SM),
+    "runs of rows, K cut": lambda: _linear(8, 4096, 14336, TI),
+    "runs of rows, half an SM": lambda: _linear(8, 14336, 1536, SM),
+    "runs of rows, half an SM, K cut": lambda: _linear(8, 4096, 4096, TI),
     "whole tiles, 128 tokens, wide layer": lambda: _linear(100, 28672, 2048, TI),
-    "split-N, 128 tokens": lambda: _linear(100, 28672, 8192, SM),
+    "runs of rows, 128 tokens": lambda: _linear(100, 28672, 8192, SM),
     "cluster, 64 tokens": lambda: _linear(40, 4096, 14336, SM),
     "K cut between CTAs, 128 tokens, generic": lambda: _linear(130, 1024, 14336, TI),
     "K cut between CTAs, 128 tokens": lambda: _linear(300, 1024, 14336, SM),

@@ -104,7 +104,7 @@ def test_gaussian_inputs_within_gates(M, N, K, asym, pc):
                                    (300, 640, 8192), (100, 512, 8192), (65, 4096, 4096), (128, 14336, 1024)])
 def test_persistent_kernel_split_tiles_and_reuse_of_workspace(M, N, K):
     # shapes whose tiles are split between CTAs in many ways (several CTAs per tile in the persistent kernel, K
-    # chunks in the split-N kernel with 16-token tiles, clusters of two to eight CTAs per tile); the workspace is shared by
+    # parts in linear_rows_kernel up to sixteen tokens, clusters of two to eight CTAs per tile); the workspace is shared by
     # consecutive calls (the kernel leaves its counters zeroed) and results repeat bit for bit
     x8, s_x, wq = _gaussian_case(M, N, K, seed=M * 3 + N + K)
     w8 = oracle.dequant_weight(*wq[:3])
@@ -130,7 +130,7 @@ def test_persistent_kernel_split_tiles_and_reuse_of_workspace(M, N, K):
     else:
         persistent = M > 128
         n_counter_bytes = 8 * ((M + 255) // 256) * ((N + 127) // 128) if persistent else 1024
-        # tile counters (persistent kernel: start of the 64 KB control area; split-N: its last 2 KB) are back to zero
+        # tile counters (persistent kernel: start of the 64 KB control area; linear_rows_kernel: its last 2 KB) are back to zero
         first = 0 if persistent else 65536 - 2048
         assert np.all(ws[first:first + n_counter_bytes].cpu().numpy() == 0)
 
@@ -362,19 +362,19 @@ def test_canonical_calls_without_a_workspace_where_none_is_used(M, N, K):
     assert worst <= 2e-3, worst
 
 
-@pytest.mark.parametrize("M,N,K,register_kernel", [(16, 6144, 2048, False), (16, 8192, 1024, False), (10, 4096, 1024, False),
+@pytest.mark.parametrize("M,N,K,small_kernel", [(16, 6144, 2048, False), (16, 8192, 1024, False), (10, 4096, 1024, False),
                                                    (9, 4096, 1024, True), (8, 2048, 2048, True)])
-def test_host_forward_on_pinned_buffers_leaves_large_outputs_to_the_split_n_kernel(M, N, K, register_kernel):
-    # The kernel for small layers writes smaller pieces over the bus: 24 us host to host at (16, 6144, 2048), 19 us with the
-    # split-N kernel.  The latter cuts K here and leaves its partial sums behind the workspace's 64 KB of control data; the
-    # former does not touch the workspace.
+def test_host_forward_on_pinned_buffers_leaves_large_outputs_to_the_kernel_that_writes_rows(M, N, K, small_kernel):
+    # The kernel for small layers writes smaller pieces over the bus: 24 us host to host at (16, 6144, 2048), 19 us with one that
+    # writes rows.  linear_rows_kernel cuts K here and leaves its partial sums behind the workspace's 64 KB of control data;
+    # the kernels for small layers (of (9, 4096, 1024): whole tiles) do not touch the workspace.
     x8, s_x, wq = _gaussian_case(M, N, K, seed=6)
     xb = inputs.make_activation(M, K, 8, 0.01, 20.0)
     fw = binding.HostForward(M, binding.prepack_weight(*weights_to_dev(*wq)))
     y = fw(torch.from_numpy(xb.view(np.int16)).view(torch.bfloat16).pin_memory())
     torch.cuda.synchronize()
     assert binding.query_device_status() == 0
-    assert bool(fw.ws[65536:].any()) != register_kernel
+    assert bool(fw.ws[65536:].any()) != small_kernel
     ok, dist = bf16_gate(bf16_bits(y), oracle.forward(xb, *wq)["y64"])
     assert ok, dist
 

@@ -4,7 +4,7 @@ against a float32 product of the dequantized operands, which is exact enough to 
 was summed from stale or missing data).  A repeat on a USED workspace cannot show such an error: a
 kernel that reads partial sums too early finds the previous launch's identical values there.  (This
 is how a barrier-phase hazard in the expansion groups showed up: wrong sums in a few tiles of the
-first launch of a process only.)  Shapes: split-N with and without a
+first launch of a process only.)  Shapes: runs of rows with and without a
 K cut, the cluster plan (K cut between two to eight CTAs of a cluster, with a ragged last tile, with as few as
 two k-blocks per CTA, with the largest number of clusters that fits), whole tiles of the persistent kernel, CTA pairs; every
 arrangement for more than 128 tokens is in test_gpu_prefill_arrangements.py."""
@@ -49,7 +49,7 @@ def test_fresh_workspace_launches_agree_and_are_right(M, N, K):
 
 
 def test_one_workspace_shared_by_layers_of_different_shapes_and_kernels():
-    # One workspace of the largest size, used by calls of different shapes one after the other -- split-N
+    # One workspace of the largest size, used by calls of different shapes one after the other -- runs of rows
     # with and without a K cut, the persistent kernel with whole tiles and with several CTAs per tile, CTA
     # pairs: whatever a call leaves behind in the data part of the workspace, the next call's
     # counters must be zero.  Every result must equal the one computed on a fresh workspace of its own.
@@ -74,9 +74,8 @@ def test_one_workspace_shared_by_layers_of_different_shapes_and_kernels():
             assert torch.equal(got.view(torch.int32), own.view(torch.int32))
     torch.cuda.synchronize()
     assert binding.query_device_status() == 0
-    # the control area is left zero-filled (but for the generation word of the split-N kernel's placement state,
-    # in its last kilobyte)
-    assert bool((shared[:65536 - 1024] == 0).all())
+    # the control area is left zero-filled
+    assert bool((shared[:65536] == 0).all())
 
 
 @pytest.mark.parametrize("M,N,K,pad", [(16, 4096, 14336, 8), (128, 4096, 4096, 8), (100, 512, 8192, 8), (300, 640, 8192, 8),
