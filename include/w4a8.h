@@ -401,7 +401,8 @@ int w4a8_quantize_weight_rtn(const float* W, int64_t N, int64_t K, int group, in
 
 /*
  * The layer Hessian the quantizer works with (Sec. 3.1; prepared as in Sec. 3.3): H = X^T X over the T
- * calibration tokens of the layer's input X (device BF16 [T][ldx]), FP32 sums, written as a full
+ * calibration tokens of the layer's input X (device BF16 [T][ldx]), FP32 sums (in an order that is the
+ * same on every call, but may change between versions), written as a full
  * symmetric matrix (device float [K][K]); accumulate != 0 adds to what H holds (batches of tokens).
  * Its diagonal is what w4a8_gar_permutation ranks by.  K <= 32768.
  */
@@ -443,12 +444,17 @@ int w4a8_gar_permutation(const float* hdiag, int64_t K, int group, int32_t* perm
  *         preparation are w4a8_hessian_accumulate / w4a8_hessian_prepare; the two factorizations
  *         in between (inverse, Cholesky) are a library matter and the caller's.
  *   perm  device int32 [K] from w4a8_gar_permutation, or NULL for the original order.  Every run
- *         of 128 positions must hold the columns of one original group (not checked on the device).
+ *         of 128 positions must hold the columns of one original group, and every group be there once
+ *         (not checked on the device: the outputs of another order are undefined, and the call may run
+ *         into its time limit).
  *   symmetric / per_channel   as in w4a8_quantize_weight_rtn (gzero may be NULL when symmetric).
  *   mse_steps  0 or 1: Eq. 8 as is; 2..11: that many shrink factors 1, 0.98, 0.96, ... are tried.
  *   workspace  device, 16-byte aligned, w4a8_dpq_workspace_bytes(N, K) bytes (scratch).
  * Every step that decides a code is a single correctly rounded fp32 operation, so the codes are
- * reproducible and independent of the launch geometry.  Enqueues about K / 128 kernels.
+ * reproducible and independent of the launch geometry.  Enqueues three kernels (per tensor, a fill as
+ * well).  The last one's blocks wait for one another's results, with a time limit; while it runs, marks of its progress stand in
+ * codes and gscale.  If a wait gives up (w4a8_query_device_status returns W4A8_ERR_TIMEOUT) codes, gscale and gzero of the
+ * call are incomplete, marks among them, and must not be used.
  */
 size_t w4a8_dpq_workspace_bytes(int64_t N, int64_t K);
 int w4a8_dpq_quantize(const float* W, int64_t N, int64_t K, int group, const float* U, const int32_t* perm,

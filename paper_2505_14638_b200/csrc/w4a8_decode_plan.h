@@ -90,7 +90,7 @@ inline bool whole_tiles_apply(int64_t M, int64_t N, int64_t K, int fmt, int sms,
 }
 
 // 17..128 tokens: whether cutting the tiles' K between the CTAs of clusters of `cl` pays for the exchange of the partial sums: the
-// k-blocks that a CTA is spared against what grows with the tokens.  Fitted to 400 shapes of up to 9472 channels (see whole_tiles_apply);
+// k-blocks that a CTA is spared against what grows with the tokens.  Fitted to 400 shapes of up to 9472 channels;
 // against linear_rows_kernel, us: (124, 7328, 512) 10.0 / 6.7, (112, 5600, 3584) 12.3 / 10.2, (20, 4096, 4096) 7.5 / 9.7, (20, 4096,
 // 14336) 12.6 / 24.9.
 inline bool cluster_kcut_pays(int64_t M, int64_t K, int cl) { return 50 * (K / 128) * (cl - 1) >= cl * (120 + 7 * M); }
@@ -135,7 +135,7 @@ inline int64_t make_direct_plan(int64_t N, int64_t K, int sms, DirPlan* plan) {
 
 // Layers at up to sixteen tokens for which the kernel above is the faster one: those of few weights, where its short start and
 // end count; its expansion does not keep up with larger ones (the FP8 fragments of its MMA are converted to 16 bits on the pipe that
-// expands), and a short K is better walked by one CTA per tile (whole_tiles_apply, with the same 1000 shapes).  Time, quantization
+// expands), and a short K is better walked by one CTA per tile (whole_tiles_apply, with the same shapes).  Time, quantization
 // and linear layer back to back, weights not in L2, this kernel / whole tiles / linear_rows_kernel, us:
 //   M <= 8   (1616, 512) 4.1 / 4.1 / 4.5, (1104, 1408) 4.4 / 5.4 / 7.1, (2160, 3328) 5.2 / 9.0 / 6.9, (7488, 2048) 7.5 / 6.7 / 7.7,
 //            (5968, 3968) 8.8 / 9.3 / 8.1, (4960, 8192) 15.4 / 20.0 / 11.2

@@ -7,7 +7,7 @@
 // U = upper Cholesky factor of the inverse Hessian in processing order.  Work is cut the way
 // GPTQ cuts it, in blocks of one group (128 columns).  Tasks of two kinds: 32 rows of a block are brought up to
 // date and quantized (group scale / zero-point, Eq. 8, optional search; the 128 columns in sequence); the errors
-// of a block or two are applied to 128 rows of a later column block, q ascending -- the same chain of fused
+// of up to eight blocks are applied to 128 rows of a later column block, q ascending -- the same chain of fused
 // multiply-adds, in the same order, that the column-by-column algorithm performs for each element.  One persistent
 // launch (dpq_kernel) takes the tasks in an order in which each follows those it waits for.
 // Every floating-point step that decides an integer is one explicitly rounded fp32 operation
@@ -528,7 +528,7 @@ __device__ __forceinline__ bool dpq_block_rows(uint8_t* sm, uint32_t sm_addr, fl
         load_err(1);
         dpq_commit();
     }
-    // The errors of the previous block first (the trailing CTAs of the previous launch left this block out): a
+    // The errors of the previous block first (the tasks that apply errors leave those to the block's own): a
     // warp takes its four rows, a lane four consecutive columns of each, so that U is read once per four rows.
     {
         const int64_t r0 = rows32 * kDpqRowsPerCta + 4 * warp;
@@ -802,8 +802,9 @@ __device__ __forceinline__ bool dpq_block_rows(uint8_t* sm, uint32_t sm_addr, fl
 // Bound by the FP32 pipes for large layers, by the chain of a block for small ones.  No CTA has to be resident for another to make
 // progress: a task waits for tasks of earlier tickets only, which running CTAs hold; any number of calls can share the device.
 // Measured, us per layer, a launch per step (whose CTAs start and drain together, with cp.async by all threads and two blocks' errors
-// at a time) / this: (N, K) = (256, 1024) 264 / 263, (256, 4096) 880 / 840, (1024, 2048) 552 / 487, (2048, 2048) 616 / 505, (4096,
-// 4096) 2390 / 2070, (8192, 8192) 14560 / 11950, (4096, 14336) 21200 / 16900 = 25 T FMA/s.  Of the last: order and waits 21200 -> 19800, tile
+// at a time) / this, search of six steps: (N, K) = (256, 1024) 266 / 263, (1024, 2048) 558 / 484, (2048, 2048) 683 / 537, (4096,
+// 4096) 2384 / 2064, (8192, 8192) 14550 / 12020, (4096, 14336) 21190 / 17000 = 25 T FMA/s; none: (256, 4096) 880 / 833, (2048, 2048)
+// 613 / 502, (4096, 14336) 20910 / 16740.  Of the last: order and waits 21200 -> 19800, tile
 // loads three stages ahead -> 17850, panels of up to eight blocks -> 16870.  A tile's loop runs at 85 % of the pipe; what is left is
 // the start and the end of tiles (13000 cycles of some 95000 at two blocks, 4 % at eight) and the tasks of the blocks, 14 % of the places.
 __global__ void __launch_bounds__(kDpqThreads, 2)

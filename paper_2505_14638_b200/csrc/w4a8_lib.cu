@@ -1568,7 +1568,7 @@ int w4a8_dpq_quantize(const float* W, int64_t N, int64_t K, int group, const flo
     steps.slots = (int)slots;
     steps.b = -1;
     // One CTA per SM where a step's tiles do not keep two busy: the chain of a block, which is what counts then, has the SM for itself.
-    // (2048, 2048) 597 us with two, 539 with one; (1024, 2048) 592 and 514.
+    // Search of six steps: (2048, 2048) 636 us with two, 537 with one; (1024, 2048) 533 and 484; but (256, 4096) without 806 and 833.
     const int64_t nb = (N + kDpqRowsPerCta - 1) / kDpqRowsPerCta, tiles = row_tiles * steps.G;
     const int64_t most = tiles <= slots ? slots / 2 : slots, useful = nb + (tiles <= slots ? tiles / 2 : tiles);
     cfg.gridDim = dim3((unsigned)(useful < most ? useful : most));

@@ -82,7 +82,8 @@ struct SkCfg {
     // Expansion with ordinary shifts and sums instead of the multipliers (see SignMagLut): a step is paced by its MMAs, barriers and the
     // latency of a row's expansion, not by the integer pipe.  us with the multipliers / so, zero-points: (256, 1584, 2432) 8.59 / 8.17,
     // (512, 4096, 4096) 16.4 / 15.5, (1100, 2048, 6016) 22.0 / 20.7, 17..128 tokens 0.6 % less on average; sign-magnitude: (384,
-    // 4096, 4096) 13.8 / 13.2, (250, 6144, 4096) 13.1 / 12.8, but clusters 0.3 % more on average.
+    // 4096, 4096) 13.8 / 13.2, (250, 6144, 4096) 13.1 / 12.8.  In clusters it makes no difference (250 shapes, each twice: 0.2 % more, with
+    // the quantization 0.0).
     static constexpr bool kPlain = FMT_ == kFmtTiled || (FMT_ == kFmtTiledSignMag && !CL_);
     static constexpr int kMeta = meta_bytes(FMT);
     static constexpr int kCodeBytes = 8192;   // packed codes of the tile's rows for one k-block

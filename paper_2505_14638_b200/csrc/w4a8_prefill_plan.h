@@ -88,9 +88,9 @@ enum PrefillKind {
 struct PlanCost {
     double step, drain, fixed, full, least;
 };
-// Sign-magnitude and generic format.  (The latter's were fitted when its expansion took twice the instructions it takes now.  With
-// every arrangement timed again at 354 shapes they choose 1.8 % above the fastest on average, a refit 2.2 %: two runs of one differ
-// by 5 %.  That was before SkCfg::kPlain took 2 to 6 % off its whole tiles.)
+// Sign-magnitude and generic format.  (The latter's were fitted when its expansion took twice the instructions it takes now.  Timed
+// again with every arrangement, 200 shapes, each 30 ms warm, they choose 2.5 % above the fastest of the eight on average, 1.18 times at
+// worst, where two timings of one arrangement lie up to 14 % apart.)
 constexpr PlanCost kPlanCost[2][kPrefillKinds] = {
     {
         {0.373, 3.16, 2.71, 0.19, 0.00},    // pairs, 256 x 256
