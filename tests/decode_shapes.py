@@ -21,7 +21,7 @@ SHAPES = {
         (8, 1008, 2304, True), (8, 4880, 640, True), (8, 3328, 640, False), (16, 2160, 1024, True), (13, 2304, 1664, True),
         (16, 4080, 2688, False), (16, 4080, 2944, True), (5, 4864, 3072, False),
         (8, 13184, 512, True), (16, 16000, 384, False),                  # more tiles than half the SMs
-        (32, 18944, 1024, True), (33, 18944, 2432, True), (128, 18944, 3072, False),
+        (32, 18944, 1024, True), (33, 18944, 2432, True), (128, 18944, 3072, False), (65, 18944, 2304, True), (65, 18944, 2304, False),
         (17, 18960, 256, False), (124, 37904, 2048, True),               # more tiles than SMs
         (128, 9472, 2944, True), (17, 640, 1280, False),                 # few tiles, short K
         (120, 2048, 2944, False), (128, 7664, 5120, False)],             # few tiles, clusters do not pay

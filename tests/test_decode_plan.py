@@ -10,6 +10,7 @@ import pytest
 
 from paper_2505_14638_b200 import build
 from decode_shapes import KINDS, RESIDENT, SHAPES, SMS
+from test_gpu_rows import ROWS as ROWS_FULL, ROWS_HALF, ROWS_SIGNMAG
 
 NONE, DIRECT, WHOLE, CLUSTER, ROWS, HALF = range(6)
 TILED, SIGNMAG = 1, 2
@@ -115,6 +116,12 @@ def test_shapes_of_the_gpu_tests_take_the_kernels_they_stand_for(lib, kind):
         assert (1, 4, 4, False, False) in rings and {r[3:] for r in rings} == {(True, False), (False, False), (False, True)}
     if kind == "rows_half":
         assert {r[3:] for r in rings} == {(True, False), (False, False), (False, True)}
+
+
+@pytest.mark.parametrize("fmt", [SIGNMAG, TILED])
+def test_the_shapes_of_rows_take_rows(lib, fmt):
+    for want, shapes in ((ROWS, ROWS_FULL), (HALF, ROWS_HALF), (ROWS if fmt == SIGNMAG else WHOLE, ROWS_SIGNMAG)):
+        assert [(s, _route(lib, *s, fmt)[0]) for s in shapes] == [(s, want) for s in shapes]
 
 
 def test_without_a_workspace_k_is_not_cut(lib):
