@@ -86,7 +86,7 @@ inline bool whole_tiles_apply(int64_t M, int64_t N, int64_t K, int fmt, int sms,
         return K <= (M <= 32 ? 1024 : (sm ? 2432 : 3072));
     }
     if (M > 16) return 100 * (K / 128) <= 800 + 12 * M;
-    return K <= (N < 1024 ? 2304 : (4 * tiles > sms ? 3072 : (sm ? 2944 : 2688)));
+    return K <= (N < 1024 ? 2304 : (sm ? 2944 : 2688));
 }
 
 // 17..128 tokens: whether cutting the tiles' K between the CTAs of clusters of `cl` pays for the exchange of the partial sums: the
@@ -133,7 +133,7 @@ inline int64_t make_direct_plan(int64_t N, int64_t K, int sms, DirPlan* plan) {
     return best;
 }
 
-// Layers at up to sixteen tokens for which the kernel above is the faster one: those of few weights, where its short start and
+// Layers at up to sixteen tokens for which linear_direct_kernel is the faster one: those of few weights, where its short start and
 // end count; its expansion does not keep up with larger ones (the FP8 fragments of its MMA are converted to 16 bits on the pipe that
 // expands), and a short K is better walked by one CTA per tile (whole_tiles_apply, with the same shapes).  Time, quantization
 // and linear layer back to back, weights not in L2, this kernel / whole tiles / linear_rows_kernel, us:
@@ -206,17 +206,20 @@ inline void make_rows_plan(int64_t M, int64_t N, int64_t K, int sms, bool may_cu
 //   more 128-channel tiles than half the SMs, K up to 1664 0.94, 0.73, to 2048 0.97, 0.80, to 3072 1.22, 0.88, to 6144 1.43, 0.93
 //   K cut, k-blocks of a part: up to 8, M <= 12 0.98, 0.91; 13..16 1.08, 1.05
 //                              9 or 10, M <= 4 1.00, 0.90; 5..12 1.05, 0.89
-//                              11 to 14, M <= 4 1.03, 0.90 (11 of K up to 4352 0.95, 0.92); 5..12 1.14, 0.92
+//                              11 to 14, M <= 4 1.03, 0.90 (11 of K up to 4352 0.95, 0.92, but see below); 5..12 1.14, 0.92
 //                              more, M <= 4 1.22, 0.93; 5..12 1.26, 0.92
 // us: (8, 4096, 4096) 7.6, 6.0 / 7.7, 7.6, (9, 4400, 3072) 7.2, 5.6 / 7.5, 7.5, (1, 5344, 3328) 7.3, 6.5 / 8.0, 7.4, (2, 13712, 1920) 6.7,
-// 5.0 / 7.1, 6.6; (8, 6144, 4096), 11 k-blocks, 8.9, 7.3 / 8.5, 7.9, (8, 4096, 14336), 28, 16.2, 10.2 / 12.5, 11.9.  With many parts of a
-// very long K more than four tokens lose as well, (8, 1296, 12288) 8.8, 7.1 / 8.3, 7.3.  (Between launches that take whole SMs nothing
-// starts beside these either: a block of qkv, o, gate_up and down with 8 tokens, o here, takes 51.2 us, o on whole SMs 50.7.)
+// 5.0 / 7.1, 6.6; (8, 6144, 4096), 11 k-blocks, 8.9, 7.3 / 8.5, 7.9, (8, 4096, 14336), 28, 16.2, 10.2 / 12.5, 11.9.
+// Between launches that take whole SMs nothing starts beside these either.  Layers of 4096 channels, with a quantization per input, from a graph, all on whole SMs / so, us: q, k and v
+// of 4096 and 1024 channels with 8 tokens 16.5 / 15.7; qkv, o, gate_up and down with 8 tokens, o here, 49.7 / 48.9 (called one by one 50.7 /
+// 51.2), with q, k, v, gate and up apart 60.7 / 61.7; but qkv (11 k-blocks) here with 1 token 46.3 / 48.4, with 4 48.4 / 49.6.
+// Hence not for a K of more than 6144, which down projections have, one layer per input: 2048 wide with 8192 between, 8 tokens, down here
+// 26.5 / 28.1; nor more channels than half the SMs' tiles and K of 2048: the same block's gate_up here with 16 tokens 30.9 / 32.9.
 inline bool half_rows_apply(int64_t M, int64_t N, int64_t K, int sms, bool may_cut) {
     if (M > 16) return false;
-    if (2 * ((N + 127) / 128) > sms) return K <= 2048;
+    if (2 * ((N + 127) / 128) > sms) return K <= 1664;
     const int64_t cut = rows_cut(N, K, sms, may_cut), blocks = (K / 128 + cut - 1) / cut;
-    return cut > 1 && (M <= 4 ? blocks <= (K <= 4352 ? 11 : 10) : (M <= 12 && blocks <= 8 && K <= 12000));
+    return cut > 1 && K <= 6144 && (M <= 4 ? blocks <= 10 : (M <= 12 && blocks <= 8));
 }
 
 enum DecodeKind {

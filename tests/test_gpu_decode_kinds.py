@@ -31,7 +31,7 @@ def test_both_sides_of_the_limits_between_kernels(kind, M, N, K, symmetric):
     assert torch.equal(yb, outs[0].to(torch.bfloat16))
 
 
-@pytest.mark.parametrize("M,N,K,asym", [(8, 4096, 3840, False), (3, 4128, 4864, True), (12, 1040, 8320, False), (1, 5248, 3200, True)])
+@pytest.mark.parametrize("M,N,K,asym", [(8, 4096, 3840, False), (3, 4128, 4864, True), (12, 1008, 5760, False), (1, 5248, 3200, True)])
 def test_launches_that_share_sms_share_a_workspace_in_turn(M, N, K, asym):
     # CTAs of half an SM, K cut: a launch starts beside the one before and uses the same counters and partial sums
     x8, s_x, tw, ref, mag = _layer(M, N, K, asym)

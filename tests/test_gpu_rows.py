@@ -14,15 +14,15 @@ pytestmark = pytest.mark.gpu
 
 # What w4a8_linear takes linear_rows_kernel for on 148 SMs (test_decode_plan.py holds decode_choice to it): CTAs of whole SMs,
 ROWS = [
-    (1, 18944, 2176), (16, 18960, 2304), (8, 37888, 2176), (3, 37904, 2304),      # 128 / 136 / 256 rows a run, two runs a CTA
+    (1, 18944, 2176), (16, 18960, 2304), (8, 37888, 1792), (3, 37904, 1920),      # 128 / 136 / 256 rows a run, two runs a CTA
     (17, 9488, 4224), (64, 19216, 2176), (65, 18944, 3200), (128, 28688, 2176), (100, 37904, 2304),
     (128, 18944, 3200),                                    # with zero-points as many stages as groups in both rings
-    (16, 1552, 14336), (13, 1024, 8320), (1, 4096, 5760), (12, 9472, 3456), (14, 128, 4096), (16, 16, 4224)]   # K cut
+    (16, 1552, 14336), (13, 1024, 8320), (1, 4096, 5760), (12, 9472, 3456), (9, 1024, 8320), (14, 128, 4096), (16, 16, 4224)]   # K cut
 # ... with zero-points whole tiles take their place (few tiles, K not cut),
 ROWS_SIGNMAG = [(128, 7664, 3072), (44, 6384, 1792)]
 # and CTAs of half an SM, the first four with K cut.
-ROWS_HALF = [(9, 1024, 8320), (12, 4400, 3200), (2, 128, 4096), (4, 16, 4224), (1, 9488, 640), (16, 18960, 1408), (5, 37904, 896),
-             (8, 37888, 1792), (3, 37904, 1920)]
+ROWS_HALF = [(9, 1008, 5888), (12, 4400, 3200), (2, 128, 4096), (4, 16, 4224), (1, 9488, 640), (16, 18960, 1408), (5, 37904, 896),
+             (8, 37888, 1664)]
 
 
 def _layer(M, N, K, asym):
